@@ -231,10 +231,11 @@ int sam_batch_dump(sam_batch_t* b, int32_t slot, int32_t* n_tokens, int32_t* n_s
 /* Pool occupancy: slabs in the pool, slabs currently free.  Synchronous. */
 int sam_batch_pool_info(sam_batch_t* b, int64_t* total_slabs, int64_t* free_slabs, void* stream);
 
-/* Number of kernels one sam_step launches for this batch: 1, or 2 for a batch larger than the GPU holds
- * at once (a small kernel first orders the slots so that those with the most tokens start first; the
+/* Number of kernels one decoding step (sam_step) launches for this batch: 1, or 2 for a batch larger than the GPU
+ * holds at once (a small kernel first orders the slots so that those with the most tokens start first; the
  * step's results do not depend on it).  sam_step_host, being synchronous, gains nothing from the order
- * when its kernel works on the host arrays in place, and then makes one launch whatever the batch.
+ * when its kernel works on the host arrays in place, and then makes one launch whatever the batch.  A step
+ * whose rows can hold a prompt (stride of 48 and more) makes two: prompts that fill an empty slot, then the rest.
  * Returns a negative sam_err_t for a null handle. */
 int sam_batch_launches_per_step(const sam_batch_t* b);
 

@@ -23,9 +23,10 @@
 //   - runs of tokens that repeat a passage of the sequence and make every Expand clone are extended by
 //     the lanes in parallel as well: the states the clones are made from are guessed (position -> state
 //     map, or ids two apart), read in one round trip and checked (dyn_repeat_run);
-//   - a static match that sits in the state of a whole corpus prefix is advanced by comparing the step's
-//     tokens with the corpus, its state read from the corpus' position -> state array (a prefix state's
-//     transition on the next corpus token always leads to the next prefix state);
+//   - the static match is not advanced token by token: all suffixes of the row are walked side by side, and a
+//     match that goes on as the corpus does is taken in one round (static_match.cuh);
+//   - a prompt that fills an empty slot is not extended token by token either: its automaton is built at once by all
+//     threads of a block (prefill_build.cuh, sam_prefill_kernel);
 //   - when the batch is larger than the GPU holds at once, the slots with the most tokens are started
 //     first (order_slots_kernel);
 //   - from 8192 slots on the two sides of a slot run as separate one-warp blocks (the static side of a slot
@@ -69,6 +70,13 @@ __device__ __forceinline__ void flush_counts(int slot, int lane, bool is_static,
 #endif
 }
 constexpr int MAX_DRAFT_REGS = 4;     // 4 x 32 lanes = 128 draft tokens
+
+}  // namespace
+
+#include "static_match.cuh"
+#include "prefill_build.cuh"
+
+namespace {
 
 struct StepArgs {
     SamStaticView S;
@@ -133,52 +141,6 @@ __device__ __forceinline__ int cut_at_stop(int32_t d[MAX_DRAFT_REGS], int dl, in
 #pragma unroll
     for (int r = 0; r < MAX_DRAFT_REGS; r++) if (r * 32 + lane >= dl) d[r] = -1;
     return dl;
-}
-
-// ------------------------------------------------------------------ static side
-// Transfer (Algorithm 1) for one token.  (s, sf, l): state, its F bit, match length.
-// root_e is root_row[t], fetched beforehand.  If have_rec, (pa, pb) is the record of s, read earlier;
-// if have_ent, pent is this lane's entry of the home bucket of (s, t), read earlier.
-__device__ __forceinline__ void static_transfer(const SamStaticView& S, uint32_t& s, uint32_t& sf, int32_t& l,
-                                                uint32_t t, uint32_t root_e, int lane, int& err,
-                                                bool have_rec, uint4 pa, uint4 pb, bool have_ent, uint4 pent, ChainCounts& kc) {
-    int guard = l + 2;                       // at most l link moves
-    bool len_from_rec = false;
-    for (;;) {
-        if (s == 0) {                        // at the root the match length is 0
-            if (root_e != SAM_NONE) { s = root_e & SAM_IDMASK; sf = root_e >> 31; l = 1; SAM_COUNT(kc.b, 1); }
-            else l = 0;
-            return;
-        }
-        uint32_t home = sam_hash2(s, t) & S.hash_mask;
-        uint4 ent = make_uint4(SAM_NONE, 0, 0, 0);
-        if (sf) ent = have_ent ? pent : __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + (lane & 7));
-        have_ent = false;
-        uint4 a = pa, b = pb;
-        if (!have_rec) { a = __ldg(S.rec + 2 * (size_t)s); b = __ldg(S.rec + 2 * (size_t)s + 1); SAM_COUNT(kc.rounds, 1); }
-        have_rec = false;
-        if (len_from_rec) { l = (int32_t)a.x; len_from_rec = false; }
-        uint32_t tgt = SAM_NONE;
-        if (a.w >= 1 && b.x == t) tgt = b.y;
-        else if (a.w >= 2 && b.z == t) tgt = b.w;
-        else if (a.w > 2) {
-            if (!sf) { ent = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + (lane & 7)); SAM_COUNT(kc.rounds, 1); }
-            for (int probe = 1;; probe++) {
-                unsigned hit = __ballot_sync(FULL, ent.x == s && ent.y == t);
-                if (hit) { tgt = __shfl_sync(FULL, ent.z, __ffs(hit) - 1); break; }
-                unsigned empty = __ballot_sync(FULL, ent.x == SAM_NONE);
-                if (empty || probe >= S.hash_max_probe) break;
-                home = (home + 1) & S.hash_mask;
-                ent = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + (lane & 7));
-                SAM_COUNT(kc.rounds, 1);
-            }
-        }
-        if (tgt != SAM_NONE) { s = tgt & SAM_IDMASK; sf = tgt >> 31; l += 1; SAM_COUNT(kc.b, 1); return; }
-        SAM_COUNT(kc.a, 1);
-        s = a.y & SAM_IDMASK; sf = a.y >> 31;            // s <- link(s), l <- len(link(s))
-        if (s == 0) l = 0; else len_from_rec = true;
-        if (--guard < 0) { err = SAM_SEQ_WALK_LIMIT; return; }
-    }
 }
 
 // ------------------------------------------------------------------ dynamic side
@@ -751,7 +713,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
     return r;
 }
 
-// The static side of one slot's step, run by one warp: Transfer (Algorithm 1) for each of the slot's m
+// The static side of one slot's step, run by one warp: the state Transfer (Algorithm 1) reaches over the slot's m
 // tokens, then the static words of the control block.  cw holds control words 0..31 as read at the start
 // of the step; on entry (ra, rb) is the copy of the match state's record kept in the control block, ntok0
 // the text length before the step.  On exit (s, sf, l) is the match state, and, if l > 0 and no error,
@@ -766,106 +728,56 @@ __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane,
     ChainCounts kc = {1, 0, 0, 0, 0};                    // one round already: the control words
     uint32_t s = __shfl_sync(FULL, cw, CB_S1), sf = __shfl_sync(FULL, cw, CB_S1FLAG);
     int32_t l = (int32_t)__shfl_sync(FULL, cw, CB_L1);
-    bool have = s != 0;
-    // The match state is the state Build-SAM created for a whole corpus prefix (len == min_endpos:
-    // not a clone), the prefix ending at e.  Its transition on the next corpus token was created
-    // solid (len + 1) and a solid transition is never redirected, so it still leads to the state of
-    // the prefix one longer, with match length l + 1.  The state may occur more than once and have
-    // other transitions too ("ab" in "ababc"): nothing is assumed about those.  The step's tokens
-    // are compared with the corpus after e; as long as they agree the state is taken from the
-    // position -> state array, and the first token that differs goes through the ordinary Transfer
-    // below.  All in one round trip, in which the draft after e + m is requested as well in case
-    // every token agrees.
-    int j0 = 0;                      // tokens already taken
+#ifdef SAM_COUNTERS
+    ChainCounts tally = {0, 0, 0, 0, 0};                 // the moves Algorithm 1 itself makes over these tokens
+    {
+        uint32_t ts = s, tsf = sf; int32_t tl = l;
+        for (int j = 0; j < m && !err; j++)
+            static_transfer(A.S, ts, tsf, tl, (uint32_t)toks[j], __ldg(A.S.root_row + toks[j]), lane, err, false, ra, rb, tally);
+    }
+#endif
     bool drafted = false;
-    if (have && m >= 1 && m <= 32 && ra.x == ra.z) {
-        const int64_t e = (int64_t)ra.z;
-        int32_t cx = -2; uint32_t px = 0;
-        if (lane < m && e + lane < A.S.n_tokens) { cx = __ldg(A.S.corpus + e + lane); px = __ldg(A.S.pstate + e + lane); }
-        const int64_t e2 = e + m;
-        const int64_t room = A.S.n_tokens - e2;
-        const int dl2 = (int)(room < L ? (room < 0 ? 0 : room) : L);
-        if (DRAFT) gather_draft<1>(A.S.corpus, e2, dl2, L, lane, d);
-        const unsigned agree = __ballot_sync(FULL, lane < m && cx == tok_first);
-        j0 = (~agree) ? __ffs(~agree) - 1 : 32;
-        SAM_COUNT(kc.rounds, 1); SAM_COUNT(kc.b, j0);
-        if (j0 > 0) {
-            const uint32_t ref = __shfl_sync(FULL, px, j0 - 1);
-            s = ref & SAM_IDMASK; sf = ref >> 31; l += j0; have = false;
-            if (j0 == m) {                                  // the whole step: the draft is in already
-                ra = __ldg(A.S.rec + 2 * (size_t)s);        // its record, for the next step
-                rb = __ldg(A.S.rec + 2 * (size_t)s + 1);
-                if (DRAFT) my_dl = cut_at_stop(d, dl2, lane, A.W.stop_token);
-                drafted = true;
-            }
-        }
-    }
-    for (int base = 0; base < m && !err && j0 < m; base += 32) {
-        const int i = base + lane;
-        uint32_t tk = 0, re = SAM_NONE;
-        if (i < m) { tk = (uint32_t)(base == 0 ? tok_first : toks[i]); re = __ldg(A.S.root_row + tk); }
-        const int cnt = min(32, m - base);
+    if (m > 32) {
+        static_suffix(A.S, toks, m, lane, s, sf, l, ra, rb, err, kc);
+    } else if (m > 0) {
+        const uint32_t tk = (uint32_t)tok_first;
+        uint32_t re = SAM_NONE;
+        if (lane < m) re = __ldg(A.S.root_row + tk);
         SAM_COUNT(kc.rounds, 1);
-        // Most tokens end a short match: the lookup misses, the link leads to the root, and the
-        // root row gives the next state u = root_row[t].  The token after that is then looked up
-        // in u — a lookup whose address is known now.  Lookups k = 0..7 (state root_row[t_k],
-        // token t_{k+1}) are read ahead here, eight lanes each: the state's record in lanes 0-1
-        // of the group, its hash bucket in all eight.  They are used if the matcher really is
-        // in that state when the token comes.
-        uint4 sp_rec[2], sp_ent[2];
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
-            const int k = 4 * r + (lane >> 3), e = lane & 7;
-            const uint32_t uref = __shfl_sync(FULL, re, k);
-            const uint32_t tnext = __shfl_sync(FULL, tk, k + 1);
-            sp_rec[r] = make_uint4(0, 0, 0, 0);
-            sp_ent[r] = make_uint4(SAM_NONE, 0, 0, 0);
-            if (k + 1 < cnt && uref != SAM_NONE) {
-                const uint32_t u = uref & SAM_IDMASK;
-                if (e < 2) sp_rec[r] = __ldg(A.S.rec + 2 * (size_t)u + e);
-                if (uref >> 31)
-                    sp_ent[r] = __ldg(A.S.hash + (size_t)(sam_hash2(u, tnext) & A.S.hash_mask) * SAM_HASH_BUCKET + e);
+        // the match so far may take the tokens in one round (with the root row, and with the draft after the last of
+        // them where it is the corpus that goes on)
+        int i0 = 0;
+        bool have = s != 0, early = false;
+        int dl2 = 0;
+        if (have) {
+            if (DRAFT && ra.x == ra.z) {
+                const int64_t e2 = (int64_t)ra.z + m, room = A.S.n_tokens - e2;
+                dl2 = (int)(room < L ? (room < 0 ? 0 : room) : L);
+                gather_draft<1>(A.S.corpus, e2, dl2, L, lane, d);
+                early = true;
             }
+            i0 = static_run(A.S, s, sf, ra, rb, have, tk, m, lane, kc);
+            l += i0;
         }
-        for (int j = j0; j < cnt && !err; j++) {
-            bool pre = false;
-            uint4 pa = ra, pb = rb, pent = make_uint4(SAM_NONE, 0, 0, 0);
-            if (j >= 1 && j <= 8 && s != 0) {
-                const uint32_t prev = __shfl_sync(FULL, re, j - 1);
-                if (prev != SAM_NONE && (prev & SAM_IDMASK) == s) {        // the state read ahead
-                    const int k = j - 1, g8 = 8 * (k & 3);
-                    const uint4 xr = (k >> 2) ? sp_rec[1] : sp_rec[0];
-                    const uint4 xe = (k >> 2) ? sp_ent[1] : sp_ent[0];
-                    pa.x = __shfl_sync(FULL, xr.x, g8); pa.y = __shfl_sync(FULL, xr.y, g8);
-                    pa.z = __shfl_sync(FULL, xr.z, g8); pa.w = __shfl_sync(FULL, xr.w, g8);
-                    pb.x = __shfl_sync(FULL, xr.x, g8 + 1); pb.y = __shfl_sync(FULL, xr.y, g8 + 1);
-                    pb.z = __shfl_sync(FULL, xr.z, g8 + 1); pb.w = __shfl_sync(FULL, xr.w, g8 + 1);
-                    const int src = g8 + (lane & 7);
-                    pent.x = __shfl_sync(FULL, xe.x, src); pent.y = __shfl_sync(FULL, xe.y, src);
-                    pent.z = __shfl_sync(FULL, xe.z, src); pent.w = __shfl_sync(FULL, xe.w, src);
-                    pre = true;
-                }
-            }
-            static_transfer(A.S, s, sf, l, __shfl_sync(FULL, tk, j), __shfl_sync(FULL, re, j), lane, err,
-                            have || pre, pa, pb, pre, pent, kc);
-            have = false;
+        if (i0 < m) {
+            static_walks(A.S, tk, re, m, lane, s != 0, i0, have, s, sf, l, ra, rb, err, kc);
+        } else {
+            if (!have) static_record(A.S, s, ra, rb);
+            if (early) { my_dl = cut_at_stop(d, dl2, lane, A.W.stop_token); drafted = true; }
         }
     }
+#ifdef SAM_COUNTERS
+    kc.a = tally.a; kc.b = tally.b;
+#endif
     l_out = l; s_out = s; sf_out = sf;
-    if (l > 0 && !err) SAM_COUNT(kc.rounds, (m > 0 ? 1 : 0) + (DRAFT && !drafted ? 1 : 0));
+    if (l > 0 && !err) SAM_COUNT(kc.rounds, DRAFT && !drafted ? 1 : 0);
     flush_counts(b, lane, true, kc, m);
-    if (l > 0 && !err && !drafted) {
-        if (m > 0) {                                    // the state moved: read its record, keep a copy
-            ra = __ldg(A.S.rec + 2 * (size_t)s);
-            rb = __ldg(A.S.rec + 2 * (size_t)s + 1);
-        }
-        if (DRAFT) {
-            const int64_t e = (int64_t)ra.z;            // min_endpos
-            int64_t room = A.S.n_tokens - e;
-            my_dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
-            gather_draft<1>(A.S.corpus, e, my_dl, L, lane, d);
-            my_dl = cut_at_stop(d, my_dl, lane, A.W.stop_token);
-        }
+    if (DRAFT && l > 0 && !err && !drafted) {
+        const int64_t e = (int64_t)ra.z;                // min_endpos
+        int64_t room = A.S.n_tokens - e;
+        my_dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
+        gather_draft<1>(A.S.corpus, e, my_dl, L, lane, d);
+        my_dl = cut_at_stop(d, my_dl, lane, A.W.stop_token);
     }
     if (m > 0 && lane == 0 && !err) {
         cb[CB_S1] = s; cb[CB_L1] = (uint32_t)l; cb[CB_S1FLAG] = sf; cb[CB_NTOK_S] = ntok0 + (uint32_t)m;
@@ -973,6 +885,39 @@ __device__ __forceinline__ void signal_done(const StepArgs& A) {
     }
 }
 
+// Both warps' results are in shared memory: choose the source, write the slot's outputs.
+template <bool VERIFY>
+__device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp, int lane, uint32_t* cb, const int32_t* sh_l, const int32_t* sh_s,
+                                             const int32_t* sh_dl, const int32_t* sh_err, const int32_t d[MAX_DRAFT_REGS], int m, int confirmed) {
+    const int L = A.L;
+    const int any_err = sh_err[0] ? sh_err[0] : sh_err[1];
+    const int l1 = sh_l[0], l2v = sh_l[1];
+    const bool use_static = A.has_static && l1 > l2v + A.W.l_bias;        // Section 3.2
+    const int lsel = use_static ? l1 : l2v;
+    const int need = A.W.min_match > 1 ? A.W.min_match : 1;
+    const int src = (any_err || lsel < need) ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
+    const int winner = src == SAM_SRC_DYNAMIC ? 1 : 0;
+
+    if (warp == winner) {
+#pragma unroll
+        for (int r = 0; r < MAX_DRAFT_REGS; r++) {
+            int j = r * 32 + lane;
+            if (j < L) A.draft_tokens[(size_t)b * L + j] = (src == SAM_SRC_NONE) ? -1 : d[r];
+        }
+    }
+    if (warp == 0 && lane == 0) {
+        if (any_err) cb[CB_STATUS] = (uint32_t)any_err;
+        A.draft_len[b] = src == SAM_SRC_NONE ? 0 : sh_dl[winner];
+        A.match_len[2 * b] = any_err ? 0 : l1;
+        A.match_len[2 * b + 1] = any_err ? 0 : l2v;
+        A.source[b] = src;
+        if (A.state) { A.state[2 * b] = any_err ? 0 : sh_s[0]; A.state[2 * b + 1] = any_err ? 0 : sh_s[1]; }
+        A.status[b] = any_err;
+        if (VERIFY && A.v_counts_out) A.v_counts_out[b] = m;
+        if (VERIFY && A.v_accepted_out) A.v_accepted_out[b] = confirmed;
+    }
+}
+
 // ------------------------------------------------------------------ the kernel
 // VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
 template <bool VERIFY>
@@ -1030,6 +975,11 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
     const uint32_t ntok0 = __shfl_sync(FULL, cw, CB_NTOK);
     const int L = A.L;
     __syncthreads();          // both warps hold the slot's state as it was before either writes any of it
+
+    if (__shfl_sync(FULL, cw, CB_ERR_S) == SAM_STEP_DONE) {      // this step is done: sam_prefill_kernel took the slot
+        if (threadIdx.x == 0) { cb[CB_ERR_S] = 0; if (A.done_flag) signal_done(A); }
+        return;
+    }
 
     // validate the whole step before any state changes (both warps reach the same verdict)
     bool fresh_fail = false;
@@ -1099,36 +1049,65 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
 
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
     __syncthreads();
-    const int any_err = sh_err[0] ? sh_err[0] : sh_err[1];
-    const int l1 = sh_l[0], l2v = sh_l[1];
-    const bool use_static = A.has_static && l1 > l2v + A.W.l_bias;        // Section 3.2
-    const int lsel = use_static ? l1 : l2v;
-    const int need = A.W.min_match > 1 ? A.W.min_match : 1;
-    const int src = (any_err || lsel < need) ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
-    const int winner = src == SAM_SRC_DYNAMIC ? 1 : 0;
-
-    if (warp == winner) {
-#pragma unroll
-        for (int r = 0; r < MAX_DRAFT_REGS; r++) {
-            int j = r * 32 + lane;
-            if (j < L) A.draft_tokens[(size_t)b * L + j] = (src == SAM_SRC_NONE) ? -1 : d[r];
-        }
-    }
-    if (warp == 0 && lane == 0) {
-        if (any_err) cb[CB_STATUS] = (uint32_t)any_err;
-        A.draft_len[b] = src == SAM_SRC_NONE ? 0 : sh_dl[winner];
-        A.match_len[2 * b] = any_err ? 0 : l1;
-        A.match_len[2 * b + 1] = any_err ? 0 : l2v;
-        A.source[b] = src;
-        if (A.state) { A.state[2 * b] = any_err ? 0 : sh_s[0]; A.state[2 * b + 1] = any_err ? 0 : sh_s[1]; }
-        A.status[b] = any_err;
-        if (VERIFY && A.v_counts_out) A.v_counts_out[b] = m;
-        if (VERIFY && A.v_accepted_out) A.v_accepted_out[b] = confirmed;
-    }
+    step_outputs<VERIFY>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, d, m, confirmed);
     if (A.done_flag) {
         __syncthreads();
         if (threadIdx.x == 0) signal_done(A);
     }
+}
+
+// ------------------------------------------------------------------ prompts
+// Launched ahead of the step kernel when the step's rows are long enough to hold prompts.  An empty slot that is given
+// SAM_PREFILL_MIN tokens or more is done here, the rest of the slots by the step kernel that follows (a word of
+// the control block tells it which).  One block per slot: warp 0 finds the static match, the other warps
+// build the automaton of the whole text (prefill_build.cuh), and the first two warps read the drafts and write the outputs.
+// From how many tokens: the build takes 14 us for its shortest texts, one Expand after the other 0.3 to 0.5 us a token.
+constexpr int SAM_PREFILL_MIN = 48;
+
+__global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant__ StepArgs A) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    extern __shared__ __align__(16) unsigned char pb_smem[];
+    __shared__ PbShared sh;
+    __shared__ int32_t sh_l[2], sh_s[2], sh_dl[2], sh_err[2];
+    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
+    const int m = A.counts[b];
+    const uint32_t cw = cb[lane];
+    if (m < SAM_PREFILL_MIN || m > A.stride || m > PB_MAX || m > A.W.max_seq_len) return;
+    if (__shfl_sync(FULL, cw, CB_STATUS) != 0 || __shfl_sync(FULL, cw, CB_NTOK) != 0) return;
+    const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
+    const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
+    bool bad = false;
+    for (int j = threadIdx.x; j < m; j += blockDim.x) { const int t = toks[j]; bad |= t < 0 || t >= vocab; }
+    if (__syncthreads_or(bad)) return;                   // the step kernel reports it
+
+    const int L = A.L;
+    int32_t d[MAX_DRAFT_REGS] = {-1, -1, -1, -1};
+    int32_t my_l = 0, my_s = 0, my_dl = 0;
+    int err = 0;
+    if (warp == 0) {
+        if (A.has_static) {
+            uint32_t s, sf; int32_t l;
+            uint4 ra = make_uint4(0, 0, 0, 0), rb = ra;
+            static_chain<true>(A, b, lane, cb, 0u, 0, toks, m, 0u, ra, rb, s, sf, l, err, d, my_dl);
+            my_l = l; my_s = (int32_t)s;
+        }
+    } else {
+        PbResult r;
+        pb_build(A.W, b, cb, toks, m, pb_smem, sh, (int)threadIdx.x - 32, (int)blockDim.x - 32, r);
+        if (warp > 1) return;
+        err = r.err; my_l = r.l2; my_s = r.s2;
+        if (r.l2 > 0) {
+            my_dl = min(m - r.e2, L);
+            gather_draft<0>(A.W.text + (size_t)b * A.W.text_stride, r.e2, my_dl, L, lane, d);
+            my_dl = cut_at_stop(d, my_dl, lane, A.W.stop_token);
+        }
+    }
+    if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
+    asm volatile("bar.sync 2, 64;" ::: "memory");
+    step_outputs<false>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, d, m, 0);
+    if (threadIdx.x == 0) cb[CB_ERR_S] = SAM_STEP_DONE;
 }
 
 // ------------------------------------------------------------------ the split step (large batches)
@@ -1625,6 +1604,8 @@ constexpr int split_big_m(int batch) { return batch >= 8192 ? 8 : 5; }
 // and shared memory would hold only a dozen of them per SM.  Once per device.
 int split_kernel_setup(int device);
 
+int prefill_kernel_setup(int device);
+
 constexpr int SAM_SPLIT_MIN_BATCH = 8192;                    // the split step is used from this many slots on
 constexpr int SAM_ORDER_MIN_BATCH = 1536;                    // more slots than a B200 holds blocks of this kernel (148 x 10)
 
@@ -1641,6 +1622,28 @@ int split_kernel_setup(int device) {
         done[device] = true;
     }
     return SAM_OK;
+}
+// The build's shared memory, once per device.
+int prefill_kernel_setup(int device) {
+    static bool done[64];
+    if (device < 0 || device >= 64) return SAM_ERR_ARG;
+    if (!done[device]) {
+        cudaError_t e = cudaFuncSetAttribute(sam_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PB_MAX * PB_BYTES_PER_TOKEN);
+        if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
+        done[device] = true;
+    }
+    return SAM_OK;
+}
+
+// Shared memory and threads of a build for rows of up to `stride` tokens: a thread for four tokens where many
+// builds share an SM, for two where each has one to itself.
+void prefill_shape(int stride, int batch, size_t* smem, unsigned* threads) {
+    int n2 = 64;
+    while (n2 < stride && n2 < PB_MAX) n2 <<= 1;
+    int t = batch <= 296 ? n2 / 2 : n2 / 4;
+    t = t < 64 ? 64 : t > 992 ? 992 : t;
+    *smem = (size_t)n2 * PB_BYTES_PER_TOKEN;
+    *threads = (unsigned)(32 + t);
 }
 }  // namespace
 
@@ -1682,9 +1685,26 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     A.order = nullptr; A.split_count = nullptr;
+    A.n_warp_blocks = A.n_lane_blocks = 0;
+    bool prompts = false;
+#ifndef SAM_COUNTERS                                       // (the counters count Expand's own operations, one Expand at a time)
+    prompts = !v_draft && stride >= SAM_PREFILL_MIN;
+#endif
+    if (prompts) {
+        int rc = prefill_kernel_setup(b->device);
+        if (rc) return rc;
+        size_t smem; unsigned threads;
+        prefill_shape(stride, b->view.batch, &smem, &threads);
+        cudaLaunchConfig_t pc;
+        memset(&pc, 0, sizeof(pc));
+        pc.gridDim = dim3((unsigned)b->view.batch); pc.blockDim = dim3(threads); pc.dynamicSmemBytes = smem; pc.stream = stream;
+        pc.attrs = attr; pc.numAttrs = 1;
+        cudaError_t pe = cudaLaunchKernelEx(&pc, sam_prefill_kernel, A);
+        if (pe != cudaSuccess) { sam_set_cuda_error(pe); return SAM_ERR_CUDA; }
+    }
     // (A host-array step is synchronous: nothing runs before it that the ordering kernel could overlap with, so it
     // would cost more than the order saves; such a step is always the one two-warp launch, slots in their own order.)
-    if (!v_draft && !done_flag_dev && b->view.batch >= SAM_ORDER_MIN_BATCH) {
+    if (!v_draft && !prompts && !done_flag_dev && b->view.batch >= SAM_ORDER_MIN_BATCH) {
         int32_t* order = b->view.order + (size_t)(b->order_phase & 1) * b->view.batch;
         cudaLaunchConfig_t oc;
         memset(&oc, 0, sizeof(oc));
@@ -1706,7 +1726,6 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)b->view.batch); cfg.blockDim = dim3(64); cfg.dynamicSmemBytes = 0; cfg.stream = stream;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    A.n_warp_blocks = A.n_lane_blocks = 0;
     cudaError_t e;
     if (A.order && A.has_static && b->view.batch >= SAM_SPLIT_MIN_BATCH) {   // the two sides of a slot in different blocks
         int rc = split_kernel_setup(b->device);

@@ -1,0 +1,101 @@
+"""GPU: steps with prompts — the whole-text build of the dynamic automaton and the static match of a long row —
+against the oracle: every output, every state of the automata, and the decoding steps that go on from them."""
+import random
+
+import numpy as np
+import pytest
+
+import oracle
+from _parity import assert_dynamic_automata_equal, assert_same, gpu_run, oracle_run
+
+pytestmark = pytest.mark.gpu
+VOCAB = 50_000
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    assert torch.cuda.is_available(), "the gpu tests need a CUDA device"
+    import paper_2411_10666_b200 as pkg
+    pkg.lib()
+    return pkg
+
+
+def _text(kind, n, rng, corpus):
+    if kind == "distinct":
+        return rng.sample(range(VOCAB), n)
+    if kind == "one":
+        return [7] * n
+    if kind == "periodic":
+        u = [rng.randrange(50) for _ in range(rng.randint(2, 40))]
+        x = (u * (n // len(u) + 1))[:n]
+        x[n // 3] = 49_999
+        return x
+    if kind == "fibonacci":                                 # many suffix links per state
+        a, b = [1], [1, 2]
+        while len(b) < n:
+            a, b = b, b + a
+        return b[:n]
+    if kind == "corpus":                                    # ends in a long passage of the corpus
+        k = rng.randint(0, len(corpus) - n)
+        x = corpus[k:k + n]
+        return [rng.randrange(400)] * min(5, n) + x[min(5, n):]
+    k = {"two": 2, "few": 30, "many": 3000, "copies": 400}[kind]
+    x = [min(int(rng.expovariate(8.0 / k)), k - 1) for _ in range(n)]
+    if kind == "copies":
+        for _ in range(n // 60):
+            m = rng.randint(5, 120)
+            src, dst = rng.randrange(n), rng.randrange(n)
+            m = min(m, n - src, n - dst)
+            x[dst:dst + m] = x[src:src + m]
+    return x
+
+
+KINDS = ("distinct", "one", "periodic", "fibonacci", "corpus", "two", "few", "many", "copies")
+
+
+@pytest.mark.parametrize("n", [47, 48, 64, 65, 127, 128, 129, 700, 1025, 2048, 4096, 4097, 8192, 8193])
+def test_prompt_builds_the_oracles_automaton(P, n):
+    rng = random.Random(n)
+    base = [rng.randrange(400) for _ in range(12_000)]
+    corpus = base + base[2000:7000] + base[1000:9000]       # passages that occur once, twice and three times
+    kinds = KINDS if n < 3000 else KINDS[1:5] + KINDS[-1:]
+    B, L, more = len(kinds), 16, 3
+    tail = [[rng.randrange(3) for _ in range(30)] for _ in range(B)]
+    rows = np.array([_text(k, n, rng, corpus) + t for k, t in zip(kinds, tail)], dtype=np.int32)
+    counts = np.full((more, B), 10, dtype=np.int32)
+    steps = rows[:, n:].reshape(B, more, 10).transpose(1, 0, 2).copy()
+    st = P.StaticSam.build(np.array(corpus, dtype=np.int32), VOCAB)
+    ref, ob, _ = oracle_run(np.array(corpus, dtype=np.int32), VOCAB, rows[:, :n], steps, counts, L, n + 30, threads=8)
+    for slab in (0,) if n > 2000 else (0, 4096):
+        got, batch = gpu_run(P, st, VOCAB, rows[:, :n], steps, counts, L, n + 30, slab_bytes=slab)
+        assert_same(got, ref, "n %d" % n)
+        assert_dynamic_automata_equal(batch, ob, range(B), n + 30)
+
+
+def test_mixed_step_with_prompts_short_rows_and_refused_slots(P):
+    """One step in which slots take a prompt, go on from one, take a few tokens, take none or are refused."""
+    import torch
+    rng = random.Random(5)
+    corpus = np.array([rng.randrange(300) for _ in range(6000)], dtype=np.int32)
+    B, n, L = 9, 300, 8
+    first = np.array([_text("copies", n, rng, []) for _ in range(B)], dtype=np.int32)
+    second = np.array([_text("copies", n, rng, []) for _ in range(B)], dtype=np.int32)
+    c1 = np.array([0, 300, 48, 47, 7, 120, 0, 300, 1], dtype=np.int32)
+    c2 = np.array([300, 60, 5, 200, 300, 0, 49, 301, -1], dtype=np.int32)
+    second[6, 20] = 300                                     # a token outside the vocabulary
+    st = P.StaticSam.build(corpus, 300)
+    S = oracle.Sam(corpus)
+    ob = oracle.Batch(S, corpus, B, 300, 700)
+    batch = P.Batch(st, B, 700, max_draft_len=L, max_host_stride=n)
+    host = P.Batch(st, B, 700, max_draft_len=L, max_host_stride=n)
+    keys = ("draft_tokens", "draft_len", "match_len", "source", "state", "status")
+    for toks, cnt in ((first, c1), (second, c2)):
+        ref = ob.step(toks, cnt, L, 1)
+        got = batch.step(torch.from_numpy(toks).cuda(), torch.from_numpy(cnt).cuda(), L).cpu()
+        o = [np.empty(s, dtype=np.int32) for s in ((B, L), (B,), (B, 2), (B,), (B, 2), (B,))]
+        P.binding.sam_step_host(host.handle, toks, n, cnt, L, *o)
+        for k, h in zip(keys, o):
+            assert np.array_equal(got[k], getattr(ref, k)), k
+            assert np.array_equal(h, getattr(ref, k)), k
+    assert set(ref.status.tolist()) == {0, 3, 4}
