@@ -350,6 +350,9 @@ extern "C" int sam_run_steps(sam_batch_t* b, const int32_t* new_tokens_dev, int3
                              match_len_dev, source_dev, status_dev);
     if (rc) return rc;
     if (n_steps < 0) return SAM_ERR_ARG;
+    if (sam_runs_in_one_launch(stride, n_steps))
+        return sam_launch_run(b, new_tokens_dev, stride, counts_dev, n_steps, L, out_per_step != 0, draft_tokens_dev, draft_len_dev,
+                              match_len_dev, source_dev, state_dev, status_dev, (cudaStream_t)stream);
     const size_t B = (size_t)b->view.batch;
     for (int32_t s = 0; s < n_steps; s++) {
         const size_t o = out_per_step ? (size_t)s : 0;

@@ -68,6 +68,12 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
                          const int32_t* v_draft, const int32_t* v_draft_len, const int32_t* v_max_new,
                          int32_t* v_counts_out, int32_t* v_accepted_out);
 
+// n_steps steps in one launch (step.cu), and whether they can be
+int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps,
+                   int32_t L, int32_t keep, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
+                   int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream);
+bool sam_runs_in_one_launch(int32_t stride, int32_t n_steps);
+
 // 1, or 2 when the batch is large enough for the slot-ordering kernel (step.cu)
 int sam_step_launch_count(const sam_batch* b);
 

@@ -713,12 +713,55 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
     return r;
 }
 
-// The static side of one slot's step, run by one warp: the state Transfer (Algorithm 1) reaches over the slot's m
-// tokens, then the static words of the control block.  cw holds control words 0..31 as read at the start
-// of the step; on entry (ra, rb) is the copy of the match state's record kept in the control block, ntok0
-// the text length before the step.  On exit (s, sf, l) is the match state, and, if l > 0 and no error,
-// (ra, rb) its record.  DRAFT: also fetch the draft after the state's first end position into d / my_dl
-// (requested early where the address is known early).
+// The static match moved over a step's m tokens (tok_first: lane k's token of the first 32), by one warp: the
+// state Transfer (Algorithm 1) reaches.  In and out: the state (s, sf, l) and, where l > 0, its record (ra, rb).
+// early(): called where the match is in the state of a corpus prefix, so that the draft after m tokens can be requested
+// with the first reads; returns true if the match did go on as the corpus does, for all m tokens.
+template <class F>
+__device__ __forceinline__ bool static_advance(const SamStaticView& S, int lane, int32_t tok_first, const int32_t* toks, int m,
+                                               uint32_t& s, uint32_t& sf, int32_t& l, uint4& ra, uint4& rb, int& err, ChainCounts& kc, F early) {
+#ifdef SAM_COUNTERS
+    ChainCounts tally = {0, 0, 0, 0, 0};                 // the moves Algorithm 1 itself makes over these tokens
+    {
+        uint32_t ts = s, tsf = sf; int32_t tl = l;
+        for (int j = 0; j < m && !err; j++)
+            static_transfer(S, ts, tsf, tl, (uint32_t)toks[j], __ldg(S.root_row + toks[j]), lane, err, false, ra, rb, tally);
+    }
+#endif
+    bool follows = false;
+    if (m > 32) {
+        static_suffix(S, toks, m, lane, s, sf, l, ra, rb, err, kc);
+    } else if (m > 0) {
+        const uint32_t tk = (uint32_t)tok_first;
+        uint32_t re = SAM_NONE;
+        if (lane < m) re = __ldg(S.root_row + tk);
+        SAM_COUNT(kc.rounds, 1);
+        int i0 = 0;
+        bool have = s != 0, prefix = false;
+        if (have) {                                      // the match so far may take the tokens in one round
+            prefix = ra.x == ra.z;
+            if (prefix) early();
+            i0 = static_run(S, s, sf, ra, rb, have, tk, m, lane, kc);
+            l += i0;
+        }
+        if (i0 < m) {
+            static_walks(S, tk, re, m, lane, s != 0, i0, have, s, sf, l, ra, rb, err, kc);
+        } else {
+            if (!have) static_record(S, s, ra, rb);
+            follows = prefix;
+        }
+    }
+#ifdef SAM_COUNTERS
+    kc.a = tally.a; kc.b = tally.b;
+#endif
+    return follows;
+}
+
+// The static side of one slot's step, run by one warp, then the static words of the control block.  cw holds
+// control words 0..31 as read at the start of the step; on entry (ra, rb) is the copy of the match state's record
+// kept in the control block, ntok0 the text length before the step.  On exit (s, sf, l) is the match state, and, if
+// l > 0 and no error, (ra, rb) its record.  DRAFT: also fetch the draft after the state's first end position into
+// d / my_dl (requested early where the address is known early).
 template <bool DRAFT>
 __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane, uint32_t* cb, uint32_t cw, int32_t tok_first,
                                              const int32_t* toks, int m, uint32_t ntok0, uint4& ra, uint4& rb,
@@ -728,55 +771,25 @@ __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane,
     ChainCounts kc = {1, 0, 0, 0, 0};                    // one round already: the control words
     uint32_t s = __shfl_sync(FULL, cw, CB_S1), sf = __shfl_sync(FULL, cw, CB_S1FLAG);
     int32_t l = (int32_t)__shfl_sync(FULL, cw, CB_L1);
-#ifdef SAM_COUNTERS
-    ChainCounts tally = {0, 0, 0, 0, 0};                 // the moves Algorithm 1 itself makes over these tokens
-    {
-        uint32_t ts = s, tsf = sf; int32_t tl = l;
-        for (int j = 0; j < m && !err; j++)
-            static_transfer(A.S, ts, tsf, tl, (uint32_t)toks[j], __ldg(A.S.root_row + toks[j]), lane, err, false, ra, rb, tally);
-    }
-#endif
-    bool drafted = false;
-    if (m > 32) {
-        static_suffix(A.S, toks, m, lane, s, sf, l, ra, rb, err, kc);
-    } else if (m > 0) {
-        const uint32_t tk = (uint32_t)tok_first;
-        uint32_t re = SAM_NONE;
-        if (lane < m) re = __ldg(A.S.root_row + tk);
-        SAM_COUNT(kc.rounds, 1);
-        // the match so far may take the tokens in one round (with the root row, and with the draft after the last of
-        // them where it is the corpus that goes on)
-        int i0 = 0;
-        bool have = s != 0, early = false;
-        int dl2 = 0;
-        if (have) {
-            if (DRAFT && ra.x == ra.z) {
-                const int64_t e2 = (int64_t)ra.z + m, room = A.S.n_tokens - e2;
-                dl2 = (int)(room < L ? (room < 0 ? 0 : room) : L);
-                gather_draft<1>(A.S.corpus, e2, dl2, L, lane, d);
-                early = true;
-            }
-            i0 = static_run(A.S, s, sf, ra, rb, have, tk, m, lane, kc);
-            l += i0;
+    int dl2 = 0;
+    const bool follows = static_advance(A.S, lane, tok_first, toks, m, s, sf, l, ra, rb, err, kc, [&]() {
+        if (DRAFT) {
+            const int64_t e2 = (int64_t)ra.z + m, room = A.S.n_tokens - e2;
+            dl2 = (int)(room < L ? (room < 0 ? 0 : room) : L);
+            gather_draft<1>(A.S.corpus, e2, dl2, L, lane, d);
         }
-        if (i0 < m) {
-            static_walks(A.S, tk, re, m, lane, s != 0, i0, have, s, sf, l, ra, rb, err, kc);
-        } else {
-            if (!have) static_record(A.S, s, ra, rb);
-            if (early) { my_dl = cut_at_stop(d, dl2, lane, A.W.stop_token); drafted = true; }
-        }
-    }
-#ifdef SAM_COUNTERS
-    kc.a = tally.a; kc.b = tally.b;
-#endif
+    });
     l_out = l; s_out = s; sf_out = sf;
-    if (l > 0 && !err) SAM_COUNT(kc.rounds, DRAFT && !drafted ? 1 : 0);
+    if (l > 0 && !err) SAM_COUNT(kc.rounds, DRAFT && !follows ? 1 : 0);
     flush_counts(b, lane, true, kc, m);
-    if (DRAFT && l > 0 && !err && !drafted) {
-        const int64_t e = (int64_t)ra.z;                // min_endpos
-        int64_t room = A.S.n_tokens - e;
-        my_dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
-        gather_draft<1>(A.S.corpus, e, my_dl, L, lane, d);
+    if (DRAFT && l > 0 && !err) {
+        if (follows) my_dl = dl2;
+        else {
+            const int64_t e = (int64_t)ra.z;            // min_endpos
+            int64_t room = A.S.n_tokens - e;
+            my_dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
+            gather_draft<1>(A.S.corpus, e, my_dl, L, lane, d);
+        }
         my_dl = cut_at_stop(d, my_dl, lane, A.W.stop_token);
     }
     if (m > 0 && lane == 0 && !err) {
@@ -785,21 +798,32 @@ __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane,
     }
 }
 
-// The dynamic side of one slot's step, run by one warp: Expand (fused with the dynamic matcher's Transfer)
-// for each of the slot's m tokens, then the slot's control words.  cw / cw2 are the slot's 64 control
-// words as read at the start of the step (lane i holds words i and 32 + i); on entry (ra, rb) is the copy
-// of the match state's record kept in the control block.  On exit (s2, l2) is the match state, ntok the
-// text length, and, if l2 > 0 and no error, (ra, rb) the record of s2 (also stored in the control block).
-__device__ __forceinline__ void dynamic_chain(const StepArgs& A, int b, int lane, uint32_t* cb, uint32_t cw, uint32_t cw2,
-                                              int32_t tok_first, const int32_t* toks, int m, uint32_t ntok0,
-                                              uint4& ra, uint4& rb, uint32_t (*sh_run)[12],
-                                              uint32_t& s2_out, uint32_t& l2_out, uint32_t& ntok_out, int& err) {
+// The copy of a match state's record that the control block keeps (its words 32.. are in cw2).
+__device__ __forceinline__ void kept_record(uint32_t cw2, int word, uint4& ra, uint4& rb) {
+    const int r = word - 32;
+    ra.x = __shfl_sync(FULL, cw2, r + 0); ra.y = __shfl_sync(FULL, cw2, r + 1);
+    ra.z = __shfl_sync(FULL, cw2, r + 2); ra.w = __shfl_sync(FULL, cw2, r + 3);
+    rb.x = __shfl_sync(FULL, cw2, r + 4); rb.y = __shfl_sync(FULL, cw2, r + 5);
+    rb.z = __shfl_sync(FULL, cw2, r + 6); rb.w = __shfl_sync(FULL, cw2, r + 7);
+}
+
+// The dynamic side of one slot: its automaton and its matcher, kept by one warp for as long as it works on the slot.
+struct DynChain {
     Dyn D;
-    D.pool = A.W.pool;
-    D.root = A.W.root_tab + (size_t)b * A.W.root_cap;
-    D.text = A.W.text + (size_t)b * A.W.text_stride;
-    D.pstate = A.W.pstate + (size_t)b * A.W.text_stride;
-    D.pool_hdr = A.W.pool_hdr; D.free_stack = A.W.free_stack; D.slab_owner = A.W.slab_owner;
+    uint32_t last, ntok, s2, l2;
+    bool have;                   // (ra, rb) is the record of s2
+    uint4 ra, rb;
+};
+
+// cw / cw2 are the slot's 64 control words as read at the start (lane i holds words i and 32 + i); (ra, rb) of X
+// is the copy of the match state's record kept there.
+__device__ __forceinline__ void dyn_open(const SamBatchView& W, int b, int lane, uint32_t* cb, uint32_t cw, uint32_t cw2, DynChain& X) {
+    Dyn& D = X.D;
+    D.pool = W.pool;
+    D.root = W.root_tab + (size_t)b * W.root_cap;
+    D.text = W.text + (size_t)b * W.text_stride;
+    D.pstate = W.pstate + (size_t)b * W.text_stride;
+    D.pool_hdr = W.pool_hdr; D.free_stack = W.free_stack; D.slab_owner = W.slab_owner;
     D.cb = cb;
     {   // slab table entry i is control word 16 + i
         uint32_t lo = __shfl_sync(FULL, cw, (lane + 16) & 31), hi = __shfl_sync(FULL, cw2, (lane + 16) & 31);
@@ -810,16 +834,22 @@ __device__ __forceinline__ void dynamic_chain(const StepArgs& A, int b, int lane
     D.blk_cur = __shfl_sync(FULL, cw, CB_BLK_CUR);
     D.blk_end = __shfl_sync(FULL, cw, CB_BLK_END);
     D.root_deg = __shfl_sync(FULL, cw, CB_ROOTDEG);
-    D.root_bmask = (uint32_t)(A.W.root_cap / SAM_ROOT_BUCKET) - 1;
-    D.slab_shift = A.W.slab_shift; D.rps_shift = A.W.slab_shift - 5;
+    D.root_bmask = (uint32_t)(W.root_cap / SAM_ROOT_BUCKET) - 1;
+    D.slab_shift = W.slab_shift; D.rps_shift = W.slab_shift - 5;
     D.seq = b; D.lane = lane; D.err = 0;
     D.pr_state = 0; D.pr_tgt = 0; D.pr_slot = 0; D.pr_bucket = SAM_NONE; D.cur = 0;
     D.kc = ChainCounts{1, 0, 0, 0, 0};                   // one round already: the control words
-    uint32_t last = __shfl_sync(FULL, cw, CB_LAST), ntok = ntok0;
-    uint32_t s2 = __shfl_sync(FULL, cw, CB_S2), l2 = __shfl_sync(FULL, cw, CB_L2);
+    X.last = __shfl_sync(FULL, cw, CB_LAST); X.ntok = __shfl_sync(FULL, cw, CB_NTOK);
+    X.s2 = __shfl_sync(FULL, cw, CB_S2); X.l2 = __shfl_sync(FULL, cw, CB_L2);
+    X.have = X.s2 != 0;
     if (D.n_states == 0) D.n_states = 1;            // the root exists implicitly (no record is read for it)
+}
 
-    bool have = s2 != 0;
+// Expand (fused with the dynamic matcher's Transfer) for each of a step's m tokens, then the slot's control words.
+// On return, unless D.err is set, (ra, rb) is the record of s2 if l2 > 0 (also stored in the control block).
+__device__ __forceinline__ void dyn_feed(DynChain& X, int32_t tok_first, const int32_t* toks, int m, uint32_t (*sh_run)[12]) {
+    Dyn& D = X.D;
+    const int lane = D.lane;
     for (int base = 0; base < m && !D.err; base += 32) {
         const int i = base + lane;
         uint32_t tk = 0;
@@ -830,43 +860,42 @@ __device__ __forceinline__ void dynamic_chain(const StepArgs& A, int b, int lane
         const int cnt = min(32, m - base);
         int j = 0;
         while (j < cnt && !D.err) {
-            if (s2 == 0) {
-                const int r = dyn_fresh_run(D, tk, j, cnt, bucket_peers, last, ntok);
-                if (r > 0) { j += r; have = false; continue; }
+            if (X.s2 == 0) {
+                const int r = dyn_fresh_run(D, tk, j, cnt, bucket_peers, X.last, X.ntok);
+                if (r > 0) { j += r; X.have = false; continue; }
                 if (D.err) break;
             }
             Pre pre;
             pre.valid = false;
-            if (s2 != 0 && have) {
-                const int r = dyn_repeat_run(D, tk, j, cnt, last, ntok, s2, l2, ra, rb, pre, sh_run);
+            if (X.s2 != 0 && X.have) {
+                const int r = dyn_repeat_run(D, tk, j, cnt, X.last, X.ntok, X.s2, X.l2, X.ra, X.rb, pre, sh_run);
                 if (r > 0) { j += r; continue; }
                 if (D.err) break;
             }
             D.cur = j;
-            dyn_extend(D, __shfl_sync(FULL, tk, j), last, ntok, s2, l2, have, ra, rb, pre);
+            dyn_extend(D, __shfl_sync(FULL, tk, j), X.last, X.ntok, X.s2, X.l2, X.have, X.ra, X.rb, pre);
             j++;
         }
     }
-    err = D.err;
-    if (m > 0 && !err) {
+    if (m > 0 && !D.err) {
         // the newest state's record, without a transition yet
-        uint4* rl = rec_ptr(D, last);
+        uint4* rl = rec_ptr(D, X.last);
+        uint32_t* cb = D.cb;
         if (lane == 0) {
-            rl[0] = make_uint4(ntok, s2, ntok, 0);
+            rl[0] = make_uint4(X.ntok, X.s2, X.ntok, 0);
             rl[1] = make_uint4(0, 0, 0, 0);
-            cb[CB_NTOK] = ntok; cb[CB_NSTATES] = D.n_states; cb[CB_LAST] = last;
-            cb[CB_S2] = s2; cb[CB_L2] = l2; cb[CB_BLK_CUR] = D.blk_cur; cb[CB_BLK_END] = D.blk_end;
+            cb[CB_NTOK] = X.ntok; cb[CB_NSTATES] = D.n_states; cb[CB_LAST] = X.last;
+            cb[CB_S2] = X.s2; cb[CB_L2] = X.l2; cb[CB_BLK_CUR] = D.blk_cur; cb[CB_BLK_END] = D.blk_end;
             cb[CB_NRECSLABS] = D.n_rec_slabs; cb[CB_ROOTDEG] = D.root_deg;
         }
         __syncwarp();
     }
-    if (l2 > 0 && !err) SAM_COUNT(D.kc.rounds, 1);       // the draft
-    if (l2 > 0 && !err && m > 0) {                      // the state moved: get its record, keep a copy
-        if (!have) { const uint4* rs = rec_ptr(D, s2); ra = rs[0]; rb = rs[1]; SAM_COUNT(D.kc.rounds, 1); }
-        if (lane == 0) { reinterpret_cast<uint4*>(cb + CB_REC2)[0] = ra; reinterpret_cast<uint4*>(cb + CB_REC2)[1] = rb; }
+    if (X.l2 > 0 && !D.err) SAM_COUNT(D.kc.rounds, 1);   // the draft
+    if (X.l2 > 0 && !D.err && m > 0) {                  // the state moved: get its record, keep a copy
+        if (!X.have) { const uint4* rs = rec_ptr(D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(D.kc.rounds, 1); }
+        if (lane == 0) { reinterpret_cast<uint4*>(D.cb + CB_REC2)[0] = X.ra; reinterpret_cast<uint4*>(D.cb + CB_REC2)[1] = X.rb; }
     }
-    s2_out = s2; l2_out = l2; ntok_out = ntok;
-    if (!err) flush_counts(b, lane, false, D.kc, m);
+    if (!D.err) flush_counts(D.seq, lane, false, D.kc, m);
 }
 
 // Called by one thread of a block after the block's outputs are written (and made known to that
@@ -882,6 +911,52 @@ __device__ __forceinline__ void signal_done(const StepArgs& A) {
         *A.done_count = 0;
         __threadfence_system();
         *reinterpret_cast<volatile int32_t*>(A.done_flag) = A.done_seq;
+    }
+}
+
+// Where a step's outputs go (step `at` of outputs that keep every step).
+struct StepOut { int32_t *draft, *draft_len, *match_len, *source, *state, *status; };
+__device__ __forceinline__ StepOut step_out(const StepArgs& A, int at) {
+    const size_t n = (size_t)at * A.W.batch;
+    return {A.draft_tokens + n * A.L, A.draft_len + n, A.match_len + 2 * n, A.source + n, A.state ? A.state + 2 * n : nullptr, A.status + n};
+}
+
+__device__ __forceinline__ void write_failed_slot(const StepOut& o, int L, int b, int lane, int status) {
+    for (int j = lane; j < L; j += 32) o.draft[(size_t)b * L + j] = -1;
+    if (lane == 0) {
+        o.draft_len[b] = 0; o.match_len[2 * b] = 0; o.match_len[2 * b + 1] = 0; o.source[b] = 0;
+        if (o.state) { o.state[2 * b] = 0; o.state[2 * b + 1] = 0; }
+        o.status[b] = status;
+    }
+}
+
+// Choose the source (Section 3.2), read the draft, write the outputs: by a whole warp that has both sides' results
+// (match length, state, first end position; ntok: the text's length).  READ: how the slot's own text is read (gather_draft).
+template <int READ>
+__device__ __forceinline__ void write_slot(const StepArgs& A, const StepOut& o, int b, int lane, int l1, int s1, int64_t e1,
+                                           int l2, int s2, int64_t e2, int64_t ntok) {
+    const int L = A.L;
+    const bool use_static = A.has_static && l1 > l2 + A.W.l_bias;
+    const int lsel = use_static ? l1 : l2;
+    const int need = A.W.min_match > 1 ? A.W.min_match : 1;
+    const int src = lsel < need ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
+    int32_t d[MAX_DRAFT_REGS] = {-1, -1, -1, -1};
+    int dl = 0;
+    if (src != SAM_SRC_NONE) {
+        const int64_t e = use_static ? e1 : e2, room = (use_static ? A.S.n_tokens : ntok) - e;
+        dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
+        gather_draft<READ>(use_static ? A.S.corpus : A.W.text + (size_t)b * A.W.text_stride, e, dl, L, lane, d);
+        dl = cut_at_stop(d, dl, lane, A.W.stop_token);
+    }
+#pragma unroll
+    for (int r = 0; r < MAX_DRAFT_REGS; r++) {
+        const int j = r * 32 + lane;
+        if (j < L) o.draft[(size_t)b * L + j] = d[r];
+    }
+    if (lane == 0) {
+        o.draft_len[b] = dl; o.match_len[2 * b] = l1; o.match_len[2 * b + 1] = l2; o.source[b] = src;
+        if (o.state) { o.state[2 * b] = s1; o.state[2 * b + 1] = s2; }
+        o.status[b] = 0;
     }
 }
 
@@ -1000,11 +1075,8 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
     if (status != 0) {
         if (warp == 0) {
             if (fresh_fail && lane == 0) cb[CB_STATUS] = (uint32_t)status;
-            for (int j = lane; j < L; j += 32) A.draft_tokens[(size_t)b * L + j] = -1;
+            write_failed_slot(step_out(A, 0), L, b, lane, status);
             if (lane == 0) {
-                A.draft_len[b] = 0; A.match_len[2 * b] = 0; A.match_len[2 * b + 1] = 0; A.source[b] = 0;
-                if (A.state) { A.state[2 * b] = 0; A.state[2 * b + 1] = 0; }
-                A.status[b] = status;
                 if (VERIFY && A.v_counts_out) A.v_counts_out[b] = m;
                 if (VERIFY && A.v_accepted_out) A.v_accepted_out[b] = confirmed;
             }
@@ -1014,13 +1086,8 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
         return;
     }
 
-    // this warp's copy of its match state's record: words CB_REC1.. (warp 0) or CB_REC2.. (warp 1)
-    const int rbase = (warp == 0 ? CB_REC1 : CB_REC2) - 32;
-    uint4 ra, rb;
-    ra.x = __shfl_sync(FULL, cw2, rbase + 0); ra.y = __shfl_sync(FULL, cw2, rbase + 1);
-    ra.z = __shfl_sync(FULL, cw2, rbase + 2); ra.w = __shfl_sync(FULL, cw2, rbase + 3);
-    rb.x = __shfl_sync(FULL, cw2, rbase + 4); rb.y = __shfl_sync(FULL, cw2, rbase + 5);
-    rb.z = __shfl_sync(FULL, cw2, rbase + 6); rb.w = __shfl_sync(FULL, cw2, rbase + 7);
+    uint4 ra, rb;             // this warp's copy of its match state's record
+    kept_record(cw2, warp == 0 ? CB_REC1 : CB_REC2, ra, rb);
 
     int32_t d[MAX_DRAFT_REGS] = {-1, -1, -1, -1};
     int32_t my_l = 0, my_s = 0, my_dl = 0;
@@ -1035,12 +1102,14 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
         }
     } else {
         // ---------------- dynamic automaton: Expand per token ----------------
-        uint32_t s2, l2, ntok;
-        dynamic_chain(A, b, lane, cb, cw, cw2, tok_first, toks, m, ntok0, ra, rb, sh_run, s2, l2, ntok, err);
-        my_l = (int32_t)l2; my_s = (int32_t)s2;
-        if (l2 > 0 && !err) {
-            const int64_t e = (int64_t)ra.z;                    // min_endpos
-            int64_t room = (int64_t)ntok - e;
+        DynChain X;
+        X.ra = ra; X.rb = rb;
+        dyn_open(A.W, b, lane, cb, cw, cw2, X);
+        dyn_feed(X, tok_first, toks, m, sh_run);
+        err = X.D.err; my_l = (int32_t)X.l2; my_s = (int32_t)X.s2;
+        if (X.l2 > 0 && !err) {
+            const int64_t e = (int64_t)X.ra.z;                  // min_endpos
+            int64_t room = (int64_t)X.ntok - e;
             my_dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
             gather_draft<0>(A.W.text + (size_t)b * A.W.text_stride, e, my_dl, L, lane, d);
             my_dl = cut_at_stop(d, my_dl, lane, A.W.stop_token);
@@ -1114,7 +1183,7 @@ __global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant
 // With more slots than the GPU holds blocks of the kernel above, throughput is set by how many chains are
 // resident, and a block of two warps holds two warps' worth of registers for as long as its slower chain
 // runs.  The split step gives the two sides of a slot to different blocks (of one warp) of one grid:
-//   - the dynamic side keeps its warp per slot (dynamic_chain);
+//   - the dynamic side keeps its warp per slot (DynChain);
 //   - the static side of a slot with few tokens needs no cooperation between lanes (a state is one 32-byte
 //     record, a hash bucket eight 16-byte entries), so one LANE carries it: a warp advances 32 slots, each
 //     round of reads serving 32 chains (static_lanes);
@@ -1128,15 +1197,6 @@ __global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant
 // A slot that fails its validation, or whose dynamic side runs into an error, is reported by the dynamic
 // side alone before it counts itself; the static side validates on its own (it keeps the text length in
 // CB_NTOK_S because CB_NTOK may change under it) and never commits a state for a step that is refused.
-
-__device__ __forceinline__ void write_failed_slot(const StepArgs& A, int b, int lane, int status) {
-    for (int j = lane; j < A.L; j += 32) A.draft_tokens[(size_t)b * A.L + j] = -1;
-    if (lane == 0) {
-        A.draft_len[b] = 0; A.match_len[2 * b] = 0; A.match_len[2 * b + 1] = 0; A.source[b] = 0;
-        if (A.state) { A.state[2 * b] = 0; A.state[2 * b + 1] = 0; }
-        A.status[b] = status;
-    }
-}
 
 // How many sides of the slot have counted themselves, read with acquire semantics: if the count is odd the
 // other side is done and everything it wrote may be read from here on (with loads that bypass the L1).
@@ -1166,50 +1226,21 @@ __device__ __forceinline__ bool arrive_warp(uint32_t* cb, int lane) {
     return (old & 1u) != 0;
 }
 
-// Both sides of slot b are done: choose the source (Section 3.2), read the draft, write the outputs.
-// Run by a whole warp.
+// Both sides of slot b are done.  Run by a whole warp.
 __device__ __forceinline__ void split_epilogue(const StepArgs& A, int b, int lane) {
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const uint32_t cw = __ldcg(cb + lane), cw2 = __ldcg(cb + 32 + lane);
     if (__shfl_sync(FULL, cw, CB_STATUS) != 0) return;                  // reported by the dynamic side
     const int err_s = (int)__shfl_sync(FULL, cw, CB_ERR_S);
+    const StepOut o = step_out(A, 0);
     if (err_s) {
-        write_failed_slot(A, b, lane, err_s);
+        write_failed_slot(o, A.L, b, lane, err_s);
         if (lane == 0) cb[CB_STATUS] = (uint32_t)err_s;
         return;
     }
-    const int l1 = (int)__shfl_sync(FULL, cw, CB_L1), l2 = (int)__shfl_sync(FULL, cw, CB_L2);
-    const int s1 = (int)__shfl_sync(FULL, cw, CB_S1), s2 = (int)__shfl_sync(FULL, cw, CB_S2);
-    const int64_t ntok = (int64_t)__shfl_sync(FULL, cw, CB_NTOK);
-    const int64_t e1 = (int64_t)__shfl_sync(FULL, cw2, CB_REC1 + 2 - 32), e2 = (int64_t)__shfl_sync(FULL, cw2, CB_REC2 + 2 - 32);
-    const int L = A.L;
-    const bool use_static = l1 > l2 + A.W.l_bias;                       // Section 3.2
-    const int lsel = use_static ? l1 : l2;
-    const int need = A.W.min_match > 1 ? A.W.min_match : 1;
-    const int src = lsel < need ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
-    int32_t d[MAX_DRAFT_REGS] = {-1, -1, -1, -1};
-    int dl = 0;
-    if (src == SAM_SRC_STATIC) {
-        const int64_t room = A.S.n_tokens - e1;
-        dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
-        gather_draft<1>(A.S.corpus, e1, dl, L, lane, d);
-        dl = cut_at_stop(d, dl, lane, A.W.stop_token);
-    } else if (src == SAM_SRC_DYNAMIC) {
-        const int64_t room = ntok - e2;
-        dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
-        gather_draft<2>(A.W.text + (size_t)b * A.W.text_stride, e2, dl, L, lane, d);
-        dl = cut_at_stop(d, dl, lane, A.W.stop_token);
-    }
-#pragma unroll
-    for (int r = 0; r < MAX_DRAFT_REGS; r++) {
-        const int j = r * 32 + lane;
-        if (j < L) A.draft_tokens[(size_t)b * L + j] = d[r];
-    }
-    if (lane == 0) {
-        A.draft_len[b] = dl; A.match_len[2 * b] = l1; A.match_len[2 * b + 1] = l2; A.source[b] = src;
-        if (A.state) { A.state[2 * b] = s1; A.state[2 * b + 1] = s2; }
-        A.status[b] = 0;
-    }
+    write_slot<2>(A, o, b, lane, (int)__shfl_sync(FULL, cw, CB_L1), (int)__shfl_sync(FULL, cw, CB_S1), (int64_t)__shfl_sync(FULL, cw2, CB_REC1 + 2 - 32),
+                  (int)__shfl_sync(FULL, cw, CB_L2), (int)__shfl_sync(FULL, cw, CB_S2), (int64_t)__shfl_sync(FULL, cw2, CB_REC2 + 2 - 32),
+                  (int64_t)__shfl_sync(FULL, cw, CB_NTOK));
 }
 
 // The same for the slots of the lanes of a static_lanes warp that found their dynamic side done (`second`).
@@ -1430,19 +1461,16 @@ __device__ __forceinline__ void dynamic_slot(const StepArgs& A, int b, int lane,
     }
     int err = 0;
     if (status == 0) {
-        const int rbase = CB_REC2 - 32;
-        uint4 ra, rb;
-        ra.x = __shfl_sync(FULL, cw2, rbase + 0); ra.y = __shfl_sync(FULL, cw2, rbase + 1);
-        ra.z = __shfl_sync(FULL, cw2, rbase + 2); ra.w = __shfl_sync(FULL, cw2, rbase + 3);
-        rb.x = __shfl_sync(FULL, cw2, rbase + 4); rb.y = __shfl_sync(FULL, cw2, rbase + 5);
-        rb.z = __shfl_sync(FULL, cw2, rbase + 6); rb.w = __shfl_sync(FULL, cw2, rbase + 7);
-        uint32_t s2, l2, ntok;
-        dynamic_chain(A, b, lane, cb, cw, cw2, tok_first, toks, m, ntok0, ra, rb, sh_run, s2, l2, ntok, err);
+        DynChain X;
+        kept_record(cw2, CB_REC2, X.ra, X.rb);
+        dyn_open(A.W, b, lane, cb, cw, cw2, X);
+        dyn_feed(X, tok_first, toks, m, sh_run);
+        err = X.D.err;
         if (err) { status = err; fresh_fail = true; }
     }
     if (status != 0) {
         if (fresh_fail && lane == 0) cb[CB_STATUS] = (uint32_t)status;
-        write_failed_slot(A, b, lane, status);
+        write_failed_slot(step_out(A, 0), A.L, b, lane, status);
         arrive_warp(cb, lane);
         return;
     }
@@ -1469,12 +1497,8 @@ __device__ __forceinline__ void static_slot(const StepArgs& A, int b, int lane) 
         run = !__any_sync(FULL, bad);
     }
     if (run) {
-        const int rbase = CB_REC1 - 32;
         uint4 ra, rb;
-        ra.x = __shfl_sync(FULL, cw2, rbase + 0); ra.y = __shfl_sync(FULL, cw2, rbase + 1);
-        ra.z = __shfl_sync(FULL, cw2, rbase + 2); ra.w = __shfl_sync(FULL, cw2, rbase + 3);
-        rb.x = __shfl_sync(FULL, cw2, rbase + 4); rb.y = __shfl_sync(FULL, cw2, rbase + 5);
-        rb.z = __shfl_sync(FULL, cw2, rbase + 6); rb.w = __shfl_sync(FULL, cw2, rbase + 7);
+        kept_record(cw2, CB_REC1, ra, rb);
         uint32_t s, sf; int32_t l, dl = 0;
         int32_t d[MAX_DRAFT_REGS];
         int err = 0;
@@ -1516,6 +1540,180 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
     if (A.done_flag) {
         __syncwarp();
         if (lane == 0) signal_done(A);
+    }
+}
+
+// ------------------------------------------------------------------ many steps in one launch
+// sam_run_steps has every step's tokens at hand and slots never meet, so a slot goes through all its steps without waiting
+// for the slowest slot of each: a launch per step costs that slowest slot (at 4096 slots 29 us a step, of which the
+// average slot needs 5), the launch, and the reads that start a step (control words, first tokens).  Both match
+// states and the automaton's head stay in registers, the next step's tokens are read a step ahead.
+struct RunArgs {
+    StepArgs A;
+    int32_t n_steps, keep;       // keep: the outputs have room for every step
+};
+
+// Whether a step's tokens can be fed to a slot: its status if not (the whole step is checked before any state changes).
+__device__ __forceinline__ int check_step(const StepArgs& A, int lane, int32_t tok_first, const int32_t* toks, int m, uint32_t ntok) {
+    if (m < 0 || m > A.stride) return SAM_SEQ_BAD_COUNT;
+    if ((int64_t)ntok + m > A.W.max_seq_len) return SAM_SEQ_CAPACITY;
+    const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
+    bool bad = false;
+    for (int base = 0; base < m; base += 32) {
+        const int i = base + lane;
+        if (i < m) { const int t = base == 0 ? tok_first : toks[i]; bad |= t < 0 || t >= vocab; }
+    }
+    return __any_sync(FULL, bad) ? SAM_SEQ_BAD_TOKEN : 0;
+}
+
+// The rows of slot b, one step after the other, read a step ahead.
+struct RunRows {
+    const int32_t *toks, *counts;
+    int32_t tok, m;
+    __device__ __forceinline__ void start(const StepArgs& A, int b, int lane) {
+        toks = A.new_tokens + (size_t)b * A.stride; counts = A.counts + b;
+        fetch(A, lane);
+    }
+    __device__ __forceinline__ void fetch(const StepArgs& A, int lane) { m = *counts; tok = lane < A.stride ? toks[lane] : 0; }
+    __device__ __forceinline__ void next(const StepArgs& A, int lane, bool more) {
+        toks += (size_t)A.W.batch * A.stride; counts += A.W.batch;
+        if (more) fetch(A, lane);
+    }
+};
+
+struct StaticSide { uint32_t s, sf; int32_t l; uint4 ra, rb; };
+__device__ __forceinline__ void static_open(uint32_t cw, uint32_t cw2, StaticSide& T) {
+    T.s = __shfl_sync(FULL, cw, CB_S1); T.sf = __shfl_sync(FULL, cw, CB_S1FLAG); T.l = (int32_t)__shfl_sync(FULL, cw, CB_L1);
+    kept_record(cw2, CB_REC1, T.ra, T.rb);
+}
+__device__ __forceinline__ void static_feed(const StepArgs& A, int b, int lane, const RunRows& in, StaticSide& T, int& err) {
+    ChainCounts kc = {1, 0, 0, 0, 0};
+    static_advance(A.S, lane, in.tok, in.toks, in.m, T.s, T.sf, T.l, T.ra, T.rb, err, kc, []() {});
+    flush_counts(b, lane, true, kc, in.m);
+}
+__device__ __forceinline__ void static_close(uint32_t* cb, int lane, uint32_t ntok, const StaticSide& T) {
+    if (lane == 0) {
+        cb[CB_S1] = T.s; cb[CB_L1] = (uint32_t)T.l; cb[CB_S1FLAG] = T.sf; cb[CB_NTOK_S] = ntok;
+        if (T.l > 0) { reinterpret_cast<uint4*>(cb + CB_REC1)[0] = T.ra; reinterpret_cast<uint4*>(cb + CB_REC1)[1] = T.rb; }
+    }
+}
+
+// One warp per slot takes both sides in turn: for batches whose slots fill the GPU, where what counts is how many
+// chains are resident (28 warps per SM).
+__global__ void __launch_bounds__(32, 28) sam_run_warp_kernel(const __grid_constant__ RunArgs R) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    __shared__ __align__(16) uint32_t sh_run[32][12];
+    const StepArgs& A = R.A;
+    const int b = blockIdx.x, lane = threadIdx.x;
+    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
+    const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
+    RunRows in;
+    in.start(A, b, lane);
+    const int status0 = (int)__shfl_sync(FULL, cw, CB_STATUS);
+    int status = status0;
+    DynChain X;
+    kept_record(cw2, CB_REC2, X.ra, X.rb);
+    dyn_open(A.W, b, lane, cb, cw, cw2, X);
+    StaticSide T;
+    static_open(cw, cw2, T);
+    for (int i = 0; i < R.n_steps; i++) {
+        const RunRows now = in;
+        in.next(A, lane, i + 1 < R.n_steps);
+        if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, X.ntok);
+        if (status == 0) {
+            int err = 0;
+            if (A.has_static) static_feed(A, b, lane, now, T, err);
+            X.D.kc = ChainCounts{1, 0, 0, 0, 0};
+            dyn_feed(X, now.tok, now.toks, now.m, sh_run);
+            status = err ? err : X.D.err;
+        }
+        const StepOut o = step_out(A, R.keep ? i : 0);
+        if (status != 0) write_failed_slot(o, A.L, b, lane, status);
+        else write_slot<0>(A, o, b, lane, T.l, (int)T.s, (int64_t)T.ra.z, (int)X.l2, (int)X.s2, (int64_t)X.ra.z, (int64_t)X.ntok);
+    }
+    if (A.has_static && status0 == 0) static_close(cb, lane, X.ntok, T);
+    if (lane == 0 && status != status0) cb[CB_STATUS] = (uint32_t)status;
+}
+
+// Three warps per slot: the static side, the dynamic side, and one that writes the outputs.  For batches that leave
+// the GPU room: each side goes on with its next step at once, at most RUN_RING steps ahead of the outputs.
+constexpr int RUN_RING = 4;
+__device__ __forceinline__ void run_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void run_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+__global__ void __launch_bounds__(96, 7) sam_run_block_kernel(const __grid_constant__ RunArgs R) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    __shared__ __align__(16) uint32_t sh_run[32][12];
+    __shared__ __align__(16) int4 from_static[RUN_RING], from_dynamic[RUN_RING];   // (l, s, first end position, error or text length)
+    __shared__ int32_t dyn_status[RUN_RING];
+    const StepArgs& A = R.A;
+    const int b = blockIdx.x, lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
+    const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
+    const int status0 = (int)__shfl_sync(FULL, cw, CB_STATUS);
+    uint32_t ntok = __shfl_sync(FULL, cw, CB_NTOK);
+    __syncthreads();                                     // all three have the slot as it was
+    // barriers: 1 + r, a side's result is in ring entry r (both sides arrive); 5 + r and 9 + r, the entry has been
+    // read and the static or the dynamic side may use it again
+    if (role == 2) {
+        int status = status0;
+        for (int i = 0; i < R.n_steps; i++) {
+            const int r = i % RUN_RING;
+            run_sync(1 + r, 96);
+            const int4 x = from_static[r], y = from_dynamic[r];
+            if (status == 0) status = dyn_status[r] ? dyn_status[r] : x.w;
+            if (i + RUN_RING < R.n_steps) { run_arrive(5 + r, 64); run_arrive(9 + r, 64); }
+            const StepOut o = step_out(A, R.keep ? i : 0);
+            if (status != 0) write_failed_slot(o, A.L, b, lane, status);
+            else write_slot<0>(A, o, b, lane, x.x, x.y, (int64_t)x.z, y.x, y.y, (int64_t)y.z, (int64_t)y.w);
+        }
+        if (lane == 0 && status != status0) cb[CB_STATUS] = (uint32_t)status;
+        return;
+    }
+    RunRows in;
+    in.start(A, b, lane);
+    int status = status0;
+    if (role == 0) {
+        StaticSide T;
+        static_open(cw, cw2, T);
+        for (int i = 0; i < R.n_steps; i++) {
+            const int r = i % RUN_RING;
+            const RunRows now = in;
+            in.next(A, lane, i + 1 < R.n_steps);
+            if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, ntok);
+            int err = 0;
+            if (status == 0) {
+                if (A.has_static) static_feed(A, b, lane, now, T, err);
+                ntok += (uint32_t)now.m;
+                status = err;
+            }
+            if (i >= RUN_RING) run_sync(5 + r, 64);
+            if (lane == 0) from_static[r] = make_int4(T.l, (int)T.s, (int)T.ra.z, err);
+            __syncwarp();
+            run_arrive(1 + r, 96);
+        }
+        if (A.has_static && status0 == 0) static_close(cb, lane, ntok, T);
+    } else {
+        DynChain X;
+        kept_record(cw2, CB_REC2, X.ra, X.rb);
+        dyn_open(A.W, b, lane, cb, cw, cw2, X);
+        for (int i = 0; i < R.n_steps; i++) {
+            const int r = i % RUN_RING;
+            const RunRows now = in;
+            in.next(A, lane, i + 1 < R.n_steps);
+            if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, X.ntok);
+            if (status == 0) {
+                X.D.kc = ChainCounts{1, 0, 0, 0, 0};
+                dyn_feed(X, now.tok, now.toks, now.m, sh_run);
+                status = X.D.err;
+            }
+            if (i >= RUN_RING) run_sync(9 + r, 64);
+            if (lane == 0) { from_dynamic[r] = make_int4((int)X.l2, (int)X.s2, (int)X.ra.z, (int)X.ntok); dyn_status[r] = status; }
+            __syncwarp();
+            run_arrive(1 + r, 96);
+        }
     }
 }
 
@@ -1618,6 +1816,7 @@ int split_kernel_setup(int device) {
     if (!done[device]) {
         cudaError_t e = cudaFuncSetAttribute(sam_step_split_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(order_slots_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_warp_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
         done[device] = true;
     }
@@ -1742,6 +1941,44 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;
 }
+
+// Steps of sam_run_steps in one launch.  Up to how many slots three warps each fit the GPU at once: 148 SMs x 7 blocks.
+constexpr int SAM_RUN_BLOCK_MAX_BATCH = 1036;
+
+int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps, int32_t L, int32_t keep,
+                   int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status,
+                   cudaStream_t stream) {
+    RunArgs R;
+    memset(&R, 0, sizeof(R));
+    StepArgs& A = R.A;
+    A.has_static = b->st != nullptr;
+    if (b->st) A.S = b->st->view; else A.S.vocab = b->view.vocab;
+    A.W = b->view;
+    A.new_tokens = new_tokens; A.stride = stride; A.counts = counts; A.L = L;
+    A.draft_tokens = draft_tokens; A.draft_len = draft_len; A.match_len = match_len; A.source = source; A.state = state; A.status = status;
+    R.n_steps = n_steps; R.keep = keep;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)b->view.batch); cfg.stream = stream; cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaError_t e;
+    if (b->view.batch <= SAM_RUN_BLOCK_MAX_BATCH) {
+        cfg.blockDim = dim3(96);
+        e = cudaLaunchKernelEx(&cfg, sam_run_block_kernel, R);
+    } else {
+        int rc = split_kernel_setup(b->device);
+        if (rc) return rc;
+        cfg.blockDim = dim3(32);
+        e = cudaLaunchKernelEx(&cfg, sam_run_warp_kernel, R);
+    }
+    if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
+    return SAM_OK;
+}
+
+// A launch per step where rows may hold prompts (the whole-text build has a kernel of its own), else one for all.
+bool sam_runs_in_one_launch(int32_t stride, int32_t n_steps) { return n_steps > 1 && stride < SAM_PREFILL_MIN; }
 
 extern "C" int sam_counters_available(void) {
 #ifdef SAM_COUNTERS
