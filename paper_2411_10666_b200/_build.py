@@ -4,6 +4,7 @@ from __future__ import annotations
 import glob
 import os
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -42,6 +43,18 @@ def build(force: bool = False, verbose: bool = False, variant: str | None = None
         subprocess.check_call(cmd, cwd=CSRC)
         os.replace(tmp, lib)
     return lib
+
+
+def build_calls(force: bool = False) -> str:
+    """Build the extension module that marshals the per-step calls (plain C API, gcc) if it is missing or stale."""
+    out, src = os.path.join(HERE, "_calls.so"), os.path.join(CSRC, "calls.c")
+    deps = (src, os.path.join(os.path.dirname(HERE), "include", "samdraft.h"))
+    if force or not os.path.exists(out) or any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps):
+        tmp = out + ".tmp%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-std=c11", "-shared", "-fPIC",
+                               "-I", sysconfig.get_paths()["include"], "-o", tmp, src])
+        os.replace(tmp, out)
+    return out
 
 
 if __name__ == "__main__":

@@ -113,6 +113,41 @@ def lib():
     return _lib
 
 
+_calls = None
+_fn = {}
+
+
+def _hot(name: str):
+    """(extension module, address of a library function): for the calls that are made every step."""
+    global _calls
+    addr = _fn.get(name)
+    if addr is None:
+        if _calls is None:
+            import importlib.machinery
+            import importlib.util
+            import torch
+            path = _build.build_calls()
+            loader = importlib.machinery.ExtensionFileLoader("_calls", path)
+            m = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
+            loader.exec_module(m)
+            m.setup(torch.int32, torch.float32, torch._C._cuda_getCurrentRawStream, _host_ptr)
+            _calls = m
+        addr = _fn[name] = ctypes.cast(getattr(lib(), name), c_void_p).value
+    return _calls, addr
+
+
+def _addr(h) -> int:
+    return 0 if h is None else h if isinstance(h, int) else h.value or 0
+
+
+def _stream_of(stream) -> int:
+    """A stream's raw handle, or -1 - device for the current stream of the current device."""
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    return -1 - torch.cuda.current_device()
+
+
 def _check(rc: int, what: str):
     if rc != SAM_OK:
         raise SamError(rc, what)
@@ -231,10 +266,9 @@ def sam_batch_destroy(h):
 
 
 def sam_step(h, new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state, status, stream=None):
-    _check(lib().sam_step(h, _dev_ptr(new_tokens, "new_tokens"), stride, _dev_ptr(counts, "counts"), L,
-                          _dev_ptr(draft_tokens, "draft_tokens"), _dev_ptr(draft_len, "draft_len"),
-                          _dev_ptr(match_len, "match_len"), _dev_ptr(source, "source"),
-                          _dev_ptr(state, "state"), _dev_ptr(status, "status"), _stream_ptr(stream)), "sam_step")
+    m, fn = _hot("sam_step")
+    _check(m.step(fn, _addr(h), new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state, status,
+                  _stream_of(stream)), "sam_step")
 
 
 def sam_run_steps(h, new_tokens, stride, counts, n_steps, L, out_per_step,
@@ -262,25 +296,24 @@ def _host_ptr(t, name):
 
 def sam_step_host(h, new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state, status,
                   stream=None):
-    _check(lib().sam_step_host(h, _host_ptr(new_tokens, "new_tokens"), stride, _host_ptr(counts, "counts"), L,
-                               _host_ptr(draft_tokens, "draft_tokens"), _host_ptr(draft_len, "draft_len"),
-                               _host_ptr(match_len, "match_len"), _host_ptr(source, "source"),
-                               _host_ptr(state, "state"), _host_ptr(status, "status"), _stream_ptr(stream)),
-           "sam_step_host")
+    m, fn = _hot("sam_step_host")
+    _check(m.step_host(fn, _addr(h), new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state, status,
+                       _stream_of(stream)), "sam_step_host")
 
 
 def sam_step_host_prepared(h, stride, L, draft_tokens, draft_len, match_len, source, state, status, stream=None):
     """The same call as sam_step_host for a loop that makes it every step: whatever does not change
     from step to step (the output arrays, stride, L, the stream) is converted once, and the returned
     function takes the step's new_tokens and counts (arrays, or plain addresses)."""
-    fn = lib().sam_step_host
-    fixed = [c_void_p(_host_ptr(x, n)) for x, n in ((draft_tokens, "draft_tokens"), (draft_len, "draft_len"),
-                                                     (match_len, "match_len"), (source, "source"), (state, "state"),
-                                                     (status, "status"))]
-    sp, hh = c_void_p(_stream_ptr(stream)), c_void_p(h) if isinstance(h, int) else h
+    m, fn = _hot("sam_step_host")
+    make = m.step_host
+    d, dl, ml, so, st, status = [_host_ptr(x, n) for x, n in ((draft_tokens, "draft_tokens"), (draft_len, "draft_len"),
+                                                              (match_len, "match_len"), (source, "source"), (state, "state"),
+                                                              (status, "status"))]
+    sp, hh = _stream_ptr(stream), _addr(h)
 
     def call(new_tokens, counts):
-        rc = fn(hh, _host_ptr(new_tokens, "new_tokens"), stride, _host_ptr(counts, "counts"), L, *fixed, sp)
+        rc = make(fn, hh, new_tokens, stride, counts, L, d, dl, ml, so, st, status, sp)
         if rc != SAM_OK:
             raise SamError(rc, "sam_step_host")
     return call
@@ -306,43 +339,32 @@ def sam_batch_pool_info(h, stream=None):
 
 def sam_accept_greedy(draft_tokens, draft_len, target_tokens, max_new, new_tokens, counts, accepted=None, stream=None):
     B, L = draft_tokens.shape
-    _check(lib().sam_accept_greedy(B, _dev_ptr(draft_tokens, "draft_tokens"), _dev_ptr(draft_len, "draft_len"), L,
-                                   _dev_ptr(target_tokens, "target_tokens"), _dev_ptr(max_new, "max_new"),
-                                   _dev_ptr(new_tokens, "new_tokens"), new_tokens.shape[1], _dev_ptr(counts, "counts"),
-                                   _dev_ptr(accepted, "accepted"), _stream_ptr(stream)), "sam_accept_greedy")
+    m, fn = _hot("sam_accept_greedy")
+    _check(m.accept_greedy(fn, B, draft_tokens, draft_len, L, target_tokens, max_new, new_tokens, new_tokens.shape[1], counts,
+                           accepted, _stream_of(stream)), "sam_accept_greedy")
 
 
 def sam_step_verified(h, target_tokens, prev_draft_tokens, prev_draft_len, max_new, L,
                       draft_tokens, draft_len, match_len, source, state, status, counts_out=None, accepted_out=None,
                       stream=None):
-    _check(lib().sam_step_verified(h, _dev_ptr(target_tokens, "target_tokens"), prev_draft_tokens.shape[1],
-                                   _dev_ptr(prev_draft_tokens, "prev_draft_tokens"), _dev_ptr(prev_draft_len, "prev_draft_len"),
-                                   _dev_ptr(max_new, "max_new"), L,
-                                   _dev_ptr(draft_tokens, "draft_tokens"), _dev_ptr(draft_len, "draft_len"),
-                                   _dev_ptr(match_len, "match_len"), _dev_ptr(source, "source"),
-                                   _dev_ptr(state, "state"), _dev_ptr(status, "status"),
-                                   _dev_ptr(counts_out, "counts_out"), _dev_ptr(accepted_out, "accepted_out"),
-                                   _stream_ptr(stream)), "sam_step_verified")
+    m, fn = _hot("sam_step_verified")
+    _check(m.step_verified(fn, _addr(h), target_tokens, prev_draft_tokens.shape[1], prev_draft_tokens, prev_draft_len, max_new, L,
+                           draft_tokens, draft_len, match_len, source, state, status, counts_out, accepted_out,
+                           _stream_of(stream)), "sam_step_verified")
 
 
 def sam_select_auxiliary(draft_tokens, draft_len, source, aux_tokens, aux_len, stream=None):
     B, L = draft_tokens.shape
-    _check(lib().sam_select_auxiliary(B, L, _dev_ptr(draft_tokens, "draft_tokens"), _dev_ptr(draft_len, "draft_len"),
-                                      _dev_ptr(source, "source"), _dev_ptr(aux_tokens, "aux_tokens"),
-                                      _dev_ptr(aux_len, "aux_len"), _stream_ptr(stream)), "sam_select_auxiliary")
+    m, fn = _hot("sam_select_auxiliary")
+    _check(m.select_auxiliary(fn, B, L, draft_tokens, draft_len, source, aux_tokens, aux_len, _stream_of(stream)),
+           "sam_select_auxiliary")
 
 
 def sam_tree_draft(static_h, states, start_tokens, max_size: int, k: int, tree_tokens, tree_parents, tree_probs,
                    tree_size, stream=None):
-    import torch
-    pp = None
-    if tree_probs is not None:
-        assert tree_probs.is_cuda and tree_probs.dtype == torch.float32 and tree_probs.is_contiguous()
-        pp = tree_probs.data_ptr()
-    _check(lib().sam_tree_draft(static_h, states.shape[0], _dev_ptr(states, "states"),
-                                _dev_ptr(start_tokens, "start_tokens"), max_size, k,
-                                _dev_ptr(tree_tokens, "tree_tokens"), _dev_ptr(tree_parents, "tree_parents"), pp,
-                                _dev_ptr(tree_size, "tree_size"), _stream_ptr(stream)), "sam_tree_draft")
+    m, fn = _hot("sam_tree_draft")
+    _check(m.tree_draft(fn, _addr(static_h), states.shape[0], states, start_tokens, max_size, k, tree_tokens, tree_parents, tree_probs,
+                        tree_size, _stream_of(stream)), "sam_tree_draft")
 
 
 def sam_static_freq(h):
@@ -355,12 +377,9 @@ def sam_static_freq(h):
 def sam_retrieve_noalloc(static_h, vocab, tokens, counts, L, l_bias, min_match,
                          draft_tokens, draft_len, match_len, source, state, status, stream=None):
     """One-shot retrieval over the library's built-in scratch array; allocates nothing."""
-    _check(lib().sam_retrieve_noalloc(static_h, vocab, tokens.shape[0], _dev_ptr(tokens, "tokens"), tokens.shape[1],
-                                      _dev_ptr(counts, "counts"), L, l_bias, min_match,
-                                      _dev_ptr(draft_tokens, "draft_tokens"), _dev_ptr(draft_len, "draft_len"),
-                                      _dev_ptr(match_len, "match_len"), _dev_ptr(source, "source"),
-                                      _dev_ptr(state, "state"), _dev_ptr(status, "status"), _stream_ptr(stream)),
-           "sam_retrieve_noalloc")
+    m, fn = _hot("sam_retrieve_noalloc")
+    _check(m.retrieve_noalloc(fn, _addr(static_h), vocab, tokens.shape[0], tokens, tokens.shape[1], counts, L, l_bias, min_match,
+                              draft_tokens, draft_len, match_len, source, state, status, _stream_of(stream)), "sam_retrieve_noalloc")
 
 
 COUNTER_NAMES = ("static_rounds", "static_link_moves", "static_next_moves", "dynamic_rounds", "walk_inserts",
@@ -517,11 +536,15 @@ class Batch:
             self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
             self.handle = sam_batch_create(static.handle if static is not None else None, self.opts, self.workspace)
         self.batch, self.max_draft_len = batch, max_draft_len
+        m, self._step_fn = _hot("sam_step")
+        self._step_call, self._addr, self._stream = m.step_out, _addr(self.handle), -1 - dev
 
     def step(self, new_tokens, counts, L: int, out: StepOutputs | None = None) -> StepOutputs:
-        out = out or StepOutputs(self.batch, L, self.device)
-        with __import__("torch").cuda.device(self.device):
-            sam_step(self.handle, new_tokens, new_tokens.shape[-1], counts, L, *out.tensors())
+        if out is None:
+            out = StepOutputs(self.batch, L, self.device)
+        rc = self._step_call(self._step_fn, self._addr, new_tokens, counts, L, out, self._stream)
+        if rc != SAM_OK:
+            raise SamError(rc, "sam_step")
         return out
 
     def run_steps(self, new_tokens, counts, L: int, per_step: bool = True, out: StepOutputs | None = None):
@@ -548,7 +571,7 @@ class Batch:
     def close(self):
         if getattr(self, "handle", None):
             sam_batch_destroy(self.handle)
-            self.handle = None
+            self.handle, self._addr = None, 0
 
     def __del__(self):
         try:

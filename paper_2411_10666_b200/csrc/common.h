@@ -38,15 +38,15 @@ void sam_set_cuda_error(cudaError_t e);
         if (_e != cudaSuccess) { sam_set_cuda_error(_e); return SAM_ERR_CUDA; } \
     } while (0)
 
-// RAII device switch
+// RAII device switch (nothing is set where the device is the current one already)
 struct SamDeviceGuard {
     int prev = -1;
-    bool ok = true;
+    bool ok = true, switched = false;
     explicit SamDeviceGuard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        if (prev != dev) { if (cudaSetDevice(dev) == cudaSuccess) switched = true; else ok = false; }
     }
-    ~SamDeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+    ~SamDeviceGuard() { if (switched) cudaSetDevice(prev); }
 };
 
 static inline size_t sam_align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

@@ -1869,6 +1869,8 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
                          int32_t* done_flag_dev, int32_t done_seq,
                          const int32_t* v_draft, const int32_t* v_draft_len, const int32_t* v_max_new,
                          int32_t* v_counts_out, int32_t* v_accepted_out) {
+    SamDeviceGuard guard(b->device);
+    if (!guard.ok) return SAM_ERR_CUDA;
     StepArgs A;
     A.v_draft = v_draft; A.v_draft_len = v_draft_len; A.v_max_new = v_max_new;
     A.v_counts_out = v_counts_out; A.v_accepted_out = v_accepted_out;
@@ -1948,6 +1950,8 @@ constexpr int SAM_RUN_BLOCK_MAX_BATCH = 1036;
 int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps, int32_t L, int32_t keep,
                    int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status,
                    cudaStream_t stream) {
+    SamDeviceGuard guard(b->device);
+    if (!guard.ok) return SAM_ERR_CUDA;
     RunArgs R;
     memset(&R, 0, sizeof(R));
     StepArgs& A = R.A;
