@@ -167,9 +167,10 @@ def _dev_ptr(t, name: str):
 
 
 def _stream_ptr(stream=None):
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 # ---------------------------------------------------------------------------------------------

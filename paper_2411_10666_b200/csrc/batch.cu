@@ -52,7 +52,7 @@ int plan(const sam_batch_opts_t* o, WsLayout* w) {
     w->off_ctrl = off;  off = sam_align_up(off + (size_t)o->batch * SAM_CTRL_WORDS * 4, 256);
     w->off_free = off;  off = sam_align_up(off + (size_t)slabs * 4, 256);
     w->off_owner = off; off = sam_align_up(off + (size_t)slabs * 4, 256);
-    w->off_reset = off; off = sam_align_up(off + (size_t)o->batch * 4 * 2, 256);   // flags + slot list
+    w->off_reset = off; off = sam_align_up(off + (size_t)o->batch * 4, 256);
     w->off_order = off; off = sam_align_up(off + (size_t)o->batch * 4 * 3 + 64, 256);   // two order buffers, the sort keys, two counts
     w->off_text = off;  off = sam_align_up(off + (size_t)o->batch * w->text_stride * 4, 256);
     w->off_pstate = off; off = sam_align_up(off + (size_t)o->batch * w->text_stride * 4, 256);
@@ -65,47 +65,66 @@ int plan(const sam_batch_opts_t* o, WsLayout* w) {
 
 // ---- kernels ----------------------------------------------------------------
 
-__global__ void init_pool_kernel(SamBatchView W) {
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t s = i; s < (size_t)W.pool_slabs; s += stride) {
-        W.free_stack[s] = (int32_t)(W.pool_slabs - 1 - s);      // slab 0 is handed out first
-        W.slab_owner[s] = -1;
-    }
-    for (size_t b = i; b < (size_t)W.batch; b += stride) W.reset_flag[b] = 0;
-    if (i == 0) { W.pool_hdr[0] = W.pool_slabs; W.pool_hdr[1] = W.pool_slabs; W.pool_hdr[4] = 0; }
-}
+constexpr int RESET_THREADS = 128;
 
-// slots == nullptr: every slot.  Clears control blocks and root tables and raises reset flags.
-__global__ void reset_slots_kernel(SamBatchView W, const int32_t* slots, int32_t n) {
-    const int which = blockIdx.x;
-    if (which >= n) return;
-    const int b = slots ? slots[which] : which;
-    if (b < 0 || b >= W.batch) return;
+__device__ __forceinline__ void clear_slot(const SamBatchView& W, int b) {
     uint32_t* cb = W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     for (int i = threadIdx.x; i < SAM_CTRL_WORDS; i += blockDim.x) cb[i] = 0;
-    uint2* root = W.root_tab + (size_t)b * W.root_cap;
-    for (int i = threadIdx.x; i < W.root_cap; i += blockDim.x) root[i] = make_uint2(SAM_NONE, 0);
-    if (threadIdx.x == 0) W.reset_flag[b] = 1;
+    // (two empty root-table entries per store; the capacity is a multiple of 64)
+    uint4* root = reinterpret_cast<uint4*>(W.root_tab + (size_t)b * W.root_cap);
+    for (int i = threadIdx.x; i < W.root_cap / 2; i += blockDim.x) root[i] = make_uint4(SAM_NONE, 0, SAM_NONE, 0);
 }
 
-// give the slabs of flagged slots back to the pool
-__global__ void release_slabs_kernel(SamBatchView W) {
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t s = i; s < (size_t)W.pool_slabs; s += stride) {
-        int owner = W.slab_owner[s];
-        if (owner >= 0 && W.reset_flag[owner]) {
+// Every slot empty, every slab free: a new batch, or a reset of all of it.  One launch: block b clears slot b, and all
+// blocks together rewrite the pool's free stack and owners (nothing of the pool is in use afterwards).
+__global__ void __launch_bounds__(RESET_THREADS) init_batch_kernel(SamBatchView W) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    for (int s = i; s < W.pool_slabs; s += stride) {
+        W.free_stack[s] = W.pool_slabs - 1 - s;                 // slab 0 is handed out first
+        W.slab_owner[s] = -1;
+    }
+    if (threadIdx.x == 0) W.reset_mark[blockIdx.x] = 0;
+    if (i == 0) { W.pool_hdr[0] = W.pool_slabs; W.pool_hdr[1] = W.pool_slabs; W.pool_hdr[4] = 0; }
+    clear_slot(W, blockIdx.x);
+}
+
+// Some slots: clear them and mark them with this reset's number; the second kernel gives the slabs of slots that carry it
+// back to the pool.  The slots come with the launch, so nothing is copied and nobody waits.
+constexpr int RESET_LIST = 900;                                 // 4 KB of launch arguments hold them
+struct ResetList { int32_t slot[RESET_LIST]; };
+
+__global__ void __launch_bounds__(RESET_THREADS) reset_slots_kernel(SamBatchView W, const __grid_constant__ ResetList list, int32_t mark) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int b = list.slot[blockIdx.x];
+    clear_slot(W, b);
+    if (threadIdx.x == 0) W.reset_mark[b] = mark;
+}
+
+__global__ void release_slabs_kernel(SamBatchView W, int32_t mark) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    for (int s = i; s < W.pool_slabs; s += stride) {
+        const int owner = W.slab_owner[s];
+        if (owner >= 0 && W.reset_mark[owner] == mark) {
             W.slab_owner[s] = -1;
-            int pos = atomicAdd(W.pool_hdr, 1);
-            W.free_stack[pos] = (int32_t)s;
+            W.free_stack[atomicAdd(W.pool_hdr, 1)] = s;
         }
     }
 }
 
-__global__ void clear_flags_kernel(SamBatchView W) {
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i < (size_t)W.batch) W.reset_flag[i] = 0;
+template <class K, class... Args>
+cudaError_t launch_after(K kernel, int blocks, int threads, cudaStream_t s, Args... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3((unsigned)threads); cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // one warp copies a slot's automaton into flat arrays
@@ -174,7 +193,7 @@ int sam_plan_view(const sam_batch_opts_t* opts, int32_t vocab, void* base, SamBa
         view->ctrl = (uint32_t*)(b + w.off_ctrl);
         view->free_stack = (int32_t*)(b + w.off_free);
         view->slab_owner = (int32_t*)(b + w.off_owner);
-        view->reset_flag = (int32_t*)(b + w.off_reset);
+        view->reset_mark = (int32_t*)(b + w.off_reset);
         view->order = (int32_t*)(b + w.off_order);
         view->text = (int32_t*)(b + w.off_text);
         view->pstate = (uint32_t*)(b + w.off_pstate);
@@ -193,10 +212,7 @@ int sam_plan_view(const sam_batch_opts_t* opts, int32_t vocab, void* base, SamBa
 
 // Put every slot of the view into the empty state and fill the slab pool's free stack.
 int sam_launch_init(const SamBatchView& V, cudaStream_t s) {
-    init_pool_kernel<<<296, 256, 0, s>>>(V);
-    reset_slots_kernel<<<V.batch, 128, 0, s>>>(V, nullptr, V.batch);
-    clear_flags_kernel<<<(V.batch + 255) / 256, 256, 0, s>>>(V);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_after(init_batch_kernel, V.batch, RESET_THREADS, s, V);
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;
 }
@@ -242,7 +258,7 @@ extern "C" int sam_batch_create(const sam_static_t* st, const sam_batch_opts_t* 
     V.ctrl = (uint32_t*)(base + w.off_ctrl);
     V.free_stack = (int32_t*)(base + w.off_free);
     V.slab_owner = (int32_t*)(base + w.off_owner);
-    V.reset_flag = (int32_t*)(base + w.off_reset);
+    V.reset_mark = (int32_t*)(base + w.off_reset);
     V.order = (int32_t*)(base + w.off_order);
     V.text = (int32_t*)(base + w.off_text);
     V.pstate = (uint32_t*)(base + w.off_pstate);
@@ -268,11 +284,7 @@ extern "C" int sam_batch_create(const sam_static_t* st, const sam_batch_opts_t* 
     }
     b->host_stage[w.stage_words] = 0;
     cudaStream_t s = (cudaStream_t)stream;
-    init_pool_kernel<<<296, 256, 0, s>>>(V);
-    reset_slots_kernel<<<V.batch, 128, 0, s>>>(V, nullptr, V.batch);
-    clear_flags_kernel<<<(V.batch + 255) / 256, 256, 0, s>>>(V);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) { sam_set_cuda_error(e); cudaFreeHost(b->host_stage); delete b; return SAM_ERR_CUDA; }
+    if (sam_launch_init(V, s) != SAM_OK) { cudaFreeHost(b->host_stage); delete b; return SAM_ERR_CUDA; }
     *out = b;
     return SAM_OK;
 }
@@ -291,20 +303,19 @@ extern "C" int sam_batch_reset(sam_batch_t* b, const int32_t* slots_host, int32_
     if (!guard.ok) return SAM_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     const SamBatchView& V = b->view;
-    if (!slots_host) {
-        reset_slots_kernel<<<V.batch, 128, 0, s>>>(V, nullptr, V.batch);
-    } else {
-        if (n > V.batch) return SAM_ERR_ARG;
-        for (int32_t i = 0; i < n; i++) if (slots_host[i] < 0 || slots_host[i] >= V.batch) return SAM_ERR_ARG;
-        if (n == 0) return SAM_OK;
-        int32_t* list_dev = V.reset_flag + V.batch;           // second half of the reset area
-        SAM_CUDA(cudaMemcpyAsync(list_dev, slots_host, (size_t)n * 4, cudaMemcpyHostToDevice, s));
-        reset_slots_kernel<<<n, 128, 0, s>>>(V, list_dev, n);
+    if (!slots_host) return sam_launch_init(V, s);
+    if (n > V.batch) return SAM_ERR_ARG;
+    for (int32_t i = 0; i < n; i++) if (slots_host[i] < 0 || slots_host[i] >= V.batch) return SAM_ERR_ARG;
+    if (n == 0) return SAM_OK;
+    if (++b->reset_count <= 0) b->reset_count = 1;              // never 0, a slot's mark before its first reset
+    for (int32_t at = 0; at < n; at += RESET_LIST) {
+        ResetList list;
+        const int32_t m = n - at < RESET_LIST ? n - at : RESET_LIST;
+        memcpy(list.slot, slots_host + at, (size_t)m * 4);
+        SAM_CUDA(launch_after(reset_slots_kernel, m, RESET_THREADS, s, V, list, b->reset_count));
     }
-    release_slabs_kernel<<<296, 256, 0, s>>>(V);
-    clear_flags_kernel<<<(V.batch + 255) / 256, 256, 0, s>>>(V);
-    SAM_CUDA(cudaGetLastError());
-    if (slots_host) SAM_CUDA(cudaStreamSynchronize(s));        // the caller's list may be reused at once
+    const int blocks = (V.pool_slabs + 255) / 256;
+    SAM_CUDA(launch_after(release_slabs_kernel, blocks < 592 ? blocks : 592, 256, s, V, b->reset_count));
     return SAM_OK;
 }
 

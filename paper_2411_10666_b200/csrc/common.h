@@ -27,6 +27,7 @@ struct sam_batch {
     int32_t* host_stage;          // pinned, device-mapped host staging area
     int32_t* host_stage_dev;      // the same memory as the device addresses it
     int32_t host_seq;             // sequence number of the last host-array step (completion flag value)
+    int32_t reset_count;          // number of the last reset of some slots
     mutable int32_t order_phase;  // which of the two slot-order buffers the next large-batch step uses
 };
 

@@ -129,7 +129,7 @@ struct SamBatchView {
     int32_t* pool_hdr;        // [0] free slabs, [1] total slabs
     int32_t* free_stack;      // [pool_slabs]
     int32_t* slab_owner;      // [pool_slabs], -1 = free
-    int32_t* reset_flag;      // [B]
+    int32_t* reset_mark;      // [B]: number of the last reset that named the slot
     int32_t* order;           // [3][B] + 16: slots sorted by their step's token count (large batches), two buffers in turn; the sort keys; per buffer, at 3B + 8 x buffer, the number of slots with many tokens
     int32_t* text;            // [B][text_stride]
     uint32_t* pstate;         // [B][text_stride]: id of the state created by each text position

@@ -4,21 +4,22 @@
 // (64 slots x 1024 tokens: 550 us, and 5.8 ms for one slot of 8191).  What it ends with is a function of the text alone,
 // and all of it can be read off the sorted order of the text's prefixes:
 //   - prefixes are sorted by their tokens from the last to the first; A[j] is the end position of the j-th, h[j]
-//     the length of the suffix it shares with its predecessor.  Sorting is by prefix doubling (ranks of 1, 4, 16,
-//     ... tokens), so a repeated passage of k tokens costs log4(k) sorts whatever the text is;
-//   - l[p], the longest suffix of prefix p that ends anywhere earlier, comes from p's nearest neighbours in
-//     sorted order with smaller end positions; e[p] is where that suffix ends first;
-//   - Expand of token p makes state c_p (the whole prefix) and, exactly if no state has that suffix as its
-//     longest string yet, one clone cl_p with length l[p] and first end position e[p].  A suffix is known by the
-//     interval of sorted positions that share it, the interval by the boundary inside it where h is smallest: the
-//     first p to claim a boundary makes the clone.  State ids follow by counting clones;
-//   - a state's suffix link is the interval around it with the next smaller length;
+//     the length of the suffix it shares with its predecessor.  Sorting is by prefix doubling: the first sort compares as many
+//     tokens as fit a 64-bit key, each further round four times as many, within groups of equal prefixes only;
+//   - the strings that are suffixes of the same set of prefixes form an interval of the sorted order.  An interval is
+//     named by the first boundary inside it where h is smallest; its length is that h, its first end position the
+//     smallest A in it, its parent the interval at the larger h just outside;
+//   - l[p], the longest suffix of prefix p that ends anywhere earlier, is the nearest interval around p that a smaller
+//     end position belongs to.  Expand of token p makes state c_p (the whole prefix) and, exactly if no state has that
+//     suffix as its longest string yet, one clone: the first p to claim an interval makes it.  State ids follow by
+//     counting clones;
+//   - suffix links are the parents;
 //   - the transitions into a state u (longest string w, link of length k) are those on w's last token from the states
 //     along the suffix links of w without that token, down to length k.
-// Nothing here depends on a guess: each of the five statements is the definition of the automaton of the text.
+// Nothing here depends on a guess: each of these statements is the definition of the automaton of the text.
 //
-// What bounds it: one block's chain of some 60 barriers and shared-memory searches (everything but the outputs
-// stays in shared memory, 28 bytes per token).
+// What bounds it: for short texts the chain of some 50 barriers, for long ones one SM's shared memory (everything but the
+// outputs stays there, 28 bytes per token).
 #pragma once
 #include "common.h"
 
@@ -32,30 +33,38 @@ constexpr uint32_t PB_ROOT = 0xFFFFu;      // handle of the root; a state is (p 
 
 struct PbShared {                          // what the threads of one build exchange besides the arrays
     int16_t chunk[PB_MAX / 32];
-    uint32_t rec_slab[SAM_MAX_REC_SLABS], blk_slab[PB_BLOCK_SLABS];
+    uint32_t slab[SAM_MAX_REC_SLABS + PB_BLOCK_SLABS];       // of the records, then of the edge blocks
     uint32_t cls_n[16], cls_base[16];
-    int groups, clones, root_deg, err, n_rec_slabs, n_blk_units;
+    int groups, clones, root_deg, err, n_rec_slabs;
 };
 
 struct PbArrays {
-    uint64_t* key;                         // sorting; its place is taken by `tree`
-    uint16_t* lev; uint16_t* A; uint16_t* H;                       // while sorting
-    uint32_t* tree; uint16_t* rank; uint16_t* L; uint16_t* E; uint16_t* idc;
-    uint32_t* first; uint16_t* link; uint32_t* deg;
+    uint64_t* key; uint16_t* lev; uint16_t* A; uint16_t* B; uint32_t* tok;      // while sorting
+    uint32_t* tree; uint16_t* rank; uint16_t* canon; uint16_t* enode; uint16_t* parent;
+    uint32_t* first; uint16_t* wnode; uint16_t* idc; uint16_t* link; uint32_t* deg;
     int N2;                                // size of the sorted order, a power of two
 };
 
+// `tree`: leaves in its upper half; `link` takes the place of the inner nodes when they are no longer needed.
 __device__ __forceinline__ PbArrays pb_arrays(unsigned char* sm, int N2) {
     PbArrays a;
     const size_t n = (size_t)N2;
     a.N2 = N2;
-    a.key = (uint64_t*)sm; a.lev = (uint16_t*)(sm + 8 * n); a.A = (uint16_t*)(sm + 20 * n); a.H = (uint16_t*)(sm + 22 * n);
-    a.tree = (uint32_t*)sm; a.rank = (uint16_t*)(sm + 8 * n); a.L = (uint16_t*)(sm + 10 * n); a.E = (uint16_t*)(sm + 12 * n);
-    a.idc = (uint16_t*)(sm + 14 * n); a.first = (uint32_t*)(sm + 16 * n); a.link = (uint16_t*)(sm + 20 * n); a.deg = (uint32_t*)(sm + 24 * n);
+    a.key = (uint64_t*)sm; a.lev = (uint16_t*)(sm + 8 * n); a.A = (uint16_t*)(sm + 20 * n); a.B = (uint16_t*)(sm + 22 * n);
+    a.tok = (uint32_t*)(sm + 24 * n);
+    a.tree = (uint32_t*)sm; a.link = (uint16_t*)sm; a.rank = (uint16_t*)(sm + 8 * n); a.canon = (uint16_t*)(sm + 10 * n);
+    a.enode = (uint16_t*)(sm + 12 * n); a.parent = (uint16_t*)(sm + 14 * n); a.first = (uint32_t*)(sm + 16 * n);
+    a.wnode = (uint16_t*)(sm + 20 * n); a.idc = (uint16_t*)(sm + 22 * n); a.deg = (uint32_t*)(sm + 24 * n);
     return a;
 }
+__device__ __forceinline__ int pb_size(int n) { return n <= 64 ? 64 : 1 << (32 - __clz(n - 1)); }
 
 __device__ __forceinline__ void pb_sync(int nt) { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); }
+__device__ __forceinline__ bool pb_sync_or(int nt, bool x) {
+    uint32_t r;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %2, 0; bar.red.or.pred q, 1, %1, p; selp.u32 %0, 1, 0, q; }" : "=r"(r) : "r"(nt), "r"((uint32_t)x) : "memory");
+    return r != 0;
+}
 
 __device__ __forceinline__ uint64_t pb_shfl_xor(uint64_t v, int s) {
     const uint32_t lo = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)v, s), hi = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)(v >> 32), s);
@@ -71,7 +80,22 @@ __device__ __forceinline__ void pb_step(uint64_t& v, int lane, int stride, bool 
 __device__ void pb_sort(uint64_t* key, int N2, int tid, int nt) {
     const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
     for (int size = 64; size <= N2; size <<= 1) {
-        for (int stride = size >> 1; stride >= 64; stride >>= 1) {
+        int stride = size >> 1;
+        for (; stride >= 128; stride >>= 2) {              // two strides a pass
+            const int half = stride >> 1;
+            for (int q = tid; q < (N2 >> 2); q += nt) {
+                const int i = ((q & ~(half - 1)) << 2) | (q & (half - 1));
+                const bool up = (i & size) == 0;
+                uint64_t x0 = key[i], x1 = key[i + half], x2 = key[i + stride], x3 = key[i + stride + half], t;
+                if ((x0 > x2) == up) { t = x0; x0 = x2; x2 = t; }
+                if ((x1 > x3) == up) { t = x1; x1 = x3; x3 = t; }
+                if ((x0 > x1) == up) { t = x0; x0 = x1; x1 = t; }
+                if ((x2 > x3) == up) { t = x2; x2 = x3; x3 = t; }
+                key[i] = x0; key[i + half] = x1; key[i + stride] = x2; key[i + stride + half] = x3;
+            }
+            pb_sync(nt);
+        }
+        for (; stride >= 64; stride >>= 1) {
             for (int q = tid; q < (N2 >> 1); q += nt) {
                 const int i = ((q & ~(stride - 1)) << 1) | (q & (stride - 1)), k = i + stride;
                 const uint64_t x = key[i], y = key[k];
@@ -173,89 +197,35 @@ __device__ __forceinline__ int pb_right(const PbArrays& a, int j, uint32_t l, ui
 }
 __device__ __forceinline__ uint32_t pb_h(const PbArrays& a, int j) { return j < a.N2 ? a.tree[a.N2 + j] >> 16 : 0u; }
 
-// Length of the suffix that p (at sorted position j) shares with its nearest neighbour on one side with a smaller end position.
-__device__ __forceinline__ uint32_t pb_earlier_left(const PbArrays& a, int j, uint32_t p) {
-    if (j == 0) return 0;
-    uint32_t m = pb_h(a, j);
-    int i = a.N2 + j - 1;
-    while (m) {
-        const uint32_t v = a.tree[i];
-        if ((v & 0xFFFFu) < p) {
-            while (i < a.N2) {
-                const uint32_t r = a.tree[2 * i + 1];
-                if ((r & 0xFFFFu) < p) i = 2 * i + 1;
-                else { m = min(m, r >> 16); i = 2 * i; }
-            }
-            return m;
-        }
-        m = min(m, v >> 16);
-        while (!(i & 1)) i >>= 1;
-        if (i == 1) return 0;
-        i -= 1;
-    }
-    return 0;
+// The interval that prefix p is alone in the middle of: the larger h on its two sides (0: none but the root).
+__device__ __forceinline__ uint32_t pb_leaf(const PbArrays& a, uint32_t p) {
+    const int j = a.rank[p];
+    const uint32_t hl = pb_h(a, j), hr = pb_h(a, j + 1);
+    return max(hl, hr) == 0 ? 0u : a.canon[hl >= hr ? j : j + 1];
 }
-__device__ __forceinline__ uint32_t pb_earlier_right(const PbArrays& a, int j, uint32_t p) {
-    if (j + 1 >= a.N2) return 0;
-    uint32_t m = 0xFFFFu;
-    int i = a.N2 + j + 1;
-    while (m) {
-        const uint32_t v = a.tree[i];
-        if ((v & 0xFFFFu) < p) {
-            while (i < a.N2) {
-                const uint32_t x = a.tree[2 * i];
-                if ((x & 0xFFFFu) < p) i = 2 * i;
-                else { m = min(m, x >> 16); i = 2 * i + 1; }
-            }
-            return min(m, a.tree[i] >> 16);
-        }
-        m = min(m, v >> 16);
-        while (i & 1) i >>= 1;
-        if (i == 0) return 0;
-        i += 1;
-    }
-    return 0;
-}
-
-struct PbNode { int lo; uint32_t len, e, up; };            // interval of the strings of length `len` around a prefix: where it
-                                                           // begins, its smallest end position, the length of its suffix link
-__device__ __forceinline__ PbNode pb_node(const PbArrays& a, int j, uint32_t len) {
-    PbNode x;
-    uint32_t e = 0xFFFFu;
-    x.lo = pb_left(a, j, len, e);
-    const int r = pb_right(a, j, len, e);
-    x.len = len; x.e = e;
-    x.up = max(pb_h(a, x.lo), pb_h(a, r));
-    return x;
-}
-// The boundary that names the interval: the first one inside it where h is as small as `len`.
-__device__ __forceinline__ int pb_boundary(const PbArrays& a, int lo, uint32_t len) {
-    uint32_t unused = 0xFFFFu;
-    return pb_right(a, lo, len + 1, unused);
-}
-__device__ __forceinline__ uint32_t pb_handle(const PbArrays& a, const PbNode& x) {
-    if (x.e + 1 == x.len) return x.e << 1;
-    const uint32_t p = a.first[pb_boundary(a, x.lo, x.len)];
-    return p == 0xFFFFFFFFu ? PB_ROOT : p << 1 | 1u;       // (every interval has been claimed)
-}
+__device__ __forceinline__ bool pb_clones(const PbArrays& a, uint32_t p) { return (a.wnode[p] & 0x8000u) != 0; }
 __device__ __forceinline__ uint32_t pb_len(const PbArrays& a, uint32_t hd) {
-    return hd == PB_ROOT ? 0u : (hd & 1) ? (uint32_t)(a.L[hd >> 1] & 0x7FFF) : (hd >> 1) + 1;
+    return hd == PB_ROOT ? 0u : (hd & 1) ? pb_h(a, a.wnode[hd >> 1] & 0x7FFF) : (hd >> 1) + 1;
 }
+__device__ __forceinline__ uint32_t pb_end(const PbArrays& a, uint32_t hd) { return (hd & 1) ? a.enode[a.wnode[hd >> 1] & 0x7FFF] : hd >> 1; }
 __device__ __forceinline__ uint32_t pb_id(const PbArrays& a, uint32_t hd) { return hd == PB_ROOT ? 0u : a.idc[hd >> 1] + (hd & 1); }
+__device__ __forceinline__ uint32_t pb_state(const PbArrays& a, uint32_t node) { return node == 0 ? PB_ROOT : a.first[node]; }
 
 // Visit every transition into state u = (p, clone): f(source handle, solid).
 template <class F>
 __device__ __forceinline__ void pb_into(const PbArrays& a, uint32_t u, F f) {
     const uint32_t p = u >> 1;
     const uint32_t len = pb_len(a, u), low = pb_len(a, a.link[u]);
-    uint32_t v = PB_ROOT;
+    uint32_t v = PB_ROOT, lv = 0;
     if (len > 1) {
         if (!(u & 1)) v = (p - 1) << 1;
-        else v = pb_handle(a, pb_node(a, a.rank[a.E[p] - 1], len - 1));
+        else {                                             // a suffix of what prefix p - 1 had in common with an earlier one
+            v = pb_state(a, a.wnode[p - 1] & 0x7FFFu);
+            while (v != PB_ROOT && pb_len(a, v) >= len) v = a.link[v];
+        }
+        lv = pb_len(a, v);
     }
-    for (uint32_t below = len;;) {
-        const uint32_t lv = pb_len(a, v);
-        if (lv < low || lv >= below) break;                // (lengths fall along suffix links)
+    for (uint32_t below = len; lv >= low && lv < below; lv = pb_len(a, v)) {        // (lengths fall along suffix links)
         below = lv;
         f(v, lv + 1 == len);
         if (v == PB_ROOT) break;
@@ -282,54 +252,104 @@ __device__ __forceinline__ uint32_t pb_take_slabs(const SamBatchView& W, int wan
 
 struct PbResult { int32_t s2, l2, e2; int err; };
 
-// The automaton of toks[0, n) for the empty slot b: every record, transition and table entry Expand would leave, and the
-// dynamic words of the slot's control block.  Run by nt threads (tid 0 .. nt - 1, whole warps, barrier 1); the
-// result is valid in all of them.  The tokens have been checked; 1 < n <= PB_MAX.
-__device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, const int32_t* toks, int n, unsigned char* smem,
+// One round of the sort: order the members of each group of equal prefixes (of `span` tokens) by the tokens before those, by
+// counting how many of the group come first.  A -> B, rank -> next.  Returns the number of groups.
+__device__ int pb_refine(const PbArrays& a, PbShared& sh, const uint16_t* A, uint16_t* B, const uint16_t* rank, uint16_t* next, int span, int n,
+                         int tid, int nt) {
+    for (int j = tid; j < n; j += nt) {
+        const int p = A[j];
+        uint64_t k = 0;
+#pragma unroll
+        for (int q = 1; q < 4; q++) { const int at = p - q * span; k = k << 16 | (at >= 0 ? (uint32_t)rank[at] + 1u : 0u); }
+        a.key[j] = k;
+    }
+    if (tid == 0) sh.groups = 0;
+    pb_sync(nt);
+    int mine = 0;
+    for (int j = tid; j < n; j += nt) {
+        const int p = A[j], g = rank[p];
+        const uint64_t k = a.key[j];
+        int less = 0, same = 0;
+        for (int i = g; i < n && rank[A[i]] == g; i++) {
+            const uint64_t x = a.key[i];
+            less += x < k; same += x == k && i < j;
+        }
+        B[g + less + same] = (uint16_t)p;
+        next[p] = (uint16_t)(g + less);
+        mine += same == 0;
+    }
+    mine = __reduce_add_sync(0xFFFFFFFFu, mine);
+    if ((tid & 31) == 0) atomicAdd(&sh.groups, mine);
+    pb_sync(nt);
+    return sh.groups;
+}
+
+// The automaton of a text of n tokens for the empty slot b: every record, transition and table entry Expand would
+// leave, and the dynamic words of the slot's control block.  Run by nt threads (tid 0 .. nt - 1, whole warps, barrier 1);
+// the result is valid in all of them.  The tokens have been checked and lie in the slot's text and in the `tok` array;
+// 1 < n <= PB_MAX.
+__device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int vocab, int n, unsigned char* smem,
                          PbShared& sh, int tid, int nt, PbResult& out) {
     const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
-    const int N2 = n <= 64 ? 64 : 1 << (32 - __clz(n - 1));
+    const int N2 = pb_size(n);
     const PbArrays a = pb_arrays(smem, N2);
-    int32_t* text = W.text + (size_t)b * W.text_stride;
-    const int ib = 32 - __clz(n - 1), rb = 32 - __clz(n);  // bits of a position, and of a rank plus one
-    const int parts = min(4, (64 - ib) / rb);
+    const int32_t* text = W.text + (size_t)b * W.text_stride;
+    const int ib = 32 - __clz(n - 1), rb = 32 - __clz(n), vb = 32 - __clz(vocab);      // bits of a position, a rank plus one, a token plus one
+    const uint32_t im = (1u << ib) - 1u;
 
     // ---- sort
+    const int span0 = min(4, (64 - ib) / vb);              // (at least one token: 13 + 31 bits)
     for (int j = tid; j < N2; j += nt) {
         uint64_t k = ~0ull;
-        if (j < n) { const int32_t t = toks[j]; text[j] = t; k = (uint64_t)(uint32_t)t << ib | (uint32_t)j; }
+        if (j < n) {
+            k = 0;
+            for (int q = 0; q < span0; q++) k = k << vb | (j - q >= 0 ? a.tok[j - q] + 1u : 0u);
+            k = k << ib | (uint32_t)j;
+        }
         a.key[j] = k;
     }
     pb_sync(nt);
     pb_sort(a.key, N2, tid, nt);
-    int top = 0, span = 1;                                 // rank level, and the tokens its ranks compare
+    uint16_t *A = a.A, *B = a.B;
+    int top = 0, span = span0;                             // rank level, and the tokens its ranks compare
     int spans[PB_LEVELS];
 #pragma unroll
-    for (int i = 0; i < PB_LEVELS; i++) spans[i] = 1;
+    for (int i = 0; i < PB_LEVELS; i++) spans[i] = span0;
+    for (int j = tid; j < n; j += nt) A[j] = (uint16_t)((uint32_t)a.key[j] & im);
     int groups = pb_rank(a, sh, a.lev, n, ib, tid, nt);
     while (groups < n && span < n) {                       // (ranks of n tokens are all different)
         const uint16_t* r = a.lev + (size_t)top * N2;
-        for (int j = tid; j < n; j += nt) {
-            uint64_t k = r[j];
-            for (int q = 1; q < parts; q++) { const int at = j - q * span; k = k << rb | (at >= 0 ? (uint32_t)r[at] + 1u : 0u); }
-            a.key[j] = k << ib | (uint32_t)j;
+        bool large = false;                                // groups of over 64: counting would take too long
+        for (int j = tid; j + 64 < n; j += nt) large |= r[A[j]] == r[A[j + 64]];
+        const int to = top < PB_LEVELS - 1 ? top + 1 : top;                          // the last array is used again for longer spans
+        if (pb_sync_or(nt, large) || to == top) {
+            const int parts = min(4, (64 - ib) / rb);
+            for (int j = tid; j < n; j += nt) {
+                uint64_t k = r[j];
+                for (int q = 1; q < parts; q++) { const int at = j - q * span; k = k << rb | (at >= 0 ? (uint32_t)r[at] + 1u : 0u); }
+                a.key[j] = k << ib | (uint32_t)j;
+            }
+            for (int j = n + tid; j < N2; j += nt) a.key[j] = ~0ull;
+            pb_sync(nt);
+            pb_sort(a.key, N2, tid, nt);
+            for (int j = tid; j < n; j += nt) A[j] = (uint16_t)((uint32_t)a.key[j] & im);
+            groups = pb_rank(a, sh, a.lev + (size_t)to * N2, n, ib, tid, nt);
+            span *= parts;
+        } else {
+            groups = pb_refine(a, sh, A, B, r, a.lev + (size_t)to * N2, span, n, tid, nt);
+            uint16_t* t = A; A = B; B = t;
+            span *= 4;
         }
-        for (int j = n + tid; j < N2; j += nt) a.key[j] = ~0ull;
-        pb_sync(nt);
-        pb_sort(a.key, N2, tid, nt);
-        span *= parts;
-        if (top < PB_LEVELS - 1) top++;                    // the last array is used again for longer spans
+        top = to;
 #pragma unroll
         for (int i = 0; i < PB_LEVELS; i++) if (i == top) spans[i] = span;
-        groups = pb_rank(a, sh, a.lev + (size_t)top * N2, n, ib, tid, nt);
     }
     // ---- sorted order, shared suffix lengths
-    const uint32_t im = (1u << ib) - 1u;
-    for (int j = tid; j < n; j += nt) {
-        const int p = (int)((uint32_t)a.key[j] & im);
-        int x = 0;
-        if (j > 0) {
-            const int q = (int)((uint32_t)a.key[j - 1] & im);
+    for (int j = tid; j < N2; j += nt) {
+        int x = 0, p = 0xFFFF;
+        if (j < n) p = A[j];
+        if (j > 0 && j < n) {
+            const int q = A[j - 1];
 #pragma unroll
             for (int i = PB_LEVELS - 1; i >= 0; i--) {
                 if (i <= top) {
@@ -337,43 +357,68 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, const int32
                     while (p - x >= 0 && q - x >= 0 && r[p - x] == r[q - x]) x += spans[i];
                 }
             }
+            while (p - x >= 0 && q - x >= 0 && a.tok[p - x] == a.tok[q - x]) x++;
         }
-        a.A[j] = (uint16_t)p; a.H[j] = (uint16_t)x;
+        a.tree[N2 + j] = (uint32_t)x << 16 | (uint32_t)p;
     }
     pb_sync(nt);
-    for (int j = tid; j < N2; j += nt) a.tree[N2 + j] = j < n ? (uint32_t)a.H[j] << 16 | a.A[j] : 0xFFFFu;
-    pb_sync(nt);
-    for (int j = tid; j < n; j += nt) { a.rank[a.A[j]] = (uint16_t)j; }
+    for (int j = tid; j < n; j += nt) a.rank[A[j]] = (uint16_t)j;
     for (int width = N2 >> 1; width >= 1; width >>= 1) {
         for (int i = tid; i < width; i += nt) a.tree[width + i] = __vminu2(a.tree[2 * (width + i)], a.tree[2 * (width + i) + 1]);
         if (width > 32) pb_sync(nt); else __syncwarp();      // the last levels are warp 0's alone
     }
+    for (int j = tid; j < N2; j += nt) { a.first[j] = 0xFFFFFFFFu; a.deg[j] = 0; }
+    if (tid == 0) { sh.root_deg = 0; sh.err = 0; }
+    if (tid < 16) sh.cls_n[tid] = 0;
+    pb_sync(nt);
+
+    // ---- intervals
+    for (int j = tid; j < n; j += nt) {
+        const uint32_t l = pb_h(a, j);
+        uint32_t c = 0;
+        if (l > 0) {
+            uint32_t e = 0xFFFFu;
+            const int i = pb_left(a, j - 1, l + 1, e);
+            c = (uint32_t)i;                               // a boundary to the left with the same h: the same interval
+            const uint32_t hi = pb_h(a, i);
+            if (hi < l) {
+                e = min(e, a.tree[N2 + j] & 0xFFFFu);
+                const int r = pb_right(a, j, l, e);
+                const uint32_t hr = pb_h(a, r);
+                a.enode[j] = (uint16_t)e;
+                a.parent[j] = (uint16_t)(hi == 0 && hr == 0 ? 0 : hi >= hr ? i : r);
+                c = (uint32_t)j;
+            }
+        }
+        a.canon[j] = (uint16_t)c;
+    }
+    for (bool moved = true; moved;) {                      // each boundary to the first of its interval, jumping over jumps
+        pb_sync(nt);
+        bool m = false;
+        for (int j = tid; j < n; j += nt) {
+            const uint32_t c = a.canon[j], d = a.canon[c];
+            if (c != d) { a.canon[j] = (uint16_t)d; m = true; }
+        }
+        moved = pb_sync_or(nt, m);
+    }
+    for (int j = tid; j < n; j += nt) if (j > 0 && a.canon[j] == j) a.parent[j] = a.canon[a.parent[j]];
     pb_sync(nt);
 
     // ---- longest suffixes that end earlier; who clones
-    for (int j = tid; j < N2; j += nt) a.first[j] = 0xFFFFFFFFu;
-    if (tid == 0) { sh.root_deg = 0; sh.err = 0; sh.n_blk_units = 0; }
-    if (tid < 16) sh.cls_n[tid] = 0;
-    pb_sync(nt);
     for (int p = tid; p < n; p += nt) {
-        const int j = a.rank[p];
-        const uint32_t l = max(pb_earlier_left(a, j, (uint32_t)p), pb_earlier_right(a, j, (uint32_t)p));
-        uint32_t e = 0, r = 0;
-        if (l > 0) {
-            const PbNode x = pb_node(a, j, l);
-            e = x.e;
-            if (e + 1 != l) { r = (uint32_t)pb_boundary(a, x.lo, l); atomicMin(&a.first[r], (uint32_t)p); }
-        }
-        a.L[p] = (uint16_t)l; a.E[p] = (uint16_t)e; a.link[p] = (uint16_t)r;        // (link holds the boundary for now)
-        a.deg[p] = 0;
+        uint32_t x = pb_leaf(a, (uint32_t)p);
+        while (x != 0 && a.enode[x] == p) x = a.parent[x]; // (as many rounds in all as there are intervals)
+        a.wnode[p] = (uint16_t)x;
+        if (x != 0 && a.enode[x] + 1u != pb_h(a, (int)x)) atomicMin(&a.first[x], (uint32_t)p);
     }
     pb_sync(nt);
     const int chunks = (n + 31) >> 5;
     for (int c = w; c < chunks; c += nw) {
         const int p = 32 * c + lane;
-        const bool cl = p < n && a.link[p] != 0 && a.first[a.link[p]] == (uint32_t)p;
+        const uint32_t x = p < n ? a.wnode[p] : 0u;
+        const bool cl = x != 0 && a.first[x] == (uint32_t)p;
         const unsigned mask = __ballot_sync(0xFFFFFFFFu, cl);
-        if (cl) a.L[p] |= 0x8000u;
+        if (cl) a.wnode[p] = (uint16_t)(x | 0x8000u);
         if (lane == 0) sh.chunk[c] = (int16_t)__popc(mask);
     }
     pb_sync(nt);
@@ -387,45 +432,35 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, const int32
             if (base + lane < chunks) sh.chunk[base + lane] = (int16_t)(run + s - v);
             run += __shfl_sync(0xFFFFFFFFu, s, 31);
         }
-        const int n_states = 1 + n + run;
-        int err = 0;
-        const int want = ((n_states - 1) >> (W.slab_shift - 5)) + 1;
-        if (want > SAM_MAX_REC_SLABS) err = SAM_SEQ_CAPACITY;
-        else pb_take_slabs(W, want, b, sh.rec_slab, lane, err);
-        if (lane == 0) { sh.clones = run; sh.n_rec_slabs = want; if (err) sh.err = err; }
+        if (lane == 0) sh.clones = run;
     }
+    for (int j = tid; j < n; j += nt)                      // from here on: the handle of the interval's state
+        if (j > 0 && a.canon[j] == j) {
+            const uint32_t e = a.enode[j];
+            a.first[j] = e + 1u == pb_h(a, j) ? e << 1 : a.first[j] << 1 | 1u;
+        }
     pb_sync(nt);
-    if (sh.err) { out.err = sh.err; out.s2 = out.l2 = out.e2 = 0; return; }
     uint32_t* pstate = W.pstate + (size_t)b * W.text_stride;
     for (int c = w; c < chunks; c += nw) {
         const int p = 32 * c + lane;
-        const bool cl = p < n && (a.L[p] & 0x8000u);
+        const bool cl = p < n && pb_clones(a, (uint32_t)p);
         const unsigned mask = __ballot_sync(0xFFFFFFFFu, cl);
         if (p < n) {
             const uint32_t id = (uint32_t)(p + 1 + sh.chunk[c] + __popc(mask & ((1u << lane) - 1u)));
             a.idc[p] = (uint16_t)id;
             pstate[p] = id;
+            // suffix links
+            uint32_t x = pb_leaf(a, (uint32_t)p);
+            if (x != 0 && pb_h(a, (int)x) == (uint32_t)p + 1u) x = a.parent[x];      // the prefix occurs again: the interval is its own
+            a.link[2 * p] = (uint16_t)pb_state(a, x);
+            if (cl) a.link[2 * p + 1] = (uint16_t)pb_state(a, a.parent[a.wnode[p] & 0x7FFFu]);
         }
     }
+    // the root's table entries are given out from a bitmap, in place of `canon`, if that is large enough
+    uint32_t* taken = reinterpret_cast<uint32_t*>(a.canon);
+    const bool bitmap = W.root_cap <= 16 * N2;
     pb_sync(nt);
-
-    // ---- suffix links
-    const int rps_shift = W.slab_shift - 5;
-    for (int p = tid; p < n; p += nt) {
-        const int j = a.rank[p];
-        {   // the state of the whole prefix
-            PbNode x;
-            x.lo = j;
-            const uint32_t hr = pb_h(a, j + 1);
-            if (hr == (uint32_t)p + 1) x = pb_node(a, j, (uint32_t)p + 1);           // it occurs again
-            else x.up = max(pb_h(a, j), hr);
-            a.link[2 * p] = (uint16_t)(x.up == 0 ? PB_ROOT : pb_handle(a, pb_node(a, x.lo, x.up)));
-        }
-        if (a.L[p] & 0x8000u) {
-            const PbNode x = pb_node(a, j, a.L[p] & 0x7FFFu);
-            a.link[2 * p + 1] = (uint16_t)(x.up == 0 ? PB_ROOT : pb_handle(a, pb_node(a, x.lo, x.up)));
-        }
-    }
+    if (bitmap) for (int j = tid; j < (N2 >> 1); j += nt) taken[j] = 0;
     pb_sync(nt);
 
     // ---- transitions: count them (the root's go to its table at once)
@@ -433,69 +468,74 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, const int32
     const uint32_t cap_mask = (uint32_t)W.root_cap - 1u, bmask = (uint32_t)(W.root_cap / SAM_ROOT_BUCKET) - 1u;
     for (int q = tid; q < 2 * n; q += nt) {
         const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1);
-        if ((u & 1) && !(a.L[u >> 1] & 0x8000u)) continue;
+        if ((u & 1) && !pb_clones(a, u >> 1)) continue;
         pb_into(a, u, [&](uint32_t v, bool solid) {
             if (v != PB_ROOT) { atomicAdd(&a.deg[v >> 1], (v & 1) ? 0x10000u : 1u); return; }
-            const uint32_t t = (uint32_t)text[(u & 1) ? a.E[u >> 1] : u >> 1];
-            const unsigned long long val = (unsigned long long)(pb_id(a, u) | (solid ? SAM_FLAG : 0u)) << 32 | t;
+            const uint32_t t = (uint32_t)text[pb_end(a, u)];
+            const uint2 val = make_uint2(t, pb_id(a, u) | (solid ? SAM_FLAG : 0u));
             uint32_t at = (sam_hash1(t) & bmask) * SAM_ROOT_BUCKET;
-            for (uint32_t i = 0; i <= cap_mask; i++, at = (at + 1) & cap_mask)
-                if (atomicCAS(reinterpret_cast<unsigned long long*>(root + at), (unsigned long long)SAM_NONE, val) == (unsigned long long)SAM_NONE) break;
+            for (uint32_t i = 0; i <= cap_mask; i++, at = (at + 1) & cap_mask) {
+                if (bitmap) {
+                    const uint32_t bit = 1u << (at & 31);
+                    if (!(atomicOr(&taken[at >> 5], bit) & bit)) { root[at] = val; break; }
+                } else if (atomicCAS(reinterpret_cast<unsigned long long*>(root + at), (unsigned long long)SAM_NONE,
+                                     (unsigned long long)val.y << 32 | val.x) == (unsigned long long)SAM_NONE) break;
+            }
             atomicAdd(&sh.root_deg, 1);
         });
     }
     pb_sync(nt);
 
-    // ---- records; edge blocks by size, largest first, so that none crosses a slab
-    // (b.x of a record holds the number of its block among those of its size until the blocks have places)
+    // ---- room: records, and edge blocks by size, largest first, so that none crosses a slab
     for (int q = tid; q < 2 * n; q += nt) {
-        const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1), p = u >> 1;
-        if ((u & 1) && !(a.L[p] & 0x8000u)) continue;
-        const uint32_t d = (u & 1) ? a.deg[p] >> 16 : a.deg[p] & 0xFFFFu;
+        const uint32_t p = (uint32_t)(q < n ? q : q - n), d = q < n ? a.deg[p] & 0xFFFFu : a.deg[p] >> 16;
         if (d > 2) {
             const int k = d <= SAM_BLOCK_MIN ? 0 : 28 - __clz(d - 1);                // 16 << k entries
-            const uint32_t id = pb_id(a, u);
-            uint4* rec = reinterpret_cast<uint4*>(W.pool + ((size_t)sh.rec_slab[id >> rps_shift] << W.slab_shift)) + 2 * (size_t)(id & ((1u << rps_shift) - 1));
-            rec[1].x = atomicAdd(&sh.cls_n[k], 1u);
+            (q < n ? a.parent : a.canon)[p] = (uint16_t)atomicAdd(&sh.cls_n[k], 1u); // its number among those of its size
         }
     }
     pb_sync(nt);
     if (w == 0) {
+        const int n_rec = ((n + sh.clones) >> (W.slab_shift - 5)) + 1;
         uint32_t units = 0;
         if (lane == 0) for (int k = 15; k >= 0; k--) { sh.cls_base[k] = units; units += sh.cls_n[k] << k; }
         units = __shfl_sync(0xFFFFFFFFu, units, 0);
         const uint32_t slab_units = 1u << (W.slab_shift - 7);
-        const int want = (int)((units + slab_units - 1) / slab_units);
+        const int n_blk = (int)((units + slab_units - 1) / slab_units);
         int err = 0;
-        if (want > PB_BLOCK_SLABS) err = SAM_SEQ_CAPACITY;
-        else if (want > 0) pb_take_slabs(W, want, b, sh.blk_slab, lane, err);
+        if (n_rec > SAM_MAX_REC_SLABS || n_blk > PB_BLOCK_SLABS) err = SAM_SEQ_CAPACITY;
+        else pb_take_slabs(W, n_rec + n_blk, b, sh.slab, lane, err);
         __syncwarp();
         if (lane == 0) {
-            if (err) sh.err = err;
-            else {
-                sh.n_blk_units = (int)units;
-                cb[CB_BLK_CUR] = want ? (sh.blk_slab[want - 1] << (W.slab_shift - 7)) + (units - (uint32_t)(want - 1) * slab_units) : 0u;
-                cb[CB_BLK_END] = want ? (sh.blk_slab[want - 1] + 1u) << (W.slab_shift - 7) : 0u;
+            sh.err = err; sh.n_rec_slabs = n_rec;
+            if (!err) {
+                const uint32_t last = sh.slab[n_rec + n_blk - 1];
+                cb[CB_BLK_CUR] = n_blk ? (last << (W.slab_shift - 7)) + (units - (uint32_t)(n_blk - 1) * slab_units) : 0u;
+                cb[CB_BLK_END] = n_blk ? (last + 1u) << (W.slab_shift - 7) : 0u;
             }
         }
     }
     pb_sync(nt);
-    // the taken record slabs belong to the slot whatever happens: they go back to the pool at its reset
     if (sh.err) { out.err = sh.err; out.s2 = out.l2 = out.e2 = 0; return; }
+    const int rps_shift = W.slab_shift - 5;
+    const uint32_t* blk_slab = sh.slab + sh.n_rec_slabs;
+    auto record = [&](uint32_t id) {
+        return reinterpret_cast<uint4*>(W.pool + ((size_t)sh.slab[id >> rps_shift] << W.slab_shift)) + 2 * (size_t)(id & ((1u << rps_shift) - 1));
+    };
+    // ---- records
     for (int q = tid; q < 2 * n; q += nt) {
         const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1), p = u >> 1;
-        if ((u & 1) && !(a.L[p] & 0x8000u)) continue;
+        if ((u & 1) && !pb_clones(a, p)) continue;
         const uint32_t d = (u & 1) ? a.deg[p] >> 16 : a.deg[p] & 0xFFFFu;
-        const uint32_t id = pb_id(a, u), e = (u & 1) ? a.E[p] : p;
-        uint4* rec = reinterpret_cast<uint4*>(W.pool + ((size_t)sh.rec_slab[id >> rps_shift] << W.slab_shift)) + 2 * (size_t)(id & ((1u << rps_shift) - 1));
         uint4 bw = make_uint4(0, 0, 0, 0);
         if (d > 2) {
             const int k = d <= SAM_BLOCK_MIN ? 0 : 28 - __clz(d - 1);
-            const uint32_t at = sh.cls_base[k] + (rec[1].x << k);
+            const uint32_t at = sh.cls_base[k] + ((uint32_t)(q < n ? a.parent : a.canon)[p] << k);
             const uint32_t us = W.slab_shift - 7;
-            bw = make_uint4((sh.blk_slab[at >> us] << us) + (at & ((1u << us) - 1u)), (uint32_t)SAM_BLOCK_MIN << k, 0, 0);
+            bw = make_uint4((blk_slab[at >> us] << us) + (at & ((1u << us) - 1u)), (uint32_t)SAM_BLOCK_MIN << k, 0, 0);
         }
-        rec[0] = make_uint4(pb_len(a, u), pb_id(a, a.link[u]), e + 1, d);
+        uint4* rec = record(pb_id(a, u));
+        rec[0] = make_uint4(pb_len(a, u), pb_id(a, a.link[u]), pb_end(a, u) + 1, d);
         rec[1] = bw;
     }
     pb_sync(nt);
@@ -508,13 +548,13 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, const int32
     // ---- transitions: write them
     for (int q = tid; q < 2 * n; q += nt) {
         const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1);
-        if ((u & 1) && !(a.L[u >> 1] & 0x8000u)) continue;
-        const uint32_t t = (uint32_t)text[(u & 1) ? a.E[u >> 1] : u >> 1], idu = pb_id(a, u);
+        if ((u & 1) && !pb_clones(a, u >> 1)) continue;
+        const uint32_t t = (uint32_t)text[pb_end(a, u)], idu = pb_id(a, u);
         pb_into(a, u, [&](uint32_t v, bool solid) {
             if (v == PB_ROOT) return;
             const uint32_t was = (v & 1) ? atomicSub(&a.deg[v >> 1], 0x10000u) >> 16 : atomicSub(&a.deg[v >> 1], 1u) & 0xFFFFu;
-            const uint32_t k = (was & 0x7FFFu) - 1u, id = pb_id(a, v);
-            uint2* rec = reinterpret_cast<uint2*>(W.pool + ((size_t)sh.rec_slab[id >> rps_shift] << W.slab_shift)) + 4 * (size_t)(id & ((1u << rps_shift) - 1));
+            const uint32_t k = (was & 0x7FFFu) - 1u;
+            uint2* rec = reinterpret_cast<uint2*>(record(pb_id(a, v)));
             uint2* at = (was & 0x8000u) ? reinterpret_cast<uint2*>(W.pool + (size_t)rec[2].x * 128) + k : rec + 2 + k;
             *at = make_uint2(t, idu | (solid ? SAM_FLAG : 0u));
         });
@@ -525,18 +565,14 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, const int32
     const uint32_t last = (uint32_t)(n - 1) << 1, s2 = a.link[last];
     out.err = 0;
     out.s2 = (int32_t)pb_id(a, s2); out.l2 = (int32_t)pb_len(a, s2);
-    out.e2 = s2 == PB_ROOT ? 0 : (int32_t)((s2 & 1) ? a.E[s2 >> 1] : s2 >> 1) + 1;
-    if (tid < sh.n_rec_slabs) cb[CB_SLABTAB + tid] = sh.rec_slab[tid];               // (nt >= SAM_MAX_REC_SLABS)
+    out.e2 = s2 == PB_ROOT ? 0 : (int32_t)pb_end(a, s2) + 1;
+    if (tid < sh.n_rec_slabs) cb[CB_SLABTAB + tid] = sh.slab[tid];                   // (nt >= SAM_MAX_REC_SLABS)
     if (tid == 0) {
         cb[CB_NTOK] = (uint32_t)n; cb[CB_NSTATES] = (uint32_t)(1 + n + sh.clones); cb[CB_LAST] = pb_id(a, last);
         cb[CB_S2] = (uint32_t)out.s2; cb[CB_L2] = (uint32_t)out.l2;
         cb[CB_NRECSLABS] = (uint32_t)sh.n_rec_slabs; cb[CB_ROOTDEG] = (uint32_t)sh.root_deg;
     }
-    if (out.l2 > 0 && tid < 2) {
-        const uint32_t id = (uint32_t)out.s2;
-        const uint4* rec = reinterpret_cast<const uint4*>(W.pool + ((size_t)sh.rec_slab[id >> rps_shift] << W.slab_shift)) + 2 * (size_t)(id & ((1u << rps_shift) - 1));
-        reinterpret_cast<uint4*>(cb + CB_REC2)[tid] = rec[tid];
-    }
+    if (out.l2 > 0 && tid < 2) reinterpret_cast<uint4*>(cb + CB_REC2)[tid] = record((uint32_t)out.s2)[tid];
 }
 
 }  // namespace

@@ -1148,7 +1148,13 @@ __global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant
     const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
     const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
     bool bad = false;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) { const int t = toks[j]; bad |= t < 0 || t >= vocab; }
+    uint32_t* tok = pb_arrays(pb_smem, pb_size(m)).tok;
+    int32_t* text = A.W.text + (size_t)b * A.W.text_stride;
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+        const int t = toks[j];
+        tok[j] = (uint32_t)t; text[j] = t;               // (the text of an empty slot is nobody's)
+        bad |= t < 0 || t >= vocab;
+    }
     if (__syncthreads_or(bad)) return;                   // the step kernel reports it
 
     const int L = A.L;
@@ -1164,7 +1170,7 @@ __global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant
         }
     } else {
         PbResult r;
-        pb_build(A.W, b, cb, toks, m, pb_smem, sh, (int)threadIdx.x - 32, (int)blockDim.x - 32, r);
+        pb_build(A.W, b, cb, vocab, m, pb_smem, sh, (int)threadIdx.x - 32, (int)blockDim.x - 32, r);
         if (warp > 1) return;
         err = r.err; my_l = r.l2; my_s = r.s2;
         if (r.l2 > 0) {
