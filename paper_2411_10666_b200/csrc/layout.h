@@ -67,14 +67,15 @@ enum {
     CB_S1FLAG, CB_BLK_CUR, CB_BLK_END, CB_NRECSLABS, CB_ROOTDEG,
     CB_ARRIVE,        // split step: how many of the slot's two sides have finished (parity: 2 per step)
     CB_NTOK_S,        // the text length as the static side keeps it (it may not read CB_NTOK while the dynamic side writes it)
-    CB_ERR_S,         // split step: error met by the static side (walk limit); SAM_STEP_DONE between the two launches of a
-                      // step with prompts, for a slot the first of them has done; 0 otherwise
+    CB_ERR_S,         // split step: error met by the static side (walk limit); SAM_STEP_DONE or SAM_STEP_BUILT between the
+                      // two launches of a step with prompts, for a slot the first of them has done or built; 0 otherwise
     CB_SLABTAB = 16,  // .. 47
     CB_REC1 = 48,     // .. 55: copy of the static match state's record (valid when s1 != 0)
     CB_REC2 = 56      // .. 63: copy of the dynamic match state's record (valid when s2 != 0)
 };
 
 #define SAM_STEP_DONE 0x80000000u
+#define SAM_STEP_BUILT 0x80000001u
 
 struct SamStaticRec {   // 32 bytes
     int32_t len; uint32_t link; int32_t min_endpos; uint32_t deg;

@@ -41,11 +41,12 @@ struct PbShared {                          // what the threads of one build exch
 struct PbArrays {
     uint64_t* key; uint16_t* lev; uint16_t* A; uint16_t* B; uint32_t* tok;      // while sorting
     uint32_t* tree; uint16_t* rank; uint16_t* canon; uint16_t* enode; uint16_t* parent;
-    uint32_t* first; uint16_t* wnode; uint16_t* idc; uint16_t* link; uint32_t* deg;
+    uint32_t* first; uint16_t* wnode; uint16_t* idc; uint16_t* link; uint32_t* deg; uint16_t* clen;
     int N2;                                // size of the sorted order, a power of two
 };
 
-// `tree`: leaves in its upper half; `link` takes the place of the inner nodes when they are no longer needed.
+// `tree`: leaves in its upper half.  When they are no longer needed, `link` takes the place of its inner nodes and `clen`,
+// the clones' lengths, that of `rank`.
 __device__ __forceinline__ PbArrays pb_arrays(unsigned char* sm, int N2) {
     PbArrays a;
     const size_t n = (size_t)N2;
@@ -55,6 +56,7 @@ __device__ __forceinline__ PbArrays pb_arrays(unsigned char* sm, int N2) {
     a.tree = (uint32_t*)sm; a.link = (uint16_t*)sm; a.rank = (uint16_t*)(sm + 8 * n); a.canon = (uint16_t*)(sm + 10 * n);
     a.enode = (uint16_t*)(sm + 12 * n); a.parent = (uint16_t*)(sm + 14 * n); a.first = (uint32_t*)(sm + 16 * n);
     a.wnode = (uint16_t*)(sm + 20 * n); a.idc = (uint16_t*)(sm + 22 * n); a.deg = (uint32_t*)(sm + 24 * n);
+    a.clen = a.rank;
     return a;
 }
 __device__ __forceinline__ int pb_size(int n) { return n <= 64 ? 64 : 1 << (32 - __clz(n - 1)); }
@@ -205,7 +207,7 @@ __device__ __forceinline__ uint32_t pb_leaf(const PbArrays& a, uint32_t p) {
 }
 __device__ __forceinline__ bool pb_clones(const PbArrays& a, uint32_t p) { return (a.wnode[p] & 0x8000u) != 0; }
 __device__ __forceinline__ uint32_t pb_len(const PbArrays& a, uint32_t hd) {
-    return hd == PB_ROOT ? 0u : (hd & 1) ? pb_h(a, a.wnode[hd >> 1] & 0x7FFF) : (hd >> 1) + 1;
+    return hd == PB_ROOT ? 0u : (hd & 1) ? a.clen[hd >> 1] : (hd >> 1) + 1;
 }
 __device__ __forceinline__ uint32_t pb_end(const PbArrays& a, uint32_t hd) { return (hd & 1) ? a.enode[a.wnode[hd >> 1] & 0x7FFF] : hd >> 1; }
 __device__ __forceinline__ uint32_t pb_id(const PbArrays& a, uint32_t hd) { return hd == PB_ROOT ? 0u : a.idc[hd >> 1] + (hd & 1); }
@@ -250,7 +252,7 @@ __device__ __forceinline__ uint32_t pb_take_slabs(const SamBatchView& W, int wan
     return (uint32_t)want;
 }
 
-struct PbResult { int32_t s2, l2, e2; int err; };
+struct PbResult { int32_t s2, l2, e2; int err; };          // e2: first end position of the match state
 
 // One round of the sort: order the members of each group of equal prefixes (of `span` tokens) by the tokens before those, by
 // counting how many of the group come first.  A -> B, rank -> next.  Returns the number of groups.
@@ -461,6 +463,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int vocab, 
     const bool bitmap = W.root_cap <= 16 * N2;
     pb_sync(nt);
     if (bitmap) for (int j = tid; j < (N2 >> 1); j += nt) taken[j] = 0;
+    for (int p = tid; p < n; p += nt) a.clen[p] = (uint16_t)pb_h(a, a.wnode[p] & 0x7FFF);
     pb_sync(nt);
 
     // ---- transitions: count them (the root's go to its table at once)

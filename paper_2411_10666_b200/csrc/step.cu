@@ -1051,14 +1051,18 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
     const int L = A.L;
     __syncthreads();          // both warps hold the slot's state as it was before either writes any of it
 
-    if (__shfl_sync(FULL, cw, CB_ERR_S) == SAM_STEP_DONE) {      // this step is done: sam_prefill_kernel took the slot
-        if (threadIdx.x == 0) { cb[CB_ERR_S] = 0; if (A.done_flag) signal_done(A); }
+    // what sam_prefill_kernel, launched before this one, has done of the slot
+    const uint32_t done = __shfl_sync(FULL, cw, CB_ERR_S);
+    const bool built = done == SAM_STEP_BUILT;
+    if (done != 0 && threadIdx.x == 0) cb[CB_ERR_S] = 0;
+    if (done == SAM_STEP_DONE) {
+        if (threadIdx.x == 0 && A.done_flag) signal_done(A);
         return;
     }
 
     // validate the whole step before any state changes (both warps reach the same verdict)
     bool fresh_fail = false;
-    if (status == 0) {
+    if (status == 0 && !built) {
         if (m < 0 || m > A.stride) status = SAM_SEQ_BAD_COUNT;
         else if ((int64_t)ntok0 + m > A.W.max_seq_len) status = SAM_SEQ_CAPACITY;
         else {
@@ -1097,7 +1101,7 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
         // ---------------- static automaton: Transfer per token ----------------
         if (A.has_static) {
             uint32_t s, sf; int32_t l;
-            static_chain<true>(A, b, lane, cb, cw, tok_first, toks, m, ntok0, ra, rb, s, sf, l, err, d, my_dl);
+            static_chain<true>(A, b, lane, cb, cw, tok_first, toks, m, built ? 0u : ntok0, ra, rb, s, sf, l, err, d, my_dl);
             my_l = l; my_s = (int32_t)s;
         }
     } else {
@@ -1105,7 +1109,7 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
         DynChain X;
         X.ra = ra; X.rb = rb;
         dyn_open(A.W, b, lane, cb, cw, cw2, X);
-        dyn_feed(X, tok_first, toks, m, sh_run);
+        dyn_feed(X, tok_first, toks, built ? 0 : m, sh_run);
         err = X.D.err; my_l = (int32_t)X.l2; my_s = (int32_t)X.s2;
         if (X.l2 > 0 && !err) {
             const int64_t e = (int64_t)X.ra.z;                  // min_endpos
@@ -1127,13 +1131,17 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
 
 // ------------------------------------------------------------------ prompts
 // Launched ahead of the step kernel when the step's rows are long enough to hold prompts.  An empty slot that is given
-// SAM_PREFILL_MIN tokens or more is done here, the rest of the slots by the step kernel that follows (a word of
-// the control block tells it which).  One block per slot: warp 0 finds the static match, the other warps
-// build the automaton of the whole text (prefill_build.cuh), and the first two warps read the drafts and write the outputs.
+// SAM_PREFILL_MIN tokens or more has its automaton built here (prefill_build.cuh), one block per slot; a word of the
+// control block tells the step kernel, which follows and does the rest of the slots.
+//   STATIC: warp 0 finds the slot's static match meanwhile, and the slot is done here, outputs included: for
+//   batches that leave the GPU room, where the step waits for the slowest slot.  Otherwise the step kernel does all but
+//   the build, and the build's blocks, without the static side's registers, are resident five to an SM instead of three
+//   (4096 prompts of 1024 tokens).
 // From how many tokens: the build takes 14 us for its shortest texts, one Expand after the other 0.3 to 0.5 us a token.
 constexpr int SAM_PREFILL_MIN = 48;
 
-__global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant__ StepArgs A) {
+template <bool STATIC, int THREADS, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __grid_constant__ StepArgs A) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(16) unsigned char pb_smem[];
@@ -1157,7 +1165,15 @@ __global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant
     }
     if (__syncthreads_or(bad)) return;                   // the step kernel reports it
 
-    const int L = A.L;
+    if (!STATIC) {
+        PbResult r;
+        pb_build(A.W, b, cb, vocab, m, pb_smem, sh, (int)threadIdx.x, (int)blockDim.x, r);
+        if (threadIdx.x == 0) {
+            if (r.err) cb[CB_STATUS] = (uint32_t)r.err;
+            cb[CB_ERR_S] = SAM_STEP_BUILT;
+        }
+        return;
+    }
     int32_t d[MAX_DRAFT_REGS] = {-1, -1, -1, -1};
     int32_t my_l = 0, my_s = 0, my_dl = 0;
     int err = 0;
@@ -1174,8 +1190,8 @@ __global__ void __launch_bounds__(1024) sam_prefill_kernel(const __grid_constant
         if (warp > 1) return;
         err = r.err; my_l = r.l2; my_s = r.s2;
         if (r.l2 > 0) {
-            my_dl = min(m - r.e2, L);
-            gather_draft<0>(A.W.text + (size_t)b * A.W.text_stride, r.e2, my_dl, L, lane, d);
+            my_dl = min(m - r.e2, A.L);
+            gather_draft<0>(text, r.e2, my_dl, A.L, lane, d);
             my_dl = cut_at_stop(d, my_dl, lane, A.W.stop_token);
         }
     }
@@ -1808,8 +1824,6 @@ constexpr int split_big_m(int batch) { return batch >= 8192 ? 8 : 5; }
 // and shared memory would hold only a dozen of them per SM.  Once per device.
 int split_kernel_setup(int device);
 
-int prefill_kernel_setup(int device);
-
 constexpr int SAM_SPLIT_MIN_BATCH = 8192;                    // the split step is used from this many slots on
 constexpr int SAM_ORDER_MIN_BATCH = 1536;                    // more slots than a B200 holds blocks of this kernel (148 x 10)
 
@@ -1828,27 +1842,30 @@ int split_kernel_setup(int device) {
     }
     return SAM_OK;
 }
-// The build's shared memory, once per device.
-int prefill_kernel_setup(int device) {
-    static bool done[64];
-    if (device < 0 || device >= 64) return SAM_ERR_ARG;
-    if (!done[device]) {
-        cudaError_t e = cudaFuncSetAttribute(sam_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PB_MAX * PB_BYTES_PER_TOKEN);
-        if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
-        done[device] = true;
-    }
-    return SAM_OK;
-}
-
-// Shared memory and threads of a build for rows of up to `stride` tokens: a thread for four tokens where many
-// builds share an SM, for two where each has one to itself.
-void prefill_shape(int stride, int batch, size_t* smem, unsigned* threads) {
+// The build for rows of up to `stride` tokens.  With the static side: two tokens a thread, four where more than two
+// builds share an SM.  Without: four tokens a thread, registers for as many blocks as the shared memory has room for.
+int launch_prefill(const StepArgs& A, int batch, int device, cudaLaunchConfig_t* cfg) {
+    using Kernel = void (*)(const StepArgs);
+    const Kernel kernels[4] = {sam_prefill_kernel<true, 1024, 1>, sam_prefill_kernel<false, 256, 5>, sam_prefill_kernel<false, 512, 3>,
+                               sam_prefill_kernel<false, 1024, 1>};
     int n2 = 64;
-    while (n2 < stride && n2 < PB_MAX) n2 <<= 1;
-    int t = batch <= 296 ? n2 / 2 : n2 / 4;
-    t = t < 64 ? 64 : t > 992 ? 992 : t;
-    *smem = (size_t)n2 * PB_BYTES_PER_TOKEN;
-    *threads = (unsigned)(32 + t);
+    while (n2 < A.stride && n2 < PB_MAX) n2 <<= 1;
+    int k = 0, threads = 32 + (n2 / 2 < 64 ? 64 : n2 / 2 > 992 ? 992 : n2 / 2);
+    if (batch > 296) {
+        k = n2 <= 1024 ? 1 : n2 <= 2048 ? 2 : 3;
+        threads = n2 / 4 < 64 ? 64 : n2 / 4 > 1024 ? 1024 : n2 / 4;
+    }
+    static bool done[64][4];                                // the kernels' shared memory, once per device
+    if (device < 0 || device >= 64) return SAM_ERR_ARG;
+    cudaError_t e = cudaSuccess;
+    if (!done[device][k]) {
+        e = cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, PB_MAX * PB_BYTES_PER_TOKEN);
+        done[device][k] = e == cudaSuccess;
+    }
+    cfg->gridDim = dim3((unsigned)batch); cfg->blockDim = dim3((unsigned)threads); cfg->dynamicSmemBytes = (size_t)n2 * PB_BYTES_PER_TOKEN;
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(cfg, kernels[k], A);
+    if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
+    return SAM_OK;
 }
 }  // namespace
 
@@ -1898,16 +1915,11 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     prompts = !v_draft && stride >= SAM_PREFILL_MIN;
 #endif
     if (prompts) {
-        int rc = prefill_kernel_setup(b->device);
-        if (rc) return rc;
-        size_t smem; unsigned threads;
-        prefill_shape(stride, b->view.batch, &smem, &threads);
         cudaLaunchConfig_t pc;
         memset(&pc, 0, sizeof(pc));
-        pc.gridDim = dim3((unsigned)b->view.batch); pc.blockDim = dim3(threads); pc.dynamicSmemBytes = smem; pc.stream = stream;
-        pc.attrs = attr; pc.numAttrs = 1;
-        cudaError_t pe = cudaLaunchKernelEx(&pc, sam_prefill_kernel, A);
-        if (pe != cudaSuccess) { sam_set_cuda_error(pe); return SAM_ERR_CUDA; }
+        pc.stream = stream; pc.attrs = attr; pc.numAttrs = 1;
+        int rc = launch_prefill(A, b->view.batch, b->device, &pc);
+        if (rc) return rc;
     }
     // (A host-array step is synchronous: nothing runs before it that the ordering kernel could overlap with, so it
     // would cost more than the order saves; such a step is always the one two-warp launch, slots in their own order.)

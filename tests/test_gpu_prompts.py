@@ -99,3 +99,19 @@ def test_mixed_step_with_prompts_short_rows_and_refused_slots(P):
             assert np.array_equal(got[k], getattr(ref, k)), k
             assert np.array_equal(h, getattr(ref, k)), k
     assert set(ref.status.tolist()) == {0, 3, 4}
+
+
+@pytest.mark.parametrize("n", [60, 1000, 1100, 2100])
+def test_many_prompts_at_once(P, n):
+    """Batches that fill the GPU build with fewer registers and leave the static side to the step kernel."""
+    rng = random.Random(n)
+    base = [rng.randrange(400) for _ in range(12_000)]
+    corpus = base + base[2000:7000]
+    B, L = 300, 16
+    rows = np.array([_text(KINDS[i % len(KINDS)], n, rng, corpus) + [rng.randrange(9) for _ in range(8)] for i in range(B)], dtype=np.int32)
+    counts = np.full((1, B), 8, dtype=np.int32)
+    st = P.StaticSam.build(np.array(corpus, dtype=np.int32), VOCAB)
+    ref, ob, _ = oracle_run(np.array(corpus, dtype=np.int32), VOCAB, rows[:, :n], rows[None, :, n:].copy(), counts, L, n + 8, threads=8)
+    got, batch = gpu_run(P, st, VOCAB, rows[:, :n], rows[None, :, n:].copy(), counts, L, n + 8)
+    assert_same(got, ref)
+    assert_dynamic_automata_equal(batch, ob, range(0, B, 37), n + 8)
