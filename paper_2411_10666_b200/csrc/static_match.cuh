@@ -8,10 +8,11 @@
 //     earliest start is the answer, and most walks end after two or three tokens (static_walks);
 //   - the match so far goes on as one more walk, which alone follows suffix links, and only for as long as it covers
 //     tokens from before the step (lane 0 of static_walks);
-//   - of a long row (a prompt) only the last 32 tokens are walked: if their first start does not reach the end no longer
+//   - of a long row (a prompt) only the last 8 tokens are walked: if their first start does not reach the end no longer
 //     suffix occurs.  If it does, the state's own first occurrence in the corpus is compared with the row leftwards,
 //     32 tokens a round: all strings of a state end at the same places, so up to the length of the state's longest
-//     string that comparison is the match (static_suffix).
+//     string that comparison is the match.  Beyond it, a longer match would have to hold the seam where that string
+//     begins, so a few tokens around the seam are walked before anything else is (static_suffix).
 #pragma once
 #include "common.h"
 
@@ -215,17 +216,19 @@ __device__ __forceinline__ void static_walks(const SamStaticView& S, uint32_t tk
 }
 
 // The longest suffix of (match so far + a row of m > 32 tokens) that occurs: (s, sf, l) and, if l > 0, its record.
+constexpr int SUFFIX_WINDOW = 8;           // tokens walked first, and on each side of a seam
 __device__ __forceinline__ void static_suffix(const SamStaticView& S, const int32_t* toks, int m, int lane, uint32_t& s, uint32_t& sf,
                                               int32_t& l, uint4& ra, uint4& rb, int& err, ChainCounts& kc) {
     const uint32_t s0 = s, sf0 = sf; const int32_t l0 = l;
     const uint4 ra0 = ra, rb0 = rb;
     {
-        const uint32_t tk = (uint32_t)toks[m - 32 + lane];
+        uint32_t tk = 0, re = SAM_NONE;
+        if (lane < SUFFIX_WINDOW) { tk = (uint32_t)toks[m - SUFFIX_WINDOW + lane]; re = __ldg(S.root_row + tk); }
         SAM_COUNT(kc.rounds, 2);
-        static_walks(S, tk, __ldg(S.root_row + tk), 32, lane, false, 0, false, s, sf, l, ra, rb, err, kc);
+        static_walks(S, tk, re, SUFFIX_WINDOW, lane, false, 0, false, s, sf, l, ra, rb, err, kc);
     }
-    if (l < 32) return;
-    for (bool again = false; !err; again = true) {
+    if (l < SUFFIX_WINDOW) return;
+    for (int turn = 0; !err; turn++) {
         bool ends = false;
         while (!ends) {                                   // the state's first occurrence, leftwards
             const int room = min((int)ra.x, m) - l;
@@ -239,15 +242,30 @@ __device__ __forceinline__ void static_suffix(const SamStaticView& S, const int3
             ends = r < min(room, 32);
         }
         if (ends || (l >= m && l0 == 0)) return;
-        // All of the state's longest string matched (or all of the row): a longer suffix would be another state's.  Look
-        // from one token further to the left, then from further and further.
-        int c = again ? m - 4 * l : m - l - 1;
+        // All of the state's longest string matched (or all of the row): a longer suffix would be another state's, and it
+        // would hold the seam between the last token matched and the one before it.
+        int c = 0, from = 0;                              // the new match begins at token c and has been taken up to token `from`
         bool have = false;
-        if (c < 0 || (c == 0 && l0 > 0)) c = 0;
-        const bool whole = c == 0;
-        s = whole ? s0 : 0; sf = whole ? sf0 : 0; l = whole ? l0 : 0;
-        if (whole && s0 != 0) { ra = ra0; rb = rb0; have = true; }
-        static_forward(S, toks, c, m, s, sf, l, ra, rb, have, lane, err, kc);
+        const int before = min(SUFFIX_WINDOW, m - l), w = before + SUFFIX_WINDOW;
+        if (before > 0 && turn < 12) {
+            uint32_t tk = 0, re = SAM_NONE, xs = 0, xsf = 0;
+            if (lane < w) { tk = (uint32_t)toks[m - l - before + lane]; re = __ldg(S.root_row + tk); }
+            SAM_COUNT(kc.rounds, 2);
+            int32_t xl = 0;
+            uint4 xa = make_uint4(0, 0, 0, 0), xb = xa;
+            static_walks(S, tk, re, w, lane, false, 0, false, xs, xsf, xl, xa, xb, err, kc);
+            if (err || xl <= SUFFIX_WINDOW) return;       // nothing that holds the seam occurs
+            from = m - l + SUFFIX_WINDOW; c = from - xl;
+            s = xs; sf = xsf; l = xl; ra = xa; rb = xb; have = true;
+        } else {                                          // (runs of one token and the like: look from further and further to the left)
+            c = from = max(0, m - 4 * l);
+            s = 0; sf = 0; l = 0;
+        }
+        const bool whole = c == 0 && l0 > 0;              // it may reach into the match so far
+        if (whole) {
+            from = 0; s = s0; sf = sf0; l = l0; ra = ra0; rb = rb0; have = true;
+        }
+        static_forward(S, toks, from, m, s, sf, l, ra, rb, have, lane, err, kc);
         if (l > 0 && !have && !err) { static_record(S, s, ra, rb); SAM_COUNT(kc.rounds, 1); }
         if (whole || l < m - c) return;
     }
