@@ -3,12 +3,19 @@
 // Appendix A.1/A.2).
 //
 // One warp per slot.  The queue lives in shared memory as plain arrays; an entry holds its path
-// probability, state, token, parent node, the state's freq and the state's successor candidates
-// (its two inline transitions, or its precomputed top-k if its transitions are hashed).  Because a
-// state's candidates travel with its entry, expanding a popped node needs exactly one round of
+// probability, its place in the order of pushes, token, parent node, the state's freq and the state's
+// successor candidates (its two inline transitions, or its precomputed top-k if its transitions are hashed).
+// Because a state's candidates travel with its entry, expanding a popped node needs exactly one round of
 // reads: lanes 0..n-1 each fetch one child's freq, record and, if flagged, top-k entry together.
-// Popping is a strided scan of the queue with a warp arg-max (larger probability first, then the
-// earlier push).  Probabilities are IEEE float32: quotient freq(child) / freq(state) rounded first,
+//   - Most nodes are states with one successor that occurs as often as they do: inside a passage the corpus holds once or
+//     several times.  Such a stretch is one entry, a path, pushed again with each pop, its tokens those of the corpus.
+//     Where the state occurs once the path goes on to the end of the corpus; otherwise its states are guessed (ids as far apart
+//     as the first two, as states made token after token along a passage are), read in one round, a few lanes
+//     for each child, and checked; the last of them is an ordinary entry again.
+//   - The entries with the largest probability are popped together as long as they are paths: each goes back to the end
+//     of the line with the same probability, so they take turns, and lane t writes the t-th node of up to 32 with one read
+//     of the corpus.
+// Probabilities are IEEE float32: quotient freq(child) / freq(state) rounded first,
 // then the product with the parent's probability.
 #include "common.h"
 
@@ -23,19 +30,15 @@ struct TreeArgs {
     int32_t* tokens; int32_t* parents; float* probs; int32_t* sizes;
 };
 
-// successor candidates of state u (id without flag) read by ONE lane: from the record when the
-// state has at most two transitions, else from the top-k table.  Returns how many; cand[] gets
-// (token, target | F) pairs.  hashed states come back in top-k order, inline ones in record order.
-__device__ __forceinline__ int load_candidates(const SamStaticView& S, uint32_t u, bool flagged, int k,
-                                               uint32_t ctok[SAM_TOPK_MAX], uint32_t ctgt[SAM_TOPK_MAX], bool& ordered) {
-    ordered = false;
-    if (!flagged) {
-        const uint4 a = __ldg(S.rec + 2 * (size_t)u), b = __ldg(S.rec + 2 * (size_t)u + 1);
-        int n = (int)(a.w < 2u ? a.w : 2u);
-        if (a.w > 2u) n = 0;                      // unflagged reference to a hashed state cannot happen
-        ctok[0] = b.x; ctgt[0] = b.y; ctok[1] = b.z; ctgt[1] = b.w;
-        return n;
-    }
+// Successor candidates of a state, by one lane: (token, target | F) pairs; returns how many.  From the record of a state
+// with at most two transitions, in record order ...
+__device__ __forceinline__ int inline_candidates(const uint4& a, const uint4& b, uint32_t ctok[SAM_TOPK_MAX], uint32_t ctgt[SAM_TOPK_MAX]) {
+    ctok[0] = b.x; ctgt[0] = b.y; ctok[1] = b.z; ctgt[1] = b.w;
+    return a.w <= 2u ? (int)a.w : 0;                        // (an unflagged reference to a hashed state cannot happen)
+}
+// ... or from the top-k table, in top-k order.
+__device__ __forceinline__ int load_topk(const SamStaticView& S, uint32_t u, int k, uint32_t ctok[SAM_TOPK_MAX], uint32_t ctgt[SAM_TOPK_MAX],
+                                         bool& ordered) {
     ordered = true;
     uint32_t at = sam_hash1(u) & S.topk_mask;
     for (uint32_t probe = 0; probe <= S.topk_mask; probe++) {
@@ -55,93 +58,200 @@ __device__ __forceinline__ int load_candidates(const SamStaticView& S, uint32_t 
     return 0;
 }
 
+constexpr int CAND_WORDS = 2 * SAM_TOPK_MAX;                // an entry's candidates: tokens, then targets
+constexpr uint32_t ENTRY_ORDERED = 256u, ENTRY_PATH = 512u, ENTRY_ENDS = 1024u;     // flags beside the number of candidates
+constexpr int PATH_LEFT = 16;                               // q_n >> PATH_LEFT: nodes left on the path; then, unless it ENDS, the entry
+constexpr int LAST_TOKEN = 2;                               // is that of its last state, whose token this word of q_cand holds
+constexpr int PATH_ENDLESS = 1024;                          // (more than any tree has nodes)
+
 __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ TreeArgs A) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ uint32_t smem[];
+    __shared__ int top[32], turn[32];                       // the entries with the largest probability, as found and in order
     const int b = blockIdx.x, lane = threadIdx.x;
+    const unsigned lt = (1u << lane) - 1u;
     const int K = A.k, M = A.max_size;
     const int Q = M * K + 1;
-    float* q_p = reinterpret_cast<float*>(smem);            // < 0: popped
-    uint32_t* q_state = smem + Q;                           // id | F
-    uint32_t* q_tok = smem + 2 * Q;
+    uint32_t* q_key = smem;                                 // bits of the probability, plus one; 0: not in the queue
+    uint32_t* q_seq = smem + Q;                             // place in the order of pushes
+    uint32_t* q_tok = smem + 2 * Q;                         // of a path: the corpus position of the next node's token
     int32_t* q_par = reinterpret_cast<int32_t*>(smem + 3 * Q);
     uint32_t* q_freq = smem + 4 * Q;
-    uint32_t* q_n = smem + 5 * Q;                           // candidates | ordered << 8
-    uint32_t* q_ctok = smem + 6 * Q;                        // [Q][SAM_TOPK_MAX]
-    uint32_t* q_ctgt = smem + 6 * Q + (size_t)Q * SAM_TOPK_MAX;
+    uint32_t* q_n = smem + 5 * Q;                           // candidates | flags
+    uint32_t* q_cand = smem + 6 * Q;                        // [Q][CAND_WORDS]
 
     int32_t* out_tok = A.tokens + (size_t)b * M;
     int32_t* out_par = A.parents + (size_t)b * M;
     float* out_p = A.probs ? A.probs + (size_t)b * M : nullptr;
-    for (int j = lane; j < M; j += 32) { out_tok[j] = -1; out_par[j] = -1; if (out_p) out_p[j] = 0.f; }
 
     const int32_t s0 = A.states[b];
-    if (s0 <= 0 || (int64_t)s0 >= A.S.n_states) { if (lane == 0) A.sizes[b] = 0; return; }
-
-    int qn = 0;
-    if (lane == 0) {                                         // the start node: probability 1
-        uint32_t ctok[SAM_TOPK_MAX], ctgt[SAM_TOPK_MAX];
-        bool ordered;
-        const bool flagged = __ldg(A.S.rec + 2 * (size_t)s0).w > 2u;
-        const int n = load_candidates(A.S, (uint32_t)s0, flagged, K, ctok, ctgt, ordered);
-        q_p[0] = 1.0f; q_state[0] = (uint32_t)s0; q_tok[0] = (uint32_t)A.start_tokens[b]; q_par[0] = -1;
-        q_freq[0] = __ldg(A.S.freq + s0); q_n[0] = (uint32_t)n | (ordered ? 256u : 0u);
-        for (int j = 0; j < SAM_TOPK_MAX; j++) { q_ctok[j] = ctok[j]; q_ctgt[j] = ctgt[j]; }
-    }
-    qn = 1;
-    __syncwarp();
-
     int n_out = 0;
-    while (n_out < M) {
-        // pop: largest probability, earliest push among equals
-        float bp = -1.0f; int bi = 0x7FFFFFFF;
-        for (int i = lane; i < qn; i += 32) { const float p = q_p[i]; if (p > bp) { bp = p; bi = i; } }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float op = __shfl_xor_sync(FULL, bp, off); const int oi = __shfl_xor_sync(FULL, bi, off);
-            if (op > bp || (op == bp && oi < bi)) { bp = op; bi = oi; }
-        }
-        if (bp < 0.0f) break;                                // queue empty
-        const int node = n_out++;
-        const uint32_t st = q_state[bi] & SAM_IDMASK, fs = q_freq[bi];
-        const uint32_t nn = q_n[bi];
-        const int n = (int)(nn & 255u); const bool ordered = (nn & 256u) != 0;
-        if (lane == 0) {
-            out_tok[node] = (int32_t)q_tok[bi]; out_par[node] = q_par[bi]; if (out_p) out_p[node] = bp;
+    if (s0 > 0 && (int64_t)s0 < A.S.n_states) {
+        if (lane == 0) {                                    // the start node: probability 1
+            uint32_t ctok[SAM_TOPK_MAX], ctgt[SAM_TOPK_MAX];
+            bool ordered = false;
+            const uint4 a = __ldg(A.S.rec + 2 * (size_t)s0), r = __ldg(A.S.rec + 2 * (size_t)s0 + 1);
+            const int n = a.w > 2u ? load_topk(A.S, (uint32_t)s0, K, ctok, ctgt, ordered) : inline_candidates(a, r, ctok, ctgt);
+            q_key[0] = __float_as_uint(1.0f) + 1u; q_seq[0] = 0; q_tok[0] = (uint32_t)A.start_tokens[b]; q_par[0] = -1;
+            q_freq[0] = __ldg(A.S.freq + s0); q_n[0] = (uint32_t)n | (ordered ? ENTRY_ORDERED : 0u);
+            for (int j = 0; j < SAM_TOPK_MAX; j++) { q_cand[j] = ctok[j]; q_cand[SAM_TOPK_MAX + j] = ctgt[j]; }
         }
         __syncwarp();
-        if (lane == 0) q_p[bi] = -1.0f;
-        if (n_out >= M) break;                               // the last node needs no expansion
-        (void)st;
-        // expand: lane j takes candidate j
-        uint32_t ctok = 0, ctgt = 0, cf = 0; int cn = 0; bool cord = false;
-        uint32_t gtok[SAM_TOPK_MAX], gtgt[SAM_TOPK_MAX];
-        if (lane < n) {
-            ctok = q_ctok[(size_t)bi * SAM_TOPK_MAX + lane]; ctgt = q_ctgt[(size_t)bi * SAM_TOPK_MAX + lane];
-            const uint32_t u = ctgt & SAM_IDMASK;
-            cf = __ldg(A.S.freq + u);
-            cn = load_candidates(A.S, u, (ctgt >> 31) != 0, K, gtok, gtgt, cord);
-        }
-        // order two inline candidates by (freq descending, token ascending); keep the first K
-        int pos = lane;
-        if (!ordered && n == 2) {
-            const uint32_t of = __shfl_xor_sync(FULL, cf, 1), ot = __shfl_xor_sync(FULL, ctok, 1);
-            if (lane < 2) {
-                const bool other_first = of > cf || (of == cf && ot < ctok);
-                pos = other_first ? 1 : 0;
+        int qn = 1;
+        uint32_t seq = 1;
+        while (n_out < M) {
+            uint32_t best = 0;
+            for (int i = lane; i < qn; i += 32) best = max(best, q_key[i]);
+            const uint32_t key = __reduce_max_sync(FULL, best);
+            if (key == 0) break;                            // queue empty
+            const float p = __uint_as_float(key - 1u);
+            int group = 0;
+            for (int base = 0; base < qn; base += 32) {
+                const bool in = base + lane < qn && q_key[base + lane] == key;
+                const unsigned mask = __ballot_sync(FULL, in);
+                const int g = group + __popc(mask & lt);
+                if (in && g < 32) top[g] = base + lane;
+                group += __popc(mask);
             }
+            __syncwarp();
+            int at = 0, paths = 0;                          // the entry to pop; the paths at the head of the line
+            if (group <= 32) {
+                int e = 0, rank = 32;
+                uint32_t sq = 0xFFFFFFFFu;
+                if (lane < group) { e = top[lane]; sq = q_seq[e]; }
+                if (group > 1) {
+                    rank = 0;
+                    for (int g = 0; g < group; g++) rank += __shfl_sync(FULL, sq, g) < sq;
+                    if (lane < group) turn[rank] = e;
+                } else if (lane == 0) { rank = 0; turn[0] = e; }
+                paths = (int)__reduce_min_sync(FULL, lane < group && !(q_n[e] & ENTRY_PATH) ? (uint32_t)rank : (uint32_t)group);
+                __syncwarp();
+                at = turn[0];
+            } else {                                        // (too many to sort: the earliest push)
+                uint32_t first = 0xFFFFFFFFu;
+                for (int i = lane; i < qn; i += 32) if (q_key[i] == key) first = min(first, q_seq[i]);
+                first = __reduce_min_sync(FULL, first);
+                for (int base = 0; base < qn; base += 32) {
+                    const unsigned m = __ballot_sync(FULL, base + lane < qn && q_key[base + lane] == key && q_seq[base + lane] == first);
+                    if (m) { at = base + __ffs(m) - 1; break; }
+                }
+                if (q_n[at] & ENTRY_PATH) { paths = 1; if (lane == 0) turn[0] = at; __syncwarp(); }
+            }
+            if (paths > 0) {
+                // lane t: the t-th pop.  Where other entries stand in line behind the paths, each path is popped once.
+                const bool alone = paths == group;
+                const int r = lane % paths, i = lane / paths, e = turn[r];
+                const int room = (int)(q_n[e] >> PATH_LEFT);
+                int count = alone ? 32 : paths;
+                count = min(count, M - n_out);
+                const int until = room * paths + r;         // the first pop this path cannot serve
+                count = (int)__reduce_min_sync(FULL, (uint32_t)(lane < paths ? min(until, count) : count));
+                if (lane < count) {
+                    out_tok[n_out + lane] = __ldg(A.S.corpus + q_tok[e] + i);
+                    out_par[n_out + lane] = i == 0 ? q_par[e] : n_out + lane - paths;
+                    if (out_p) out_p[n_out + lane] = p;
+                }
+                __syncwarp();
+                if (lane < paths && lane < count) {         // lane r: path r, popped `c` times
+                    const int c = (count - lane + paths - 1) / paths, last = lane + (c - 1) * paths;
+                    q_tok[e] += (uint32_t)c; q_par[e] = n_out + last; q_seq[e] = seq + (uint32_t)last;
+                    const uint32_t nn = q_n[e] - ((uint32_t)c << PATH_LEFT);
+                    q_n[e] = nn;
+                    if ((nn >> PATH_LEFT) == 0) {
+                        if (nn & ENTRY_ENDS) q_key[e] = 0;
+                        else { q_n[e] = nn & 255u; q_tok[e] = q_cand[(size_t)e * CAND_WORDS + LAST_TOKEN]; }
+                    }
+                }
+                n_out += count; seq += (uint32_t)count;
+                __syncwarp();
+                continue;
+            }
+            const int node = n_out++;
+            if (lane == 0) {
+                out_tok[node] = (int32_t)q_tok[at]; out_par[node] = q_par[at];
+                if (out_p) out_p[node] = p;
+                q_key[at] = 0;
+            }
+            if (n_out >= M) break;                          // the last node needs no expansion
+            // expand: lane j takes candidate j
+            const uint32_t nn = q_n[at], fs = q_freq[at];
+            const int n = (int)(nn & 255u);
+            if (n == 0) { __syncwarp(); continue; }
+            uint32_t ctok = 0, ctgt = 0, cf = 0;
+            int cn = 0; bool cord = false;
+            uint4 ra = make_uint4(0, 0, 0, 0), rb = ra;
+            uint32_t gtok[SAM_TOPK_MAX], gtgt[SAM_TOPK_MAX];
+            if (lane < n) {
+                ctok = q_cand[(size_t)at * CAND_WORDS + lane]; ctgt = q_cand[(size_t)at * CAND_WORDS + SAM_TOPK_MAX + lane];
+                const uint32_t u = ctgt & SAM_IDMASK;
+                cf = __ldg(A.S.freq + u);
+                if (ctgt >> 31) cn = load_topk(A.S, u, K, gtok, gtgt, cord);
+                else {
+                    ra = __ldg(A.S.rec + 2 * (size_t)u); rb = __ldg(A.S.rec + 2 * (size_t)u + 1);
+                    cn = inline_candidates(ra, rb, gtok, gtgt);
+                }
+            }
+            // order two inline candidates by (freq descending, token ascending); keep the first K
+            int pos = lane;
+            if (!(nn & ENTRY_ORDERED) && n == 2) {
+                const uint32_t of = __shfl_xor_sync(FULL, cf, 1), ot = __shfl_xor_sync(FULL, ctok, 1);
+                if (lane < 2) pos = of > cf || (of == cf && ot < ctok) ? 1 : 0;
+            }
+            const int keep = n < K ? n : K;
+            // paths: lane k of child c's lanes takes the k-th state after the child
+            const int width = n == 1 ? 32 : n == 2 ? 16 : n <= 4 ? 8 : 4, c = lane / width, k = lane % width;
+            const uint32_t u = ctgt & SAM_IDMASK, far = (rb.y & SAM_IDMASK) - u;
+            const uint32_t step = lane < n && !(ctgt >> 31) && ra.w == 1u && cf > 1 ? far : 0u;
+            const uint32_t step_c = __shfl_sync(FULL, step, c), u_c = __shfl_sync(FULL, u, c), cf_c = __shfl_sync(FULL, cf, c);
+            const int pos_c = __shfl_sync(FULL, pos, c);
+            const uint4 ra_c = make_uint4(0, 0, __shfl_sync(FULL, ra.z, c), __shfl_sync(FULL, ra.w, c));
+            const uint2 rb_c = make_uint2(__shfl_sync(FULL, rb.x, c), __shfl_sync(FULL, rb.y, c));
+            int run = 1;                                    // states of child c's path
+            if (__any_sync(FULL, step != 0)) {
+                const uint32_t id = u_c + step_c * (uint32_t)k;
+                uint32_t deg = ra_c.w, f = cf_c, t0 = rb_c.x, g0 = rb_c.y;
+                uint4 r1 = make_uint4(0, 0, 0, 0);
+                if (k > 0) {
+                    deg = 3; f = 0;
+                    if (step_c != 0 && (int64_t)id < A.S.n_states) {
+                        deg = __ldg(&A.S.rec[2 * (size_t)id].w); r1 = __ldg(A.S.rec + 2 * (size_t)id + 1); f = __ldg(A.S.freq + id);
+                        t0 = r1.x; g0 = r1.y;
+                    }
+                }
+                const uint32_t deg_n = __shfl_down_sync(FULL, deg, 1), f_n = __shfl_down_sync(FULL, f, 1), t_p = __shfl_up_sync(FULL, t0, 1);
+                const bool on = step_c != 0 && k + 1 < width && deg == 1 && g0 == id + step_c && f_n == cf_c && deg_n <= 2;
+                const unsigned m = __ballot_sync(FULL, on) >> (c * width);
+                run = (~m ? __ffs(~m) - 1 : 32) + 1;
+                if (run > 1 && k == run - 1 && c < n && pos_c < keep) {              // the last state's lane
+                    const int e = qn + pos_c;
+                    uint32_t* to = q_cand + (size_t)e * CAND_WORDS;
+                    to[0] = r1.x; to[1] = r1.z; to[SAM_TOPK_MAX] = r1.y; to[SAM_TOPK_MAX + 1] = r1.w; to[LAST_TOKEN] = t_p;
+                    q_n[e] = deg | ENTRY_PATH | (uint32_t)(run - 1) << PATH_LEFT;
+                    q_tok[e] = ra_c.z - 1u;                 // (its first end position: the token itself is the one before)
+                }
+            }
+            run = __shfl_sync(FULL, run, (lane * width) & 31);                        // of child `lane`
+            if (lane < n && pos < keep) {
+                const int e = qn + pos;
+                q_key[e] = __float_as_uint(__fmul_rn(p, __fdiv_rn(__uint2float_rn(cf), __uint2float_rn(fs)))) + 1u;
+                q_seq[e] = seq + (uint32_t)pos; q_par[e] = node; q_freq[e] = cf;
+                if (cf == 1) {
+                    const int64_t room = A.S.n_tokens - (int64_t)ra.z + 1;
+                    q_tok[e] = ra.z - 1u;
+                    q_n[e] = ENTRY_PATH | ENTRY_ENDS | (uint32_t)(room < PATH_ENDLESS ? room : PATH_ENDLESS) << PATH_LEFT;
+                } else if (run == 1) {
+                    q_tok[e] = ctok; q_n[e] = (uint32_t)cn | (cord ? ENTRY_ORDERED : 0u);
+                    uint32_t* to = q_cand + (size_t)e * CAND_WORDS;
+                    for (int j = 0; j < SAM_TOPK_MAX; j++) { to[j] = gtok[j]; to[SAM_TOPK_MAX + j] = gtgt[j]; }
+                }
+            }
+            qn += keep; seq += (uint32_t)keep;
+            __syncwarp();
         }
-        const int keep = n < K ? n : K;
-        if (lane < n && pos < keep) {
-            const int e = qn + pos;
-            q_p[e] = __fmul_rn(bp, __fdiv_rn(__uint2float_rn(cf), __uint2float_rn(fs)));
-            q_state[e] = ctgt; q_tok[e] = ctok; q_par[e] = node; q_freq[e] = cf;
-            q_n[e] = (uint32_t)cn | (cord ? 256u : 0u);
-            for (int j = 0; j < SAM_TOPK_MAX; j++) { q_ctok[(size_t)e * SAM_TOPK_MAX + j] = gtok[j]; q_ctgt[(size_t)e * SAM_TOPK_MAX + j] = gtgt[j]; }
-        }
-        qn += keep;
-        __syncwarp();
     }
     if (lane == 0) A.sizes[b] = n_out;
+    for (int j = n_out + lane; j < M; j += 32) { out_tok[j] = -1; out_par[j] = -1; if (out_p) out_p[j] = 0.f; }
 }
 
 }  // namespace
@@ -165,7 +275,12 @@ extern "C" int sam_tree_draft(const sam_static_t* st, int32_t batch, const int32
         cudaError_t e = cudaFuncSetAttribute(tree_draft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     }
-    tree_draft_kernel<<<batch, 32, smem, (cudaStream_t)stream>>>(A);
-    SAM_CUDA(cudaGetLastError());
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)batch); cfg.blockDim = dim3(32); cfg.dynamicSmemBytes = smem; cfg.stream = (cudaStream_t)stream;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    SAM_CUDA(cudaLaunchKernelEx(&cfg, tree_draft_kernel, A));
     return SAM_OK;
 }
