@@ -25,6 +25,7 @@
 //     map, or ids two apart), read in one round trip and checked (dyn_repeat_run);
 //   - the static match is not advanced token by token: all suffixes of the row are walked side by side, and a
 //     match that goes on as the corpus does is taken in one round (static_match.cuh);
+//   - steps whose tokens are all at hand (sam_run_steps) run in one launch, no slot waiting for another;
 //   - a prompt that fills an empty slot is not extended token by token either: its automaton is built at once by all
 //     threads of a block (prefill_build.cuh, sam_prefill_kernel);
 //   - when the batch is larger than the GPU holds at once, the slots with the most tokens are started
@@ -717,7 +718,8 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
 // state Transfer (Algorithm 1) reaches.  In and out: the state (s, sf, l) and, where l > 0, its record (ra, rb).
 // early(): called where the match is in the state of a corpus prefix, so that the draft after m tokens can be requested
 // with the first reads; returns true if the match did go on as the corpus does, for all m tokens.
-template <class F>
+// LONG: rows of more than 32 tokens are prompts, as a rule; otherwise they are taken token by token.
+template <bool LONG, class F>
 __device__ __forceinline__ bool static_advance(const SamStaticView& S, int lane, int32_t tok_first, const int32_t* toks, int m,
                                                uint32_t& s, uint32_t& sf, int32_t& l, uint4& ra, uint4& rb, int& err, ChainCounts& kc, F early) {
 #ifdef SAM_COUNTERS
@@ -730,7 +732,12 @@ __device__ __forceinline__ bool static_advance(const SamStaticView& S, int lane,
 #endif
     bool follows = false;
     if (m > 32) {
-        static_suffix(S, toks, m, lane, s, sf, l, ra, rb, err, kc);
+        if (LONG) static_suffix(S, toks, m, lane, s, sf, l, ra, rb, err, kc);
+        else {
+            bool have = s != 0;
+            static_forward(S, toks, 0, m, s, sf, l, ra, rb, have, lane, err, kc);
+            if (l > 0 && !have && !err) static_record(S, s, ra, rb);
+        }
     } else if (m > 0) {
         const uint32_t tk = (uint32_t)tok_first;
         uint32_t re = SAM_NONE;
@@ -772,7 +779,7 @@ __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane,
     uint32_t s = __shfl_sync(FULL, cw, CB_S1), sf = __shfl_sync(FULL, cw, CB_S1FLAG);
     int32_t l = (int32_t)__shfl_sync(FULL, cw, CB_L1);
     int dl2 = 0;
-    const bool follows = static_advance(A.S, lane, tok_first, toks, m, s, sf, l, ra, rb, err, kc, [&]() {
+    const bool follows = static_advance<true>(A.S, lane, tok_first, toks, m, s, sf, l, ra, rb, err, kc, [&]() {
         if (DRAFT) {
             const int64_t e2 = (int64_t)ra.z + m, room = A.S.n_tokens - e2;
             dl2 = (int)(room < L ? (room < 0 ? 0 : room) : L);
@@ -1610,7 +1617,7 @@ __device__ __forceinline__ void static_open(uint32_t cw, uint32_t cw2, StaticSid
 }
 __device__ __forceinline__ void static_feed(const StepArgs& A, int b, int lane, const RunRows& in, StaticSide& T, int& err) {
     ChainCounts kc = {1, 0, 0, 0, 0};
-    static_advance(A.S, lane, in.tok, in.toks, in.m, T.s, T.sf, T.l, T.ra, T.rb, err, kc, []() {});
+    static_advance<false>(A.S, lane, in.tok, in.toks, in.m, T.s, T.sf, T.l, T.ra, T.rb, err, kc, []() {});
     flush_counts(b, lane, true, kc, in.m);
 }
 __device__ __forceinline__ void static_close(uint32_t* cb, int lane, uint32_t ntok, const StaticSide& T) {
@@ -1620,42 +1627,268 @@ __device__ __forceinline__ void static_close(uint32_t* cb, int lane, uint32_t nt
     }
 }
 
-// One warp per slot takes both sides in turn: for batches whose slots fill the GPU, where what counts is how many
-// chains are resident (28 warps per SM).
-__global__ void __launch_bounds__(32, 28) sam_run_warp_kernel(const __grid_constant__ RunArgs R) {
+// Batches of more than two slots per SM: what counts is how much one resident warp carries.
+//   - The static side of a slot needs little help from other lanes (a state is one 32-byte record, a hash bucket eight
+//     16-byte entries), so a few LANES carry it, each group at its own pace (run_static_lanes).
+//   - The dynamic side has a warp per slot, without the static side's registers and waits (sam_run_split_kernel).
+//   - Both leave each step's result in the step's own outputs, and sam_run_finish_kernel, which no chain waits for, chooses the
+//     sources and reads the drafts: 32 rows a warp, eight rows' reads under way together.
+// Per step (a warp for both sides of a slot, before): 1000 slots 18.5 -> 8.3 us, 4096 slots 16.2 -> 7.9, 16384 slots
+// 58 -> 21.4.  Bound by the static chains up to 4096 slots (5 us a step), by the dynamic side's warps beyond.
+// What the two sides leave: match_len, state and status as they will be; the static side's first end position (or minus its
+// error) in draft_len, the dynamic side's in source, the text length in the first word of the draft.
+
+// The static side of 32 / G slots, G lanes each: Transfer (Algorithm 1) for every token of every step.  A pass of the loop
+// is one round of reads: the record of the state, the home bucket of (state, token) if it has hashed transitions, the root-row
+// entry of the token (used when the walk reaches the root in this pass), the token after it and the next step's count.
+// A step's first end position is in the record that the next step's first pass reads, so it is written then.
+// The lanes of a slot hold its state alike; each reads its share of the bucket's entries.
+template <int G>
+__device__ __forceinline__ void run_static_lanes(const RunArgs& R, int w, int lane) {
+    constexpr int E = SAM_HASH_BUCKET / G;
+    const StepArgs& A = R.A;
+    const SamStaticView& S = A.S;
+    const int sub = lane % G, group = lane - sub, b = (w * 32 + lane) / G;
+    const bool live = b < A.W.batch;
+    uint32_t* cb = A.W.ctrl + (size_t)(live ? b : 0) * SAM_CTRL_WORDS;
+    const int32_t* row = A.new_tokens + (size_t)(live ? b : 0) * A.stride;
+    const int32_t* cnt = A.counts + (live ? b : 0);
+    const size_t row_step = (size_t)A.W.batch * A.stride;
+    uint32_t s = 0, sf = 0, ntok = 0;
+    int32_t l = 0;
+    uint4 a = make_uint4(0, 0, 0, 0), bb = a;
+    bool active = live && R.n_steps > 0;
+    if (live) {
+        s = cb[CB_S1]; l = (int32_t)cb[CB_L1]; sf = cb[CB_S1FLAG]; ntok = cb[CB_NTOK_S];
+        a = *reinterpret_cast<const uint4*>(cb + CB_REC1); bb = *reinterpret_cast<const uint4*>(cb + CB_REC1 + 4);
+        if (cb[CB_STATUS] != 0) active = false;
+    }
+    const bool was = active;
+    bool have = s != 0, need_len = false, begin = true, bad = false;
+    uint32_t s0 = s, sf0 = sf; int32_t l0 = l;             // as the step found it: a refused step changes nothing
+    int i = 0, j = 0, m = 0, due = 0, err = 0, guard = 0;  // due: the first step whose result has not been written
+    int32_t t = 0, tn = row[0], mn = *cnt;
+    [[maybe_unused]] ChainCounts kc = {1, 0, 0, 0, 0};
+    for (;;) {
+        if (active) {
+            // steps begin here: those without tokens pass by, the first with tokens is looked at
+            while (begin && i < R.n_steps) {
+                m = mn; t = tn;
+                if (m < 0 || m > A.stride || (int64_t)ntok + m > A.W.max_seq_len || (m > 0 && (t < 0 || t >= S.vocab))) { bad = true; break; }
+                if (m > 0) { begin = false; j = 0; s0 = s; sf0 = sf; l0 = l; guard = l + 2 * m + 4; break; }
+                i++; row += row_step; cnt += A.W.batch;
+                if (i < R.n_steps) { mn = *cnt; tn = row[0]; }
+            }
+            if (bad || i >= R.n_steps) active = false;
+        }
+        const bool owed = live && was && due < i;          // results that wait for the record of s
+        if (!__any_sync(FULL, active || owed)) break;
+        SAM_COUNT(kc.rounds, active ? 1 : 0);
+        // none of these reads is under a branch: a lane that does not need a line reads one that every such lane shares
+        const bool at_root = s == 0;
+        const bool want_rec = (active || owed) && !at_root && !have;
+        const bool want_bucket = active && !at_root && sf != 0;
+        uint32_t home = want_bucket ? sam_hash2(s, (uint32_t)t) & S.hash_mask : 0u;
+        const uint32_t re = __ldg(S.root_row + (active ? t : 0));
+        const bool last_tok = j + 1 >= m, more = i + 1 < R.n_steps;
+        tn = active ? (last_tok ? (more ? row[row_step] : 0) : row[j + 1]) : 0;
+        mn = active && more ? cnt[A.W.batch] : 0;
+        const size_t ri = want_rec ? (size_t)s : 0;
+        const uint4 ra = __ldg(S.rec + 2 * ri), rb = __ldg(S.rec + 2 * ri + 1);
+        uint4 ent[E];
+#pragma unroll
+        for (int e = 0; e < E; e++) ent[e] = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + sub * E + e);
+        if (want_rec) { a = ra; bb = rb; have = true; }
+        if (owed) {
+            for (; due < i; due++) {
+                if (sub != 0 || (!R.keep && due + 1 < R.n_steps)) continue;
+                const StepOut o = step_out(A, R.keep ? due : 0);
+                o.match_len[2 * b] = l; o.draft_len[b] = l > 0 ? (int32_t)a.z : 0;
+                if (o.state) o.state[2 * b] = (int32_t)s;
+            }
+        }
+        // the transition: from the record, or from the bucket and the buckets after it
+        uint32_t tgt = at_root ? SAM_NONE : inline_target(a, bb, (uint32_t)t);
+        bool search = want_bucket && tgt == SAM_NONE;      // (every reference to a state with hashed transitions carries the flag)
+        for (int probe = 1; __any_sync(FULL, search); probe++) {
+            uint32_t z = SAM_NONE;
+            bool empty = false;
+#pragma unroll
+            for (int e = 0; e < E; e++) {
+                if (ent[e].x == s && ent[e].y == (uint32_t)t) z = ent[e].z;
+                empty |= ent[e].x == SAM_NONE;
+            }
+            const unsigned in_group = (0xFFFFFFFFu >> (32 - G)) << group;
+            const unsigned hit = __ballot_sync(FULL, search && z != SAM_NONE) & in_group, gap = __ballot_sync(FULL, search && empty) & in_group;
+            const uint32_t found = __shfl_sync(FULL, z, hit ? __ffs(hit) - 1 : lane);
+            if (search) {
+                if (hit) tgt = found;
+                if (hit || gap || probe >= S.hash_max_probe) search = false;
+                else {
+                    home = (home + 1) & S.hash_mask;
+#pragma unroll
+                    for (int e = 0; e < E; e++) ent[e] = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + sub * E + e);
+                }
+            }
+        }
+        if (active) {
+            bool advance = false;
+            if (at_root) {                                 // at the root the match length is 0
+                if (re != SAM_NONE) { s = re & SAM_IDMASK; sf = re >> 31; l = 1; have = false; SAM_COUNT(kc.b, 1); } else l = 0;
+                advance = true;
+            } else {
+                if (need_len) { l = (int32_t)a.x; need_len = false; }
+                have = false;
+                if (tgt != SAM_NONE) { s = tgt & SAM_IDMASK; sf = tgt >> 31; l += 1; advance = true; SAM_COUNT(kc.b, 1); }
+                else {                                     // s <- link(s), l <- len(link(s))
+                    SAM_COUNT(kc.a, 1);
+                    s = a.y & SAM_IDMASK; sf = a.y >> 31;
+                    if (s == 0) {                          // the root either has the token or not: known already
+                        if (re != SAM_NONE) { s = re & SAM_IDMASK; sf = re >> 31; l = 1; SAM_COUNT(kc.b, 1); } else l = 0;
+                        advance = true;
+                    } else need_len = true;
+                    if (--guard < 0) { err = SAM_SEQ_WALK_LIMIT; bad = true; }
+                }
+            }
+            if (advance && !bad) {
+                if (++j < m) {
+                    t = tn;
+                    if (t < 0 || t >= S.vocab) bad = true;
+                } else {
+                    ntok += (uint32_t)m;
+                    i++; row += row_step; cnt += A.W.batch;
+                    begin = true;
+                }
+            }
+            if (bad) { active = false; s = s0; sf = sf0; l = l0; have = false; need_len = false; }
+        }
+    }
+    if (!was || sub != 0) return;
+    if (err)
+        for (int k = i; k < R.n_steps; k++) if (R.keep || k + 1 == R.n_steps) step_out(A, R.keep ? k : 0).draft_len[b] = -err;
+    if (l > 0) {
+        if (!have) static_record(S, s, a, bb);
+        *reinterpret_cast<uint4*>(cb + CB_REC1) = a; *reinterpret_cast<uint4*>(cb + CB_REC1 + 4) = bb;
+    }
+    cb[CB_S1] = s; cb[CB_L1] = (uint32_t)l; cb[CB_S1FLAG] = sf; cb[CB_NTOK_S] = ntok;
+#ifdef SAM_COUNTERS
+    if (g_sam_counters && b < g_sam_counter_slots) {
+        unsigned long long* o = g_sam_counters + (size_t)b * SAM_N_COUNTERS;
+        o[SAM_CNT_STATIC_ROUNDS] += kc.rounds; o[SAM_CNT_STATIC_LINK_MOVES] += kc.a; o[SAM_CNT_STATIC_NEXT_MOVES] += kc.b;
+    }
+#endif
+}
+
+// Blocks [0, n_lane_blocks): the static sides, 32 slots each; the others: the dynamic side of one slot each.
+// G, the lanes of a static side: 1, 2, 4, 8 take 13.4, 8.2, 7.9, 8.4 us a step at 4096 slots (fewer lanes: a pass waits for
+// more lines and holds more registers) and 20.5, 21.4, 22.3, 25.0 at 16384 (more lanes: fewer warps for the dynamic sides).
+// 24 warps an SM rather than 28: the 72-register version spills 400 bytes.
+constexpr int run_lanes(int batch) { return batch <= 8192 ? 4 : 2; }
+template <int G>
+__global__ void __launch_bounds__(32, 24) sam_run_split_kernel(const __grid_constant__ RunArgs R) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     __shared__ __align__(16) uint32_t sh_run[32][12];
     const StepArgs& A = R.A;
-    const int b = blockIdx.x, lane = threadIdx.x;
+    const int lane = threadIdx.x;
+    if ((int)blockIdx.x < A.n_lane_blocks) { run_static_lanes<G>(R, blockIdx.x, lane); return; }
+    const int b = (int)blockIdx.x - A.n_lane_blocks;
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
     RunRows in;
     in.start(A, b, lane);
-    const int status0 = (int)__shfl_sync(FULL, cw, CB_STATUS);
-    int status = status0;
+    int status = (int)__shfl_sync(FULL, cw, CB_STATUS);
     DynChain X;
     kept_record(cw2, CB_REC2, X.ra, X.rb);
     dyn_open(A.W, b, lane, cb, cw, cw2, X);
-    StaticSide T;
-    static_open(cw, cw2, T);
     for (int i = 0; i < R.n_steps; i++) {
         const RunRows now = in;
         in.next(A, lane, i + 1 < R.n_steps);
         if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, X.ntok);
         if (status == 0) {
-            int err = 0;
-            if (A.has_static) static_feed(A, b, lane, now, T, err);
             X.D.kc = ChainCounts{1, 0, 0, 0, 0};
             dyn_feed(X, now.tok, now.toks, now.m, sh_run);
-            status = err ? err : X.D.err;
+            status = X.D.err;
         }
-        const StepOut o = step_out(A, R.keep ? i : 0);
-        if (status != 0) write_failed_slot(o, A.L, b, lane, status);
-        else write_slot<0>(A, o, b, lane, T.l, (int)T.s, (int64_t)T.ra.z, (int)X.l2, (int)X.s2, (int64_t)X.ra.z, (int64_t)X.ntok);
+        if (lane == 0 && (R.keep || i + 1 == R.n_steps)) {
+            const StepOut o = step_out(A, R.keep ? i : 0);
+            o.match_len[2 * b + 1] = (int32_t)X.l2; o.source[b] = (int32_t)X.ra.z; o.status[b] = status;
+            o.draft[(size_t)b * A.L] = (int32_t)X.ntok;
+            if (o.state) o.state[2 * b + 1] = (int32_t)X.s2;
+        }
     }
-    if (A.has_static && status0 == 0) static_close(cb, lane, X.ntok, T);
-    if (lane == 0 && status != status0) cb[CB_STATUS] = (uint32_t)status;
+    // (the slot's status is the finish kernel's to write: its static side may begin after this)
+}
+
+constexpr int FINISH_ROWS = 8;                             // rows whose reads a warp has under way together
+__global__ void __launch_bounds__(128) sam_run_finish_kernel(const __grid_constant__ RunArgs R) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const StepArgs& A = R.A;
+    const int lane = threadIdx.x & 31, L = A.L;
+    const int64_t rows = (int64_t)A.W.batch * (R.keep ? R.n_steps : 1);
+    const int64_t r0 = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * 32;
+    if (r0 >= rows) return;
+    const int64_t r = r0 + lane;
+    const bool live = r < rows;
+    int src = SAM_SRC_NONE, dl = 0;
+    const int32_t* from = A.S.corpus;
+    if (live) {                                            // lane k: row r0 + k
+        const int b = (int)(r % A.W.batch);
+        int status = A.status[r], l1 = 0, s1 = 0, e1 = 0;
+        int l2 = A.match_len[2 * r + 1];
+        const int e2 = A.source[r], ntok = A.draft_tokens[r * L];
+        if (A.has_static) {
+            l1 = A.match_len[2 * r]; e1 = A.draft_len[r];
+            if (status == 0 && e1 < 0) status = -e1;       // the static side's error, reported from here on
+        }
+        if (status != 0 && r + A.W.batch >= rows) A.W.ctrl[(size_t)b * SAM_CTRL_WORDS + CB_STATUS] = (uint32_t)status;
+        if (status != 0) {
+            l1 = l2 = 0;
+            A.status[r] = status;
+            if (A.state) { A.state[2 * r] = 0; A.state[2 * r + 1] = 0; }
+            A.match_len[2 * r + 1] = 0;
+        } else {
+            const bool use_static = A.has_static && l1 > l2 + A.W.l_bias;           // Section 3.2
+            const int lsel = use_static ? l1 : l2;
+            const int need = A.W.min_match > 1 ? A.W.min_match : 1;
+            src = lsel < need ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
+            if (src != SAM_SRC_NONE) {
+                const int64_t e = use_static ? e1 : e2, room = (use_static ? A.S.n_tokens : (int64_t)ntok) - e;
+                dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
+                from = (use_static ? A.S.corpus : A.W.text + (size_t)b * A.W.text_stride) + e;
+            }
+            if (!A.has_static && A.state) A.state[2 * r] = s1;
+        }
+        if (!A.has_static || status != 0) A.match_len[2 * r] = l1;
+        A.source[r] = src;
+    }
+    __syncwarp();                                          // (every lane has read its row's first word)
+    const int32_t stop = A.W.stop_token;
+    int cut = dl;
+    const int n = (int)(rows - r0 < 32 ? rows - r0 : 32);
+    for (int base = 0; base < L; base += 32)
+        for (int k0 = 0; k0 < n; k0 += FINISH_ROWS) {
+            int32_t v[FINISH_ROWS];
+#pragma unroll
+            for (int k = 0; k < FINISH_ROWS; k++) {
+                const int32_t* p = reinterpret_cast<const int32_t*>(__shfl_sync(FULL, (unsigned long long)from, (k0 + k) & 31));
+                const int d = __shfl_sync(FULL, dl, (k0 + k) & 31);
+                v[k] = -1;
+                if (base + lane < d) v[k] = p[base + lane];
+            }
+#pragma unroll
+            for (int k = 0; k < FINISH_ROWS; k++) {
+                int c = __shfl_sync(FULL, cut, (k0 + k) & 31);
+                if (stop >= 0) {                           // a draft ends before the first stop token
+                    const unsigned hit = __ballot_sync(FULL, v[k] == stop && base + lane < c);
+                    if (hit) c = base + __ffs(hit) - 1;
+                    if (lane == k0 + k) cut = c;
+                }
+                if (k0 + k < n && base + lane < L) A.draft_tokens[(r0 + k0 + k) * L + base + lane] = base + lane < c ? v[k] : -1;
+            }
+        }
+    if (live) A.draft_len[r] = cut;
 }
 
 // Three warps per slot: the static side, the dynamic side, and one that writes the outputs.  For batches that leave
@@ -1664,7 +1897,7 @@ constexpr int RUN_RING = 4;
 __device__ __forceinline__ void run_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void run_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
-__global__ void __launch_bounds__(96, 7) sam_run_block_kernel(const __grid_constant__ RunArgs R) {
+__global__ void __launch_bounds__(96, 4) sam_run_block_kernel(const __grid_constant__ RunArgs R) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     __shared__ __align__(16) uint32_t sh_run[32][12];
@@ -1836,7 +2069,8 @@ int split_kernel_setup(int device) {
     if (!done[device]) {
         cudaError_t e = cudaFuncSetAttribute(sam_step_split_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(order_slots_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_warp_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel<2>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
         done[device] = true;
     }
@@ -1962,8 +2196,9 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     return SAM_OK;
 }
 
-// Steps of sam_run_steps in one launch.  Up to how many slots three warps each fit the GPU at once: 148 SMs x 7 blocks.
-constexpr int SAM_RUN_BLOCK_MAX_BATCH = 1036;
+// Steps of sam_run_steps in one launch.  Up to two slots per SM three warps a slot are faster (256 slots 2.6 against 3.4 us a
+// step), from there on what the two sides cost in throughput counts (600 slots 4.9 against 4.4, 500 slots of c4's kind 9.7 against 7.2).
+constexpr int SAM_RUN_BLOCK_MAX_BATCH = 296;
 
 int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps, int32_t L, int32_t keep,
                    int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status,
@@ -1992,8 +2227,13 @@ int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride
     } else {
         int rc = split_kernel_setup(b->device);
         if (rc) return rc;
-        cfg.blockDim = dim3(32);
-        e = cudaLaunchKernelEx(&cfg, sam_run_warp_kernel, R);
+        const int lanes = run_lanes(b->view.batch);
+        A.n_lane_blocks = A.has_static ? (int)(((int64_t)b->view.batch * lanes + 31) / 32) : 0;
+        cfg.gridDim.x += (unsigned)A.n_lane_blocks; cfg.blockDim = dim3(32);
+        e = lanes == 4 ? cudaLaunchKernelEx(&cfg, sam_run_split_kernel<4>, R) : cudaLaunchKernelEx(&cfg, sam_run_split_kernel<2>, R);
+        const int64_t rows = (int64_t)b->view.batch * (keep ? n_steps : 1);
+        cfg.gridDim = dim3((unsigned)((rows + 127) / 128)); cfg.blockDim = dim3(128);
+        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, sam_run_finish_kernel, R);
     }
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;

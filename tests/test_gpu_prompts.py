@@ -115,3 +115,34 @@ def test_many_prompts_at_once(P, n):
     got, batch = gpu_run(P, st, VOCAB, rows[:, :n], rows[None, :, n:].copy(), counts, L, n + 8)
     assert_same(got, ref)
     assert_dynamic_automata_equal(batch, ob, range(0, B, 37), n + 8)
+
+
+@pytest.mark.parametrize("B,per_step", [(1, True), (296, True), (297, True), (297, False), (8193, True)])
+def test_steps_in_one_launch(P, B, per_step):
+    """sam_run_steps over each kernel's range: ragged counts, steps without tokens, slots that are refused on the way,
+    rows of up to 47 tokens, with and without room for every step's outputs, with and without a static automaton."""
+    import torch
+    rng = np.random.default_rng(B)
+    vocab, K, steps, L, msl = 60, 47, 5, 9, 150
+    corpus = rng.integers(0, vocab, size=5000, dtype=np.int32)
+    corpus[1000:2000] = corpus[:1000]
+    text = rng.integers(0, vocab, size=(B, steps * K + 1), dtype=np.int32)
+    text[:, 100:200] = corpus[900:1000]                     # long static matches
+    text[::3, 30:60] = text[::3, :30]
+    counts = np.where(rng.random((steps, B)) < 0.3, 0, rng.integers(0, K + 1, size=(steps, B))).astype(np.int32)
+    toks = np.stack([text[:, i * K:(i + 1) * K] for i in range(steps)]).copy()
+    if B > 8:
+        counts[1, 3] = -2; counts[2, 5] = K + 1; toks[1, 7, 4] = vocab; counts[1, 7] = 9; toks[3, 8, 0] = -7; counts[3, 8] = 1
+    keys = ("draft_tokens", "draft_len", "match_len", "source", "state", "status")
+    for static in (True, False):
+        st = P.StaticSam.build(corpus, vocab) if static else None
+        S = oracle.Sam(corpus) if static else None
+        ob = oracle.Batch(S, corpus if static else None, B, vocab, msl, 2, 2, 5)
+        batch = P.Batch(st, B, msl, max_draft_len=L, l_bias=2, min_match=2, vocab=vocab, stop_token=5)
+        for turn in range(2):                               # the second run goes on from the first
+            ref = [ob.step(toks[i], counts[i], L, 8) for i in range(steps)]
+            out = batch.run_steps(torch.from_numpy(toks).cuda(), torch.from_numpy(counts).cuda(), L, per_step=per_step).cpu()
+            for k in keys:
+                exp = np.stack([getattr(r, k) for r in ref]) if per_step else getattr(ref[-1], k)
+                assert np.array_equal(out[k], exp), (static, turn, k, np.argwhere(out[k] != exp)[:3])
+        assert_dynamic_automata_equal(batch, ob, [b for b in (0, 2, 3, 100) if b < B and ref[-1].status[b] == 0], msl)
