@@ -967,6 +967,102 @@ __device__ __forceinline__ void write_slot(const StepArgs& A, const StepOut& o, 
     }
 }
 
+// A third warp that reads ahead of the dynamic side, for batches that leave the GPU room for it.  It goes through the step's
+// tokens as the dynamic side will, from every token on along the transitions of the tokens after it, but only reads: the slot's root-table buckets, records and edge blocks come into the
+// SM's L1, where the dynamic side, which reads them one after the other, then finds them (a record from the L2 or beyond takes
+// it 520 cycles, an edge block 810).  The dynamic side changes these structures meanwhile, so what is read here may be of
+// any age; it is used for addresses only, each checked against the pool, and for no result.
+// The same reads made by the dynamic side itself, before its first token, cost what they saved; following the match
+// state's suffix links as well gave nothing.  Per step: 4 slots 6.2 -> 5.5 us, 64 slots 6.0 -> 5.5, 1000 slots 22.1 -> 20.8, 256
+// slots fed by verified drafts 26.2 -> 21.5.
+struct Ahead {
+    const unsigned char* pool;
+    uint32_t tab, n_states, n_units;      // lane i: slab index of state slab i; states and 128-byte units that may be read
+    int slab_shift, lane;
+};
+__device__ __forceinline__ uint4 ahead_load(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.ca.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+// The record of state s of each lane that wants one.
+__device__ __forceinline__ void ahead_records(const Ahead& H, bool want, uint32_t s, uint4& a, uint4& b) {
+    want = want && s != 0 && s < H.n_states;
+    const int rps_shift = H.slab_shift - 5;
+    const uint32_t slab = __shfl_sync(FULL, H.tab, want ? (int)(s >> rps_shift) : 0);
+    a = b = make_uint4(0, 0, 0, 0);
+    if (want) {
+        const unsigned char* p = H.pool + ((size_t)slab << H.slab_shift) + ((size_t)(s & ((1u << rps_shift) - 1)) << 5);
+        a = ahead_load(p); b = ahead_load(p + 16);
+    }
+}
+// Where each lane's state (record a, b) leads on token t: looked for in all lanes' edge blocks.
+__device__ __forceinline__ uint32_t ahead_targets(const Ahead& H, const uint4& a, const uint4& b, uint32_t t) {
+    uint32_t q = 0;
+    if (a.w >= 1 && a.w <= 2) { if (b.x == t) q = b.y; else if (a.w == 2 && b.z == t) q = b.w; }
+    const bool wide = a.w > 2 && a.w <= 512 && b.x + ((a.w + 15) >> 4) <= H.n_units && b.x < H.n_units;
+    const unsigned todo = __ballot_sync(FULL, wide);
+    for (unsigned w = todo; w; w &= w - 1) {               // every line of every block asked for ...
+        const int k = __ffs(w) - 1;
+        const uint32_t deg = __shfl_sync(FULL, a.w, k), off = __shfl_sync(FULL, b.x, k);
+        if ((uint32_t)H.lane * 16u < deg) asm volatile("prefetch.global.L1 [%0];" ::"l"(H.pool + ((size_t)off + H.lane) * 128));
+    }
+    for (unsigned w = todo; w; w &= w - 1) {               // ... before any is looked through
+        const int k = __ffs(w) - 1;
+        const uint32_t deg = __shfl_sync(FULL, a.w, k), off = __shfl_sync(FULL, b.x, k), tk = __shfl_sync(FULL, t, k);
+        for (uint32_t base = 0; base < deg; base += 64) {  // two entries a lane
+            const uint32_t i = base + 2u * H.lane;
+            uint4 e = make_uint4(SAM_NONE, 0, SAM_NONE, 0);
+            if (i < deg) e = ahead_load(H.pool + (size_t)off * 128 + (size_t)i * 8);
+            const bool first = e.x == tk, second = e.z == tk && i + 1 < deg;
+            const unsigned hit = __ballot_sync(FULL, first || second);
+            if (hit) {
+                const uint32_t v = __shfl_sync(FULL, first ? e.y : e.w, __ffs(hit) - 1);
+                if (H.lane == k) q = v;
+                break;
+            }
+        }
+    }
+    return q & SAM_IDMASK;
+}
+constexpr int AHEAD_MIN_TOKENS = 2, AHEAD_LEVELS = 4;
+__device__ __forceinline__ void read_ahead(const SamBatchView& W, int b, int lane, uint32_t cw, uint32_t cw2, int32_t tok_first, int m) {
+    const int n = m < 32 ? m : 32;
+    if (n < AHEAD_MIN_TOKENS) return;
+    Ahead H;
+    H.pool = W.pool; H.slab_shift = W.slab_shift; H.lane = lane;
+    {
+        const uint32_t lo = __shfl_sync(FULL, cw, (lane + 16) & 31), hi = __shfl_sync(FULL, cw2, (lane + 16) & 31);
+        H.tab = lane < 16 ? lo : hi;
+        if (H.tab >= (uint32_t)W.pool_slabs) H.tab = 0;
+    }
+    H.n_states = min(__shfl_sync(FULL, cw, CB_NSTATES), __shfl_sync(FULL, cw, CB_NRECSLABS) << (W.slab_shift - 5));
+    H.n_units = (uint32_t)W.pool_slabs << (W.slab_shift - 7);
+    const uint32_t t = (uint32_t)tok_first;
+    // the token's entry in the root table, from its home bucket
+    uint32_t u = 0;
+    if (lane < n) {
+        const uint32_t home = sam_hash1(t) & ((uint32_t)(W.root_cap / SAM_ROOT_BUCKET) - 1u);
+        const uint2* bucket = W.root_tab + (size_t)b * W.root_cap + (size_t)home * SAM_ROOT_BUCKET;
+#pragma unroll
+        for (int i = 0; i < SAM_ROOT_BUCKET / 2; i++) {
+            const uint4 e = ahead_load(bucket + 2 * i);
+            if (e.x == t) u = e.y & SAM_IDMASK;
+            if (e.z == t) u = e.w & SAM_IDMASK;
+        }
+    }
+    // level by level: lane k is at the state of tokens k .. k + level - 1 and looks up token k + level
+    uint4 a, bb;
+    ahead_records(H, lane < n, u, a, bb);
+    for (int level = 1; level <= AHEAD_LEVELS; level++) {
+        const uint32_t next = __shfl_sync(FULL, t, (lane + level) & 31);
+        if (lane + level >= n) a.w = 0;
+        if (!__any_sync(FULL, a.w != 0)) break;
+        u = ahead_targets(H, a, bb, next);
+        ahead_records(H, u != 0, u, a, bb);
+    }
+}
+
 // Both warps' results are in shared memory: choose the source, write the slot's outputs.
 template <bool VERIFY>
 __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp, int lane, uint32_t* cb, const int32_t* sh_l, const int32_t* sh_s,
@@ -1002,8 +1098,12 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
 
 // ------------------------------------------------------------------ the kernel
 // VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
-template <bool VERIFY>
-__global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ StepArgs A) {
+// The two warps that work on the slot.
+__device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+
+// AHEAD: a third warp reads ahead of the dynamic side (read_ahead).
+template <bool VERIFY, bool AHEAD>
+__global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_constant__ StepArgs A) {
     // Programmatic dependent launch: this grid may be scheduled while the previous kernel of the stream
     // is still finishing.  Nothing is read before that kernel has completed and flushed; the kernel
     // after this one is allowed to get scheduled right away (it waits in the same way).
@@ -1056,7 +1156,11 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
     int status = (int)__shfl_sync(FULL, cw, CB_STATUS);
     const uint32_t ntok0 = __shfl_sync(FULL, cw, CB_NTOK);
     const int L = A.L;
-    __syncthreads();          // both warps hold the slot's state as it was before either writes any of it
+    if (AHEAD && warp == 2) {
+        if (status == 0 && m <= A.stride && __shfl_sync(FULL, cw, CB_ERR_S) == 0) read_ahead(A.W, b, lane, cw, cw2, tok_first, m);
+        return;
+    }
+    step_sync();              // both warps hold the slot's state as it was before either writes any of it
 
     // what sam_prefill_kernel, launched before this one, has done of the slot
     const uint32_t done = __shfl_sync(FULL, cw, CB_ERR_S);
@@ -1128,10 +1232,10 @@ __global__ void __launch_bounds__(64) sam_step_kernel(const __grid_constant__ St
     }
 
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
-    __syncthreads();
+    step_sync();
     step_outputs<VERIFY>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, d, m, confirmed);
     if (A.done_flag) {
-        __syncthreads();
+        step_sync();
         if (threadIdx.x == 0) signal_done(A);
     }
 }
@@ -2058,6 +2162,7 @@ constexpr int split_big_m(int batch) { return batch >= 8192 ? 8 : 5; }
 int split_kernel_setup(int device);
 
 constexpr int SAM_SPLIT_MIN_BATCH = 8192;                    // the split step is used from this many slots on
+constexpr int SAM_AHEAD_MAX_BATCH = 1036;                    // three warps a slot, all slots resident at once (148 x 7)
 constexpr int SAM_ORDER_MIN_BATCH = 1536;                    // more slots than a B200 holds blocks of this kernel (148 x 10)
 
 }  // namespace
@@ -2188,8 +2293,10 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
         cfg.gridDim = dim3((unsigned)(b->view.batch + A.n_warp_blocks + A.n_lane_blocks)); cfg.blockDim = dim3(32);
         e = cudaLaunchKernelEx(&cfg, sam_step_split_kernel, A);
     } else {
-        e = v_draft ? cudaLaunchKernelEx(&cfg, sam_step_kernel<true>, A)
-                    : cudaLaunchKernelEx(&cfg, sam_step_kernel<false>, A);
+        const bool ahead = b->view.batch <= SAM_AHEAD_MAX_BATCH;
+        if (ahead) cfg.blockDim = dim3(96);
+        e = v_draft ? (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<true, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<true, false>, A))
+                    : (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<false, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<false, false>, A));
     }
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
