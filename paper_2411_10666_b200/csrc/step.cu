@@ -173,6 +173,7 @@ struct Look {                    // result of looking a token up in a non-root s
     uint32_t tgt;                // transition target with its S bit, valid if found
     uint32_t idx;                // 0 / 1 inline slot, or index in the edge block
     bool found;
+    uint4* rp;                   // the record
 };
 
 __device__ __forceinline__ uint4* rec_ptr(const Dyn& D, uint32_t s) {
@@ -225,8 +226,9 @@ __device__ __forceinline__ Look lookup_state(const Dyn& D, uint32_t p, uint32_t 
                                              bool have_rec = false, uint4 pa = make_uint4(0, 0, 0, 0),
                                              uint4 pb = make_uint4(0, 0, 0, 0)) {
     uint4 a = pa, b = pb;
-    if (!have_rec) { const uint4* rp = rec_ptr(D, p); a = rp[0]; b = rp[1]; SAM_COUNT(D.kc.rounds, 1); }
     Look r;
+    r.rp = rec_ptr(D, p);
+    if (!have_rec) { a = r.rp[0]; b = r.rp[1]; SAM_COUNT(D.kc.rounds, 1); }
     r.len = a.x; r.link = a.y; r.deg = a.w; r.b0 = b.x; r.b1 = b.y; r.b2 = b.z; r.b3 = b.w;
     r.found = false; r.tgt = 0; r.idx = 0;
     if (a.w <= 2) {
@@ -234,33 +236,31 @@ __device__ __forceinline__ Look lookup_state(const Dyn& D, uint32_t p, uint32_t 
         else if (a.w == 2 && b.z == t) { r.found = true; r.tgt = b.w; r.idx = 1; }
         return r;
     }
-    // 128 entries per round trip: the four reads of a lane are independent and go out together
-    const uint2* blk = blk_ptr(D, b.x);
+    // 128 entries per round trip, four a lane in two reads that go out together
+    const uint4* blk = reinterpret_cast<const uint4*>(blk_ptr(D, b.x));
     for (uint32_t base = 0; base < a.w; base += 128) {
         SAM_COUNT(D.kc.rounds, 1);
-        uint2 e[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const uint32_t i = base + 32 * u + D.lane;
-            e[u] = make_uint2(SAM_NONE, 0);
-            if (i < a.w) e[u] = blk[i];
+        const uint32_t i0 = base + 2u * D.lane, i1 = i0 + 64;
+        uint4 e0 = make_uint4(SAM_NONE, 0, SAM_NONE, 0), e1 = e0;
+        if (i0 < a.w) e0 = blk[i0 >> 1];
+        if (i1 < a.w) e1 = blk[i1 >> 1];
+        const bool x0 = e0.x == t, x1 = e1.x == t;                       // (what lies past the last transition is not looked at)
+        const bool m0 = x0 || (e0.z == t && i0 + 1 < a.w), m1 = x1 || (e1.z == t && i1 + 1 < a.w);
+        const unsigned hit = __ballot_sync(FULL, m0 || m1);
+        if (hit) {
+            const int src = __ffs(hit) - 1;
+            r.found = true;
+            r.tgt = __shfl_sync(FULL, m0 ? (x0 ? e0.y : e0.w) : (x1 ? e1.y : e1.w), src);
+            r.idx = __shfl_sync(FULL, m0 ? i0 + !x0 : i1 + !x1, src);
+            break;
         }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const unsigned hit = __ballot_sync(FULL, e[u].x == t);
-            if (hit && !r.found) {
-                const int src = __ffs(hit) - 1;
-                r.found = true; r.tgt = __shfl_sync(FULL, e[u].y, src); r.idx = base + 32 * u + src;
-            }
-        }
-        if (r.found) break;
     }
     return r;
 }
 
 // add the transition (p, t) -> tgt to a non-root state whose record is in lk
-__device__ __forceinline__ void insert_edge(Dyn& D, uint32_t p, const Look& lk, uint32_t t, uint32_t tgt) {
-    uint4* rp = rec_ptr(D, p);
+__device__ __forceinline__ void insert_edge(Dyn& D, const Look& lk, uint32_t t, uint32_t tgt) {
+    uint4* rp = lk.rp;
     uint32_t* rw = reinterpret_cast<uint32_t*>(rp);
     if (lk.deg < 2) {
         if (D.lane == 0) {
@@ -381,7 +381,7 @@ __device__ __forceinline__ void redirect_walk(Dyn& D, uint32_t pp, uint32_t t, u
         first = false;
         if (!l2k.found) { D.err = SAM_SEQ_WALK_LIMIT; return; }   // every state up the chain has t
         if ((l2k.tgt & SAM_IDMASK) != q) return;
-        uint32_t* rw2 = reinterpret_cast<uint32_t*>(rec_ptr(D, pp));
+        uint32_t* rw2 = reinterpret_cast<uint32_t*>(l2k.rp);
         if (D.lane == 0) {
             if (l2k.deg <= 2) rw2[5 + 2 * l2k.idx] = cl;
             else blk_ptr(D, l2k.b0)[l2k.idx].y = cl;
@@ -426,7 +426,7 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
     bool found = false, at_root = false;
     uint32_t qt = 0, plen = 0, root_slot = 0;
     Look lk;
-    lk.len = lk.link = lk.deg = lk.b0 = lk.b1 = lk.b2 = lk.b3 = lk.tgt = lk.idx = 0; lk.found = false;
+    lk.len = lk.link = lk.deg = lk.b0 = lk.b1 = lk.b2 = lk.b3 = lk.tgt = lk.idx = 0; lk.found = false; lk.rp = nullptr;
     int guard = (int)k + 2;
     for (;;) {
         if (p == 0) {
@@ -442,7 +442,7 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
         lk = lookup_state(D, p, t, use_rec, pa, pb);
         use_rec = false;
         if (lk.found) { found = true; qt = lk.tgt; plen = lk.len; break; }
-        insert_edge(D, p, lk, t, c);                   // len[p] + 1 < k: not solid
+        insert_edge(D, lk, t, c);                   // len[p] + 1 < k: not solid
         SAM_COUNT(D.kc.a, 1);
         if (D.err) return;
         p = lk.link;
@@ -497,7 +497,7 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
             if (at_root) {
                 root_retarget(D, root_slot, cl | SAM_FLAG);
             } else {
-                uint32_t* rw = reinterpret_cast<uint32_t*>(rec_ptr(D, p));
+                uint32_t* rw = reinterpret_cast<uint32_t*>(lk.rp);
                 if (D.lane == 0) {
                     if (lk.deg <= 2) rw[5 + 2 * lk.idx] = cl | SAM_FLAG;
                     else blk_ptr(D, lk.b0)[lk.idx].y = cl | SAM_FLAG;
@@ -1886,10 +1886,10 @@ __device__ __forceinline__ void run_static_lanes(const RunArgs& R, int w, int la
 // Blocks [0, n_lane_blocks): the static sides, 32 slots each; the others: the dynamic side of one slot each.
 // G, the lanes of a static side: 1, 2, 4, 8 take 13.4, 8.2, 7.9, 8.4 us a step at 4096 slots (fewer lanes: a pass waits for
 // more lines and holds more registers) and 20.5, 21.4, 22.3, 25.0 at 16384 (more lanes: fewer warps for the dynamic sides).
-// 24 warps an SM rather than 28: the 72-register version spills 400 bytes.
+// 20 warps an SM: with 96 registers nothing spills (28 or 24 warps, 72 or 80 registers: 9 and 5 % slower).
 constexpr int run_lanes(int batch) { return batch <= 8192 ? 4 : 2; }
 template <int G>
-__global__ void __launch_bounds__(32, 24) sam_run_split_kernel(const __grid_constant__ RunArgs R) {
+__global__ void __launch_bounds__(32, 20) sam_run_split_kernel(const __grid_constant__ RunArgs R) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     __shared__ __align__(16) uint32_t sh_run[32][12];
