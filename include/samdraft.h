@@ -206,12 +206,12 @@ int sam_run_steps(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t stride,
                   int32_t* source_dev, int32_t* state_dev, int32_t* status_dev, void* stream);
 
 /* sam_step with HOST arrays: copies new_tokens and counts to the device, runs the step, copies
- * every output back and waits for the stream — the end-to-end call a serving loop that keeps its
+ * every output back and waits for them — the end-to-end call a serving loop that keeps its
  * tokens on the host would make.  stride <= max_host_stride.  Any host memory works.  How the
- * bytes travel depends on the step's size: small steps go through a page-locked staging area that
- * the kernel reads and writes itself; from 64 KiB of arrays on, arrays that are ALL page-locked and
- * device-addressable (cudaHostAlloc, cudaHostRegister, a pinned torch tensor) are read and written
- * in place by the kernel, and any others are copied through the staging area.  state_host may be
+ * bytes travel depends on the step's size: few rows are carried by the launch, few outputs come back
+ * through a page-locked staging area word by word, each with the step's number; from 64 KiB of arrays on, arrays
+ * that are ALL page-locked and device-addressable (cudaHostAlloc, cudaHostRegister, a pinned torch tensor)
+ * are read and written in place by kernels, and any others are copied through the staging area.  state_host may be
  * NULL.  Synchronous: the results are in the arrays when the call returns.  Errors: as sam_step,
  * plus CUDA. */
 int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int32_t stride,
@@ -234,8 +234,8 @@ int sam_batch_pool_info(sam_batch_t* b, int64_t* total_slabs, int64_t* free_slab
 
 /* Number of kernels one decoding step (sam_step) launches for this batch: 1, or 2 for a batch larger than the GPU
  * holds at once (a small kernel first orders the slots so that those with the most tokens start first; the
- * step's results do not depend on it).  sam_step_host, being synchronous, gains nothing from the order
- * when its kernel works on the host arrays in place, and then makes one launch whatever the batch.  A step
+ * step's results do not depend on it).  sam_step_host, being synchronous, gains nothing from the order and
+ * never makes that launch; with many rows it makes another that brings them to the device.  A step
  * whose rows can hold a prompt (stride of 48 and more) makes two: prompts that fill an empty slot, then the rest.
  * Returns a negative sam_err_t for a null handle. */
 int sam_batch_launches_per_step(const sam_batch_t* b);

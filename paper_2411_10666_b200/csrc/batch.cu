@@ -2,6 +2,7 @@
 // the host-array step, the step replay loop and the inspection calls.
 #include "common.h"
 
+#include <atomic>
 #include <chrono>
 #include <cstring>
 #include <new>
@@ -10,6 +11,13 @@
 namespace {
 
 constexpr size_t SAM_ZERO_COPY_MAX_BYTES = 4u << 20;     // larger host steps go through two DMA copies
+// Outputs of a host step that come back as (word, number) pairs: no fence and no flag, twice the bytes.  With the rows in the
+// launch's arguments, 16 slots take 13.9 us a call instead of 18.5, 64 slots (1472 words) 15.3 instead of 19.8, 64 slots
+// of 47 words 21.0 instead of 24.6; from there on the bytes cost more.
+constexpr size_t SAM_TAGGED_MAX_WORDS = 4096;
+// From how many words of rows on a kernel brings them over ahead of the step's: 250 slots (3250 words) take 28.7 us without
+// and 30.6 with it, 1000 slots (13000) 39.2 without and 36.5 with it, 4000 slots 76 and 68.
+constexpr size_t SAM_FETCH_MIN_WORDS = 8192;
 constexpr size_t SAM_DIRECT_MIN_BYTES = 64u << 10;       // from this size on, page-locked caller arrays are used in place
 constexpr int SAM_POLL_LIMIT_US = 2000;                  // how long a host step polls its completion flag
 
@@ -274,7 +282,11 @@ extern "C" int sam_batch_create(const sam_static_t* st, const sam_batch_opts_t* 
 
     SamDeviceGuard guard(b->device);
     if (!guard.ok) { delete b; return SAM_ERR_CUDA; }
-    e = cudaHostAlloc((void**)&b->host_stage, (w.stage_words + 16) * 4, cudaHostAllocMapped);   // + the completion flag
+    // the staging area, the completion flag, and (word, number) pairs for the outputs of a small step
+    const size_t per_step = (size_t)opts->batch * ((size_t)opts->max_draft_len + 7);
+    const size_t pairs = per_step < SAM_TAGGED_MAX_WORDS ? per_step : SAM_TAGGED_MAX_WORDS;
+    const size_t pairs_at = sam_align_up(w.stage_words + 16, 16);
+    e = cudaHostAlloc((void**)&b->host_stage, (pairs_at + 2 * pairs) * 4, cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&b->host_stage_dev, b->host_stage, 0);
     if (e != cudaSuccess) {
         sam_set_cuda_error(e); cudaGetLastError();
@@ -283,6 +295,8 @@ extern "C" int sam_batch_create(const sam_static_t* st, const sam_batch_opts_t* 
         return SAM_ERR_NOMEM;
     }
     b->host_stage[w.stage_words] = 0;
+    b->host_tagged = b->host_stage + pairs_at; b->host_tagged_dev = b->host_stage_dev + pairs_at;
+    memset(b->host_tagged, 0, 2 * pairs * 4);             // no step has the number 0
     cudaStream_t s = (cudaStream_t)stream;
     if (sam_launch_init(V, s) != SAM_OK) { cudaFreeHost(b->host_stage); delete b; return SAM_ERR_CUDA; }
     *out = b;
@@ -326,6 +340,14 @@ static int check_step_args(const sam_batch* b, const void* toks, int32_t stride,
     return SAM_OK;
 }
 
+static SamStepIo step_io(const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t L, int32_t* draft_tokens,
+                         int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status) {
+    SamStepIo io{};
+    io.new_tokens = new_tokens; io.stride = stride; io.counts = counts; io.L = L;
+    io.draft_tokens = draft_tokens; io.draft_len = draft_len; io.match_len = match_len; io.source = source; io.state = state; io.status = status;
+    return io;
+}
+
 extern "C" int sam_step(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t stride,
                         const int32_t* counts_dev, int32_t L,
                         int32_t* draft_tokens_dev, int32_t* draft_len_dev, int32_t* match_len_dev,
@@ -333,8 +355,8 @@ extern "C" int sam_step(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t s
     int rc = check_step_args(b, new_tokens_dev, stride, counts_dev, L, draft_tokens_dev, draft_len_dev,
                              match_len_dev, source_dev, status_dev);
     if (rc) return rc;
-    return sam_launch_step(b, new_tokens_dev, stride, counts_dev, L, draft_tokens_dev, draft_len_dev,
-                           match_len_dev, source_dev, state_dev, status_dev, (cudaStream_t)stream);
+    return sam_launch_step(b, step_io(new_tokens_dev, stride, counts_dev, L, draft_tokens_dev, draft_len_dev, match_len_dev, source_dev,
+                                      state_dev, status_dev), (cudaStream_t)stream);
 }
 
 extern "C" int sam_step_verified(sam_batch_t* b, const int32_t* target_tokens_dev, int32_t prev_L,
@@ -348,9 +370,10 @@ extern "C" int sam_step_verified(sam_batch_t* b, const int32_t* target_tokens_de
     if (rc) return rc;
     if (!prev_draft_tokens_dev || prev_L < 1 || prev_L > 128) return SAM_ERR_ARG;
     if (prev_draft_tokens_dev == draft_tokens_dev || prev_draft_len_dev == draft_len_dev) return SAM_ERR_ARG;
-    return sam_launch_step_full(b, target_tokens_dev, prev_L + 1, nullptr, L, draft_tokens_dev, draft_len_dev,
-                                match_len_dev, source_dev, state_dev, status_dev, (cudaStream_t)stream, nullptr, 0,
-                                prev_draft_tokens_dev, prev_draft_len_dev, max_new_dev, counts_out_dev, accepted_out_dev);
+    SamStepIo io = step_io(target_tokens_dev, prev_L + 1, nullptr, L, draft_tokens_dev, draft_len_dev, match_len_dev, source_dev, state_dev, status_dev);
+    io.v_draft = prev_draft_tokens_dev; io.v_draft_len = prev_draft_len_dev; io.v_max_new = max_new_dev;
+    io.v_counts_out = counts_out_dev; io.v_accepted_out = accepted_out_dev;
+    return sam_launch_step(b, io, (cudaStream_t)stream);
 }
 
 extern "C" int sam_run_steps(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t stride,
@@ -367,10 +390,10 @@ extern "C" int sam_run_steps(sam_batch_t* b, const int32_t* new_tokens_dev, int3
     const size_t B = (size_t)b->view.batch;
     for (int32_t s = 0; s < n_steps; s++) {
         const size_t o = out_per_step ? (size_t)s : 0;
-        rc = sam_launch_step(b, new_tokens_dev + (size_t)s * B * stride, stride, counts_dev + (size_t)s * B, L,
-                             draft_tokens_dev + o * B * L, draft_len_dev + o * B, match_len_dev + o * B * 2,
-                             source_dev + o * B, state_dev ? state_dev + o * B * 2 : nullptr,
-                             status_dev + o * B, (cudaStream_t)stream);
+        rc = sam_launch_step(b, step_io(new_tokens_dev + (size_t)s * B * stride, stride, counts_dev + (size_t)s * B, L,
+                                        draft_tokens_dev + o * B * L, draft_len_dev + o * B, match_len_dev + o * B * 2,
+                                        source_dev + o * B, state_dev ? state_dev + o * B * 2 : nullptr, status_dev + o * B),
+                             (cudaStream_t)stream);
         if (rc) return rc;
     }
     return SAM_OK;
@@ -389,13 +412,78 @@ extern "C" int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int
     cudaStream_t s = (cudaStream_t)stream;
     const size_t B = (size_t)b->view.batch;
     // staging layout (int32 words): inputs [tokens B*stride | counts B], then outputs
-    // [draft B*L | draft_len B | match_len 2B | source B | state 2B | status B]
+    // [draft B*L | draft_len B | match_len 2B | source B | state 2B | status B], or B rows of L + 7 (word, number) pairs
     int32_t* dev = b->view.stage;
     int32_t* hst = b->host_stage;
-    const size_t in_words = B * stride + B;
-    const size_t out_words = B * L + 7 * B;
+    const size_t in_words = B * stride + B, out_words = B * L + 7 * B;
+    const int32_t seq = ++b->host_seq == 0 ? ++b->host_seq : b->host_seq;
+    // The waits below poll: the bytes are there sooner than a stream synchronisation returns.  They are bounded; past the
+    // bound (other work queued ahead on the stream, or a failed launch) the stream is synchronised, after which
+    // everything has to be there.
+    const auto t0 = std::chrono::steady_clock::now();
+    uint32_t spin = 0;
+    bool synced = false;
+    auto not_yet = [&]() -> int {
+        if ((++spin & 1023u) != 1023u || std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(SAM_POLL_LIMIT_US)) return SAM_OK;
+        if (synced) return SAM_ERR_CUDA;
+        SAM_CUDA(cudaStreamSynchronize(s));
+        synced = true;
+        return SAM_OK;
+    };
+
+    if (out_words <= SAM_TAGGED_MAX_WORDS) {
+        // Small steps: the rows and counts come with the launch, or are read by the kernel from the mapped staging area.  Each
+        // output word comes back with the step's number beside it, in one 8-byte store, so the kernel neither fences nor
+        // signals: a word whose number is the step's is there.
+        SamStepIo io = step_io(b->host_stage_dev, stride, b->host_stage_dev + B * stride, L, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
+        io.from_host = true; io.done_seq = seq; io.tagged = b->host_tagged_dev;
+        if (sam_step_is_inline(b, stride)) { io.inline_rows = new_tokens_host; io.inline_counts = counts_host; }
+        else {
+            memcpy(hst, new_tokens_host, B * stride * 4);
+            memcpy(hst + B * stride, counts_host, B * 4);
+        }
+        rc = sam_launch_step(b, io, s);
+        if (rc) return rc;
+        const volatile uint64_t* w = reinterpret_cast<const volatile uint64_t*>(b->host_tagged);
+        const size_t R = (size_t)L + 7;
+        for (size_t i = 0; i < B; i++, w += R) {
+            int32_t* draft = draft_tokens_host + i * L;
+            int32_t rest[7];
+            for (size_t k = 0; k < R; k++) {
+                uint64_t v;
+                while ((v = w[k]) >> 32 != (uint64_t)(uint32_t)seq) if ((rc = not_yet()) != SAM_OK) return rc;
+                if (k < (size_t)L) draft[k] = (int32_t)v; else rest[k - L] = (int32_t)v;
+            }
+            draft_len_host[i] = rest[0]; match_len_host[2 * i] = rest[1]; match_len_host[2 * i + 1] = rest[2]; source_host[i] = rest[3];
+            if (state_host) { state_host[2 * i] = rest[4]; state_host[2 * i + 1] = rest[5]; }
+            status_host[i] = rest[6];
+        }
+        return SAM_OK;
+    }
+
+    // Larger steps: the kernel writes to host memory itself, and the last block to finish writes this step's number into the
+    // flag word behind the staging area.  Rows and counts come with the launch where they fit, are brought over ahead of it
+    // where they are many, and are read by the kernel in between.
+    int32_t* flag_dev = b->host_stage_dev + b->stage_words;
+    const volatile int32_t* flag = b->host_stage + b->stage_words;
+    auto run = [&](const int32_t* rows, const int32_t* cnt, int32_t* d, int32_t* dl, int32_t* ml, int32_t* so, int32_t* st, int32_t* sta,
+                   const int32_t* rows_host, const int32_t* cnt_host) -> int {
+        SamStepIo io = step_io(rows, stride, cnt, L, d, dl, ml, so, st, sta);
+        io.from_host = true; io.done_flag = flag_dev; io.done_seq = seq;
+        if (sam_step_is_inline(b, stride)) { io.inline_rows = rows_host; io.inline_counts = cnt_host; }
+        else if (in_words >= SAM_FETCH_MIN_WORDS) {
+            int r = sam_launch_fetch(b, rows, cnt, dev, stride, s);
+            if (r) return r;
+            io.new_tokens = dev; io.counts = dev + B * stride;
+        }
+        int r = sam_launch_step(b, io, s);
+        if (r) return r;
+        while (*flag != seq) if ((r = not_yet()) != SAM_OK) return r;
+        std::atomic_thread_fence(std::memory_order_acquire);
+        return SAM_OK;
+    };
     if ((in_words + out_words) * 4 >= SAM_DIRECT_MIN_BYTES) {
-        // Large steps: copying the arrays through the staging area on the host costs more than the step.
+        // Copying the arrays through the staging area on the host costs more than the step.
         // If every array the caller passed is page-locked memory the device can address (cudaHostAlloc /
         // cudaHostRegister: what a pinned torch tensor is), the kernel reads and writes them in place.
         const void* hp[8] = {new_tokens_host, counts_host, draft_tokens_host, draft_len_host, match_len_host,
@@ -406,53 +494,23 @@ extern "C" int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int
             if (!hp[i]) continue;                              // state_host may be null
             if (cudaHostGetDevicePointer(&dp[i], const_cast<void*>(hp[i]), 0) != cudaSuccess) { cudaGetLastError(); direct = false; }
         }
-        if (direct) {
-            volatile int32_t* flag = b->host_stage + b->stage_words;
-            const int32_t seq = ++b->host_seq == 0 ? ++b->host_seq : b->host_seq;
-            rc = sam_launch_step_signal(b, (const int32_t*)dp[0], stride, (const int32_t*)dp[1], L, (int32_t*)dp[2], (int32_t*)dp[3],
-                                        (int32_t*)dp[4], (int32_t*)dp[5], (int32_t*)dp[7], (int32_t*)dp[6], s,
-                                        b->host_stage_dev + b->stage_words, seq);
-            if (rc) return rc;
-            const auto t0 = std::chrono::steady_clock::now();
-            bool seen = false;
-            for (uint32_t spin = 0;; spin++) {
-                if (*flag == seq) { seen = true; break; }
-                if ((spin & 1023u) == 1023u &&
-                    std::chrono::steady_clock::now() - t0 > std::chrono::microseconds(SAM_POLL_LIMIT_US)) break;
-            }
-            if (!seen) SAM_CUDA(cudaStreamSynchronize(s));
-            return SAM_OK;
-        }
+        if (direct)
+            return run((const int32_t*)dp[0], (const int32_t*)dp[1], (int32_t*)dp[2], (int32_t*)dp[3], (int32_t*)dp[4], (int32_t*)dp[5],
+                       (int32_t*)dp[7], (int32_t*)dp[6], new_tokens_host, counts_host);
     }
     memcpy(hst, new_tokens_host, B * stride * 4);
     memcpy(hst + B * stride, counts_host, B * 4);
     int32_t* ho = hst + in_words;
     if ((in_words + out_words) * 4 <= SAM_ZERO_COPY_MAX_BYTES) {
-        // small steps: the kernel reads its inputs from, and writes its outputs to, the mapped host
-        // staging area directly; the bytes cross the bus inside the kernel instead of in two copies
         int32_t* zd = b->host_stage_dev;
         int32_t* zo = zd + in_words;
-        // completion: the last block writes this step's sequence number into the flag word behind the
-        // staging area; polling it costs less than a stream synchronisation.  The poll is bounded;
-        // past the bound (other work queued ahead on the stream, or a failed launch) it falls back.
-        volatile int32_t* flag = b->host_stage + b->stage_words;
-        const int32_t seq = ++b->host_seq == 0 ? ++b->host_seq : b->host_seq;
-        rc = sam_launch_step_signal(b, zd, stride, zd + B * stride, L, zo, zo + B * L, zo + B * L + B, zo + B * L + 3 * B,
-                                    zo + B * L + 4 * B, zo + B * L + 6 * B, s, b->host_stage_dev + b->stage_words, seq);
+        rc = run(zd, zd + B * stride, zo, zo + B * L, zo + B * L + B, zo + B * L + 3 * B, zo + B * L + 4 * B, zo + B * L + 6 * B, hst, hst + B * stride);
         if (rc) return rc;
-        const auto t0 = std::chrono::steady_clock::now();
-        bool seen = false;
-        for (uint32_t spin = 0;; spin++) {
-            if (*flag == seq) { seen = true; break; }
-            if ((spin & 1023u) == 1023u &&
-                std::chrono::steady_clock::now() - t0 > std::chrono::microseconds(SAM_POLL_LIMIT_US)) break;
-        }
-        if (!seen) SAM_CUDA(cudaStreamSynchronize(s));
     } else {
         SAM_CUDA(cudaMemcpyAsync(dev, hst, in_words * 4, cudaMemcpyHostToDevice, s));
         int32_t* o = dev + in_words;
-        rc = sam_launch_step(b, dev, stride, dev + B * stride, L, o, o + B * L, o + B * L + B, o + B * L + 3 * B,
-                             o + B * L + 4 * B, o + B * L + 6 * B, s);
+        rc = sam_launch_step(b, step_io(dev, stride, dev + B * stride, L, o, o + B * L, o + B * L + B, o + B * L + 3 * B,
+                                        o + B * L + 4 * B, o + B * L + 6 * B), s);
         if (rc) return rc;
         SAM_CUDA(cudaMemcpyAsync(ho, o, out_words * 4, cudaMemcpyDeviceToHost, s));
         SAM_CUDA(cudaStreamSynchronize(s));

@@ -26,6 +26,8 @@ struct sam_batch {
     size_t stage_words;           // int32 words of device staging
     int32_t* host_stage;          // pinned, device-mapped host staging area
     int32_t* host_stage_dev;      // the same memory as the device addresses it
+    int32_t* host_tagged;         // part of it: (word, step number) pairs, and as the device addresses them
+    int32_t* host_tagged_dev;
     int32_t host_seq;             // sequence number of the last host-array step (completion flag value)
     int32_t reset_count;          // number of the last reset of some slots
     mutable int32_t order_phase;  // which of the two slot-order buffers the next large-batch step uses
@@ -52,22 +54,24 @@ struct SamDeviceGuard {
 
 static inline size_t sam_align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// launchers implemented in step.cu
-int sam_launch_step(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts,
-                    int32_t L, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
-                    int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream);
-
-int sam_launch_step_signal(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts,
-                           int32_t L, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
-                           int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream,
-                           int32_t* done_flag_dev, int32_t done_seq);
-
-int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts,
-                         int32_t L, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
-                         int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream,
-                         int32_t* done_flag_dev, int32_t done_seq,
-                         const int32_t* v_draft, const int32_t* v_draft_len, const int32_t* v_max_new,
-                         int32_t* v_counts_out, int32_t* v_accepted_out);
+// What one step reads and writes (launchers in step.cu).
+struct SamStepIo {
+    const int32_t* new_tokens; int32_t stride; const int32_t* counts; int32_t L;
+    int32_t *draft_tokens, *draft_len, *match_len, *source, *state, *status;
+    // sam_step_verified
+    const int32_t *v_draft, *v_draft_len, *v_max_new;
+    int32_t *v_counts_out, *v_accepted_out;
+    // sam_step_host: rows and counts to carry with the launch, if any; completion: either the last block writes done_seq to
+    // *done_flag, or every output word goes to `tagged` with done_seq beside it
+    bool from_host;
+    const int32_t *inline_rows, *inline_counts;
+    int32_t* done_flag; int32_t done_seq;
+    void* tagged;
+};
+int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream);
+bool sam_step_is_inline(const sam_batch* b, int32_t stride);
+// host-mapped rows and counts to device memory, one behind the other
+int sam_launch_fetch(const sam_batch* b, const int32_t* rows, const int32_t* counts, int32_t* to, int32_t stride, cudaStream_t stream);
 
 // n_steps steps in one launch (step.cu), and whether they can be
 int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps,

@@ -82,6 +82,9 @@ extern "C" int sam_retrieve_noalloc(const sam_static_t* st, int32_t vocab, int32
     cudaStream_t s = (cudaStream_t)stream;
     rc = sam_launch_init(tmp.view, s);                        // the array keeps the last call's contents: start clean
     if (rc) return rc;
-    return sam_launch_step(&tmp, tokens_dev, stride, counts_dev, L, draft_tokens_dev, draft_len_dev,
-                           match_len_dev, source_dev, state_dev, status_dev, s);
+    SamStepIo io{};
+    io.new_tokens = tokens_dev; io.stride = stride; io.counts = counts_dev; io.L = L;
+    io.draft_tokens = draft_tokens_dev; io.draft_len = draft_len_dev; io.match_len = match_len_dev;
+    io.source = source_dev; io.state = state_dev; io.status = status_dev;
+    return sam_launch_step(&tmp, io, s);
 }

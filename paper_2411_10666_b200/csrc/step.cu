@@ -89,6 +89,9 @@ struct StepArgs {
     // optional completion signal for the host-array step: the last block to finish writes done_seq to
     // *done_flag (host-mapped memory) so the host can poll instead of synchronising the stream
     int32_t* done_count; int32_t* done_flag; int32_t done_seq;
+    // small host-array steps: where set, slot b's outputs go to row b of this host-mapped buffer, L + 7 words (draft,
+    // draft_len, match_len[2], source, state[2], status), each with the step's number beside it (sam_step_host)
+    uint2* tagged; uint32_t tag;
     // optional fused greedy verification (Section 2.2): when v_draft is set, new_tokens holds the target
     // model's tokens [B, stride] with stride = previous draft length limit + 1, and each slot's count is
     // derived here: the confirmed prefix of its previous draft plus the target's next token
@@ -928,6 +931,11 @@ __device__ __forceinline__ StepOut step_out(const StepArgs& A, int at) {
     return {A.draft_tokens + n * A.L, A.draft_len + n, A.match_len + 2 * n, A.source + n, A.state ? A.state + 2 * n : nullptr, A.status + n};
 }
 
+__device__ __forceinline__ void write_failed_tagged(const StepArgs& A, int b, int lane, int status) {
+    uint2* row = A.tagged + (size_t)b * (A.L + 7);
+    for (int j = lane; j < A.L + 7; j += 32) row[j] = make_uint2(j < A.L ? 0xFFFFFFFFu : j == A.L + 6 ? (uint32_t)status : 0u, A.tag);
+}
+
 __device__ __forceinline__ void write_failed_slot(const StepOut& o, int L, int b, int lane, int status) {
     for (int j = lane; j < L; j += 32) o.draft[(size_t)b * L + j] = -1;
     if (lane == 0) {
@@ -1076,6 +1084,23 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
     const int src = (any_err || lsel < need) ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
     const int winner = src == SAM_SRC_DYNAMIC ? 1 : 0;
 
+    if (A.tagged) {
+        uint2* row = A.tagged + (size_t)b * (L + 7);
+        if (warp == winner) {
+#pragma unroll
+            for (int r = 0; r < MAX_DRAFT_REGS; r++) {
+                const int j = r * 32 + lane;
+                if (j < L) row[j] = make_uint2((uint32_t)(src == SAM_SRC_NONE ? -1 : d[r]), A.tag);
+            }
+        }
+        if (warp == 0) {
+            const int v = lane == 0 ? (src == SAM_SRC_NONE ? 0 : sh_dl[winner]) : lane == 3 ? src : lane == 6 ? any_err : any_err ? 0 :
+                          lane == 1 ? l1 : lane == 2 ? l2v : lane == 4 ? sh_s[0] : sh_s[1];
+            if (lane < 7) row[L + lane] = make_uint2((uint32_t)v, A.tag);
+            if (any_err && lane == 0) cb[CB_STATUS] = (uint32_t)any_err;
+        }
+        return;
+    }
     if (warp == winner) {
 #pragma unroll
         for (int r = 0; r < MAX_DRAFT_REGS; r++) {
@@ -1102,8 +1127,9 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
 __device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 
 // AHEAD: a third warp reads ahead of the dynamic side (read_ahead).
-template <bool VERIFY, bool AHEAD>
-__global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_constant__ StepArgs A) {
+// INLINE: the rows and counts came with the launch (sam_step_host).
+template <bool VERIFY, bool AHEAD, bool INLINE>
+__device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_tokens, const int32_t* counts) {
     // Programmatic dependent launch: this grid may be scheduled while the previous kernel of the stream
     // is still finishing.  Nothing is read before that kernel has completed and flushed; the kernel
     // after this one is allowed to get scheduled right away (it waits in the same way).
@@ -1112,10 +1138,10 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_
         // block reads first, so that their address translations and L2 lines are at hand after the wait.
         const int pb_ = blockIdx.x, pl_ = threadIdx.x & 31;
         const char* p0 = reinterpret_cast<const char*>(A.W.ctrl + (size_t)pb_ * SAM_CTRL_WORDS);
-        const char* p1 = reinterpret_cast<const char*>(A.new_tokens + (size_t)pb_ * A.stride);
-        const char* p2 = reinterpret_cast<const char*>(VERIFY ? A.v_draft_len + pb_ : A.counts + pb_);
+        const char* p1 = reinterpret_cast<const char*>(new_tokens + (size_t)pb_ * A.stride);
+        const char* p2 = reinterpret_cast<const char*>(VERIFY ? A.v_draft_len + pb_ : counts + pb_);
         const char* pp_ = pl_ == 0 ? p0 : pl_ == 1 ? p0 + 128 : pl_ == 2 ? p1 : p2;
-        if (pl_ < 4) asm volatile("prefetch.global.L2 [%0];" ::"l"(pp_));
+        if (pl_ < (INLINE ? 2 : 4)) asm volatile("prefetch.global.L2 [%0];" ::"l"(pp_));
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
@@ -1128,7 +1154,7 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_
     // words (state, slab table, copies of the two match states' records), its count, and the
     // first 32 tokens of its row (read before the count is known; unused lanes are ignored).
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
-    const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
+    const int32_t* toks = new_tokens + (size_t)b * A.stride;
     const uint32_t cw = cb[lane];                       // control words 0..31
     const uint32_t cw2 = cb[32 + lane];                 // control words 32..63
     int32_t tok_first = 0;
@@ -1151,7 +1177,7 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_
         if (A.v_max_new) { int cap = A.v_max_new[b]; cap = cap < 0 ? 0 : cap; m = m < cap ? m : cap; }
         confirmed = a < m ? a : m;
     } else {
-        m = A.counts[b];
+        m = counts[b];
     }
     int status = (int)__shfl_sync(FULL, cw, CB_STATUS);
     const uint32_t ntok0 = __shfl_sync(FULL, cw, CB_NTOK);
@@ -1190,7 +1216,8 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_
     if (status != 0) {
         if (warp == 0) {
             if (fresh_fail && lane == 0) cb[CB_STATUS] = (uint32_t)status;
-            write_failed_slot(step_out(A, 0), L, b, lane, status);
+            if (A.tagged) write_failed_tagged(A, b, lane, status);
+            else write_failed_slot(step_out(A, 0), L, b, lane, status);
             if (lane == 0) {
                 if (VERIFY && A.v_counts_out) A.v_counts_out[b] = m;
                 if (VERIFY && A.v_accepted_out) A.v_accepted_out[b] = confirmed;
@@ -1237,6 +1264,39 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_
     if (A.done_flag) {
         step_sync();
         if (threadIdx.x == 0) signal_done(A);
+    }
+}
+
+template <bool VERIFY, bool AHEAD>
+__global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_constant__ StepArgs A) {
+    step_body<VERIFY, AHEAD, false>(A, A.new_tokens, A.counts);
+}
+
+// A host-array step whose rows and counts fit the launch's arguments: reading them from host memory, in the kernel's first
+// round, costs 1.1 us for 4 slots and 3.2 us for 64 (many small requests on the bus), carrying them with the launch nothing.
+// (With 32 KB of arguments, for 250 slots, it costs 3 us more than it saves.)
+constexpr int SAM_INLINE_WORDS = 896;                    // within 4 KB of arguments
+struct StepArgsInline { StepArgs A; int32_t in[SAM_INLINE_WORDS]; };                // rows, then counts
+__global__ void __launch_bounds__(96) sam_step_inline_kernel(const __grid_constant__ StepArgsInline I) {
+    step_body<false, true, true>(I.A, I.in, I.in + (size_t)I.A.W.batch * I.A.stride);
+}
+
+// Larger ones: the rows and counts are brought over in whole lines by this kernel, launched ahead of the step's.
+__global__ void __launch_bounds__(128) fetch_inputs_kernel(const int32_t* rows, const int32_t* counts, int32_t* to, uint32_t n_rows, uint32_t n_counts) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const int32_t* from = k ? counts : rows;
+        int32_t* dst = k ? to + n_rows : to;
+        const uint32_t n = k ? n_counts : n_rows;
+        uint32_t done = 0;
+        if (((reinterpret_cast<uintptr_t>(from) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+            for (uint32_t i = t; i < n / 4; i += all) reinterpret_cast<int4*>(dst)[i] = reinterpret_cast<const int4*>(from)[i];
+            done = n & ~3u;
+        }
+        for (uint32_t i = done + t; i < n; i += all) dst[i] = from[i];
     }
 }
 
@@ -1669,10 +1729,6 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
     } else {
         // the dynamic side's time hardly depends on the token count: slots in their own order, one read less
         dynamic_slot(A, i - A.n_warp_blocks - A.n_lane_blocks, lane, sh_run);
-    }
-    if (A.done_flag) {
-        __syncwarp();
-        if (lane == 0) signal_done(A);
     }
 }
 
@@ -2210,40 +2266,24 @@ int launch_prefill(const StepArgs& A, int batch, int device, cudaLaunchConfig_t*
 
 int sam_step_launch_count(const sam_batch* b) { return b->view.batch >= SAM_ORDER_MIN_BATCH ? 2 : 1; }
 
-int sam_launch_step(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts,
-                    int32_t L, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
-                    int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream) {
-    return sam_launch_step_signal(b, new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state,
-                                  status, stream, nullptr, 0);
-}
-
-int sam_launch_step_signal(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts,
-                           int32_t L, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
-                           int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream,
-                           int32_t* done_flag_dev, int32_t done_seq) {
-    return sam_launch_step_full(b, new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state,
-                                status, stream, done_flag_dev, done_seq, nullptr, nullptr, nullptr, nullptr, nullptr);
-}
-
-int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts,
-                         int32_t L, int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len,
-                         int32_t* source, int32_t* state, int32_t* status, cudaStream_t stream,
-                         int32_t* done_flag_dev, int32_t done_seq,
-                         const int32_t* v_draft, const int32_t* v_draft_len, const int32_t* v_max_new,
-                         int32_t* v_counts_out, int32_t* v_accepted_out) {
+int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream) {
     SamDeviceGuard guard(b->device);
     if (!guard.ok) return SAM_ERR_CUDA;
     StepArgs A;
-    A.v_draft = v_draft; A.v_draft_len = v_draft_len; A.v_max_new = v_max_new;
-    A.v_counts_out = v_counts_out; A.v_accepted_out = v_accepted_out;
-    A.done_count = b->view.pool_hdr + 4; A.done_flag = done_flag_dev; A.done_seq = done_seq;
+    const bool verify = io.v_draft != nullptr;
+    A.v_draft = io.v_draft; A.v_draft_len = io.v_draft_len; A.v_max_new = io.v_max_new;
+    A.v_counts_out = io.v_counts_out; A.v_accepted_out = io.v_accepted_out;
+    A.done_count = b->view.pool_hdr + 4; A.done_flag = io.done_flag; A.done_seq = io.done_seq;
+    A.tagged = reinterpret_cast<uint2*>(io.tagged); A.tag = (uint32_t)io.done_seq;
     A.has_static = b->st != nullptr;
     if (b->st) A.S = b->st->view;
     else { A.S = SamStaticView(); A.S.vocab = b->view.vocab; }
     A.W = b->view;
-    A.new_tokens = new_tokens; A.stride = stride; A.counts = counts; A.L = L;
-    A.draft_tokens = draft_tokens; A.draft_len = draft_len; A.match_len = match_len;
-    A.source = source; A.state = state; A.status = status;
+    const int32_t stride = io.stride;
+    const int32_t* counts = io.counts;
+    A.new_tokens = io.new_tokens; A.stride = stride; A.counts = counts; A.L = io.L;
+    A.draft_tokens = io.draft_tokens; A.draft_len = io.draft_len; A.match_len = io.match_len;
+    A.source = io.source; A.state = io.state; A.status = io.status;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -2251,7 +2291,7 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     A.n_warp_blocks = A.n_lane_blocks = 0;
     bool prompts = false;
 #ifndef SAM_COUNTERS                                       // (the counters count Expand's own operations, one Expand at a time)
-    prompts = !v_draft && stride >= SAM_PREFILL_MIN;
+    prompts = !verify && stride >= SAM_PREFILL_MIN;
 #endif
     if (prompts) {
         cudaLaunchConfig_t pc;
@@ -2262,7 +2302,7 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     }
     // (A host-array step is synchronous: nothing runs before it that the ordering kernel could overlap with, so it
     // would cost more than the order saves; such a step is always the one two-warp launch, slots in their own order.)
-    if (!v_draft && !prompts && !done_flag_dev && b->view.batch >= SAM_ORDER_MIN_BATCH) {
+    if (!verify && !prompts && !io.from_host && b->view.batch >= SAM_ORDER_MIN_BATCH) {
         int32_t* order = b->view.order + (size_t)(b->order_phase & 1) * b->view.batch;
         cudaLaunchConfig_t oc;
         memset(&oc, 0, sizeof(oc));
@@ -2295,11 +2335,36 @@ int sam_launch_step_full(const sam_batch* b, const int32_t* new_tokens, int32_t 
     } else {
         const bool ahead = b->view.batch <= SAM_AHEAD_MAX_BATCH;
         if (ahead) cfg.blockDim = dim3(96);
-        e = v_draft ? (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<true, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<true, false>, A))
-                    : (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<false, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<false, false>, A));
+        if (io.inline_rows && ahead && !prompts) {
+            const size_t rows = (size_t)b->view.batch * stride;
+            StepArgsInline I;
+            I.A = A;
+            memcpy(I.in, io.inline_rows, rows * 4);
+            memcpy(I.in + rows, io.inline_counts, (size_t)b->view.batch * 4);
+            e = cudaLaunchKernelEx(&cfg, sam_step_inline_kernel, I);
+        } else
+            e = verify ? (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<true, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<true, false>, A))
+                       : (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<false, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<false, false>, A));
     }
-    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
+    return SAM_OK;
+}
+
+// Whether a host-array step's rows and counts can come with the launch.
+bool sam_step_is_inline(const sam_batch* b, int32_t stride) {
+    return stride < SAM_PREFILL_MIN && b->view.batch <= SAM_AHEAD_MAX_BATCH &&
+           (size_t)b->view.batch * (stride + 1) <= (size_t)SAM_INLINE_WORDS;
+}
+
+int sam_launch_fetch(const sam_batch* b, const int32_t* rows, const int32_t* counts, int32_t* to, int32_t stride, cudaStream_t stream) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    const size_t n = (size_t)b->view.batch * stride, blocks = (n + 511) / 512;      // a 16-byte read a thread
+    cfg.gridDim = dim3((unsigned)(blocks < 592 ? blocks : 592)); cfg.blockDim = dim3(128); cfg.stream = stream; cfg.attrs = attr; cfg.numAttrs = 1;
+    SAM_CUDA(cudaLaunchKernelEx(&cfg, fetch_inputs_kernel, rows, counts, to, (uint32_t)n, (uint32_t)b->view.batch));
     return SAM_OK;
 }
 

@@ -146,3 +146,34 @@ def test_steps_in_one_launch(P, B, per_step):
                 exp = np.stack([getattr(r, k) for r in ref]) if per_step else getattr(ref[-1], k)
                 assert np.array_equal(out[k], exp), (static, turn, k, np.argwhere(out[k] != exp)[:3])
         assert_dynamic_automata_equal(batch, ob, [b for b in (0, 2, 3, 100) if b < B and ref[-1].status[b] == 0], msl)
+
+
+@pytest.mark.parametrize("B,stride,L", [(1, 1, 1), (16, 47, 9), (18, 48, 9), (74, 11, 40), (75, 11, 40), (86, 11, 40), (87, 11, 41), (700, 12, 40), (1037, 7, 3)])
+def test_host_steps_of_every_size(P, B, stride, L):
+    """Host arrays at the edges of each way their bytes travel (in the launch, as pairs, fetched ahead, in place), pageable and
+    page-locked, with refused slots among them."""
+    import torch
+    rng = np.random.default_rng(B * 100 + stride)
+    vocab, steps = 40, 4
+    msl = stride * steps
+    corpus = rng.integers(0, vocab, size=3000, dtype=np.int32)
+    st, S = P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)
+    toks = rng.integers(0, vocab, size=(steps, B, stride), dtype=np.int32)
+    counts = rng.integers(0, stride + 1, size=(steps, B)).astype(np.int32)
+    if B > 10:
+        counts[1, 3] = -1; counts[2, 9] = stride + 1; toks[1, 5, 0] = vocab; counts[1, 5] = 1
+    shapes = ((B, L), (B,), (B, 2), (B,), (B, 2), (B,))
+    for pinned in (False, True):
+        ob = oracle.Batch(S, corpus, B, vocab, msl)
+        batch = P.Batch(st, B, msl, max_draft_len=L, max_host_stride=stride)
+        out = [torch.empty(s, dtype=torch.int32) for s in shapes]
+        tt, ct = torch.from_numpy(toks), torch.from_numpy(counts)
+        if pinned:
+            out, tt, ct = [o.pin_memory() for o in out], tt.pin_memory(), ct.pin_memory()
+        for i in range(steps):
+            ref = ob.step(toks[i], counts[i], L, 8)
+            for o in out:
+                o.fill_(-77)
+            P.binding.sam_step_host(batch.handle, tt[i], stride, ct[i], L, *out)
+            for o, k in zip(out, ("draft_tokens", "draft_len", "match_len", "source", "state", "status")):
+                assert np.array_equal(o.numpy(), getattr(ref, k)), (pinned, i, k)
