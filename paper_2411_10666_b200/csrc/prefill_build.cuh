@@ -4,8 +4,8 @@
 // (64 slots x 1024 tokens: 550 us, and 5.8 ms for one slot of 8191).  What it ends with is a function of the text alone,
 // and all of it can be read off the sorted order of the text's prefixes:
 //   - prefixes are sorted by their tokens from the last to the first; A[j] is the end position of the j-th, h[j]
-//     the length of the suffix it shares with its predecessor.  Sorting is by prefix doubling: the first sort compares as many
-//     tokens as fit a 64-bit key, each further round four times as many, within groups of equal prefixes only;
+//     the length of the suffix it shares with its predecessor.  Sorting is by prefix doubling: positions are grouped by their
+//     token, and each round orders the groups of equal prefixes by four times as many tokens;
 //   - the strings that are suffixes of the same set of prefixes form an interval of the sorted order.  An interval is
 //     named by the first boundary inside it where h is smallest; its length is that h, its first end position the
 //     smallest A in it, its parent the interval at the larger h just outside;
@@ -79,7 +79,8 @@ __device__ __forceinline__ void pb_step(uint64_t& v, int lane, int stride, bool 
 }
 
 // Bitonic sort of key[0, N2).  Strides below 64 stay in the registers of one warp (two keys a lane).
-__device__ void pb_sort(uint64_t* key, int N2, int tid, int nt) {
+// (One copy, out of line: with builds in different phases on an SM, fetching instructions is what they wait for most.)
+__device__ __noinline__ void pb_sort(uint64_t* key, int N2, int tid, int nt) {
     const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
     for (int size = 64; size <= N2; size <<= 1) {
         int stride = size >> 1;
@@ -254,27 +255,92 @@ __device__ __forceinline__ uint32_t pb_take_slabs(const SamBatchView& W, int wan
 
 struct PbResult { int32_t s2, l2, e2; int err; };          // e2: first end position of the match state
 
+// The first round: positions grouped by their token, the groups in the order of a hash table (any order of the tokens will do).
+// A: the positions, group after group; rank 0 of `lev`: where a position's group begins.  Returns the number of groups.
+// (Counting in a table costs 3 us for 1024 tokens; sorting keys of three tokens cost 10.)
+__device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, int n, int tid, int nt) {
+    const int lane = tid & 31, w = tid >> 5, nw = nt >> 5, N2 = a.N2, size = 2 * N2;
+    uint32_t* key = reinterpret_cast<uint32_t*>(a.key);                              // [size]: tokens
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + 10 * (size_t)N2);             // [size]: positions, then where they begin
+    uint16_t* at = reinterpret_cast<uint16_t*>(smem + 18 * (size_t)N2);              // [N2]: a position's table entry
+    for (int i = tid; i < size; i += nt) { key[i] = SAM_NONE; cnt[i] = 0; }
+    if (tid == 0) sh.groups = 0;
+    pb_sync(nt);
+    for (int p = tid; p < n; p += nt) {
+        const uint32_t t = a.tok[p];
+        uint32_t h = sam_hash1(t) & (size - 1);
+        for (int probe = 0; probe < size; probe++) {       // (at most half full)
+            const uint32_t old = atomicCAS(&key[h], SAM_NONE, t);
+            if (old == SAM_NONE || old == t) break;
+            h = (h + 1) & (size - 1);
+        }
+        at[p] = (uint16_t)h;
+        a.B[p] = (uint16_t)atomicAdd(&cnt[h], 1u);
+    }
+    pb_sync(nt);
+    const int chunks = size >> 6;                          // of 64 entries, two a lane
+    for (int c = w; c < chunks; c += nw) {
+        const uint32_t x = cnt[64 * c + 2 * lane], y = cnt[64 * c + 2 * lane + 1];
+        const int sum = __reduce_add_sync(0xFFFFFFFFu, (int)(x + y)), used = __reduce_add_sync(0xFFFFFFFFu, (x != 0) + (y != 0));
+        if (lane == 0) { sh.chunk[c] = (int16_t)sum; if (used) atomicAdd(&sh.groups, used); }
+    }
+    pb_sync(nt);
+    if (w == 0) {
+        int run = 0;
+        for (int base = 0; base < chunks; base += 32) {
+            const int v = base + lane < chunks ? sh.chunk[base + lane] : 0;
+            int s = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
+            if (base + lane < chunks) sh.chunk[base + lane] = (int16_t)(run + s - v);
+            run += __shfl_sync(0xFFFFFFFFu, s, 31);
+        }
+    }
+    pb_sync(nt);
+    for (int c = w; c < chunks; c += nw) {
+        const int x = (int)cnt[64 * c + 2 * lane], y = (int)cnt[64 * c + 2 * lane + 1];
+        int s = x + y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
+        const int begin = sh.chunk[c] + s - x - y;
+        cnt[64 * c + 2 * lane] = (uint32_t)begin; cnt[64 * c + 2 * lane + 1] = (uint32_t)(begin + x);
+    }
+    pb_sync(nt);
+    for (int p = tid; p < n; p += nt) {
+        const uint32_t begin = cnt[at[p]];
+        a.A[begin + a.B[p]] = (uint16_t)p;
+        a.lev[p] = (uint16_t)begin;
+    }
+    pb_sync(nt);
+    return sh.groups;
+}
+
 // One round of the sort: order the members of each group of equal prefixes (of `span` tokens) by the tokens before those, by
-// counting how many of the group come first.  A -> B, rank -> next.  Returns the number of groups.
-__device__ int pb_refine(const PbArrays& a, PbShared& sh, const uint16_t* A, uint16_t* B, const uint16_t* rank, uint16_t* next, int span, int n,
-                         int tid, int nt) {
+// counting how many of the group come first.  A -> B, rank -> next; end: room for where each group ends.  Returns the number
+// of groups.
+__device__ int pb_refine(const PbArrays& a, PbShared& sh, const uint16_t* A, uint16_t* B, const uint16_t* rank, uint16_t* next, uint16_t* end,
+                         int span, int n, int tid, int nt) {
     for (int j = tid; j < n; j += nt) {
-        const int p = A[j];
+        const int p = A[j], g = rank[p];
         uint64_t k = 0;
 #pragma unroll
         for (int q = 1; q < 4; q++) { const int at = p - q * span; k = k << 16 | (at >= 0 ? (uint32_t)rank[at] + 1u : 0u); }
         a.key[j] = k;
+        if (j + 1 == n || rank[A[j + 1]] != g) end[g] = (uint16_t)(j + 1);
     }
     if (tid == 0) sh.groups = 0;
     pb_sync(nt);
     int mine = 0;
     for (int j = tid; j < n; j += nt) {
-        const int p = A[j], g = rank[p];
-        const uint64_t k = a.key[j];
+        const int p = A[j], g = rank[p], e = end[g];
         int less = 0, same = 0;
-        for (int i = g; i < n && rank[A[i]] == g; i++) {
-            const uint64_t x = a.key[i];
-            less += x < k; same += x == k && i < j;
+        if (e - g > 1) {
+            const uint64_t k = a.key[j];
+#pragma unroll 4
+            for (int i = g; i < e; i++) {
+                const uint64_t x = a.key[i];
+                less += x < k; same += x == k && i < j;
+            }
         }
         B[g + less + same] = (uint16_t)p;
         next[p] = (uint16_t)(g + less);
@@ -290,39 +356,27 @@ __device__ int pb_refine(const PbArrays& a, PbShared& sh, const uint16_t* A, uin
 // leave, and the dynamic words of the slot's control block.  Run by nt threads (tid 0 .. nt - 1, whole warps, barrier 1);
 // the result is valid in all of them.  The tokens have been checked and lie in the slot's text and in the `tok` array;
 // 1 < n <= PB_MAX.
-__device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int vocab, int n, unsigned char* smem,
+__device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsigned char* smem,
                          PbShared& sh, int tid, int nt, PbResult& out) {
     const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
     const int N2 = pb_size(n);
     const PbArrays a = pb_arrays(smem, N2);
     const int32_t* text = W.text + (size_t)b * W.text_stride;
-    const int ib = 32 - __clz(n - 1), rb = 32 - __clz(n), vb = 32 - __clz(vocab);      // bits of a position, a rank plus one, a token plus one
+    const int ib = 32 - __clz(n - 1), rb = 32 - __clz(n);  // bits of a position, and of a rank plus one
     const uint32_t im = (1u << ib) - 1u;
 
     // ---- sort
-    const int span0 = min(4, (64 - ib) / vb);              // (at least one token: 13 + 31 bits)
-    for (int j = tid; j < N2; j += nt) {
-        uint64_t k = ~0ull;
-        if (j < n) {
-            k = 0;
-            for (int q = 0; q < span0; q++) k = k << vb | (j - q >= 0 ? a.tok[j - q] + 1u : 0u);
-            k = k << ib | (uint32_t)j;
-        }
-        a.key[j] = k;
-    }
-    pb_sync(nt);
-    pb_sort(a.key, N2, tid, nt);
     uint16_t *A = a.A, *B = a.B;
-    int top = 0, span = span0;                             // rank level, and the tokens its ranks compare
+    int top = 0, span = 1;                                 // rank level, and the tokens its ranks compare
     int spans[PB_LEVELS];
 #pragma unroll
-    for (int i = 0; i < PB_LEVELS; i++) spans[i] = span0;
-    for (int j = tid; j < n; j += nt) A[j] = (uint16_t)((uint32_t)a.key[j] & im);
-    int groups = pb_rank(a, sh, a.lev, n, ib, tid, nt);
+    for (int i = 0; i < PB_LEVELS; i++) spans[i] = 1;
+    int groups = pb_group(a, sh, smem, n, tid, nt);
     while (groups < n && span < n) {                       // (ranks of n tokens are all different)
         const uint16_t* r = a.lev + (size_t)top * N2;
-        bool large = false;                                // groups of over 64: counting would take too long
-        for (int j = tid; j + 64 < n; j += nt) large |= r[A[j]] == r[A[j + 64]];
+        bool large = false;                                // groups so large that counting would take longer than sorting all
+        const int most = min(max(64, N2 >> 3), 384);       // (1 x 8191 with groups of 650: 266 us counted, 222 sorted)
+        for (int j = tid; j + most < n; j += nt) large |= r[A[j]] == r[A[j + most]];
         const int to = top < PB_LEVELS - 1 ? top + 1 : top;                          // the last array is used again for longer spans
         if (pb_sync_or(nt, large) || to == top) {
             const int parts = min(4, (64 - ib) / rb);
@@ -338,7 +392,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int vocab, 
             groups = pb_rank(a, sh, a.lev + (size_t)to * N2, n, ib, tid, nt);
             span *= parts;
         } else {
-            groups = pb_refine(a, sh, A, B, r, a.lev + (size_t)to * N2, span, n, tid, nt);
+            groups = pb_refine(a, sh, A, B, r, a.lev + (size_t)to * N2, a.lev + (to == 1 ? 2 * (size_t)N2 : 0), span, n, tid, nt);
             uint16_t* t = A; A = B; B = t;
             span *= 4;
         }
@@ -353,7 +407,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int vocab, 
         if (j > 0 && j < n) {
             const int q = A[j - 1];
 #pragma unroll
-            for (int i = PB_LEVELS - 1; i >= 0; i--) {
+            for (int i = PB_LEVELS - 1; i >= 1; i--) {     // (level 0 is not kept: its place is used by later rounds)
                 if (i <= top) {
                     const uint16_t* r = a.lev + (size_t)i * N2;
                     while (p - x >= 0 && q - x >= 0 && r[p - x] == r[q - x]) x += spans[i];

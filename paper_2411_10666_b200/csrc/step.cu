@@ -1338,7 +1338,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
 
     if (!STATIC) {
         PbResult r;
-        pb_build(A.W, b, cb, vocab, m, pb_smem, sh, (int)threadIdx.x, (int)blockDim.x, r);
+        pb_build(A.W, b, cb, m, pb_smem, sh, (int)threadIdx.x, (int)blockDim.x, r);
         if (threadIdx.x == 0) {
             if (r.err) cb[CB_STATUS] = (uint32_t)r.err;
             cb[CB_ERR_S] = SAM_STEP_BUILT;
@@ -1357,7 +1357,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
         }
     } else {
         PbResult r;
-        pb_build(A.W, b, cb, vocab, m, pb_smem, sh, (int)threadIdx.x - 32, (int)blockDim.x - 32, r);
+        pb_build(A.W, b, cb, m, pb_smem, sh, (int)threadIdx.x - 32, (int)blockDim.x - 32, r);
         if (warp > 1) return;
         err = r.err; my_l = r.l2; my_s = r.s2;
         if (r.l2 > 0) {
