@@ -23,6 +23,9 @@
 //   freq, topk: optional, for tree drafts — the occurrence count of every state, and for states
 //               with hashed transitions their k most frequent successors (a state with at most two
 //               transitions has them all in its record).
+//   path      : with them, per state: over how many transitions the state's only successor occurs as often as it
+//               does, and so on, and the state where that ends.  A tree's best-first expansion goes along such a
+//               stretch without a choice.  Derived on the device after each upload.
 //
 // DYNAMIC automata (one per sequence slot, written by the slot's own warp only)
 //   rec       : 32 bytes per state, in slabs from the shared pool, addressed through the slot's
@@ -121,6 +124,7 @@ struct SamStaticView {
     const uint4* topk;        // SamTopkEnt table, four 16-byte words per entry
     uint32_t topk_mask;       // entries - 1
     int32_t tree_k;           // successors kept per hashed state (0: no tree data)
+    const uint2* path;        // tree drafts: {steps, end | F} per state, see above
     const uint32_t* pstate;   // [n_tokens]: id | F of the state of the prefix ending with corpus token i
 };
 

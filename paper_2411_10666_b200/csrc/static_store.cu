@@ -43,6 +43,8 @@ void layout_sections(sam_static* st) {
     // derived on the device after every upload, never stored in a file: position -> prefix state
     st->len_pstate = sam_align_up(((size_t)st->info.n_tokens + CORPUS_PAD_TOKENS) * 4, 8);
     st->off_pstate = off; off = sam_align_up(off + st->len_pstate, 256);
+    st->len_path = st->info.tree_topk ? (size_t)st->info.n_states * 8 : 0;
+    st->off_path = off;   off = sam_align_up(off + st->len_path, 256);
     st->dev_bytes = off;
 }
 
@@ -62,6 +64,7 @@ void make_view(sam_static* st) {
     st->view.topk_mask = st->len_topk ? (uint32_t)(st->len_topk / sizeof(SamTopkEnt) - 1) : 0;
     st->view.tree_k = st->info.tree_topk;
     st->view.pstate = (const uint32_t*)(base + st->off_pstate);
+    st->view.path = (const uint2*)(base + st->off_path);
 }
 
 // pstate[i] = id | F of the state Build-SAM created for corpus token i, the state of the whole prefix
@@ -75,12 +78,38 @@ __global__ void derive_pstate_kernel(const uint4* rec, int64_t n_states, uint32_
     }
 }
 
-int derive_pstate(sam_static* st) {
+// path[s] = {steps, state it ends in (with its F bit)}: how far a state's only successor occurs as often as the state itself,
+// and that one's, and so on (0 steps for a state that occurs once: its path is the rest of the corpus).  One step for each
+// state first, then the steps of the state arrived at are added, over and over: what a pair says stays true while others
+// change (it is read and written as one word), and each pass at least doubles it.
+__global__ void derive_path_kernel(const uint4* rec, const uint32_t* freq, int64_t n_states, unsigned long long* path, int pass) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_states; s += stride) {
+        if (pass == 0) {
+            const uint4 a = rec[2 * s], b = rec[2 * s + 1];
+            const uint32_t f = freq[s];
+            const bool on = s > 0 && a.w == 1 && f > 1 && freq[b.y & SAM_IDMASK] == f;
+            path[s] = on ? (unsigned long long)b.y << 32 | 1u : (unsigned long long)(uint32_t)s << 32;
+        } else {
+            const unsigned long long p = *(volatile unsigned long long*)(path + s);
+            const uint32_t steps = (uint32_t)p;
+            if (steps == 0 || steps >= 1024) continue;
+            const unsigned long long q = *(volatile unsigned long long*)(path + ((uint32_t)(p >> 32) & SAM_IDMASK));
+            if ((uint32_t)q != 0) *(volatile unsigned long long*)(path + s) = (q >> 32) << 32 | (steps + (uint32_t)q);
+        }
+    }
+}
+constexpr int PATH_PASSES = 7;             // 2^7 steps: the largest tree has 128 nodes
+
+// The sections that are not part of the saved file.
+int derive_sections(sam_static* st) {
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, st->device);
     if (e != cudaSuccess || sms < 1) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
-    derive_pstate_kernel<<<sms * 8, 256>>>(st->view.rec, st->info.n_states,
-                                           (uint32_t*)((char*)st->dev_base + st->off_pstate), st->info.n_tokens);
+    char* base = (char*)st->dev_base;
+    derive_pstate_kernel<<<sms * 8, 256>>>(st->view.rec, st->info.n_states, (uint32_t*)(base + st->off_pstate), st->info.n_tokens);
+    for (int pass = 0; st->len_path && pass <= PATH_PASSES; pass++)
+        derive_path_kernel<<<sms * 8, 256>>>(st->view.rec, st->view.freq, st->info.n_states, (unsigned long long*)(base + st->off_path), pass);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
@@ -193,7 +222,7 @@ extern "C" int sam_build_static(const int32_t* corpus_host, int64_t n_tokens, in
     if (e == cudaSuccess && !img.topk.empty()) e = cudaMemcpy(base + st->off_topk, img.topk.data(), st->len_topk, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { sam_set_cuda_error(e); cudaFree(st->dev_base); delete st; return SAM_ERR_CUDA; }
     make_view(st);
-    if (derive_pstate(st) != SAM_OK) { cudaFree(st->dev_base); delete st; return SAM_ERR_CUDA; }
+    if (derive_sections(st) != SAM_OK) { cudaFree(st->dev_base); delete st; return SAM_ERR_CUDA; }
     *out = st;
     return SAM_OK;
 }
@@ -310,7 +339,7 @@ extern "C" int sam_static_load(const char* path, int device, sam_static_t** out)
     if (rc == SAM_OK && sum != h.checksum) rc = SAM_ERR_FORMAT;
     if (rc != SAM_OK) { cudaFree(st->dev_base); delete st; return rc; }
     make_view(st);
-    if (derive_pstate(st) != SAM_OK) { cudaFree(st->dev_base); delete st; return SAM_ERR_CUDA; }
+    if (derive_sections(st) != SAM_OK) { cudaFree(st->dev_base); delete st; return SAM_ERR_CUDA; }
     *out = st;
     return SAM_OK;
 }

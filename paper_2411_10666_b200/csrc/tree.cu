@@ -9,12 +9,13 @@
 // reads: lanes 0..n-1 each fetch one child's freq, record and, if flagged, top-k entry together.
 //   - Most nodes are states with one successor that occurs as often as they do: inside a passage the corpus holds once or
 //     several times.  Such a stretch is one entry, a path, pushed again with each pop, its tokens those of the corpus.
-//     Where the state occurs once the path goes on to the end of the corpus; otherwise its states are guessed (ids as far apart
-//     as the first two, as states made token after token along a passage are), read in one round, a few lanes
-//     for each child, and checked; the last of them is an ordinary entry again.
+//     Where the state occurs once the path goes on to the end of the corpus, otherwise over as many states as the
+//     automaton's `path` says; the state it ends in is then an ordinary entry whose candidates are read when it is popped.
 //   - The entries with the largest probability are popped together as long as they are paths: each goes back to the end
 //     of the line with the same probability, so they take turns, and lane t writes the t-th node of up to 32 with one read
 //     of the corpus.
+// 64 slots of 40 nodes, k = 4: 18 to 31 us from seed to seed (32 to 34 with one pop and one round of reads for each node), 4096
+// slots of 100 nodes 90 us (315).  Bound by the pops that are left, one after the other, 1 us each.
 // Probabilities are IEEE float32: quotient freq(child) / freq(state) rounded first,
 // then the product with the parent's probability.
 #include "common.h"
@@ -59,9 +60,10 @@ __device__ __forceinline__ int load_topk(const SamStaticView& S, uint32_t u, int
 }
 
 constexpr int CAND_WORDS = 2 * SAM_TOPK_MAX;                // an entry's candidates: tokens, then targets
-constexpr uint32_t ENTRY_ORDERED = 256u, ENTRY_PATH = 512u, ENTRY_ENDS = 1024u;     // flags beside the number of candidates
+constexpr uint32_t ENTRY_ORDERED = 256u, ENTRY_PATH = 512u, ENTRY_ENDS = 1024u, ENTRY_LATE = 2048u;   // flags beside the number of candidates
 constexpr int PATH_LEFT = 16;                               // q_n >> PATH_LEFT: nodes left on the path; then, unless it ENDS, the entry
-constexpr int LAST_TOKEN = 2;                               // is that of its last state, whose token this word of q_cand holds
+                                                            // is that of its last state (q_cand[0]), LATE: its token is in the corpus at
+                                                            // q_tok, its candidates have not been read
 constexpr int PATH_ENDLESS = 1024;                          // (more than any tree has nodes)
 
 __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ TreeArgs A) {
@@ -160,7 +162,7 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
                     q_n[e] = nn;
                     if ((nn >> PATH_LEFT) == 0) {
                         if (nn & ENTRY_ENDS) q_key[e] = 0;
-                        else { q_n[e] = nn & 255u; q_tok[e] = q_cand[(size_t)e * CAND_WORDS + LAST_TOKEN]; }
+                        else q_n[e] = ENTRY_LATE;
                     }
                 }
                 n_out += count; seq += (uint32_t)count;
@@ -168,81 +170,64 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
                 continue;
             }
             const int node = n_out++;
+            const uint32_t nn = q_n[at], fs = q_freq[at], tok = q_tok[at];
             if (lane == 0) {
-                out_tok[node] = (int32_t)q_tok[at]; out_par[node] = q_par[at];
+                out_tok[node] = nn & ENTRY_LATE ? __ldg(A.S.corpus + tok) : (int32_t)tok;
+                out_par[node] = q_par[at];
                 if (out_p) out_p[node] = p;
                 q_key[at] = 0;
             }
             if (n_out >= M) break;                          // the last node needs no expansion
             // expand: lane j takes candidate j
-            const uint32_t nn = q_n[at], fs = q_freq[at];
-            const int n = (int)(nn & 255u);
-            if (n == 0) { __syncwarp(); continue; }
+            int n = (int)(nn & 255u);
+            bool ordered = (nn & ENTRY_ORDERED) != 0;
             uint32_t ctok = 0, ctgt = 0, cf = 0;
-            int cn = 0; bool cord = false;
-            uint4 ra = make_uint4(0, 0, 0, 0), rb = ra;
             uint32_t gtok[SAM_TOPK_MAX], gtgt[SAM_TOPK_MAX];
-            if (lane < n) {
+            if (nn & ENTRY_LATE) {                          // every lane reads the candidates and picks its own
+                const uint32_t end = q_cand[(size_t)at * CAND_WORDS], u = end & SAM_IDMASK;
+                if (end >> 31) n = load_topk(A.S, u, K, gtok, gtgt, ordered);
+                else n = inline_candidates(__ldg(A.S.rec + 2 * (size_t)u), __ldg(A.S.rec + 2 * (size_t)u + 1), gtok, gtgt);
+#pragma unroll
+                for (int j = 0; j < SAM_TOPK_MAX; j++) if (lane == j && j < n) { ctok = gtok[j]; ctgt = gtgt[j]; }
+            } else if (lane < n) {
                 ctok = q_cand[(size_t)at * CAND_WORDS + lane]; ctgt = q_cand[(size_t)at * CAND_WORDS + SAM_TOPK_MAX + lane];
+            }
+            if (n == 0) { __syncwarp(); continue; }
+            int cn = 0; bool cord = false;
+            uint32_t end1 = 0;                              // first end position
+            uint2 path = make_uint2(0, 0);
+            if (lane < n) {
                 const uint32_t u = ctgt & SAM_IDMASK;
                 cf = __ldg(A.S.freq + u);
                 if (ctgt >> 31) cn = load_topk(A.S, u, K, gtok, gtgt, cord);
                 else {
-                    ra = __ldg(A.S.rec + 2 * (size_t)u); rb = __ldg(A.S.rec + 2 * (size_t)u + 1);
+                    const uint4 ra = __ldg(A.S.rec + 2 * (size_t)u), rb = __ldg(A.S.rec + 2 * (size_t)u + 1);
+                    path = __ldg(A.S.path + u);
+                    end1 = ra.z;
                     cn = inline_candidates(ra, rb, gtok, gtgt);
                 }
             }
             // order two inline candidates by (freq descending, token ascending); keep the first K
             int pos = lane;
-            if (!(nn & ENTRY_ORDERED) && n == 2) {
+            if (!ordered && n == 2) {
                 const uint32_t of = __shfl_xor_sync(FULL, cf, 1), ot = __shfl_xor_sync(FULL, ctok, 1);
                 if (lane < 2) pos = of > cf || (of == cf && ot < ctok) ? 1 : 0;
             }
             const int keep = n < K ? n : K;
-            // paths: lane k of child c's lanes takes the k-th state after the child
-            const int width = n == 1 ? 32 : n == 2 ? 16 : n <= 4 ? 8 : 4, c = lane / width, k = lane % width;
-            const uint32_t u = ctgt & SAM_IDMASK, far = (rb.y & SAM_IDMASK) - u;
-            const uint32_t step = lane < n && !(ctgt >> 31) && ra.w == 1u && cf > 1 ? far : 0u;
-            const uint32_t step_c = __shfl_sync(FULL, step, c), u_c = __shfl_sync(FULL, u, c), cf_c = __shfl_sync(FULL, cf, c);
-            const int pos_c = __shfl_sync(FULL, pos, c);
-            const uint4 ra_c = make_uint4(0, 0, __shfl_sync(FULL, ra.z, c), __shfl_sync(FULL, ra.w, c));
-            const uint2 rb_c = make_uint2(__shfl_sync(FULL, rb.x, c), __shfl_sync(FULL, rb.y, c));
-            int run = 1;                                    // states of child c's path
-            if (__any_sync(FULL, step != 0)) {
-                const uint32_t id = u_c + step_c * (uint32_t)k;
-                uint32_t deg = ra_c.w, f = cf_c, t0 = rb_c.x, g0 = rb_c.y;
-                uint4 r1 = make_uint4(0, 0, 0, 0);
-                if (k > 0) {
-                    deg = 3; f = 0;
-                    if (step_c != 0 && (int64_t)id < A.S.n_states) {
-                        deg = __ldg(&A.S.rec[2 * (size_t)id].w); r1 = __ldg(A.S.rec + 2 * (size_t)id + 1); f = __ldg(A.S.freq + id);
-                        t0 = r1.x; g0 = r1.y;
-                    }
-                }
-                const uint32_t deg_n = __shfl_down_sync(FULL, deg, 1), f_n = __shfl_down_sync(FULL, f, 1), t_p = __shfl_up_sync(FULL, t0, 1);
-                const bool on = step_c != 0 && k + 1 < width && deg == 1 && g0 == id + step_c && f_n == cf_c && deg_n <= 2;
-                const unsigned m = __ballot_sync(FULL, on) >> (c * width);
-                run = (~m ? __ffs(~m) - 1 : 32) + 1;
-                if (run > 1 && k == run - 1 && c < n && pos_c < keep) {              // the last state's lane
-                    const int e = qn + pos_c;
-                    uint32_t* to = q_cand + (size_t)e * CAND_WORDS;
-                    to[0] = r1.x; to[1] = r1.z; to[SAM_TOPK_MAX] = r1.y; to[SAM_TOPK_MAX + 1] = r1.w; to[LAST_TOKEN] = t_p;
-                    q_n[e] = deg | ENTRY_PATH | (uint32_t)(run - 1) << PATH_LEFT;
-                    q_tok[e] = ra_c.z - 1u;                 // (its first end position: the token itself is the one before)
-                }
-            }
-            run = __shfl_sync(FULL, run, (lane * width) & 31);                        // of child `lane`
             if (lane < n && pos < keep) {
                 const int e = qn + pos;
+                uint32_t* to = q_cand + (size_t)e * CAND_WORDS;
                 q_key[e] = __float_as_uint(__fmul_rn(p, __fdiv_rn(__uint2float_rn(cf), __uint2float_rn(fs)))) + 1u;
                 q_seq[e] = seq + (uint32_t)pos; q_par[e] = node; q_freq[e] = cf;
                 if (cf == 1) {
-                    const int64_t room = A.S.n_tokens - (int64_t)ra.z + 1;
-                    q_tok[e] = ra.z - 1u;
+                    const int64_t room = A.S.n_tokens - (int64_t)end1 + 1;
+                    q_tok[e] = end1 - 1u;                   // (the token itself is the one before its end position)
                     q_n[e] = ENTRY_PATH | ENTRY_ENDS | (uint32_t)(room < PATH_ENDLESS ? room : PATH_ENDLESS) << PATH_LEFT;
-                } else if (run == 1) {
+                } else if (path.x > 0) {
+                    q_tok[e] = end1 - 1u; to[0] = path.y;
+                    q_n[e] = ENTRY_PATH | path.x << PATH_LEFT;
+                } else {
                     q_tok[e] = ctok; q_n[e] = (uint32_t)cn | (cord ? ENTRY_ORDERED : 0u);
-                    uint32_t* to = q_cand + (size_t)e * CAND_WORDS;
                     for (int j = 0; j < SAM_TOPK_MAX; j++) { to[j] = gtok[j]; to[SAM_TOPK_MAX + j] = gtgt[j]; }
                 }
             }
