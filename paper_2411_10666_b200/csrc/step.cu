@@ -1267,9 +1267,13 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
     }
 }
 
-template <bool VERIFY, bool AHEAD>
-__global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_constant__ StepArgs A) {
-    step_body<VERIFY, AHEAD, false>(A, A.new_tokens, A.counts);
+// AHEAD: blocks of three warps an SM has to hold, 0 for blocks of two.  Registers come in quarters of an SM: 5 blocks (740
+// slots) have 120 a thread and spill nothing, 6 (888) have 96, 8 (1184) have 80 and spill 330 bytes.  Prompt-copying
+// slots, us a step with 5 / 6 / 8 blocks: 740 slots 14.6 / 15.0 / -, 880 slots - / 15.5 / 16.4, 1000 slots (in two
+// waves: 20.5 / 18.5) 17.0, 1180 slots with two warps a slot 19.2, with three 17.4.
+template <bool VERIFY, int AHEAD>
+__global__ void __launch_bounds__(AHEAD ? 96 : 64, AHEAD ? AHEAD : 10) sam_step_kernel(const __grid_constant__ StepArgs A) {
+    step_body<VERIFY, AHEAD != 0, false>(A, A.new_tokens, A.counts);
 }
 
 // A host-array step whose rows and counts fit the launch's arguments: reading them from host memory, in the kernel's first
@@ -1277,7 +1281,7 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64) sam_step_kernel(const __grid_
 // (With 32 KB of arguments, for 250 slots, it costs 3 us more than it saves.)
 constexpr int SAM_INLINE_WORDS = 896;                    // within 4 KB of arguments
 struct StepArgsInline { StepArgs A; int32_t in[SAM_INLINE_WORDS]; };                // rows, then counts
-__global__ void __launch_bounds__(96) sam_step_inline_kernel(const __grid_constant__ StepArgsInline I) {
+__global__ void __launch_bounds__(96, 5) sam_step_inline_kernel(const __grid_constant__ StepArgsInline I) {
     step_body<false, true, true>(I.A, I.in, I.in + (size_t)I.A.W.batch * I.A.stride);
 }
 
@@ -2218,7 +2222,8 @@ constexpr int split_big_m(int batch) { return batch >= 8192 ? 8 : 5; }
 int split_kernel_setup(int device);
 
 constexpr int SAM_SPLIT_MIN_BATCH = 8192;                    // the split step is used from this many slots on
-constexpr int SAM_AHEAD_MAX_BATCH = 1036;                    // three warps a slot, all slots resident at once (148 x 7)
+constexpr int SAM_SMS = 148;
+constexpr int SAM_AHEAD_MAX_BATCH = SAM_SMS * 8;             // three warps a slot, all slots resident at once
 constexpr int SAM_ORDER_MIN_BATCH = 1536;                    // more slots than a B200 holds blocks of this kernel (148 x 10)
 
 }  // namespace
@@ -2342,9 +2347,13 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
             memcpy(I.in, io.inline_rows, rows * 4);
             memcpy(I.in + rows, io.inline_counts, (size_t)b->view.batch * 4);
             e = cudaLaunchKernelEx(&cfg, sam_step_inline_kernel, I);
-        } else
-            e = verify ? (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<true, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<true, false>, A))
-                       : (ahead ? cudaLaunchKernelEx(&cfg, sam_step_kernel<false, true>, A) : cudaLaunchKernelEx(&cfg, sam_step_kernel<false, false>, A));
+        } else {
+            using Kernel = void (*)(const StepArgs);
+            const Kernel kernels[2][4] = {{sam_step_kernel<false, 0>, sam_step_kernel<false, 5>, sam_step_kernel<false, 6>, sam_step_kernel<false, 8>},
+                                          {sam_step_kernel<true, 0>, sam_step_kernel<true, 5>, sam_step_kernel<true, 6>, sam_step_kernel<true, 8>}};
+            const int B = b->view.batch, k = !ahead ? 0 : B <= SAM_SMS * 5 ? 1 : B <= SAM_SMS * 6 ? 2 : 3;
+            e = cudaLaunchKernelEx(&cfg, kernels[verify][k], A);
+        }
     }
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;

@@ -177,3 +177,30 @@ def test_host_steps_of_every_size(P, B, stride, L):
             P.binding.sam_step_host(batch.handle, tt[i], stride, ct[i], L, *out)
             for o, k in zip(out, ("draft_tokens", "draft_len", "match_len", "source", "state", "status")):
                 assert np.array_equal(o.numpy(), getattr(ref, k)), (pinned, i, k)
+
+
+@pytest.mark.parametrize("B", [740, 741, 889, 1184, 1185])
+def test_steps_at_the_edges_of_the_register_budgets(P, B):
+    """One step kernel for each number of blocks an SM holds: plain and verified steps at the first and last batch of each."""
+    import torch
+    rng = np.random.default_rng(B)
+    vocab, K, L, steps, msl = 25, 7, 6, 3, 60
+    corpus = rng.integers(0, vocab, size=4000, dtype=np.int32)
+    st, S = P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)
+    toks = rng.integers(0, vocab, size=(steps, B, K), dtype=np.int32)
+    counts = rng.integers(0, K + 1, size=(steps, B)).astype(np.int32)
+    ob, batch = oracle.Batch(S, corpus, B, vocab, msl), P.Batch(st, B, msl, max_draft_len=L)
+    keys = ("draft_tokens", "draft_len", "match_len", "source", "state", "status")
+    out = [P.StepOutputs(B, L, batch.device) for _ in range(2)]
+    for i in range(steps):
+        ref = ob.step(toks[i], counts[i], L, 8)
+        batch.step(torch.from_numpy(toks[i]).cuda(), torch.from_numpy(counts[i]).cuda(), L, out[0])
+        for k, v in out[0].cpu().items():
+            assert np.array_equal(v, getattr(ref, k)), k
+    dr, dl = out[0].draft_tokens.cpu().numpy(), out[0].draft_len.cpu().numpy()
+    target = np.where(rng.random((B, L + 1)) < 0.8, np.concatenate([dr, dr[:, :1]], 1), 1).clip(0, vocab - 1).astype(np.int32)
+    m = np.array([next((j for j in range(n) if dr[b, j] != target[b, j]), n) + 1 for b, n in enumerate(dl)], dtype=np.int32)
+    P.binding.sam_step_verified(batch.handle, torch.from_numpy(target).cuda(), out[0].draft_tokens, out[0].draft_len, None, L, *out[1].tensors())
+    ref = ob.step(target, m, L, 8)
+    for k in keys:
+        assert np.array_equal(getattr(out[1], k).cpu().numpy(), getattr(ref, k)), k
