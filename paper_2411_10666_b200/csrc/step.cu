@@ -188,15 +188,17 @@ __device__ __forceinline__ uint2* blk_ptr(const Dyn& D, uint32_t off) {
     return reinterpret_cast<uint2*>(D.pool + (size_t)off * 128);
 }
 
-__device__ __forceinline__ int alloc_slab(Dyn& D) {
+// (Out of line: it is needed in nine places and seldom runs.)
+__device__ __noinline__ int take_slab(int32_t* pool_hdr, int32_t* free_stack, int32_t* slab_owner, int seq) {
     int idx = -1;
-    if (D.lane == 0) {
-        int old = atomicSub(D.pool_hdr, 1);
-        if (old <= 0) atomicAdd(D.pool_hdr, 1);
-        else { idx = D.free_stack[old - 1]; D.slab_owner[idx] = D.seq; }
+    if ((threadIdx.x & 31) == 0) {
+        int old = atomicSub(pool_hdr, 1);
+        if (old <= 0) atomicAdd(pool_hdr, 1);
+        else { idx = free_stack[old - 1]; slab_owner[idx] = seq; }
     }
     return __shfl_sync(FULL, idx, 0);
 }
+__device__ __forceinline__ int alloc_slab(Dyn& D) { return take_slab(D.pool_hdr, D.free_stack, D.slab_owner, D.seq); }
 
 // make sure state id s has a record to live in
 __device__ __forceinline__ void ensure_rec(Dyn& D, uint32_t s) {
