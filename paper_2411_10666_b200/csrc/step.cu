@@ -330,6 +330,23 @@ __device__ __forceinline__ void root_precompute(Dyn& D, uint32_t tk, bool valid)
     if (D.pr_state == 0 && first_empty >= 0) { D.pr_state = 2; D.pr_slot = home * SAM_ROOT_BUCKET + first_empty; }
 }
 
+// A lookup that was not settled ahead of time, 32 entries a round: {found (2: table full), target, slot, rounds}
+__device__ __noinline__ uint4 root_probe(const uint2* root, uint32_t bmask, uint32_t t) {
+    const uint32_t cap_mask = (bmask + 1) * SAM_ROOT_BUCKET - 1, base = (sam_hash1(t) & bmask) * SAM_ROOT_BUCKET;
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t off = 0; off <= cap_mask; off += 32) {
+        const uint2 e = root[(base + off + lane) & cap_mask];
+        const unsigned hit = __ballot_sync(FULL, e.x == t);
+        if (hit) {
+            const int src = __ffs(hit) - 1;
+            return make_uint4(1, __shfl_sync(FULL, e.y, src), (base + off + src) & cap_mask, off / 32 + 1);
+        }
+        const unsigned empty = __ballot_sync(FULL, e.x == SAM_NONE);
+        if (empty) return make_uint4(0, 0, (base + off + (__ffs(empty) - 1)) & cap_mask, off / 32 + 1);
+    }
+    return make_uint4(2, 0, 0, 0);
+}
+
 __device__ __forceinline__ RootLook root_lookup(Dyn& D, uint32_t t) {
     RootLook r; r.found = false; r.tgt = 0; r.slot = 0;
     const uint32_t st = __shfl_sync(FULL, D.pr_state, D.cur);
@@ -339,21 +356,10 @@ __device__ __forceinline__ RootLook root_lookup(Dyn& D, uint32_t t) {
         r.slot = __shfl_sync(FULL, D.pr_slot, D.cur);
         return r;
     }
-    const uint32_t cap_mask = (D.root_bmask + 1) * SAM_ROOT_BUCKET - 1;
-    const uint32_t base = (sam_hash1(t) & D.root_bmask) * SAM_ROOT_BUCKET;
-    for (uint32_t off = 0; off <= cap_mask; off += 32) {
-        SAM_COUNT(D.kc.rounds, 1);
-        uint2 e = D.root[(base + off + D.lane) & cap_mask];
-        unsigned hit = __ballot_sync(FULL, e.x == t);
-        if (hit) {
-            int src = __ffs(hit) - 1;
-            r.found = true; r.tgt = __shfl_sync(FULL, e.y, src); r.slot = (base + off + src) & cap_mask;
-            return r;
-        }
-        unsigned empty = __ballot_sync(FULL, e.x == SAM_NONE);
-        if (empty) { r.slot = (base + off + (__ffs(empty) - 1)) & cap_mask; return r; }
-    }
-    D.err = SAM_SEQ_WALK_LIMIT;           // table full: cannot happen with root_cap >= 2 * distinct tokens
+    const uint4 x = root_probe(D.root, D.root_bmask, t);
+    SAM_COUNT(D.kc.rounds, x.w);
+    r.found = x.x == 1; r.tgt = x.y; r.slot = x.z;
+    if (x.x == 2) D.err = SAM_SEQ_WALK_LIMIT;             // table full: cannot happen with root_cap >= 2 * distinct tokens
     return r;
 }
 
