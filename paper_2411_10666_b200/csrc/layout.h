@@ -92,6 +92,15 @@ struct SamHashEnt { uint32_t state, tok, tgt, pad; };   // 16 bytes
 // Kept in an open-addressing table keyed by state (linear probing, state == SAM_NONE is empty).
 struct SamTopkEnt { uint32_t state, n, pad0, pad1; uint32_t tok[SAM_TOPK_MAX]; uint32_t tgt[SAM_TOPK_MAX]; };
 
+// path entries: {steps in the low half, end | F in the high half}.  From SAM_PATH_MAX steps on (a tree has at most 128 nodes)
+// a path counts as endless: its steps stay at that number and its end says nothing.
+#define SAM_PATH_MAX 1024u
+// The path p, shorter than that, prolonged by the path q of the state it ends in.
+SAM_HD uint64_t sam_path_join(uint64_t p, uint64_t q) {
+    const uint32_t steps = (uint32_t)p + ((uint32_t)q < SAM_PATH_MAX ? (uint32_t)q : SAM_PATH_MAX);
+    return (q >> 32) << 32 | (steps < SAM_PATH_MAX ? steps : SAM_PATH_MAX);
+}
+
 // 64-bit multiplicative mix of (state, token); upper half is the hash.
 SAM_HD uint32_t sam_hash2(uint32_t state, uint32_t tok) {
     uint64_t k = ((uint64_t)state << 32) | tok;

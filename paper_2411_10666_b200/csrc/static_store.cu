@@ -81,7 +81,8 @@ __global__ void derive_pstate_kernel(const uint4* rec, int64_t n_states, uint32_
 // path[s] = {steps, state it ends in (with its F bit)}: how far a state's only successor occurs as often as the state itself,
 // and that one's, and so on (0 steps for a state that occurs once: its path is the rest of the corpus).  One step for each
 // state first, then the steps of the state arrived at are added, over and over: what a pair says stays true while others
-// change (it is read and written as one word), and each pass at least doubles it.
+// change (it is read and written as one word), and each pass at least doubles it.  The successor's steps may have grown in
+// the same pass, by any number of states on the way: the sum is bounded where it is made (sam_path_join).
 __global__ void derive_path_kernel(const uint4* rec, const uint32_t* freq, int64_t n_states, unsigned long long* path, int pass) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_states; s += stride) {
@@ -93,9 +94,9 @@ __global__ void derive_path_kernel(const uint4* rec, const uint32_t* freq, int64
         } else {
             const unsigned long long p = *(volatile unsigned long long*)(path + s);
             const uint32_t steps = (uint32_t)p;
-            if (steps == 0 || steps >= 1024) continue;
+            if (steps == 0 || steps >= SAM_PATH_MAX) continue;
             const unsigned long long q = *(volatile unsigned long long*)(path + ((uint32_t)(p >> 32) & SAM_IDMASK));
-            if ((uint32_t)q != 0) *(volatile unsigned long long*)(path + s) = (q >> 32) << 32 | (steps + (uint32_t)q);
+            if ((uint32_t)q != 0) *(volatile unsigned long long*)(path + s) = sam_path_join(p, q);
         }
     }
 }

@@ -64,7 +64,8 @@ constexpr uint32_t ENTRY_ORDERED = 256u, ENTRY_PATH = 512u, ENTRY_ENDS = 1024u, 
 constexpr int PATH_LEFT = 16;                               // q_n >> PATH_LEFT: nodes left on the path; then, unless it ENDS, the entry
                                                             // is that of its last state (q_cand[0]), LATE: its token is in the corpus at
                                                             // q_tok, its candidates have not been read
-constexpr int PATH_ENDLESS = 1024;                          // (more than any tree has nodes)
+constexpr uint32_t PATH_ENDLESS = SAM_PATH_MAX;             // (more than any tree has nodes)
+static_assert(PATH_ENDLESS > 128 && PATH_ENDLESS < 1u << (32 - PATH_LEFT), "nodes left fit beside the flags");
 
 __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ TreeArgs A) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -222,10 +223,10 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
                 if (cf == 1) {
                     const int64_t room = A.S.n_tokens - (int64_t)end1 + 1;
                     q_tok[e] = end1 - 1u;                   // (the token itself is the one before its end position)
-                    q_n[e] = ENTRY_PATH | ENTRY_ENDS | (uint32_t)(room < PATH_ENDLESS ? room : PATH_ENDLESS) << PATH_LEFT;
+                    q_n[e] = ENTRY_PATH | ENTRY_ENDS | (room < (int64_t)PATH_ENDLESS ? (uint32_t)room : PATH_ENDLESS) << PATH_LEFT;
                 } else if (path.x > 0) {
                     q_tok[e] = end1 - 1u; to[0] = path.y;
-                    q_n[e] = ENTRY_PATH | path.x << PATH_LEFT;
+                    q_n[e] = ENTRY_PATH | min(path.x, PATH_ENDLESS) << PATH_LEFT;
                 } else {
                     q_tok[e] = ctok; q_n[e] = (uint32_t)cn | (cord ? ENTRY_ORDERED : 0u);
                     for (int j = 0; j < SAM_TOPK_MAX; j++) { to[j] = gtok[j]; to[SAM_TOPK_MAX + j] = gtgt[j]; }
