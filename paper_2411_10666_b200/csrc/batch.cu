@@ -88,9 +88,9 @@ __device__ __forceinline__ void clear_slot(const SamBatchView& W, int b) {
 __global__ void __launch_bounds__(RESET_THREADS) init_batch_kernel(SamBatchView W) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    for (int s = i; s < W.pool_slabs; s += stride) {
-        W.free_stack[s] = W.pool_slabs - 1 - s;                 // slab 0 is handed out first
+    const size_t i = sam_grid_index(blockIdx.x, blockDim.x, threadIdx.x), stride = sam_grid_size(gridDim.x, blockDim.x);
+    for (size_t s = i; s < (size_t)W.pool_slabs; s += stride) {
+        W.free_stack[s] = W.pool_slabs - 1 - (int32_t)s;               // slab 0 is handed out first
         W.slab_owner[s] = -1;
     }
     if (threadIdx.x == 0) W.reset_mark[blockIdx.x] = 0;
@@ -114,12 +114,12 @@ __global__ void __launch_bounds__(RESET_THREADS) reset_slots_kernel(SamBatchView
 __global__ void release_slabs_kernel(SamBatchView W, int32_t mark) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    for (int s = i; s < W.pool_slabs; s += stride) {
+    const size_t i = sam_grid_index(blockIdx.x, blockDim.x, threadIdx.x), stride = sam_grid_size(gridDim.x, blockDim.x);
+    for (size_t s = i; s < (size_t)W.pool_slabs; s += stride) {
         const int owner = W.slab_owner[s];
         if (owner >= 0 && W.reset_mark[owner] == mark) {
             W.slab_owner[s] = -1;
-            W.free_stack[atomicAdd(W.pool_hdr, 1)] = s;
+            W.free_stack[atomicAdd(W.pool_hdr, 1)] = (int32_t)s;
         }
     }
 }

@@ -45,6 +45,7 @@
 //               (the state of the whole prefix of length i + 1), so the states along an earlier
 //               occurrence of a passage can be addressed without following their transitions.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 #include <vector_types.h>
 
@@ -100,6 +101,10 @@ SAM_HD uint64_t sam_path_join(uint64_t p, uint64_t q) {
     const uint32_t steps = (uint32_t)p + ((uint32_t)q < SAM_PATH_MAX ? (uint32_t)q : SAM_PATH_MAX);
     return (q >> 32) << 32 | (steps < SAM_PATH_MAX ? steps : SAM_PATH_MAX);
 }
+
+// A thread's number in a one-dimensional grid, and the grid's size: 2^24 slots with 128 threads each are 2^31 threads.
+SAM_HD size_t sam_grid_index(uint32_t block, uint32_t threads, uint32_t thread) { return (size_t)block * threads + thread; }
+SAM_HD size_t sam_grid_size(uint32_t blocks, uint32_t threads) { return (size_t)blocks * threads; }
 
 // 64-bit multiplicative mix of (state, token); upper half is the hash.
 SAM_HD uint32_t sam_hash2(uint32_t state, uint32_t tok) {

@@ -1294,21 +1294,21 @@ __global__ void __launch_bounds__(96, 5) sam_step_inline_kernel(const __grid_con
 }
 
 // Larger ones: the rows and counts are brought over in whole lines by this kernel, launched ahead of the step's.
-__global__ void __launch_bounds__(128) fetch_inputs_kernel(const int32_t* rows, const int32_t* counts, int32_t* to, uint32_t n_rows, uint32_t n_counts) {
+__global__ void __launch_bounds__(128) fetch_inputs_kernel(const int32_t* rows, const int32_t* counts, int32_t* to, size_t n_rows, size_t n_counts) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
+    const size_t t = sam_grid_index(blockIdx.x, blockDim.x, threadIdx.x), all = sam_grid_size(gridDim.x, blockDim.x);
 #pragma unroll
     for (int k = 0; k < 2; k++) {
         const int32_t* from = k ? counts : rows;
         int32_t* dst = k ? to + n_rows : to;
-        const uint32_t n = k ? n_counts : n_rows;
-        uint32_t done = 0;
+        const size_t n = k ? n_counts : n_rows;
+        size_t done = 0;
         if (((reinterpret_cast<uintptr_t>(from) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
-            for (uint32_t i = t; i < n / 4; i += all) reinterpret_cast<int4*>(dst)[i] = reinterpret_cast<const int4*>(from)[i];
-            done = n & ~3u;
+            for (size_t i = t; i < n / 4; i += all) reinterpret_cast<int4*>(dst)[i] = reinterpret_cast<const int4*>(from)[i];
+            done = n & ~(size_t)3;
         }
-        for (uint32_t i = done + t; i < n; i += all) dst[i] = from[i];
+        for (size_t i = done + t; i < n; i += all) dst[i] = from[i];
     }
 }
 
@@ -2381,7 +2381,7 @@ int sam_launch_fetch(const sam_batch* b, const int32_t* rows, const int32_t* cou
     memset(&cfg, 0, sizeof(cfg));
     const size_t n = (size_t)b->view.batch * stride, blocks = (n + 511) / 512;      // a 16-byte read a thread
     cfg.gridDim = dim3((unsigned)(blocks < 592 ? blocks : 592)); cfg.blockDim = dim3(128); cfg.stream = stream; cfg.attrs = attr; cfg.numAttrs = 1;
-    SAM_CUDA(cudaLaunchKernelEx(&cfg, fetch_inputs_kernel, rows, counts, to, (uint32_t)n, (uint32_t)b->view.batch));
+    SAM_CUDA(cudaLaunchKernelEx(&cfg, fetch_inputs_kernel, rows, counts, to, n, (size_t)b->view.batch));
     return SAM_OK;
 }
 

@@ -9,6 +9,8 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2411_10666_b200", "csrc")
 SOURCE = """
 #include "layout.h"
+extern "C" int64_t grid_index(uint32_t block, uint32_t threads, uint32_t thread) { return (int64_t)sam_grid_index(block, threads, thread); }
+extern "C" int64_t grid_size(uint32_t blocks, uint32_t threads) { return (int64_t)sam_grid_size(blocks, threads); }
 extern "C" uint64_t path_max() { return SAM_PATH_MAX; }
 // pointer jumping over the chain 0 -> 1 -> ... -> n, one state after the other in the order given
 extern "C" void path_pass(uint64_t* path, const int64_t* order, int64_t n) {
@@ -32,6 +34,7 @@ def lib(tmp_path_factory):
     subprocess.check_call([os.environ.get("NVCC", "nvcc"), "-O1", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", CSRC, "-o", out, src])
     L = ctypes.CDLL(out)
     L.path_max.restype = ctypes.c_uint64
+    L.grid_index.restype = L.grid_size.restype = ctypes.c_int64
     return L
 
 
@@ -53,3 +56,10 @@ def test_a_path_never_has_more_steps_than_a_tree_entry_holds(lib, order):
     assert most < 1 << 16 and (steps >= np.minimum(left, 128)).all() and (steps <= most).all()
     exact = steps < most
     assert np.array_equal(end[exact], np.arange(n)[exact] + steps[exact]) and (steps[exact] <= left[exact]).all()
+
+
+def test_thread_numbers_at_the_largest_batch(lib):
+    """2^24 slots, a block of 128 threads each, clear the batch: thread numbers and the grid's size pass 2^31."""
+    slots, threads = 1 << 24, 128
+    assert lib.grid_size(slots, threads) == slots * threads == 1 << 31
+    assert lib.grid_index(slots - 1, threads, threads - 1) == (1 << 31) - 1
