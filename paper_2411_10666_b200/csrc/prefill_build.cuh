@@ -237,11 +237,16 @@ __device__ __forceinline__ void pb_into(const PbArrays& a, uint32_t u, F f) {
 }
 
 __device__ __forceinline__ uint32_t pb_take_slabs(const SamBatchView& W, int want, int b, uint32_t* out, int lane, int& err) {
-    // by one warp: all of them with one addition; nothing is taken if they are not all there
+    // by one warp: all of them at once, or none.  (Never taken first and given back if they are too few: in between, other
+    // blocks would find the pool short and fail prompts that it has room for.)
     int old = 0;
     if (lane == 0) {
-        old = atomicSub(W.pool_hdr, want);
-        if (old < want) atomicAdd(W.pool_hdr, want);
+        old = *reinterpret_cast<volatile int32_t*>(W.pool_hdr);
+        while (old >= want) {                              // (each round that fails, another block has taken its slabs)
+            const int seen = atomicCAS(W.pool_hdr, old, old - want);
+            if (seen == old) break;
+            old = seen;
+        }
     }
     old = __shfl_sync(0xFFFFFFFFu, old, 0);
     if (old < want) { err = SAM_SEQ_CAPACITY; return 0; }

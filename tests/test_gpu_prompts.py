@@ -204,3 +204,30 @@ def test_steps_at_the_edges_of_the_register_budgets(P, B):
     ref = ob.step(target, m, L, 8)
     for k in keys:
         assert np.array_equal(getattr(out[1], k).cpu().numpy(), getattr(ref, k)), k
+
+
+@pytest.mark.parametrize("B", [64, 400])
+def test_prompts_beside_others_the_pool_cannot_hold(P, B):
+    """Prompts the pool has room for are taken, whatever others that never fit ask for at the same time."""
+    import torch
+    rng = np.random.default_rng(B)
+    vocab, n, L, fits = 2000, 1000, 8, (B // 3, B - 5)
+    rows = rng.integers(0, 25, size=(B, n), dtype=np.int32)
+    for b in fits:
+        rows[b] = rng.permutation(vocab)[:n]                # one state a token, no edge blocks
+    toks, counts = torch.from_numpy(rows).cuda(), torch.full((B,), n, dtype=torch.int32, device="cuda")
+
+    def takes(b):
+        one = P.Batch(None, 1, n, max_draft_len=L, vocab=vocab, slab_bytes=4096)
+        assert one.step(toks[b:b + 1], counts[:1], L).cpu()["status"][0] == 0
+        total, free = one.pool_info()
+        return total - free
+
+    pool = sum(takes(b) for b in fits)
+    assert all(takes(b) > pool for b in (0, 1, B // 2, B - 1))
+    for turn in range(30):
+        batch = P.Batch(None, B, n, max_draft_len=L, vocab=vocab, slab_bytes=4096, pool_slabs=pool)
+        status = batch.step(toks, counts, L).cpu()["status"]
+        assert np.flatnonzero(status == 0).tolist() == list(fits), (turn, np.flatnonzero(status == 0))
+        assert batch.pool_info() == (pool, 0)
+        batch.close()
