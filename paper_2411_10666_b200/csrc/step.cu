@@ -34,6 +34,7 @@
 //     with few tokens on a single lane), neither waiting for the other, and whichever finishes last writes
 //     the slot's outputs (sam_step_split_kernel, further down).
 #include "common.h"
+#include "once.h"
 
 #include <cstring>
 
@@ -2237,17 +2238,19 @@ constexpr int SAM_ORDER_MIN_BATCH = 1536;                    // more slots than 
 }  // namespace
 
 namespace {
+constexpr int SAM_MAX_DEVICES = 64;
+SamOncePerDevice<SAM_MAX_DEVICES> g_split_setup, g_prefill_setup[4];
+
 int split_kernel_setup(int device) {
-    static bool done[64];
-    if (device < 0 || device >= 64) return SAM_ERR_ARG;
-    if (!done[device]) {
+    if (device < 0 || device >= SAM_MAX_DEVICES) return SAM_ERR_ARG;
+    cudaError_t e = (cudaError_t)g_split_setup(device, []() -> int {
         cudaError_t e = cudaFuncSetAttribute(sam_step_split_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(order_slots_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel<2>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-        if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
-        done[device] = true;
-    }
+        return (int)e;
+    });
+    if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;
 }
 // The build for rows of up to `stride` tokens.  With the static side: two tokens a thread, four where more than two
@@ -2263,13 +2266,10 @@ int launch_prefill(const StepArgs& A, int batch, int device, cudaLaunchConfig_t*
         k = n2 <= 1024 ? 1 : n2 <= 2048 ? 2 : 3;
         threads = n2 / 4 < 64 ? 64 : n2 / 4 > 1024 ? 1024 : n2 / 4;
     }
-    static bool done[64][4];                                // the kernels' shared memory, once per device
-    if (device < 0 || device >= 64) return SAM_ERR_ARG;
-    cudaError_t e = cudaSuccess;
-    if (!done[device][k]) {
-        e = cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, PB_MAX * PB_BYTES_PER_TOKEN);
-        done[device][k] = e == cudaSuccess;
-    }
+    if (device < 0 || device >= SAM_MAX_DEVICES) return SAM_ERR_ARG;
+    cudaError_t e = (cudaError_t)g_prefill_setup[k](device, [&]() -> int {
+        return (int)cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, PB_MAX * PB_BYTES_PER_TOKEN);
+    });
     cfg->gridDim = dim3((unsigned)batch); cfg->blockDim = dim3((unsigned)threads); cfg->dynamicSmemBytes = (size_t)n2 * PB_BYTES_PER_TOKEN;
     if (e == cudaSuccess) e = cudaLaunchKernelEx(cfg, kernels[k], A);
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
