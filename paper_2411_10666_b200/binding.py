@@ -1,4 +1,5 @@
-"""ctypes binding of libsamdraft.so: the same calls as include/samdraft.h, argument marshalling only.
+"""Binding of libsamdraft.so: the same calls as include/samdraft.h, argument marshalling only.  The calls a serving loop makes
+every step are marshalled in C (csrc/calls.c) where that can be compiled, the others, and all where it cannot, by ctypes.
 
 Every step of the retrieval path runs inside the CUDA library.  PyTorch is used here for device
 memory (the batch workspace and the I/O tensors) and for the current stream, nothing else.  If the
@@ -117,23 +118,99 @@ _calls = None
 _fn = {}
 
 
+def _load_calls():
+    """The extension module that marshals the per-step calls, or, where it is not there and cannot be compiled (no C
+    compiler, no Python headers, a directory that cannot be written), the same by ctypes: some 8 us more a call."""
+    import importlib.machinery
+    import importlib.util
+    import subprocess
+    import warnings
+    import torch
+    try:
+        loader = importlib.machinery.ExtensionFileLoader("_calls", _build.build_calls())
+        m = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
+        loader.exec_module(m)
+    except (OSError, subprocess.CalledProcessError, ImportError) as e:
+        warnings.warn("per-step calls are marshalled by ctypes, some 8 us more each: %s" % e, RuntimeWarning)
+        return _PlainCalls
+    m.setup(torch.int32, torch.float32, torch._C._cuda_getCurrentRawStream, _host_ptr)
+    return m
+
+
 def _hot(name: str):
-    """(extension module, address of a library function): for the calls that are made every step."""
+    """(marshalling module, address of a library function): for the calls that are made every step."""
     global _calls
     addr = _fn.get(name)
     if addr is None:
         if _calls is None:
-            import importlib.machinery
-            import importlib.util
-            import torch
-            path = _build.build_calls()
-            loader = importlib.machinery.ExtensionFileLoader("_calls", path)
-            m = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
-            loader.exec_module(m)
-            m.setup(torch.int32, torch.float32, torch._C._cuda_getCurrentRawStream, _host_ptr)
-            _calls = m
+            _calls = _load_calls()
         addr = _fn[name] = ctypes.cast(getattr(lib(), name), c_void_p).value
     return _calls, addr
+
+
+class _PlainCalls:
+    """What csrc/calls.c does, by ctypes: the same functions with the same arguments."""
+
+    @staticmethod
+    def _stream(x):
+        import torch
+        return x if x >= 0 else torch._C._cuda_getCurrentRawStream(-1 - x)
+
+    @staticmethod
+    def _outputs(tensors):
+        return [_dev_ptr(t, n) for t, n in zip(tensors, ("draft_tokens", "draft_len", "match_len", "source", "state", "status"))]
+
+    @staticmethod
+    def step_out(fn, h, new_tokens, counts, L, out, stream):
+        return _PlainCalls.step(fn, h, new_tokens, new_tokens.shape[-1] if new_tokens.dim() else 0, counts, L, *out.tensors(), stream)
+
+    @staticmethod
+    def step(fn, h, new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state, status, stream):
+        c = _PlainCalls
+        return lib().sam_step(h, _dev_ptr(new_tokens, "new_tokens"), stride, _dev_ptr(counts, "counts"), L,
+                              *c._outputs((draft_tokens, draft_len, match_len, source, state, status)), c._stream(stream))
+
+    @staticmethod
+    def step_host(fn, h, new_tokens, stride, counts, L, draft_tokens, draft_len, match_len, source, state, status, stream):
+        p = [_host_ptr(t, n) for t, n in ((new_tokens, "new_tokens"), (counts, "counts"), (draft_tokens, "draft_tokens"),
+                                          (draft_len, "draft_len"), (match_len, "match_len"), (source, "source"), (state, "state"),
+                                          (status, "status"))]
+        return lib().sam_step_host(h, p[0], stride, p[1], L, *p[2:], _PlainCalls._stream(stream))
+
+    @staticmethod
+    def step_verified(fn, h, target, prev_L, prev_draft, prev_len, max_new, L, draft_tokens, draft_len, match_len, source, state,
+                      status, counts_out, accepted_out, stream):
+        c = _PlainCalls
+        return lib().sam_step_verified(h, _dev_ptr(target, "target_tokens"), prev_L, _dev_ptr(prev_draft, "prev_draft_tokens"),
+                                       _dev_ptr(prev_len, "prev_draft_len"), _dev_ptr(max_new, "max_new"), L,
+                                       *c._outputs((draft_tokens, draft_len, match_len, source, state, status)),
+                                       _dev_ptr(counts_out, "counts_out"), _dev_ptr(accepted_out, "accepted_out"), c._stream(stream))
+
+    @staticmethod
+    def select_auxiliary(fn, batch, L, draft, draft_len, source, aux, aux_len, stream):
+        return lib().sam_select_auxiliary(batch, L, _dev_ptr(draft, "draft_tokens"), _dev_ptr(draft_len, "draft_len"),
+                                          _dev_ptr(source, "source"), _dev_ptr(aux, "aux_tokens"), _dev_ptr(aux_len, "aux_len"),
+                                          _PlainCalls._stream(stream))
+
+    @staticmethod
+    def accept_greedy(fn, batch, draft, draft_len, L, target, max_new, new_tokens, stride, counts, accepted, stream):
+        return lib().sam_accept_greedy(batch, _dev_ptr(draft, "draft_tokens"), _dev_ptr(draft_len, "draft_len"), L,
+                                       _dev_ptr(target, "target_tokens"), _dev_ptr(max_new, "max_new"), _dev_ptr(new_tokens, "new_tokens"),
+                                       stride, _dev_ptr(counts, "counts"), _dev_ptr(accepted, "accepted"), _PlainCalls._stream(stream))
+
+    @staticmethod
+    def tree_draft(fn, static, batch, states, starts, max_size, k, tokens, parents, probs, sizes, stream):
+        return lib().sam_tree_draft(static, batch, _dev_ptr(states, "states"), _dev_ptr(starts, "start_tokens"), max_size, k,
+                                    _dev_ptr(tokens, "tree_tokens"), _dev_ptr(parents, "tree_parents"), _dev_ptr(probs, "tree_probs", "float32"),
+                                    _dev_ptr(sizes, "tree_size"), _PlainCalls._stream(stream))
+
+    @staticmethod
+    def retrieve_noalloc(fn, static, vocab, batch, tokens, stride, counts, L, l_bias, min_match, draft_tokens, draft_len, match_len,
+                         source, state, status, stream):
+        c = _PlainCalls
+        return lib().sam_retrieve_noalloc(static, vocab, batch, _dev_ptr(tokens, "tokens"), stride, _dev_ptr(counts, "counts"), L, l_bias,
+                                          min_match, *c._outputs((draft_tokens, draft_len, match_len, source, state, status)),
+                                          c._stream(stream))
 
 
 def _addr(h) -> int:
@@ -157,12 +234,12 @@ def _np32(a) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
 
-def _dev_ptr(t, name: str):
+def _dev_ptr(t, name: str, dtype: str = "int32"):
     import torch
     if t is None:
         return None
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.int32 and t.is_contiguous()):
-        raise TypeError("%s must be a contiguous int32 CUDA tensor" % name)
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == getattr(torch, dtype) and t.is_contiguous()):
+        raise TypeError("%s must be a contiguous %s CUDA tensor" % (name, dtype))
     return t.data_ptr()
 
 

@@ -267,3 +267,48 @@ def test_stop_token_matches_oracle(P):
     plain, _ = gpu_run(P, st, spec.vocab, w.prompts, w.new_tokens, w.counts, L, msl)
     assert (got["draft_len"] < plain["draft_len"]).any()    # some drafts were cut
     assert not (got["draft_tokens"] == stop).any()
+
+
+def test_per_step_calls_without_the_extension_module(P, monkeypatch):
+    """A machine that cannot compile csrc/calls.c: every call it marshals gives the same results through ctypes."""
+    import torch
+    rng = np.random.default_rng(12)
+    vocab, B, n, L = 30, 6, 80, 8
+    corpus = rng.integers(0, vocab, size=3000, dtype=np.int32)
+    st = P.StaticSam.build(corpus, vocab, tree_topk=3)
+    toks = torch.from_numpy(rng.integers(0, vocab, size=(B, n), dtype=np.int32)).cuda()
+    counts, few = (torch.full((B,), k, dtype=torch.int32, device="cuda") for k in (n, 5))
+    x = P.binding
+
+    def all_calls():
+        i32 = dict(dtype=torch.int32, device="cuda")
+        b = P.Batch(st, B, 4 * n, max_draft_len=L)
+        first, second, host = b.step(toks, counts, L), P.StepOutputs(B, L, "cuda"), P.StepOutputs(B, L, "cpu")
+        x.sam_step(b.handle, toks[:, :5].contiguous(), 5, few, L, *second.tensors())
+        new, cnt, acc = torch.empty(B, L + 1, **i32), torch.empty(B, **i32), torch.empty(B, **i32)
+        target = torch.cat([first.draft_tokens, first.draft_tokens[:, :1]], 1).clamp_(0, vocab - 1).contiguous()
+        x.sam_accept_greedy(first.draft_tokens, first.draft_len, target, None, new, cnt, acc)
+        third = P.StepOutputs(B, L, "cuda")
+        x.sam_step_verified(b.handle, target, first.draft_tokens, first.draft_len, None, L, *third.tensors(), counts_out=cnt, accepted_out=acc)
+        x.sam_select_auxiliary(third.draft_tokens, third.draft_len, third.source, target[:, :L].contiguous(), few)
+        x.sam_step_host(b.handle, toks[:, :5].cpu(), 5, few.cpu(), L, *host.tensors())
+        again = P.StepOutputs(B, L, "cpu")
+        x.sam_step_host_prepared(b.handle, 5, L, *again.tensors())(toks[:, 5:10].cpu().contiguous(), few.cpu())
+        tree = [torch.empty(B, 12, **i32), torch.empty(B, 12, **i32), torch.empty(B, 12, device="cuda"), torch.empty(B, **i32)]
+        x.sam_tree_draft(st.handle, first.state[:, 0].contiguous(), toks[:, -1].contiguous(), 12, 3, *tree)
+        once = P.StepOutputs(B, L, "cuda")
+        x.sam_retrieve_noalloc(st.handle, vocab, toks, counts, L, 0, 1, *once.tensors())
+        return [t.cpu().numpy() for o in (first, second, third, host, again, once) for t in o.tensors()] + [t.cpu().numpy() for t in (new, cnt, acc, *tree)]
+
+    expected = all_calls()
+
+    def build_calls(force=False):
+        raise FileNotFoundError("gcc")
+
+    monkeypatch.setattr(x, "_calls", None)
+    monkeypatch.setattr(x, "_fn", {})
+    monkeypatch.setattr(x._build, "build_calls", build_calls)
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        got = all_calls()
+    assert x._calls is x._PlainCalls
+    assert len(got) == len(expected) and all(np.array_equal(a, b) for a, b in zip(got, expected))
