@@ -61,7 +61,8 @@ NCU_TRAFFIC = {
            "10 M-token corpus (3.80 MB read + 1.17 MB written per launch of 4096 slots) and carried over per slot: the "
            "full-size corpus changes which lines are read, not how many"),
 }
-KERNEL_SOURCES = ("paper_2411_10666_b200/csrc/step.cu", "paper_2411_10666_b200/csrc/static_match.cuh", "paper_2411_10666_b200/csrc/layout.h")
+KERNEL_SOURCES = tuple("paper_2411_10666_b200/csrc/" + f for f in
+                       ("step.cu", "static_match.cuh", "prefill_build.cuh", "common.h", "layout.h", "once.h"))
 
 
 def kernel_digest() -> str:

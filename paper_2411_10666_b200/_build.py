@@ -26,7 +26,7 @@ def _stale(lib: str) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = _sources() + glob.glob(os.path.join(CSRC, "*.h")) + \
+    deps = _sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(os.path.dirname(HERE), "include", "samdraft.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 

@@ -110,3 +110,33 @@ def test_byte_model_and_workload_naming_of_the_benchmark():
     assert cfg["workload"] == "c4 (recipe run with 77 sequences)" and cfg["global_batch"] == 154 and cfg["batch_per_gpu"] == 77
     assert set(cfg) >= {"workload", "batch_per_gpu", "global_batch", "prompt_len", "gen_len", "draft_len", "corpus_tokens", "vocab", "l2"}
     assert len(bench.kernel_digest()) == 16
+
+
+def test_the_kernel_digest_covers_every_file_the_step_kernels_are_made_of():
+    import re
+    sys.path.insert(0, ROOT)
+    import bench
+    csrc, seen, todo = os.path.join(ROOT, "paper_2411_10666_b200", "csrc"), set(), ["step.cu"]
+    while todo:
+        name = todo.pop()
+        if name in seen or not os.path.exists(os.path.join(csrc, name)):
+            continue
+        seen.add(name)
+        todo += re.findall(r'^#include "([^"]+)"', open(os.path.join(csrc, name)).read(), re.M)
+    assert {os.path.basename(f) for f in bench.KERNEL_SOURCES} == seen
+
+
+def test_the_library_is_rebuilt_when_any_of_its_sources_changes():
+    from paper_2411_10666_b200 import _build
+    _build.build()
+    for name in sorted(os.listdir(_build.CSRC)):
+        if not name.endswith((".cu", ".cuh", ".cpp", ".h")):
+            continue
+        path = os.path.join(_build.CSRC, name)
+        was = os.stat(path)
+        try:
+            os.utime(path, ns=(was.st_atime_ns, os.stat(_build.LIB).st_mtime_ns + 10 ** 9))
+            assert _build._stale(_build.LIB), name
+        finally:
+            os.utime(path, ns=(was.st_atime_ns, was.st_mtime_ns))
+    assert not _build._stale(_build.LIB)
