@@ -119,8 +119,8 @@ def test_the_kernel_digest_covers_every_file_the_step_kernels_are_made_of():
     csrc, seen, todo = os.path.join(ROOT, "paper_2411_10666_b200", "csrc"), set(), ["step.cu"]
     while todo:
         name = todo.pop()
-        if name in seen or not os.path.exists(os.path.join(csrc, name)):
-            continue
+        if name in seen or "/" in name or not os.path.exists(os.path.join(csrc, name)):
+            continue                                        # (the public header declares calls, and counters the kernels index)
         seen.add(name)
         todo += re.findall(r'^#include "([^"]+)"', open(os.path.join(csrc, name)).read(), re.M)
     assert {os.path.basename(f) for f in bench.KERNEL_SOURCES} == seen
