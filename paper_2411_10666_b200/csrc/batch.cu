@@ -536,7 +536,7 @@ extern "C" int sam_batch_pool_info(sam_batch_t* b, int64_t* total_slabs, int64_t
     int32_t hdr[2] = {0, 0};
     SAM_CUDA(cudaMemcpyAsync(hdr, b->view.pool_hdr, 8, cudaMemcpyDeviceToHost, (cudaStream_t)stream));
     SAM_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
-    *free_slabs = hdr[0]; *total_slabs = hdr[1];
+    *free_slabs = hdr[0]; *total_slabs = b->view.pool_slabs;
     return SAM_OK;
 }
 

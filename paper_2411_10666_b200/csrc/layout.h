@@ -145,7 +145,7 @@ struct SamStaticView {
 // Device-side view of a batch workspace.
 struct SamBatchView {
     uint32_t* ctrl;           // [B][SAM_CTRL_WORDS]
-    int32_t* pool_hdr;        // [0] free slabs, [1] total slabs
+    int32_t* pool_hdr;        // [0] free slabs, [1] total slabs (plus takers under way, see pb_take_slabs), [4] blocks of a host step that are done
     int32_t* free_stack;      // [pool_slabs]
     int32_t* slab_owner;      // [pool_slabs], -1 = free
     int32_t* reset_mark;      // [B]: number of the last reset that named the slot

@@ -231,3 +231,32 @@ def test_prompts_beside_others_the_pool_cannot_hold(P, B):
         assert np.flatnonzero(status == 0).tolist() == list(fits), (turn, np.flatnonzero(status == 0))
         assert batch.pool_info() == (pool, 0)
         batch.close()
+
+
+@pytest.mark.parametrize("B", [64, 400])
+def test_as_many_prompts_as_the_pool_holds(P, B):
+    """Prompts of one text against a pool that holds half of them and a rest too small for one more: that many are taken, and
+    they are the oracle's; the others fail without holding anything."""
+    import torch
+    rng = np.random.default_rng(B + 1)
+    vocab, n, L, holds = 60, 700, 8, B // 2
+    row = rng.integers(0, vocab, size=n, dtype=np.int32)
+    toks = torch.from_numpy(np.tile(row, (B, 1))).cuda()
+    counts = torch.full((B,), n, dtype=torch.int32, device="cuda")
+    ref = oracle.Batch(None, None, 1, vocab, n).step(row[None], np.array([n], dtype=np.int32), L, 1)
+    one = P.Batch(None, 1, n, max_draft_len=L, vocab=vocab, slab_bytes=4096)
+    one.step(toks[:1], counts[:1], L)
+    total, free = one.pool_info()
+    takes = total - free
+    assert takes > 4
+    for turn in range(10):
+        batch = P.Batch(None, B, n, max_draft_len=L, vocab=vocab, slab_bytes=4096, pool_slabs=holds * takes + takes - 1)
+        out = batch.step(toks, counts, L).cpu()
+        done = out["status"] == 0
+        assert done.sum() == holds and (out["status"][~done] == 1).all()
+        assert batch.pool_info() == (holds * takes + takes - 1, takes - 1)
+        for k in ("draft_tokens", "draft_len", "match_len", "source", "state"):
+            assert (out[k][done] == getattr(ref, k)[0]).all(), k
+        batch.reset()
+        assert batch.pool_info() == (holds * takes + takes - 1,) * 2
+        batch.close()
