@@ -1042,10 +1042,22 @@ __device__ __forceinline__ uint32_t ahead_targets(const Ahead& H, const uint4& a
     }
     return q & SAM_IDMASK;
 }
+// A barrier of all three warps; whether x holds for any thread.  (Not the barrier of step_sync: the third warp may come to this
+// one before the others have passed that.)
+__device__ __forceinline__ bool step_join(bool x) {
+    uint32_t r;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %1, 0; bar.red.or.pred q, 2, 96, p; selp.u32 %0, 1, 0, q; }" : "=r"(r) : "r"((uint32_t)x) : "memory");
+    return r != 0;
+}
+// The third warp's part in it, once what it read last has arrived: its vote depends on that (and says nothing).  Out of line,
+// so that a step nobody waits for in this way does not wait for those reads.
+__device__ __noinline__ void ahead_join(uint32_t x, uint32_t y, uint32_t z) { step_join(x + (y ^ z) == 0xFFFFFFFFu); }
+
 constexpr int AHEAD_MIN_TOKENS = 2, AHEAD_LEVELS = 4;
-__device__ __forceinline__ void read_ahead(const SamBatchView& W, int b, int lane, uint32_t cw, uint32_t cw2, int32_t tok_first, int m) {
+// join: end with ahead_join.
+__device__ __forceinline__ void read_ahead(const SamBatchView& W, int b, int lane, uint32_t cw, uint32_t cw2, int32_t tok_first, int m, bool join) {
     const int n = m < 32 ? m : 32;
-    if (n < AHEAD_MIN_TOKENS) return;
+    if (n < AHEAD_MIN_TOKENS) { if (join) ahead_join((uint32_t)tok_first, 0, 0); return; }
     Ahead H;
     H.pool = W.pool; H.slab_shift = W.slab_shift; H.lane = lane;
     {
@@ -1078,14 +1090,15 @@ __device__ __forceinline__ void read_ahead(const SamBatchView& W, int b, int lan
         u = ahead_targets(H, a, bb, next);
         ahead_records(H, u != 0, u, a, bb);
     }
+    if (join) ahead_join(t, a.w, bb.w);
 }
 
-// Both warps' results are in shared memory: choose the source, write the slot's outputs.
+// Both warps' results are in shared memory: choose the source, write the slot's outputs.  Not failed: both errors are 0.
 template <bool VERIFY>
 __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp, int lane, uint32_t* cb, const int32_t* sh_l, const int32_t* sh_s,
-                                             const int32_t* sh_dl, const int32_t* sh_err, const int32_t d[MAX_DRAFT_REGS], int m, int confirmed) {
+                                             const int32_t* sh_dl, const int32_t* sh_err, bool failed, const int32_t d[MAX_DRAFT_REGS], int m, int confirmed) {
     const int L = A.L;
-    const int any_err = sh_err[0] ? sh_err[0] : sh_err[1];
+    const int any_err = !failed ? 0 : sh_err[0] ? sh_err[0] : sh_err[1];
     const int l1 = sh_l[0], l2v = sh_l[1];
     const bool use_static = A.has_static && l1 > l2v + A.W.l_bias;        // Section 3.2
     const int lsel = use_static ? l1 : l2v;
@@ -1134,7 +1147,6 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
 // VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
 // The two warps that work on the slot.
 __device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
-
 // AHEAD: a third warp reads ahead of the dynamic side (read_ahead).
 // INLINE: the rows and counts came with the launch (sam_step_host).
 template <bool VERIFY, bool AHEAD, bool INLINE>
@@ -1191,8 +1203,12 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
     int status = (int)__shfl_sync(FULL, cw, CB_STATUS);
     const uint32_t ntok0 = __shfl_sync(FULL, cw, CB_NTOK);
     const int L = A.L;
+    const bool host = AHEAD && !VERIFY && (A.tagged != nullptr || A.done_flag != nullptr);
     if (AHEAD && warp == 2) {
-        if (status == 0 && m <= A.stride && __shfl_sync(FULL, cw, CB_ERR_S) == 0) read_ahead(A.W, b, lane, cw, cw2, tok_first, m);
+        // A host-array step's caller goes on before this kernel has ended, but not before this warp's reads have: of the caller's
+        // arrays, which kernels may read in place, and of the batch's memory.
+        if (status == 0 && m <= A.stride && __shfl_sync(FULL, cw, CB_ERR_S) == 0) read_ahead(A.W, b, lane, cw, cw2, tok_first, m, host);
+        else if (host) ahead_join((uint32_t)tok_first, 0, 0);
         return;
     }
     step_sync();              // both warps hold the slot's state as it was before either writes any of it
@@ -1202,6 +1218,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
     const bool built = done == SAM_STEP_BUILT;
     if (done != 0 && threadIdx.x == 0) cb[CB_ERR_S] = 0;
     if (done == SAM_STEP_DONE) {
+        if (host) step_join(false);
         if (threadIdx.x == 0 && A.done_flag) signal_done(A);
         return;
     }
@@ -1223,6 +1240,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
         fresh_fail = status != 0;
     }
     if (status != 0) {
+        if (host) step_join(false);
         if (warp == 0) {
             if (fresh_fail && lane == 0) cb[CB_STATUS] = (uint32_t)status;
             if (A.tagged) write_failed_tagged(A, b, lane, status);
@@ -1268,10 +1286,11 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
     }
 
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
-    step_sync();
-    step_outputs<VERIFY>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, d, m, confirmed);
-    if (A.done_flag) {
-        step_sync();
+    bool failed = true;
+    if (AHEAD && !VERIFY && A.tagged) failed = step_join(err != 0); else step_sync();
+    step_outputs<VERIFY>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, failed, d, m, confirmed);
+    if (!VERIFY && A.done_flag) {
+        if (AHEAD) step_join(false); else step_sync();
         if (threadIdx.x == 0) signal_done(A);
     }
 }
@@ -1381,7 +1400,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
     }
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
     asm volatile("bar.sync 2, 64;" ::: "memory");
-    step_outputs<false>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, d, m, 0);
+    step_outputs<false>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, true, d, m, 0);
     if (threadIdx.x == 0) cb[CB_ERR_S] = SAM_STEP_DONE;
 }
 

@@ -312,3 +312,37 @@ def test_per_step_calls_without_the_extension_module(P, monkeypatch):
         got = all_calls()
     assert x._calls is x._PlainCalls
     assert len(got) == len(expected) and all(np.array_equal(a, b) for a, b in zip(got, expected))
+
+
+@pytest.mark.parametrize("B,K,L", [(100, 40, 128), (200, 16, 128), (700, 8, 24)])
+def test_host_arrays_are_the_callers_again_when_the_call_returns(P, B, K, L):
+    """Page-locked arrays that kernels work on in place (64 KiB and more in all, rows too few to be fetched ahead): every step has
+    arrays of its own, unregistered and overwritten as soon as the call returns; the batch is dropped after the last."""
+    import torch
+    assert B * (K + 1) < 8192 and B * (K + 1 + L + 7) * 4 >= 65536
+    rt = torch.cuda.cudart()
+    rng = np.random.default_rng(B)
+    vocab, steps = 30, 12
+    corpus = rng.integers(0, vocab, size=4000, dtype=np.int32)
+    st, S = P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)
+    ob, batch = oracle.Batch(S, corpus, B, vocab, K * steps), P.Batch(st, B, K * steps, max_draft_len=L, max_host_stride=K)
+    shapes = ((B, K), (B,), (B, L), (B,), (B, 2), (B,), (B, 2), (B,))
+    words = [int(np.prod(s)) for s in shapes]
+    for i in range(steps):
+        toks = rng.integers(0, vocab, size=(B, K), dtype=np.int32)
+        counts = rng.integers(0, K + 1, size=B).astype(np.int32)
+        raw = np.full(sum(words) + 1024, -9, dtype=np.int32)
+        at = (-(raw.ctypes.data // 4)) % 1024                # a page of its own
+        assert int(rt.cudaHostRegister(raw.ctypes.data + 4 * at, 4 * sum(words), 0)) == 0
+        views = []
+        for s, n in zip(shapes, words):
+            views.append(raw[at:at + n].reshape(s)); at += n
+        views[0][:], views[1][:] = toks, counts
+        P.binding.sam_step_host(batch.handle, views[0], K, views[1], L, *views[2:])
+        assert int(rt.cudaHostUnregister(views[0].ctypes.data)) == 0
+        got = [v.copy() for v in views[2:]]
+        raw[:] = -5
+        ref = ob.step(toks, counts, L, 4)
+        for k, v in zip(KEYS, got):
+            assert np.array_equal(v, getattr(ref, k)), (i, k)
+    batch.close()
