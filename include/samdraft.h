@@ -212,8 +212,9 @@ int sam_run_steps(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t stride,
  * through a page-locked staging area word by word, each with the step's number; from 64 KiB of arrays on, arrays
  * that are ALL page-locked and device-addressable (cudaHostAlloc, cudaHostRegister, a pinned torch tensor)
  * are read and written in place by kernels, and any others are copied through the staging area.  state_host may be
- * NULL.  Synchronous: the results are in the arrays when the call returns.  Errors: as sam_step,
- * plus CUDA. */
+ * NULL.  Synchronous: when the call returns the results are in the arrays, the arrays are the caller's again,
+ * and the batch is as the step leaves it for any later work, on this stream or another.  Errors: as
+ * sam_step, plus CUDA. */
 int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int32_t stride,
                   const int32_t* counts_host, int32_t L,
                   int32_t* draft_tokens_host, int32_t* draft_len_host, int32_t* match_len_host,

@@ -344,6 +344,7 @@ static SamStepIo step_io(const int32_t* new_tokens, int32_t stride, const int32_
                          int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status) {
     SamStepIo io{};
     io.new_tokens = new_tokens; io.stride = stride; io.counts = counts; io.L = L;
+    io.prompts = stride >= SAM_PREFILL_MIN;
     io.draft_tokens = draft_tokens; io.draft_len = draft_len; io.match_len = match_len; io.source = source; io.state = state; io.status = status;
     return io;
 }
@@ -371,6 +372,7 @@ extern "C" int sam_step_verified(sam_batch_t* b, const int32_t* target_tokens_de
     if (!prev_draft_tokens_dev || prev_L < 1 || prev_L > 128) return SAM_ERR_ARG;
     if (prev_draft_tokens_dev == draft_tokens_dev || prev_draft_len_dev == draft_len_dev) return SAM_ERR_ARG;
     SamStepIo io = step_io(target_tokens_dev, prev_L + 1, nullptr, L, draft_tokens_dev, draft_len_dev, match_len_dev, source_dev, state_dev, status_dev);
+    io.prompts = false;
     io.v_draft = prev_draft_tokens_dev; io.v_draft_len = prev_draft_len_dev; io.v_max_new = max_new_dev;
     io.v_counts_out = counts_out_dev; io.v_accepted_out = accepted_out_dev;
     return sam_launch_step(b, io, (cudaStream_t)stream);
@@ -417,6 +419,9 @@ extern "C" int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int
     int32_t* hst = b->host_stage;
     const size_t in_words = B * stride + B, out_words = B * L + 7 * B;
     const int32_t seq = ++b->host_seq == 0 ? ++b->host_seq : b->host_seq;
+    bool prompts = false;
+    for (size_t i = 0; i < B; i++) prompts |= counts_host[i] >= SAM_PREFILL_MIN;
+    const bool with_launch = !prompts && sam_step_is_inline(b, stride);
     // The waits below poll: the bytes are there sooner than a stream synchronisation returns.  They are bounded; past the
     // bound (other work queued ahead on the stream, or a failed launch) the stream is synchronised, after which
     // everything has to be there.
@@ -431,13 +436,14 @@ extern "C" int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int
         return SAM_OK;
     };
 
-    if (out_words <= SAM_TAGGED_MAX_WORDS) {
+    if (out_words <= SAM_TAGGED_MAX_WORDS && !prompts) {
         // Small steps: the rows and counts come with the launch, or are read by the kernel from the mapped staging area.  Each
-        // output word comes back with the step's number beside it, in one 8-byte store, so the kernel neither fences nor
-        // signals: a word whose number is the step's is there.
+        // output word comes back with the step's number beside it, in one 8-byte store, so no block waits for another or for its
+        // stores to host memory: a word whose number is the step's is there.  (A step with prompts takes two launches, and is
+        // done when the second is.)
         SamStepIo io = step_io(b->host_stage_dev, stride, b->host_stage_dev + B * stride, L, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
-        io.from_host = true; io.done_seq = seq; io.tagged = b->host_tagged_dev;
-        if (sam_step_is_inline(b, stride)) { io.inline_rows = new_tokens_host; io.inline_counts = counts_host; }
+        io.from_host = true; io.prompts = false; io.done_seq = seq; io.tagged = b->host_tagged_dev;
+        if (with_launch) { io.inline_rows = new_tokens_host; io.inline_counts = counts_host; }
         else {
             memcpy(hst, new_tokens_host, B * stride * 4);
             memcpy(hst + B * stride, counts_host, B * 4);
@@ -469,8 +475,8 @@ extern "C" int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int
     auto run = [&](const int32_t* rows, const int32_t* cnt, int32_t* d, int32_t* dl, int32_t* ml, int32_t* so, int32_t* st, int32_t* sta,
                    const int32_t* rows_host, const int32_t* cnt_host) -> int {
         SamStepIo io = step_io(rows, stride, cnt, L, d, dl, ml, so, st, sta);
-        io.from_host = true; io.done_flag = flag_dev; io.done_seq = seq;
-        if (sam_step_is_inline(b, stride)) { io.inline_rows = rows_host; io.inline_counts = cnt_host; }
+        io.from_host = true; io.prompts = prompts; io.done_flag = flag_dev; io.done_seq = seq;
+        if (with_launch) { io.inline_rows = rows_host; io.inline_counts = cnt_host; }
         else if (in_words >= SAM_FETCH_MIN_WORDS) {
             int r = sam_launch_fetch(b, rows, cnt, dev, stride, s);
             if (r) return r;
@@ -509,8 +515,9 @@ extern "C" int sam_step_host(sam_batch_t* b, const int32_t* new_tokens_host, int
     } else {
         SAM_CUDA(cudaMemcpyAsync(dev, hst, in_words * 4, cudaMemcpyHostToDevice, s));
         int32_t* o = dev + in_words;
-        rc = sam_launch_step(b, step_io(dev, stride, dev + B * stride, L, o, o + B * L, o + B * L + B, o + B * L + 3 * B,
-                                        o + B * L + 4 * B, o + B * L + 6 * B), s);
+        SamStepIo io = step_io(dev, stride, dev + B * stride, L, o, o + B * L, o + B * L + B, o + B * L + 3 * B, o + B * L + 4 * B, o + B * L + 6 * B);
+        io.prompts = prompts;
+        rc = sam_launch_step(b, io, s);
         if (rc) return rc;
         SAM_CUDA(cudaMemcpyAsync(ho, o, out_words * 4, cudaMemcpyDeviceToHost, s));
         SAM_CUDA(cudaStreamSynchronize(s));

@@ -54,9 +54,13 @@ struct SamDeviceGuard {
 
 static inline size_t sam_align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// From how many tokens an empty slot's row is a prompt, whose automaton is built at once (step.cu).
+constexpr int32_t SAM_PREFILL_MIN = 48;
+
 // What one step reads and writes (launchers in step.cu).
 struct SamStepIo {
     const int32_t* new_tokens; int32_t stride; const int32_t* counts; int32_t L;
+    bool prompts;                 // some counts may be SAM_PREFILL_MIN or more
     int32_t *draft_tokens, *draft_len, *match_len, *source, *state, *status;
     // sam_step_verified
     const int32_t *v_draft, *v_draft_len, *v_max_new;

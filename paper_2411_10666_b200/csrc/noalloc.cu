@@ -84,6 +84,7 @@ extern "C" int sam_retrieve_noalloc(const sam_static_t* st, int32_t vocab, int32
     if (rc) return rc;
     SamStepIo io{};
     io.new_tokens = tokens_dev; io.stride = stride; io.counts = counts_dev; io.L = L;
+    io.prompts = stride >= SAM_PREFILL_MIN;
     io.draft_tokens = draft_tokens_dev; io.draft_len = draft_len_dev; io.match_len = match_len_dev;
     io.source = source_dev; io.state = state_dev; io.status = status_dev;
     return sam_launch_step(&tmp, io, s);

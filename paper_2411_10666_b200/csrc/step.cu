@@ -942,6 +942,7 @@ __device__ __forceinline__ StepOut step_out(const StepArgs& A, int at) {
 
 __device__ __forceinline__ void write_failed_tagged(const StepArgs& A, int b, int lane, int status) {
     uint2* row = A.tagged + (size_t)b * (A.L + 7);
+    __threadfence();                                       // as in step_outputs
     for (int j = lane; j < A.L + 7; j += 32) row[j] = make_uint2(j < A.L ? 0xFFFFFFFFu : j == A.L + 6 ? (uint32_t)status : 0u, A.tag);
 }
 
@@ -1108,6 +1109,12 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
 
     if (A.tagged) {
         uint2* row = A.tagged + (size_t)b * (L + 7);
+        if (warp == 0) {
+            if (any_err && lane == 0) cb[CB_STATUS] = (uint32_t)any_err;
+            // The host takes the step for done when it has all words, of which some are this warp's: what the block has changed of
+            // the slot is there before them, for whatever stream the batch is used on next.
+            __threadfence();
+        }
         if (warp == winner) {
 #pragma unroll
             for (int r = 0; r < MAX_DRAFT_REGS; r++) {
@@ -1119,7 +1126,6 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
             const int v = lane == 0 ? (src == SAM_SRC_NONE ? 0 : sh_dl[winner]) : lane == 3 ? src : lane == 6 ? any_err : any_err ? 0 :
                           lane == 1 ? l1 : lane == 2 ? l2v : lane == 4 ? sh_s[0] : sh_s[1];
             if (lane < 7) row[L + lane] = make_uint2((uint32_t)v, A.tag);
-            if (any_err && lane == 0) cb[CB_STATUS] = (uint32_t)any_err;
         }
         return;
     }
@@ -1340,8 +1346,8 @@ __global__ void __launch_bounds__(128) fetch_inputs_kernel(const int32_t* rows, 
 //   batches that leave the GPU room, where the step waits for the slowest slot.  Otherwise the step kernel does all but
 //   the build, and the build's blocks, without the static side's registers, are resident five to an SM instead of three
 //   (4096 prompts of 1024 tokens).
-// From how many tokens: the build takes 14 us for its shortest texts, one Expand after the other 0.3 to 0.5 us a token.
-constexpr int SAM_PREFILL_MIN = 48;
+// From how many tokens (SAM_PREFILL_MIN): the build takes 14 us for its shortest texts, one Expand after the other 0.3 to 0.5
+// us a token.
 
 template <bool STATIC, int THREADS, int BLOCKS>
 __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __grid_constant__ StepArgs A) {
@@ -2323,7 +2329,7 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
     A.n_warp_blocks = A.n_lane_blocks = 0;
     bool prompts = false;
 #ifndef SAM_COUNTERS                                       // (the counters count Expand's own operations, one Expand at a time)
-    prompts = !verify && stride >= SAM_PREFILL_MIN;
+    prompts = io.prompts;
 #endif
     if (prompts) {
         cudaLaunchConfig_t pc;
@@ -2386,10 +2392,9 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
     return SAM_OK;
 }
 
-// Whether a host-array step's rows and counts can come with the launch.
+// Whether a host-array step's rows and counts, without prompts, can come with the launch.
 bool sam_step_is_inline(const sam_batch* b, int32_t stride) {
-    return stride < SAM_PREFILL_MIN && b->view.batch <= SAM_AHEAD_MAX_BATCH &&
-           (size_t)b->view.batch * (stride + 1) <= (size_t)SAM_INLINE_WORDS;
+    return b->view.batch <= SAM_AHEAD_MAX_BATCH && (size_t)b->view.batch * ((size_t)stride + 1) <= (size_t)SAM_INLINE_WORDS;
 }
 
 int sam_launch_fetch(const sam_batch* b, const int32_t* rows, const int32_t* counts, int32_t* to, int32_t stride, cudaStream_t stream) {

@@ -346,3 +346,39 @@ def test_host_arrays_are_the_callers_again_when_the_call_returns(P, B, K, L):
         for k, v in zip(KEYS, got):
             assert np.array_equal(v, getattr(ref, k)), (i, k)
     batch.close()
+
+
+@pytest.mark.parametrize("B,K,L", [(1, 8, 16), (16, 60, 16), (60, 16, 32), (64, 100, 50), (300, 12, 40), (1300, 8, 24)])
+def test_a_host_step_is_followed_by_work_on_another_stream(P, B, K, L):
+    """Nothing but the host call's return orders the stream of the next call behind it: device steps, dumps and resets there see
+    the batch as the host step left it, prompts (rows of 60 and 100) included."""
+    import torch
+    rng = np.random.default_rng(B)
+    vocab, rounds, msl = 12, 25, 400
+    corpus = rng.integers(0, vocab, size=4000, dtype=np.int32)
+    st, S = P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)
+    batch = P.Batch(st, B, msl, max_draft_len=L, max_host_stride=K)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    ob = oracle.Batch(S, corpus, B, vocab, msl)
+    out = [np.empty(s, dtype=np.int32) for s in ((B, L), (B,), (B, 2), (B,), (B, 2), (B,))]
+    dev = P.StepOutputs(B, L, "cuda")
+    torch.cuda.synchronize()
+    for i in range(rounds):
+        toks = rng.integers(0, vocab, size=(2, B, K), dtype=np.int32)
+        counts = np.stack([np.full(B, K if i % 3 == 0 else 3), rng.integers(0, 3, size=B)]).astype(np.int32)
+        d = [torch.from_numpy(x).cuda() for x in (toks[1], counts[1])]
+        torch.cuda.synchronize()
+        P.binding.sam_step_host(batch.handle, toks[0], K, counts[0], L, *out, stream=streams[0])
+        with torch.cuda.stream(streams[1]):
+            P.binding.sam_step(batch.handle, d[0], K, d[1], L, *dev.tensors(), stream=streams[1])
+            ref = ob.step(toks[0], counts[0], L, 4)
+            for k, v in zip(KEYS, out):
+                assert np.array_equal(v, getattr(ref, k)), (i, k)
+            ref = ob.step(toks[1], counts[1], L, 4)
+            streams[1].synchronize()
+        for k, v in dev.cpu().items():
+            assert np.array_equal(v, getattr(ref, k)), (i, k)
+        if i % 3 == 2:                                      # start over: the next host step brings prompts again
+            P.binding.sam_batch_reset(batch.handle, None, streams[0])
+            streams[0].synchronize()
+            ob = oracle.Batch(S, corpus, B, vocab, msl)
