@@ -57,6 +57,9 @@ static inline size_t sam_align_up(size_t x, size_t a) { return (x + a - 1) / a *
 // From how many tokens an empty slot's row is a prompt, whose automaton is built at once (step.cu).
 constexpr int32_t SAM_PREFILL_MIN = 48;
 
+// From how many slots a step's slots are ordered by their token counts: more than a B200 holds blocks of the step kernel (148 x 10).
+constexpr int32_t SAM_ORDER_MIN_BATCH = 1536;
+
 // What one step reads and writes (launchers in step.cu).
 struct SamStepIo {
     const int32_t* new_tokens; int32_t stride; const int32_t* counts; int32_t L;

@@ -71,13 +71,14 @@ enum {
     CB_S1FLAG, CB_BLK_CUR, CB_BLK_END, CB_NRECSLABS, CB_ROOTDEG,
     CB_ARRIVE,        // split step: how many of the slot's two sides have finished (parity: 2 per step)
     CB_NTOK_S,        // the text length as the static side keeps it (it may not read CB_NTOK while the dynamic side writes it)
-    CB_ERR_S,         // split step: error met by the static side (walk limit); SAM_STEP_DONE or SAM_STEP_BUILT between the
-                      // two launches of a step with prompts, for a slot the first of them has done or built; 0 otherwise
+    CB_ERR_S,         // split step: error met by the static side (walk limit)
     CB_SLABTAB = 16,  // .. 47
     CB_REC1 = 48,     // .. 55: copy of the static match state's record (valid when s1 != 0)
     CB_REC2 = 56      // .. 63: copy of the dynamic match state's record (valid when s2 != 0)
 };
 
+// What CB_STATUS says between the launches of a step with prompts, of a slot whose prompt has been done or built; it is 0 again
+// when the step has ended.
 #define SAM_STEP_DONE 0x80000000u
 #define SAM_STEP_BUILT 0x80000001u
 
@@ -150,6 +151,7 @@ struct SamBatchView {
     int32_t* slab_owner;      // [pool_slabs], -1 = free
     int32_t* reset_mark;      // [B]: number of the last reset that named the slot
     int32_t* order;           // [3][B] + 16: slots sorted by their step's token count (large batches), two buffers in turn; the sort keys; per buffer, at 3B + 8 x buffer, the number of slots with many tokens
+    int32_t* prompts;         // [B] + 2, batches that are ordered: the slots with prompts in the step to come, how many, and how many have been taken
     int32_t* text;            // [B][text_stride]
     uint32_t* pstate;         // [B][text_stride]: id of the state created by each text position
     uint2* root_tab;          // [B][root_cap]

@@ -105,6 +105,9 @@ struct StepArgs {
     // side of 32 slots each, the remaining blocks the dynamic side of one slot each
     int32_t n_warp_blocks, n_lane_blocks;
     const int32_t* split_count;
+    // optional: the *n_prompts slots that sam_prefill_kernel is to look at (order_slots_kernel), and behind that number how many of
+    // them, beyond one for each of its blocks, have been taken; without it, all slots
+    const int32_t* prompts; int32_t* n_prompts;
 };
 
 // ------------------------------------------------------------------ draft read
@@ -1213,20 +1216,22 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
     if (AHEAD && warp == 2) {
         // A host-array step's caller goes on before this kernel has ended, but not before this warp's reads have: of the caller's
         // arrays, which kernels may read in place, and of the batch's memory.
-        if (status == 0 && m <= A.stride && __shfl_sync(FULL, cw, CB_ERR_S) == 0) read_ahead(A.W, b, lane, cw, cw2, tok_first, m, host);
+        if (status == 0 && m <= A.stride) read_ahead(A.W, b, lane, cw, cw2, tok_first, m, host);
         else if (host) ahead_join((uint32_t)tok_first, 0, 0);
         return;
     }
     step_sync();              // both warps hold the slot's state as it was before either writes any of it
 
-    // what sam_prefill_kernel, launched before this one, has done of the slot
-    const uint32_t done = __shfl_sync(FULL, cw, CB_ERR_S);
-    const bool built = done == SAM_STEP_BUILT;
-    if (done != 0 && threadIdx.x == 0) cb[CB_ERR_S] = 0;
-    if (done == SAM_STEP_DONE) {
-        if (host) step_join(false);
-        if (threadIdx.x == 0 && A.done_flag) signal_done(A);
-        return;
+    // what sam_prefill_kernel, launched before this one where a step may have prompts, has done of the slot
+    const bool built = !VERIFY && !INLINE && (uint32_t)status == SAM_STEP_BUILT;
+    if (!VERIFY && !INLINE && status < 0) {
+        if (threadIdx.x == 0) cb[CB_STATUS] = 0;
+        if ((uint32_t)status == SAM_STEP_DONE) {
+            if (host) step_join(false);
+            if (threadIdx.x == 0 && A.done_flag) signal_done(A);
+            return;
+        }
+        status = 0;
     }
 
     // validate the whole step before any state changes (both warps reach the same verdict)
@@ -1340,14 +1345,77 @@ __global__ void __launch_bounds__(128) fetch_inputs_kernel(const int32_t* rows, 
 
 // ------------------------------------------------------------------ prompts
 // Launched ahead of the step kernel when the step's rows are long enough to hold prompts.  An empty slot that is given
-// SAM_PREFILL_MIN tokens or more has its automaton built here (prefill_build.cuh), one block per slot; a word of the
-// control block tells the step kernel, which follows and does the rest of the slots.
-//   STATIC: warp 0 finds the slot's static match meanwhile, and the slot is done here, outputs included: for
-//   batches that leave the GPU room, where the step waits for the slowest slot.  Otherwise the step kernel does all but
-//   the build, and the build's blocks, without the static side's registers, are resident five to an SM instead of three
-//   (4096 prompts of 1024 tokens).
+// SAM_PREFILL_MIN tokens or more has its automaton built here (prefill_build.cuh); the slot's status tells the step kernel,
+// which follows and does the rest of the slots.
+//   STATIC: a block per slot.  Warp 0 finds the slot's static match meanwhile, and the slot is done here, outputs included: for
+//   batches that leave the GPU room, where the step waits for the slowest slot.
+//   Otherwise the step kernel does all but the build, and the build's blocks, without the static side's registers, are resident
+//   five to an SM instead of three (4096 prompts of 1024 tokens).  There are as many blocks as are resident at once, and they share
+//   out the slots with prompts: those that order_slots_kernel has listed, or, in batches that are not ordered, what they find in the counts.
+//   (A block per slot costs an ordinary step of 1000 slots with rows of 8192 tokens 3 us.)
 // From how many tokens (SAM_PREFILL_MIN): the build takes 14 us for its shortest texts, one Expand after the other 0.3 to 0.5
 // us a token.
+__device__ __forceinline__ bool is_prompt(const StepArgs& A, int m) {
+    return m >= SAM_PREFILL_MIN && m <= A.stride && m <= PB_MAX && m <= A.W.max_seq_len;
+}
+// The prompt's tokens to shared memory and to the slot's text (the text of an empty slot is nobody's); whether all of them are
+// in the vocabulary (if not, the step kernel reports it).  Run by the whole block.
+__device__ __forceinline__ bool load_prompt(const StepArgs& A, int b, int m, uint32_t* tok) {
+    const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
+    int32_t* text = A.W.text + (size_t)b * A.W.text_stride;
+    const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
+    bool bad = false;
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+        const int t = toks[j];
+        tok[j] = (uint32_t)t; text[j] = t;
+        bad |= t < 0 || t >= vocab;
+    }
+    return !__syncthreads_or(bad);
+}
+// Which prompts a block builds, one after the other, kept by its first thread in shared memory:
+//   - those that order_slots_kernel has listed: the blockIdx.x-th, then whichever is next;
+//   - in batches that are not ordered, those among every gridDim.x-th slot (with 740 blocks, at most three), or,
+//   - where rows are so wide that only few blocks are resident, every gridDim.x-th of those that a look at all counts finds.
+constexpr int PROMPT_SHARE = 128;                          // (more than 18944 slots, not ordered: the others' prompts go token by token)
+struct PromptTake { int32_t share[PROMPT_SHARE]; int turn, found, slot; };
+template <bool LOOK>
+__device__ __forceinline__ void prompts_begin(const StepArgs& A, PromptTake& T) {
+    if (threadIdx.x == 0) T.turn = T.found = 0;
+    if (!LOOK || A.prompts) return;
+    const int B = A.W.batch, lane = threadIdx.x & 31;
+    bool any = false;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < B; i += blockDim.x) any |= is_prompt(A, A.counts[i]);
+    if (!__syncthreads_or(any) || threadIdx.x >= 32) return;
+    int rank = 0, mine = 0;
+#pragma unroll 4
+    for (int base = 0; base < B; base += 32) {
+        const bool is = base + lane < B && is_prompt(A, A.counts[base + lane]);
+        const unsigned mask = __ballot_sync(FULL, is);
+        const int r = rank + __popc(mask & ((1u << lane) - 1u)), k = r / (int)gridDim.x;
+        if (is && r % (int)gridDim.x == (int)blockIdx.x && k < PROMPT_SHARE) { T.share[k] = base + lane; mine = k + 1; }
+        rank += __popc(mask);
+    }
+    mine = __reduce_max_sync(FULL, mine);
+    if (lane == 0) T.found = mine;
+    __syncwarp();
+}
+// The next one's slot, -1 if there is none; by the first thread.
+template <bool LOOK>
+__device__ __forceinline__ int prompts_next(const StepArgs& A, PromptTake& T) {
+    if (A.prompts) {
+        int at = blockIdx.x;
+        if (T.turn++ > 0) at = (int)gridDim.x + atomicAdd(A.n_prompts + 1, 1);
+        return at < *A.n_prompts ? A.prompts[at] : -1;
+    }
+    if constexpr (LOOK) return T.turn < T.found ? T.share[T.turn++] : -1;
+    else
+        for (;;) {
+            const int b = (int)blockIdx.x + T.turn++ * (int)gridDim.x;
+            if (b >= A.W.batch) return -1;
+            if (is_prompt(A, A.counts[b])) return b;
+        }
+}
 
 template <bool STATIC, int THREADS, int BLOCKS>
 __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __grid_constant__ StepArgs A) {
@@ -1355,34 +1423,38 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
     asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(16) unsigned char pb_smem[];
     __shared__ PbShared sh;
-    __shared__ int32_t sh_l[2], sh_s[2], sh_dl[2], sh_err[2];
-    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
-    const int m = A.counts[b];
-    const uint32_t cw = cb[lane];
-    if (m < SAM_PREFILL_MIN || m > A.stride || m > PB_MAX || m > A.W.max_seq_len) return;
-    if (__shfl_sync(FULL, cw, CB_STATUS) != 0 || __shfl_sync(FULL, cw, CB_NTOK) != 0) return;
-    const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
-    const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
-    bool bad = false;
-    uint32_t* tok = pb_arrays(pb_smem, pb_size(m)).tok;
-    int32_t* text = A.W.text + (size_t)b * A.W.text_stride;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        const int t = toks[j];
-        tok[j] = (uint32_t)t; text[j] = t;               // (the text of an empty slot is nobody's)
-        bad |= t < 0 || t >= vocab;
-    }
-    if (__syncthreads_or(bad)) return;                   // the step kernel reports it
-
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (!STATIC) {
-        PbResult r;
-        pb_build(A.W, b, cb, m, pb_smem, sh, (int)threadIdx.x, (int)blockDim.x, r);
-        if (threadIdx.x == 0) {
-            if (r.err) cb[CB_STATUS] = (uint32_t)r.err;
-            cb[CB_ERR_S] = SAM_STEP_BUILT;
+        constexpr bool LOOK = THREADS > 256;
+        __shared__ PromptTake take;
+        prompts_begin<LOOK>(A, take);
+        for (;;) {
+            if (threadIdx.x == 0) take.slot = prompts_next<LOOK>(A, take);
+            __syncthreads();
+            if (take.slot < 0) break;
+            {
+                const int b = take.slot, m = A.counts[b];
+                uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
+                if (is_prompt(A, m) && cb[CB_STATUS] == 0 && cb[CB_NTOK] == 0 && load_prompt(A, b, m, pb_arrays(pb_smem, pb_size(m)).tok)) {
+                    PbResult r;
+                    pb_build(A.W, b, cb, m, pb_smem, sh, (int)threadIdx.x, (int)blockDim.x, r);
+                    if (threadIdx.x == 0) A.W.ctrl[(size_t)take.slot * SAM_CTRL_WORDS + CB_STATUS] = r.err ? (uint32_t)r.err : SAM_STEP_BUILT;
+                }
+            }
+            __syncthreads();
         }
         return;
     }
+    __shared__ int32_t sh_l[2], sh_s[2], sh_dl[2], sh_err[2];
+    const int b = blockIdx.x;
+    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
+    const int m = A.counts[b];
+    const uint32_t cw = cb[lane];
+    if (!is_prompt(A, m)) return;
+    if (__shfl_sync(FULL, cw, CB_STATUS) != 0 || __shfl_sync(FULL, cw, CB_NTOK) != 0) return;
+    const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
+    const int32_t* text = A.W.text + (size_t)b * A.W.text_stride;
+    if (!load_prompt(A, b, m, pb_arrays(pb_smem, pb_size(m)).tok)) return;
     int32_t d[MAX_DRAFT_REGS] = {-1, -1, -1, -1};
     int32_t my_l = 0, my_s = 0, my_dl = 0;
     int err = 0;
@@ -1407,7 +1479,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
     asm volatile("bar.sync 2, 64;" ::: "memory");
     step_outputs<false>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, true, d, m, 0);
-    if (threadIdx.x == 0) cb[CB_ERR_S] = SAM_STEP_DONE;
+    if (threadIdx.x == 0 && sh_err[0] == 0 && sh_err[1] == 0) cb[CB_STATUS] = SAM_STEP_DONE;     // (a failed slot is reported again)
 }
 
 // ------------------------------------------------------------------ the split step (large batches)
@@ -1461,7 +1533,9 @@ __device__ __forceinline__ bool arrive_warp(uint32_t* cb, int lane) {
 __device__ __forceinline__ void split_epilogue(const StepArgs& A, int b, int lane) {
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const uint32_t cw = __ldcg(cb + lane), cw2 = __ldcg(cb + 32 + lane);
-    if (__shfl_sync(FULL, cw, CB_STATUS) != 0) return;                  // reported by the dynamic side
+    const uint32_t status = __shfl_sync(FULL, cw, CB_STATUS);
+    if (status == SAM_STEP_BUILT) { if (lane == 0) cb[CB_STATUS] = 0; } // (both sides have seen it)
+    else if (status != 0) return;                                       // reported by the dynamic side
     const int err_s = (int)__shfl_sync(FULL, cw, CB_ERR_S);
     const StepOut o = step_out(A, 0);
     if (err_s) {
@@ -1492,7 +1566,12 @@ __device__ __forceinline__ void split_epilogue_lanes(const StepArgs& A, bool sec
         const uint32_t st = __ldcg(cb + CB_STATUS);
         l2 = (int)__ldcg(cb + CB_L2); s2 = (int)__ldcg(cb + CB_S2);
         const int64_t ntok = (int64_t)__ldcg(cb + CB_NTOK), e2 = (int64_t)__ldcg(cb + CB_REC2 + 2);
-        if (st != 0) mine = false;                                       // reported by the dynamic side
+        if (st == SAM_STEP_BUILT) {                                      // both sides are the other warp's
+            l1 = (int)__ldcg(cb + CB_L1); s1 = (int)__ldcg(cb + CB_S1); e1 = (int64_t)__ldcg(cb + CB_REC1 + 2);
+            err_s = (int)__ldcg(cb + CB_ERR_S);
+            cb[CB_STATUS] = 0;
+        }
+        if (st != 0 && st != SAM_STEP_BUILT) mine = false;               // reported by the dynamic side
         else if (err_s) { status = err_s; l1 = l2 = 0; s1 = s2 = 0; cb[CB_STATUS] = (uint32_t)err_s; }
         else {
             const bool use_static = l1 > l2 + A.W.l_bias;               // Section 3.2
@@ -1665,8 +1744,10 @@ __device__ __forceinline__ void static_lanes(const StepArgs& A, int w, int lane)
     split_epilogue_lanes(A, second, b, lane, l, (int32_t)s, e1, err);
 }
 
-// The dynamic side of one slot (one warp), including everything that reports a slot as failed.
-__device__ __forceinline__ void dynamic_slot(const StepArgs& A, int b, int lane, uint32_t (*sh_run)[12]) {
+// The dynamic side of one slot (one warp), including everything that reports a slot as failed.  Of a slot whose prompt
+// has been built it does the static side as well (true: nothing else is left of its own side), for which the lanes of
+// static_lanes would be slow; the static side's blocks see the slot's status and only count themselves.
+__device__ __forceinline__ bool dynamic_slot(const StepArgs& A, int b, int lane, uint32_t (*sh_run)[12]) {
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
     const uint32_t cw = cb[lane];
@@ -1675,6 +1756,7 @@ __device__ __forceinline__ void dynamic_slot(const StepArgs& A, int b, int lane,
     if (lane < A.stride) tok_first = toks[lane];
     const int m = A.counts[b];
     int status = (int)__shfl_sync(FULL, cw, CB_STATUS);
+    if ((uint32_t)status == SAM_STEP_BUILT) return true;
     const uint32_t ntok0 = __shfl_sync(FULL, cw, CB_NTOK);
     bool fresh_fail = false;
     if (status == 0) {                                   // validate the whole step before any state changes
@@ -1703,13 +1785,14 @@ __device__ __forceinline__ void dynamic_slot(const StepArgs& A, int b, int lane,
         if (fresh_fail && lane == 0) cb[CB_STATUS] = (uint32_t)status;
         write_failed_slot(step_out(A, 0), A.L, b, lane, status);
         arrive_warp(cb, lane);
-        return;
+        return false;
     }
     if (arrive_warp(cb, lane)) split_epilogue(A, b, lane);
+    return false;
 }
 
-// The static side of one slot with a warp of its own.
-__device__ __forceinline__ void static_slot(const StepArgs& A, int b, int lane) {
+// The static side of one slot with a warp of its own.  built: of a slot whose prompt has been built and checked.
+__device__ __forceinline__ void static_slot(const StepArgs& A, int b, int lane, bool built) {
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const int32_t* toks = A.new_tokens + (size_t)b * A.stride;
     const uint32_t cw = cb[lane];
@@ -1718,8 +1801,8 @@ __device__ __forceinline__ void static_slot(const StepArgs& A, int b, int lane) 
     if (lane < A.stride) tok_first = toks[lane];
     const int m = A.counts[b];
     const uint32_t ntok_s = __shfl_sync(FULL, cw, CB_NTOK_S);
-    bool run = __shfl_sync(FULL, cw, CB_STATUS) == 0 && m >= 0 && m <= A.stride && (int64_t)ntok_s + m <= A.W.max_seq_len;
-    if (run) {                                           // the dynamic side reports a refused step; this side only keeps out
+    bool run = __shfl_sync(FULL, cw, CB_STATUS) == (built ? SAM_STEP_BUILT : 0u) && m >= 0 && m <= A.stride && (int64_t)ntok_s + m <= A.W.max_seq_len;
+    if (run && !built) {                                 // the dynamic side reports a refused step; this side only keeps out
         bool bad = false;
         for (int base = 0; base < m; base += 32) {
             const int i = base + lane;
@@ -1755,19 +1838,22 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
     asm volatile("griddepcontrol.launch_dependents;");
     __shared__ __align__(16) uint32_t sh_run[32][12];   // per-token staging of a repeat run (dynamic side)
     const int lane = threadIdx.x;
-    int i = (int)blockIdx.x;
-    if (i < A.n_warp_blocks + A.n_lane_blocks) {
+    const int i = (int)blockIdx.x;
+    int b = -1;                                          // the slot whose static side this warp does
+    bool built = false;
+    if (i < A.n_warp_blocks) {
         // slots whose static side gets a warp: the first n_big of the sorted order (read together with order[])
-        if (i < A.n_warp_blocks) {
-            const int b = A.order[i];
-            if (i < min(*A.split_count, A.n_warp_blocks)) static_slot(A, b, lane);
-        } else {
-            static_lanes(A, i - A.n_warp_blocks, lane);
-        }
+        const int ob = A.order[i];
+        if (i < min(*A.split_count, A.n_warp_blocks)) b = ob;
+    } else if (i < A.n_warp_blocks + A.n_lane_blocks) {
+        static_lanes(A, i - A.n_warp_blocks, lane);
     } else {
         // the dynamic side's time hardly depends on the token count: slots in their own order, one read less
-        dynamic_slot(A, i - A.n_warp_blocks - A.n_lane_blocks, lane, sh_run);
+        const int db = i - A.n_warp_blocks - A.n_lane_blocks;
+        built = dynamic_slot(A, db, lane, sh_run);
+        if (built) b = db;
     }
+    if (b >= 0) static_slot(A, b, lane, built);
 }
 
 // ------------------------------------------------------------------ many steps in one launch
@@ -2187,7 +2273,7 @@ constexpr int SAM_ORDER_THREADS = 1024;
 // memory, because kernels that want different ones do not share an SM.)
 template <bool SPLIT>
 __global__ void __launch_bounds__(SAM_ORDER_THREADS) order_slots_kernel(const int32_t* counts, int32_t B, int32_t* order,
-                                                                        int32_t* keys, int32_t big_m, int32_t* n_big) {
+                                                                        int32_t* keys, int32_t big_m, int32_t* n_big, int32_t* prompts) {
     asm volatile("griddepcontrol.launch_dependents;");
     __shared__ int hist[SAM_ORDER_KEYS];
     const int lane = threadIdx.x & 31;
@@ -2244,6 +2330,30 @@ __global__ void __launch_bounds__(SAM_ORDER_THREADS) order_slots_kernel(const in
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!prompts) return;
+    // Now the counts are final: the slots with prompts, for sam_prefill_kernel, which looks at nothing else.
+    __shared__ int n;
+    if (threadIdx.x == 0) n = 0;
+    __syncthreads();
+    for (int base = 0; base < B; base += U * SAM_ORDER_THREADS) {
+        int m[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int i = base + u * SAM_ORDER_THREADS + (int)threadIdx.x;
+            m[u] = i < B ? __ldcg(counts + i) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const unsigned mask = __ballot_sync(FULL, m[u] >= SAM_PREFILL_MIN);
+            if (!mask) continue;
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&n, __popc(mask));
+            at = __shfl_sync(FULL, at, 0);
+            if (m[u] >= SAM_PREFILL_MIN) prompts[at + __popc(mask & lt)] = base + u * SAM_ORDER_THREADS + (int)threadIdx.x;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) { prompts[B] = n; prompts[B + 1] = 0; }
 }
 
 // From how many tokens on a slot's static side gets a warp of its own in the split step.  A lane's chain costs
@@ -2258,7 +2368,6 @@ int split_kernel_setup(int device);
 constexpr int SAM_SPLIT_MIN_BATCH = 8192;                    // the split step is used from this many slots on
 constexpr int SAM_SMS = 148;
 constexpr int SAM_AHEAD_MAX_BATCH = SAM_SMS * 8;             // three warps a slot, all slots resident at once
-constexpr int SAM_ORDER_MIN_BATCH = 1536;                    // more slots than a B200 holds blocks of this kernel (148 x 10)
 
 }  // namespace
 
@@ -2286,16 +2395,18 @@ int launch_prefill(const StepArgs& A, int batch, int device, cudaLaunchConfig_t*
                                sam_prefill_kernel<false, 1024, 1>};
     int n2 = 64;
     while (n2 < A.stride && n2 < PB_MAX) n2 <<= 1;
-    int k = 0, threads = 32 + (n2 / 2 < 64 ? 64 : n2 / 2 > 992 ? 992 : n2 / 2);
-    if (batch > 296) {
+    int k = 0, threads = 32 + (n2 / 2 < 64 ? 64 : n2 / 2 > 992 ? 992 : n2 / 2), blocks = batch;
+    if (batch > 2 * SAM_SMS) {
         k = n2 <= 1024 ? 1 : n2 <= 2048 ? 2 : 3;
-        threads = n2 / 4 < 64 ? 64 : n2 / 4 > 1024 ? 1024 : n2 / 4;
+        threads = n2 / 4 < 128 ? 128 : n2 / 4 > 1024 ? 1024 : n2 / 4;
+        const int resident = SAM_SMS * (k == 1 ? (threads < 256 ? 10 : 5) : k == 2 ? 3 : 1);
+        if (blocks > resident) blocks = resident;
     }
     if (device < 0 || device >= SAM_MAX_DEVICES) return SAM_ERR_ARG;
     cudaError_t e = (cudaError_t)g_prefill_setup[k](device, [&]() -> int {
         return (int)cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, PB_MAX * PB_BYTES_PER_TOKEN);
     });
-    cfg->gridDim = dim3((unsigned)batch); cfg->blockDim = dim3((unsigned)threads); cfg->dynamicSmemBytes = (size_t)n2 * PB_BYTES_PER_TOKEN;
+    cfg->gridDim = dim3((unsigned)blocks); cfg->blockDim = dim3((unsigned)threads); cfg->dynamicSmemBytes = (size_t)n2 * PB_BYTES_PER_TOKEN;
     if (e == cudaSuccess) e = cudaLaunchKernelEx(cfg, kernels[k], A);
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;
@@ -2325,38 +2436,40 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    A.order = nullptr; A.split_count = nullptr;
+    A.order = nullptr; A.split_count = nullptr; A.prompts = A.n_prompts = nullptr;
     A.n_warp_blocks = A.n_lane_blocks = 0;
     bool prompts = false;
 #ifndef SAM_COUNTERS                                       // (the counters count Expand's own operations, one Expand at a time)
     prompts = io.prompts;
 #endif
+    // (A host-array step is synchronous: nothing runs before it that the ordering kernel could overlap with, so it
+    // would cost more than the order saves; such a step is always the one two-warp launch, slots in their own order.)
+    if (!verify && !io.from_host && b->view.batch >= SAM_ORDER_MIN_BATCH) {
+        int32_t* order = b->view.order + (size_t)(b->order_phase & 1) * b->view.batch;
+        cudaLaunchConfig_t oc;
+        memset(&oc, 0, sizeof(oc));
+        oc.gridDim = dim3(1); oc.blockDim = dim3(SAM_ORDER_THREADS); oc.stream = stream; oc.attrs = attr; oc.numAttrs = 1;
+        int32_t* n_big = b->view.order + 3 * (size_t)b->view.batch + 8 * (b->order_phase & 1);
+        int32_t* list = prompts ? b->view.prompts : nullptr;
+        if (list) { A.prompts = list; A.n_prompts = list + b->view.batch; }
+        const bool split = A.has_static && b->view.batch >= SAM_SPLIT_MIN_BATCH;
+        if (split) { int rc = split_kernel_setup(b->device); if (rc) return rc; }
+        cudaError_t oe = split
+            ? cudaLaunchKernelEx(&oc, order_slots_kernel<true>, counts, (int32_t)b->view.batch, order,
+                                 b->view.order + 2 * (size_t)b->view.batch, split_big_m(b->view.batch), n_big, list)
+            : cudaLaunchKernelEx(&oc, order_slots_kernel<false>, counts, (int32_t)b->view.batch, order,
+                                 b->view.order + 2 * (size_t)b->view.batch, split_big_m(b->view.batch), n_big, list);
+        A.split_count = n_big;
+        b->order_phase ^= 1;
+        if (oe != cudaSuccess) { sam_set_cuda_error(oe); return SAM_ERR_CUDA; }
+        A.order = order;
+    }
     if (prompts) {
         cudaLaunchConfig_t pc;
         memset(&pc, 0, sizeof(pc));
         pc.stream = stream; pc.attrs = attr; pc.numAttrs = 1;
         int rc = launch_prefill(A, b->view.batch, b->device, &pc);
         if (rc) return rc;
-    }
-    // (A host-array step is synchronous: nothing runs before it that the ordering kernel could overlap with, so it
-    // would cost more than the order saves; such a step is always the one two-warp launch, slots in their own order.)
-    if (!verify && !prompts && !io.from_host && b->view.batch >= SAM_ORDER_MIN_BATCH) {
-        int32_t* order = b->view.order + (size_t)(b->order_phase & 1) * b->view.batch;
-        cudaLaunchConfig_t oc;
-        memset(&oc, 0, sizeof(oc));
-        oc.gridDim = dim3(1); oc.blockDim = dim3(SAM_ORDER_THREADS); oc.stream = stream; oc.attrs = attr; oc.numAttrs = 1;
-        int32_t* n_big = b->view.order + 3 * (size_t)b->view.batch + 8 * (b->order_phase & 1);
-        const bool split = A.has_static && b->view.batch >= SAM_SPLIT_MIN_BATCH;
-        if (split) { int rc = split_kernel_setup(b->device); if (rc) return rc; }
-        cudaError_t oe = split
-            ? cudaLaunchKernelEx(&oc, order_slots_kernel<true>, counts, (int32_t)b->view.batch, order,
-                                 b->view.order + 2 * (size_t)b->view.batch, split_big_m(b->view.batch), n_big)
-            : cudaLaunchKernelEx(&oc, order_slots_kernel<false>, counts, (int32_t)b->view.batch, order,
-                                 b->view.order + 2 * (size_t)b->view.batch, split_big_m(b->view.batch), n_big);
-        A.split_count = n_big;
-        b->order_phase ^= 1;
-        if (oe != cudaSuccess) { sam_set_cuda_error(oe); return SAM_ERR_CUDA; }
-        A.order = order;
     }
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));

@@ -51,6 +51,7 @@ def _text(kind, n, rng, corpus):
     return x
 
 
+KEYS = ("draft_tokens", "draft_len", "match_len", "source", "state", "status")
 KINDS = ("distinct", "one", "periodic", "fibonacci", "corpus", "two", "few", "many", "copies")
 
 
@@ -216,15 +217,16 @@ def test_prompts_beside_others_the_pool_cannot_hold(P, B):
     for b in fits:
         rows[b] = rng.permutation(vocab)[:n]                # one state a token, no edge blocks
     toks, counts = torch.from_numpy(rows).cuda(), torch.full((B,), n, dtype=torch.int32, device="cuda")
+    counts[list(fits)] = n // 2
 
     def takes(b):
         one = P.Batch(None, 1, n, max_draft_len=L, vocab=vocab, slab_bytes=4096)
-        assert one.step(toks[b:b + 1], counts[:1], L).cpu()["status"][0] == 0
+        assert one.step(toks[b:b + 1], counts[b:b + 1], L).cpu()["status"][0] == 0
         total, free = one.pool_info()
         return total - free
 
     pool = sum(takes(b) for b in fits)
-    assert all(takes(b) > pool for b in (0, 1, B // 2, B - 1))
+    assert pool == 2 * (n // 2 * 32 // 4096 + 1) and min(takes(b) for b in (0, 1, B // 2, B - 1)) >= pool + 6    # (they differ by one or two)
     for turn in range(30):
         batch = P.Batch(None, B, n, max_draft_len=L, vocab=vocab, slab_bytes=4096, pool_slabs=pool)
         status = batch.step(toks, counts, L).cpu()["status"]
@@ -260,3 +262,82 @@ def test_as_many_prompts_as_the_pool_holds(P, B):
         batch.reset()
         assert batch.pool_info() == (holds * takes + takes - 1,) * 2
         batch.close()
+
+
+@pytest.mark.parametrize("B,static", [(7, True), (296, True), (297, True), (297, False), (1300, True), (1700, False), (8300, True)])
+@pytest.mark.parametrize("wide", [48, 129, 300])
+def test_wide_rows_with_and_without_prompts(P, B, static, wide):
+    """A server that keeps one row width: steps whose rows could hold prompts and do not, steps where a few slots change hands,
+    refused rows among both, narrow rows and several steps in one call in between.  Every output of every step, and the
+    automata at the end, at the edges of the kernels' ranges."""
+    import torch
+    rng = np.random.default_rng(B * 1000 + wide)
+    vocab, L, msl = 50, 9, 900
+    corpus = rng.integers(0, vocab, size=6000, dtype=np.int32)
+    corpus[2000:3000] = corpus[:1000]
+    st, S = (P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)) if static else (None, None)
+    ob = oracle.Batch(S, corpus if static else None, B, vocab, msl, 1, 2, 5)
+    batch = P.Batch(st, B, msl, max_draft_len=L, l_bias=1, min_match=2, vocab=vocab, stop_token=5)
+
+    def rows(width, counts):
+        t = rng.integers(0, vocab, size=(B, width), dtype=np.int32)
+        for b in np.flatnonzero(counts > 20):               # passages of the corpus, and repeats
+            k = rng.integers(0, 5000)
+            t[b, 10:20] = corpus[k:k + 10]
+            if width > 60:
+                t[b, 45:60] = t[b, 20:35]
+        return t
+
+    def compare(toks, counts, got):
+        ref = ob.step(toks, counts, L, 8)
+        for k in KEYS:
+            assert np.array_equal(got[k], getattr(ref, k)), (k, np.argwhere(got[k] != getattr(ref, k))[:3])
+
+    def step(toks, counts):
+        compare(toks, counts, batch.step(torch.from_numpy(toks).cuda(), torch.from_numpy(counts).cuda(), L).cpu())
+
+    few = lambda: rng.integers(0, 7, size=B).astype(np.int32)
+    counts = np.where(rng.random(B) < 0.8, rng.integers(48, wide + 1, size=B), few()).astype(np.int32)
+    toks = rows(wide, counts)
+    counts[1], counts[2], toks[3, 20] = wide + 1, -1, vocab       # refused: too many, fewer than none, a token out of range
+    counts[3] = wide
+    step(toks, counts)
+    for i in range(3):                                      # no prompts, rows that could hold them
+        c = few()
+        step(rows(wide, c), c)
+    c = few()
+    step(rows(16, c), c)
+    gone = np.unique(rng.integers(0, B, size=max(2, B // 20))).astype(np.int32)
+    batch.reset(gone)
+    for b in gone:
+        ob.reset(b)
+    c = few()
+    c[gone] = rng.integers(40, wide + 1, size=len(gone))
+    toks = rows(wide, c)
+    toks[gone[0], 30], c[gone[0]] = -4, wide                # a new slot's prompt is refused
+    step(toks, c)
+    many = np.stack([few() for _ in range(3)])
+    toks = np.stack([rows(wide, c) for c in many])
+    out = batch.run_steps(torch.from_numpy(toks).cuda(), torch.from_numpy(many).cuda(), L).cpu()
+    for i in range(3):
+        compare(toks[i], many[i], {k: out[k][i] for k in KEYS})
+    ok = [b for b in list(range(0, B, max(1, B // 6))) + gone.tolist()[1:3] if out["status"][-1][b] == 0]
+    assert_dynamic_automata_equal(batch, ob, ok, msl)
+
+
+def test_host_steps_with_prompts_in_a_batch_that_lists_them(P):
+    """Host arrays, more than two slots an SM: the completion flag is the last launch's, with prompts in every, in some and in no
+    row of a wide step."""
+    rng = np.random.default_rng(3)
+    vocab, B, W, L, msl = 30, 400, 90, 7, 500
+    corpus = rng.integers(0, vocab, size=4000, dtype=np.int32)
+    st, S = P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)
+    ob, batch = oracle.Batch(S, corpus, B, vocab, msl), P.Batch(st, B, msl, max_draft_len=L, max_host_stride=W)
+    out = [np.empty(s, dtype=np.int32) for s in ((B, L), (B,), (B, 2), (B,), (B, 2), (B,))]
+    for i, share in enumerate((0.5, 0.0, 0.5, 0.0, 1.0)):
+        toks = rng.integers(0, vocab, size=(B, W), dtype=np.int32)
+        counts = np.where(rng.random(B) < share, rng.integers(48, W + 1, size=B), rng.integers(0, 5, size=B)).astype(np.int32)
+        ref = ob.step(toks, counts, L, 8)
+        P.binding.sam_step_host(batch.handle, toks, W, counts, L, *out)
+        for k, v in zip(KEYS, out):
+            assert np.array_equal(v, getattr(ref, k)), (i, k)
