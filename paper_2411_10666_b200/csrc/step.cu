@@ -1098,7 +1098,8 @@ __device__ __forceinline__ void read_ahead(const SamBatchView& W, int b, int lan
 }
 
 // Both warps' results are in shared memory: choose the source, write the slot's outputs.  Not failed: both errors are 0.
-template <bool VERIFY>
+// PAIRS: to the host, each with the step's number beside it, where A.tagged says so.
+template <bool VERIFY, bool PAIRS>
 __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp, int lane, uint32_t* cb, const int32_t* sh_l, const int32_t* sh_s,
                                              const int32_t* sh_dl, const int32_t* sh_err, bool failed, const int32_t d[MAX_DRAFT_REGS], int m, int confirmed) {
     const int L = A.L;
@@ -1110,7 +1111,7 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
     const int src = (any_err || lsel < need) ? SAM_SRC_NONE : (use_static ? SAM_SRC_STATIC : SAM_SRC_DYNAMIC);
     const int winner = src == SAM_SRC_DYNAMIC ? 1 : 0;
 
-    if (A.tagged) {
+    if (PAIRS && A.tagged) {
         uint2* row = A.tagged + (size_t)b * (L + 7);
         if (warp == 0) {
             if (any_err && lane == 0) cb[CB_STATUS] = (uint32_t)any_err;
@@ -1254,14 +1255,14 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
         if (host) step_join(false);
         if (warp == 0) {
             if (fresh_fail && lane == 0) cb[CB_STATUS] = (uint32_t)status;
-            if (A.tagged) write_failed_tagged(A, b, lane, status);
+            if (AHEAD && !VERIFY && A.tagged) write_failed_tagged(A, b, lane, status);
             else write_failed_slot(step_out(A, 0), L, b, lane, status);
             if (lane == 0) {
                 if (VERIFY && A.v_counts_out) A.v_counts_out[b] = m;
                 if (VERIFY && A.v_accepted_out) A.v_accepted_out[b] = confirmed;
             }
             __syncwarp();
-            if (A.done_flag && lane == 0) signal_done(A);
+            if (!VERIFY && A.done_flag && lane == 0) signal_done(A);
         }
         return;
     }
@@ -1299,7 +1300,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
     bool failed = true;
     if (AHEAD && !VERIFY && A.tagged) failed = step_join(err != 0); else step_sync();
-    step_outputs<VERIFY>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, failed, d, m, confirmed);
+    step_outputs<VERIFY, AHEAD && !VERIFY>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, failed, d, m, confirmed);
     if (!VERIFY && A.done_flag) {
         if (AHEAD) step_join(false); else step_sync();
         if (threadIdx.x == 0) signal_done(A);
@@ -1478,7 +1479,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
     }
     if (lane == 0) { sh_l[warp] = my_l; sh_s[warp] = my_s; sh_dl[warp] = my_dl; sh_err[warp] = err; }
     asm volatile("bar.sync 2, 64;" ::: "memory");
-    step_outputs<false>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, true, d, m, 0);
+    step_outputs<false, false>(A, b, warp, lane, cb, sh_l, sh_s, sh_dl, sh_err, true, d, m, 0);
     if (threadIdx.x == 0 && sh_err[0] == 0 && sh_err[1] == 0) cb[CB_STATUS] = SAM_STEP_DONE;     // (a failed slot is reported again)
 }
 
