@@ -13,9 +13,12 @@
 //     automaton's `path` says; the state it ends in is then an ordinary entry whose candidates are read when it is popped.
 //   - The entries with the largest probability are popped together as long as they are paths: each goes back to the end
 //     of the line with the same probability, so they take turns, and lane t writes the t-th node of up to 32 with one read
-//     of the corpus.
-// 64 slots of 40 nodes, k = 4: 18 to 31 us from seed to seed (32 to 34 with one pop and one round of reads for each node), 4096
-// slots of 100 nodes 90 us (315).  Bound by the pops that are left, one after the other, 1 us each.
+//     of the corpus, which the pops after it do not wait for.  Who else has the probability of the first in line is only looked
+//     up where that is a path: an entry that is none costs one look through the queue, as if there were no paths.
+// us, seeds of 64 slots with k = 4 (one pop and one round of reads for each node): 8 nodes 11.7, 7.8, 8.1 (10.4), 20 nodes 24.2,
+// 11.6, 12.6 (18.6 to 20.6), 40 nodes 26.4, 15.8, 15.8 (33 to 35); 4096 slots: 8 nodes 12.2 (14.5), 100 nodes 74 (316).  Bound by the
+// pops that are not paths, one after the other, 0.7 to 1.2 us each; a call is as long as its slowest tree, and a tree whose paths
+// are all one or two tokens long (24.2) gains nothing by them.
 // Probabilities are IEEE float32: quotient freq(child) / freq(state) rounded first,
 // then the product with the parent's probability.
 #include "common.h"
@@ -103,43 +106,46 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
         __syncwarp();
         int qn = 1;
         uint32_t seq = 1;
+        int32_t late_tok = 0; int late_at = -1;             // a token of the corpus on its way, and the node it is for: the pops after do not wait
         while (n_out < M) {
-            uint32_t best = 0;
-            for (int i = lane; i < qn; i += 32) best = max(best, q_key[i]);
+            // the most probable entry, of equal ones the one pushed first
+            uint32_t best = 0, first = 0xFFFFFFFFu;
+            int at = 0, ties = 0;
+            for (int i = lane; i < qn; i += 32) {
+                const uint32_t k = q_key[i], sq = q_seq[i];
+                if (k > best) { best = k; first = sq; at = i; ties = 1; }
+                else if (k == best) { ties++; if (sq < first) { first = sq; at = i; } }
+            }
             const uint32_t key = __reduce_max_sync(FULL, best);
             if (key == 0) break;                            // queue empty
             const float p = __uint_as_float(key - 1u);
-            int group = 0;
-            for (int base = 0; base < qn; base += 32) {
-                const bool in = base + lane < qn && q_key[base + lane] == key;
-                const unsigned mask = __ballot_sync(FULL, in);
-                const int g = group + __popc(mask & lt);
-                if (in && g < 32) top[g] = base + lane;
-                group += __popc(mask);
-            }
-            __syncwarp();
-            int at = 0, paths = 0;                          // the entry to pop; the paths at the head of the line
-            if (group <= 32) {
-                int e = 0, rank = 32;
-                uint32_t sq = 0xFFFFFFFFu;
-                if (lane < group) { e = top[lane]; sq = q_seq[e]; }
-                if (group > 1) {
-                    rank = 0;
+            const uint32_t front = __reduce_min_sync(FULL, best == key ? first : 0xFFFFFFFFu);
+            at = __shfl_sync(FULL, at, __ffs(__ballot_sync(FULL, best == key && first == front)) - 1);
+            const uint32_t nn = q_n[at];
+            int group = 1, paths = 0;                       // entries as probable as it; the paths at the head of their line
+            if (nn & ENTRY_PATH) {
+                group = __reduce_add_sync(FULL, best == key ? ties : 0);
+                if (group == 1 || group > 32) {             // (more are too many to sort: the first alone)
+                    paths = 1;
+                    if (lane == 0) turn[0] = at;
+                    __syncwarp();
+                } else {
+                    int found = 0;
+                    for (int base = 0; base < qn; base += 32) {
+                        const bool in = base + lane < qn && q_key[base + lane] == key;
+                        const unsigned mask = __ballot_sync(FULL, in);
+                        if (in) top[found + __popc(mask & lt)] = base + lane;
+                        found += __popc(mask);
+                    }
+                    __syncwarp();
+                    int e = 0, rank = 0;
+                    uint32_t sq = 0xFFFFFFFFu;
+                    if (lane < group) { e = top[lane]; sq = q_seq[e]; }
                     for (int g = 0; g < group; g++) rank += __shfl_sync(FULL, sq, g) < sq;
                     if (lane < group) turn[rank] = e;
-                } else if (lane == 0) { rank = 0; turn[0] = e; }
-                paths = (int)__reduce_min_sync(FULL, lane < group && !(q_n[e] & ENTRY_PATH) ? (uint32_t)rank : (uint32_t)group);
-                __syncwarp();
-                at = turn[0];
-            } else {                                        // (too many to sort: the earliest push)
-                uint32_t first = 0xFFFFFFFFu;
-                for (int i = lane; i < qn; i += 32) if (q_key[i] == key) first = min(first, q_seq[i]);
-                first = __reduce_min_sync(FULL, first);
-                for (int base = 0; base < qn; base += 32) {
-                    const unsigned m = __ballot_sync(FULL, base + lane < qn && q_key[base + lane] == key && q_seq[base + lane] == first);
-                    if (m) { at = base + __ffs(m) - 1; break; }
+                    paths = (int)__reduce_min_sync(FULL, lane < group && !(q_n[e] & ENTRY_PATH) ? (uint32_t)rank : (uint32_t)group);
+                    __syncwarp();
                 }
-                if (q_n[at] & ENTRY_PATH) { paths = 1; if (lane == 0) turn[0] = at; __syncwarp(); }
             }
             if (paths > 0) {
                 // lane t: the t-th pop.  Where other entries stand in line behind the paths, each path is popped once.
@@ -150,8 +156,10 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
                 count = min(count, M - n_out);
                 const int until = room * paths + r;         // the first pop this path cannot serve
                 count = (int)__reduce_min_sync(FULL, (uint32_t)(lane < paths ? min(until, count) : count));
+                if (late_at >= 0) out_tok[late_at] = late_tok;
+                late_at = -1;
                 if (lane < count) {
-                    out_tok[n_out + lane] = __ldg(A.S.corpus + q_tok[e] + i);
+                    late_tok = __ldg(A.S.corpus + q_tok[e] + i); late_at = n_out + lane;
                     out_par[n_out + lane] = i == 0 ? q_par[e] : n_out + lane - paths;
                     if (out_p) out_p[n_out + lane] = p;
                 }
@@ -159,10 +167,10 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
                 if (lane < paths && lane < count) {         // lane r: path r, popped `c` times
                     const int c = (count - lane + paths - 1) / paths, last = lane + (c - 1) * paths;
                     q_tok[e] += (uint32_t)c; q_par[e] = n_out + last; q_seq[e] = seq + (uint32_t)last;
-                    const uint32_t nn = q_n[e] - ((uint32_t)c << PATH_LEFT);
-                    q_n[e] = nn;
-                    if ((nn >> PATH_LEFT) == 0) {
-                        if (nn & ENTRY_ENDS) q_key[e] = 0;
+                    const uint32_t left = q_n[e] - ((uint32_t)c << PATH_LEFT);
+                    q_n[e] = left;
+                    if ((left >> PATH_LEFT) == 0) {
+                        if (left & ENTRY_ENDS) q_key[e] = 0;
                         else q_n[e] = ENTRY_LATE;
                     }
                 }
@@ -171,9 +179,12 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
                 continue;
             }
             const int node = n_out++;
-            const uint32_t nn = q_n[at], fs = q_freq[at], tok = q_tok[at];
+            const uint32_t fs = q_freq[at], tok = q_tok[at];
             if (lane == 0) {
-                out_tok[node] = nn & ENTRY_LATE ? __ldg(A.S.corpus + tok) : (int32_t)tok;
+                if (nn & ENTRY_LATE) {
+                    if (late_at >= 0) out_tok[late_at] = late_tok;
+                    late_tok = __ldg(A.S.corpus + tok); late_at = node;
+                } else out_tok[node] = (int32_t)tok;
                 out_par[node] = q_par[at];
                 if (out_p) out_p[node] = p;
                 q_key[at] = 0;
@@ -235,6 +246,7 @@ __global__ void __launch_bounds__(32) tree_draft_kernel(const __grid_constant__ 
             qn += keep; seq += (uint32_t)keep;
             __syncwarp();
         }
+        if (late_at >= 0) out_tok[late_at] = late_tok;
     }
     if (lane == 0) A.sizes[b] = n_out;
     for (int j = n_out + lane; j < M; j += 32) { out_tok[j] = -1; out_par[j] = -1; if (out_p) out_p[j] = 0.f; }

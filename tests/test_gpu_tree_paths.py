@@ -33,3 +33,24 @@ def test_paths_of_every_length(P, length, tmp_path):  # noqa: F811
     for st in (built, P.StaticSam.load(str(tmp_path / "image"))):
         for max_size, k in ((128, 4), (40, 2), (33, 1), (5, 4)):
             _check(P, S, f, st, states, starts, max_size, k)
+
+
+@pytest.mark.parametrize("fan", [(1, 1), (2, 3), (5, 6), (6, 6)])
+@pytest.mark.parametrize("repeats", [1, 2, 3])
+def test_many_equally_probable_entries(P, fan, repeats):  # noqa: F811
+    """Up to 36 entries of one probability in the queue: paths of several lengths, states with a choice after one token, and
+    both in one line, in the order in which they were pushed."""
+    rng = random.Random(fan[0] * 10 + fan[1] + repeats)
+    x, s = [], 5000
+    for i in range(fan[0]):
+        for j in range(fan[1]):
+            tail = [rng.randrange(100, 5000) for _ in range((i + j) % 5)]
+            for _ in range(repeats):
+                x += [s, 10 + i, 30 + j] + tail + [rng.randrange(100, 5000), 6000 + len(x) % 900]
+    x = np.array(x, dtype=np.int32)
+    S = oracle.Sam(x)
+    st = P.StaticSam.build(x, 8000, tree_topk=6)
+    states = [S.edges(0)[s]] * 2 + [rng.randrange(1, S.n_states) for _ in range(30)]
+    starts = [rng.randrange(8000) for _ in states]
+    for max_size, k in ((128, 6), (50, 5), (9, 6), (2, 1)):
+        _check(P, S, S.freq(), st, states, starts, max_size, k)
