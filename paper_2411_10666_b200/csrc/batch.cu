@@ -11,12 +11,12 @@
 namespace {
 
 constexpr size_t SAM_ZERO_COPY_MAX_BYTES = 4u << 20;     // larger host steps go through two DMA copies
-// Outputs of a host step that come back as (word, number) pairs: no fence and no flag, twice the bytes.  With the rows in the
-// launch's arguments, 16 slots take 13.9 us a call instead of 18.5, 64 slots (1472 words) 15.3 instead of 19.8, 64 slots
-// of 47 words 21.0 instead of 24.6; from there on the bytes cost more.
-constexpr size_t SAM_TAGGED_MAX_WORDS = 4096;
-// From how many words of rows on a kernel brings them over ahead of the step's: 250 slots (3250 words) take 28.7 us without
-// and 30.6 with it, 1000 slots (13000) 39.2 without and 36.5 with it, 4000 slots 76 and 68.
+// Outputs of a host step that come back as (word, number) pairs: a fence a slot and no flag, twice the bytes.  us a call as
+// pairs / behind the flag: 16 slots (368 words) 15.3 to 16.9 / 16.7 to 17.2, 43 slots (2021 words) 17.9 / 17.9, 44 (2068) 18.0 /
+// 17.7, 64 slots of 47 words (3008) 19.5 / 18.5, 87 (4089) 20.5 / 18.8.
+constexpr size_t SAM_TAGGED_MAX_WORDS = 2048;
+// From how many words of rows on a kernel brings them over ahead of the step's, us a call without / with it: 200 slots (1800
+// words) 22.0 / 25.0, 300 (2700) 23.7 / 24.0, 500 (6500) 25.9 / 26.0, 620 (8060) 27.3 / 26.4; 1000 (13000) 39.2 / 36.5.
 constexpr size_t SAM_FETCH_MIN_WORDS = 8192;
 constexpr size_t SAM_DIRECT_MIN_BYTES = 64u << 10;       // from this size on, page-locked caller arrays are used in place
 constexpr int SAM_POLL_LIMIT_US = 2000;                  // how long a host step polls its completion flag

@@ -1,6 +1,6 @@
 // The hot kernel: one decoding step of SAM-Decoding's draft retrieval for a batch of sequences.
 //
-// One block of two warps per sequence slot.  Warp 0 advances the slot's match state through the
+// One block per sequence slot, of two warps and, up to 1184 slots, a third that reads ahead of them.  Warp 0 advances the slot's match state through the
 // STATIC automaton (Transfer, Algorithm 1) for each accepted token; warp 1 extends the slot's own
 // DYNAMIC automaton (Expand, Algorithm 3) with the same tokens and keeps its match state, which
 // after each Expand is link[last] with length len[link[last]] (the state Transfer would reach on
@@ -994,7 +994,7 @@ __device__ __forceinline__ void write_slot(const StepArgs& A, const StepOut& o, 
 // it 520 cycles, an edge block 810).  The dynamic side changes these structures meanwhile, so what is read here may be of
 // any age; it is used for addresses only, each checked against the pool, and for no result.
 // The same reads made by the dynamic side itself, before its first token, cost what they saved; following the match
-// state's suffix links as well gave nothing.  Per step: 4 slots 6.2 -> 5.5 us, 64 slots 6.0 -> 5.5, 1000 slots 22.1 -> 20.8, 256
+// state's suffix links as well gave nothing.  Per step: 4 slots 6.2 -> 5.5 us, 64 slots 6.0 -> 5.5, 1000 slots 18.5 -> 17.0, 256
 // slots fed by verified drafts 26.2 -> 21.5.
 struct Ahead {
     const unsigned char* pool;
@@ -1154,9 +1154,9 @@ __device__ __forceinline__ void step_outputs(const StepArgs& A, int b, int warp,
 }
 
 // ------------------------------------------------------------------ the kernel
-// VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
 // The two warps that work on the slot.
 __device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+// VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
 // AHEAD: a third warp reads ahead of the dynamic side (read_ahead).
 // INLINE: the rows and counts came with the launch (sam_step_host).
 template <bool VERIFY, bool AHEAD, bool INLINE>
@@ -1308,7 +1308,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
 }
 
 // AHEAD: blocks of three warps an SM has to hold, 0 for blocks of two.  Registers come in quarters of an SM: 5 blocks (740
-// slots) have 120 a thread and spill nothing, 6 (888) have 96, 8 (1184) have 80 and spill 330 bytes.  Prompt-copying
+// slots) have 120 a thread and spill nothing, 6 (888) have 96, 8 (1184) have 80 and spill 188 bytes.  Prompt-copying
 // slots, us a step with 5 / 6 / 8 blocks: 740 slots 14.6 / 15.0 / -, 880 slots - / 15.5 / 16.4, 1000 slots (in two
 // waves: 20.5 / 18.5) 17.0, 1180 slots with two warps a slot 19.2, with three 17.4.
 template <bool VERIFY, int AHEAD>
@@ -1492,7 +1492,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sam_prefill_kernel(const __gr
 //     record, a hash bucket eight 16-byte entries), so one LANE carries it: a warp advances 32 slots, each
 //     round of reads serving 32 chains (static_lanes);
 //   - the static side of a slot with many tokens is what a step waits for, so it keeps a warp of its own
-//     and everything that shortens the chain (static_chain: read-ahead lookups, prefix states).
+//     and everything that shortens the chain (static_chain: suffixes side by side, prefix states).
 // The slots come sorted by token count (order_slots_kernel), which also says how many of them have "many".
 // Neither side waits for the other.  Each writes its result to the slot's control block and then counts
 // itself in CB_ARRIVE; the side that finds the other already counted (an odd count) reads both results,
@@ -1918,8 +1918,8 @@ __device__ __forceinline__ void static_close(uint32_t* cb, int lane, uint32_t nt
 //   - The dynamic side has a warp per slot, without the static side's registers and waits (sam_run_split_kernel).
 //   - Both leave each step's result in the step's own outputs, and sam_run_finish_kernel, which no chain waits for, chooses the
 //     sources and reads the drafts: 32 rows a warp, eight rows' reads under way together.
-// Per step (a warp for both sides of a slot, before): 1000 slots 18.5 -> 8.3 us, 4096 slots 16.2 -> 7.9, 16384 slots
-// 58 -> 21.4.  Bound by the static chains up to 4096 slots (5 us a step), by the dynamic side's warps beyond.
+// Per step (a warp for both sides of a slot, before): 1000 slots 18.5 -> 7.3 us, 4096 slots 16.2 -> 7.2, 16384 slots
+// 58 -> 20.3.  Bound by the static chains up to 4096 slots (5 us a step), by the dynamic side's warps beyond.
 // What the two sides leave: match_len, state and status as they will be; the static side's first end position (or minus its
 // error) in draft_len, the dynamic side's in source, the text length in the first word of the draft.
 
@@ -2444,7 +2444,7 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
     prompts = io.prompts;
 #endif
     // (A host-array step is synchronous: nothing runs before it that the ordering kernel could overlap with, so it
-    // would cost more than the order saves; such a step is always the one two-warp launch, slots in their own order.)
+    // would cost more than the order saves; its slots are in their own order.)
     if (!verify && !io.from_host && b->view.batch >= SAM_ORDER_MIN_BATCH) {
         int32_t* order = b->view.order + (size_t)(b->order_phase & 1) * b->view.batch;
         cudaLaunchConfig_t oc;

@@ -341,3 +341,9 @@ def test_host_steps_with_prompts_in_a_batch_that_lists_them(P):
         P.binding.sam_step_host(batch.handle, toks, W, counts, L, *out)
         for k, v in zip(KEYS, out):
             assert np.array_equal(v, getattr(ref, k)), (i, k)
+
+
+@pytest.mark.parametrize("B,stride,L", [(43, 8, 40), (44, 8, 40), (127, 100, 9), (128, 3, 9), (129, 3, 9)])
+def test_host_steps_at_the_edge_of_the_pairs(P, B, stride, L):
+    """Outputs of at most 2048 words come back as pairs, more behind the completion flag; rows of 100 tokens hold prompts."""
+    test_host_steps_of_every_size(P, B, stride, L)
