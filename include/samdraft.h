@@ -237,7 +237,9 @@ int sam_batch_pool_info(sam_batch_t* b, int64_t* total_slabs, int64_t* free_slab
  * holds at once (a small kernel first orders the slots so that those with the most tokens start first; the
  * step's results do not depend on it).  sam_step_host, being synchronous, gains nothing from the order and
  * never makes that launch; with many rows it makes another that brings them to the device.  A step
- * whose rows can hold a prompt (stride of 48 and more) makes two: prompts that fill an empty slot, then the rest.
+ * whose rows can hold a prompt (stride of 48 and more; in sam_step_host a count of 48 and more) makes one more,
+ * for prompts that fill an empty slot; where there is none it costs 1 to 4 us (a step of 64 slots 6.9 -> 8.2,
+ * of 4096 32.3 -> 35.8).
  * Returns a negative sam_err_t for a null handle. */
 int sam_batch_launches_per_step(const sam_batch_t* b);
 

@@ -22,7 +22,7 @@ constexpr size_t SAM_DIRECT_MIN_BYTES = 64u << 10;       // from this size on, p
 constexpr int SAM_POLL_LIMIT_US = 2000;                  // how long a host step polls its completion flag
 
 struct WsLayout {
-    size_t off_hdr, off_ctrl, off_free, off_owner, off_reset, off_order, off_prompts, off_text, off_pstate, off_root, off_stage, off_pool, total;
+    size_t off_hdr, off_ctrl, off_free, off_owner, off_reset, off_order, off_text, off_pstate, off_root, off_stage, off_pool, total;
     int32_t text_stride, root_cap, slab_shift, pool_slabs, max_host_stride;
     size_t stage_words;
 };
@@ -61,9 +61,10 @@ int plan(const sam_batch_opts_t* o, WsLayout* w) {
     w->off_free = off;  off = sam_align_up(off + (size_t)slabs * 4, 256);
     w->off_owner = off; off = sam_align_up(off + (size_t)slabs * 4, 256);
     w->off_reset = off; off = sam_align_up(off + (size_t)o->batch * 4, 256);
-    w->off_order = off; off = sam_align_up(off + (size_t)o->batch * 4 * 3 + 64, 256);   // two order buffers, the sort keys, two counts
-    w->off_prompts = off;
-    if (o->batch >= SAM_ORDER_MIN_BATCH) off = sam_align_up(off + ((size_t)o->batch + 2) * 4, 256);
+    // two order buffers, the sort keys, two counts; the list of prompts
+    w->off_order = off; off += ((size_t)o->batch * 3 + SAM_ORDER_WORDS) * 4;
+    if (o->batch >= SAM_ORDER_MIN_BATCH) off += ((size_t)o->batch + 2) * 4;
+    off = sam_align_up(off, 256);
     w->off_text = off;  off = sam_align_up(off + (size_t)o->batch * w->text_stride * 4, 256);
     w->off_pstate = off; off = sam_align_up(off + (size_t)o->batch * w->text_stride * 4, 256);
     w->off_root = off;  off = sam_align_up(off + (size_t)o->batch * w->root_cap * 8, 256);
@@ -205,7 +206,6 @@ int sam_plan_view(const sam_batch_opts_t* opts, int32_t vocab, void* base, SamBa
         view->slab_owner = (int32_t*)(b + w.off_owner);
         view->reset_mark = (int32_t*)(b + w.off_reset);
         view->order = (int32_t*)(b + w.off_order);
-        view->prompts = (int32_t*)(b + w.off_prompts);
         view->text = (int32_t*)(b + w.off_text);
         view->pstate = (uint32_t*)(b + w.off_pstate);
         view->root_tab = (uint2*)(b + w.off_root);
@@ -271,7 +271,6 @@ extern "C" int sam_batch_create(const sam_static_t* st, const sam_batch_opts_t* 
     V.slab_owner = (int32_t*)(base + w.off_owner);
     V.reset_mark = (int32_t*)(base + w.off_reset);
     V.order = (int32_t*)(base + w.off_order);
-    V.prompts = (int32_t*)(base + w.off_prompts);
     V.text = (int32_t*)(base + w.off_text);
     V.pstate = (uint32_t*)(base + w.off_pstate);
     V.root_tab = (uint2*)(base + w.off_root);

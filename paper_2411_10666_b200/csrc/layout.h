@@ -77,6 +77,8 @@ enum {
     CB_REC2 = 56      // .. 63: copy of the dynamic match state's record (valid when s2 != 0)
 };
 
+#define SAM_ORDER_WORDS 16         // words behind the slot orders and the sort keys
+
 // What CB_STATUS says between the launches of a step with prompts, of a slot whose prompt has been done or built; it is 0 again
 // when the step has ended.
 #define SAM_STEP_DONE 0x80000000u
@@ -150,8 +152,7 @@ struct SamBatchView {
     int32_t* free_stack;      // [pool_slabs]
     int32_t* slab_owner;      // [pool_slabs], -1 = free
     int32_t* reset_mark;      // [B]: number of the last reset that named the slot
-    int32_t* order;           // [3][B] + 16: slots sorted by their step's token count (large batches), two buffers in turn; the sort keys; per buffer, at 3B + 8 x buffer, the number of slots with many tokens
-    int32_t* prompts;         // [B] + 2, batches that are ordered: the slots with prompts in the step to come, how many, and how many have been taken
+    int32_t* order;           // [3][B] + 16: slots sorted by their step's token count (large batches), two buffers in turn; the sort keys; per buffer, at 3B + 8 x buffer, the number of slots with many tokens; in batches that are ordered, behind them [2 + B]: prompts listed, taken, their slots
     int32_t* text;            // [B][text_stride]
     uint32_t* pstate;         // [B][text_stride]: id of the state created by each text position
     uint2* root_tab;          // [B][root_cap]

@@ -105,9 +105,6 @@ struct StepArgs {
     // side of 32 slots each, the remaining blocks the dynamic side of one slot each
     int32_t n_warp_blocks, n_lane_blocks;
     const int32_t* split_count;
-    // optional: the *n_prompts slots that sam_prefill_kernel is to look at (order_slots_kernel), and behind that number how many of
-    // them, beyond one for each of its blocks, have been taken; without it, all slots
-    const int32_t* prompts; int32_t* n_prompts;
 };
 
 // ------------------------------------------------------------------ draft read
@@ -1373,6 +1370,9 @@ __device__ __forceinline__ bool load_prompt(const StepArgs& A, int b, int m, uin
     }
     return !__syncthreads_or(bad);
 }
+// The list of prompts of a batch that is ordered: how many, how many have been taken beyond one for each block, the slots.
+__host__ __device__ __forceinline__ int32_t* prompt_list(const SamBatchView& W) { return W.order + 3 * (size_t)W.batch + SAM_ORDER_WORDS; }
+
 // Which prompts a block builds, one after the other, kept by its first thread in shared memory:
 //   - those that order_slots_kernel has listed: the blockIdx.x-th, then whichever is next;
 //   - in batches that are not ordered, those among every gridDim.x-th slot (with 740 blocks, at most three), or,
@@ -1382,7 +1382,7 @@ struct PromptTake { int32_t share[PROMPT_SHARE]; int turn, found, slot; };
 template <bool LOOK>
 __device__ __forceinline__ void prompts_begin(const StepArgs& A, PromptTake& T) {
     if (threadIdx.x == 0) T.turn = T.found = 0;
-    if (!LOOK || A.prompts) return;
+    if (!LOOK || A.order) return;
     const int B = A.W.batch, lane = threadIdx.x & 31;
     bool any = false;
 #pragma unroll 4
@@ -1404,10 +1404,11 @@ __device__ __forceinline__ void prompts_begin(const StepArgs& A, PromptTake& T) 
 // The next one's slot, -1 if there is none; by the first thread.
 template <bool LOOK>
 __device__ __forceinline__ int prompts_next(const StepArgs& A, PromptTake& T) {
-    if (A.prompts) {
+    if (A.order) {
+        int32_t* list = prompt_list(A.W);
         int at = blockIdx.x;
-        if (T.turn++ > 0) at = (int)gridDim.x + atomicAdd(A.n_prompts + 1, 1);
-        return at < *A.n_prompts ? A.prompts[at] : -1;
+        if (T.turn++ > 0) at = (int)gridDim.x + atomicAdd(list + 1, 1);
+        return at < list[0] ? list[2 + at] : -1;
     }
     if constexpr (LOOK) return T.turn < T.found ? T.share[T.turn++] : -1;
     else
@@ -2274,7 +2275,7 @@ constexpr int SAM_ORDER_THREADS = 1024;
 // memory, because kernels that want different ones do not share an SM.)
 template <bool SPLIT>
 __global__ void __launch_bounds__(SAM_ORDER_THREADS) order_slots_kernel(const int32_t* counts, int32_t B, int32_t* order,
-                                                                        int32_t* keys, int32_t big_m, int32_t* n_big, int32_t* prompts) {
+                                                                        int32_t* keys, int32_t big_m, int32_t* n_big, int32_t* list) {
     asm volatile("griddepcontrol.launch_dependents;");
     __shared__ int hist[SAM_ORDER_KEYS];
     const int lane = threadIdx.x & 31;
@@ -2331,7 +2332,7 @@ __global__ void __launch_bounds__(SAM_ORDER_THREADS) order_slots_kernel(const in
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!prompts) return;
+    if (!list) return;
     // Now the counts are final: the slots with prompts, for sam_prefill_kernel, which looks at nothing else.
     __shared__ int n;
     if (threadIdx.x == 0) n = 0;
@@ -2350,11 +2351,11 @@ __global__ void __launch_bounds__(SAM_ORDER_THREADS) order_slots_kernel(const in
             int at = 0;
             if (lane == 0) at = atomicAdd(&n, __popc(mask));
             at = __shfl_sync(FULL, at, 0);
-            if (m[u] >= SAM_PREFILL_MIN) prompts[at + __popc(mask & lt)] = base + u * SAM_ORDER_THREADS + (int)threadIdx.x;
+            if (m[u] >= SAM_PREFILL_MIN) list[2 + at + __popc(mask & lt)] = base + u * SAM_ORDER_THREADS + (int)threadIdx.x;
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) { prompts[B] = n; prompts[B + 1] = 0; }
+    if (threadIdx.x == 0) { list[0] = n; list[1] = 0; }
 }
 
 // From how many tokens on a slot's static side gets a warp of its own in the split step.  A lane's chain costs
@@ -2437,7 +2438,7 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    A.order = nullptr; A.split_count = nullptr; A.prompts = A.n_prompts = nullptr;
+    A.order = nullptr; A.split_count = nullptr;
     A.n_warp_blocks = A.n_lane_blocks = 0;
     bool prompts = false;
 #ifndef SAM_COUNTERS                                       // (the counters count Expand's own operations, one Expand at a time)
@@ -2451,8 +2452,7 @@ int sam_launch_step(const sam_batch* b, const SamStepIo& io, cudaStream_t stream
         memset(&oc, 0, sizeof(oc));
         oc.gridDim = dim3(1); oc.blockDim = dim3(SAM_ORDER_THREADS); oc.stream = stream; oc.attrs = attr; oc.numAttrs = 1;
         int32_t* n_big = b->view.order + 3 * (size_t)b->view.batch + 8 * (b->order_phase & 1);
-        int32_t* list = prompts ? b->view.prompts : nullptr;
-        if (list) { A.prompts = list; A.n_prompts = list + b->view.batch; }
+        int32_t* list = prompts ? prompt_list(b->view) : nullptr;
         const bool split = A.has_static && b->view.batch >= SAM_SPLIT_MIN_BATCH;
         if (split) { int rc = split_kernel_setup(b->device); if (rc) return rc; }
         cudaError_t oe = split

@@ -347,3 +347,41 @@ def test_host_steps_with_prompts_in_a_batch_that_lists_them(P):
 def test_host_steps_at_the_edge_of_the_pairs(P, B, stride, L):
     """Outputs of at most 2048 words come back as pairs, more behind the completion flag; rows of 100 tokens hold prompts."""
     test_host_steps_of_every_size(P, B, stride, L)
+
+
+@pytest.mark.parametrize("B", [64, 400, 1700, 8200])
+def test_steps_with_prompts_replayed_from_a_graph(P, B):
+    """A reset, a step with prompts and two wide steps without, captured once and replayed on other inputs: nothing of one pass
+    (marks, the list of prompts, which buffer holds the order) is left over for the next."""
+    import torch
+    rng = np.random.default_rng(B)
+    vocab, W, L, msl = 40, 70, 8, 200
+    corpus = rng.integers(0, vocab, size=4000, dtype=np.int32)
+    st, S = P.StaticSam.build(corpus, vocab), oracle.Sam(corpus)
+    batch = P.Batch(st, B, msl, max_draft_len=L)
+    toks = torch.zeros(3, B, W, dtype=torch.int32, device="cuda")
+    counts = torch.zeros(3, B, dtype=torch.int32, device="cuda")
+    outs = [P.StepOutputs(B, L, "cuda") for _ in range(3)]
+
+    def one_pass():
+        batch.reset()
+        for i in range(3):
+            batch.step(toks[i], counts[i], L, outs[i])
+
+    one_pass()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        one_pass()
+    for share in (0.5, 0.0, 1.0, 0.1):
+        t = rng.integers(0, vocab, size=(3, B, W), dtype=np.int32)
+        c = rng.integers(0, 6, size=(3, B)).astype(np.int32)
+        c[0] = np.where(rng.random(B) < share, rng.integers(48, W + 1, size=B), c[0])
+        toks.copy_(torch.from_numpy(t)); counts.copy_(torch.from_numpy(c))
+        graph.replay()
+        torch.cuda.synchronize()
+        ob = oracle.Batch(S, corpus, B, vocab, msl)
+        for i in range(3):
+            ref = ob.step(t[i], c[i], L, 8)
+            for k, v in outs[i].cpu().items():
+                assert np.array_equal(v, getattr(ref, k)), (share, i, k)
