@@ -19,7 +19,9 @@
 // Nothing here depends on a guess: each of these statements is the definition of the automaton of the text.
 //
 // What bounds it: for short texts the chain of some 50 barriers, for long ones one SM's shared memory (everything but the
-// outputs stays there, 28 bytes per token).
+// outputs stays there, 28 bytes per token), and a step waits for its slowest build.  Walking the suffix links' chains with one
+// read a link, and the longest of them by whole warps (pb_walk), took the slowest of 64 x 1024 tokens from 70 us to 47, of
+// 256 x 1024 from 110 to 53.
 #pragma once
 #include "common.h"
 
@@ -41,12 +43,13 @@ struct PbShared {                          // what the threads of one build exch
 struct PbArrays {
     uint64_t* key; uint16_t* lev; uint16_t* A; uint16_t* B; uint32_t* tok;      // while sorting
     uint32_t* tree; uint16_t* rank; uint16_t* canon; uint16_t* enode; uint16_t* parent;
-    uint32_t* first; uint16_t* wnode; uint16_t* idc; uint16_t* link; uint32_t* deg; uint16_t* clen;
+    uint32_t* first; uint16_t* wnode; uint16_t* idc; uint16_t* link; uint16_t* llen; uint32_t* deg; uint16_t* clen;
     int N2;                                // size of the sorted order, a power of two
 };
 
-// `tree`: leaves in its upper half.  When they are no longer needed, `link` takes the place of its inner nodes and `clen`,
-// the clones' lengths, that of `rank`.
+// `tree`: leaves in its upper half.  When they are no longer needed, `link` takes the place of its inner nodes, `deg` that of its
+// leaves, `llen` (the lengths of the states that `link` names) that of the tokens, and `clen` (of each position the length of
+// `wnode`'s interval, for a position that clones the clone's) that of `rank`.
 __device__ __forceinline__ PbArrays pb_arrays(unsigned char* sm, int N2) {
     PbArrays a;
     const size_t n = (size_t)N2;
@@ -55,7 +58,7 @@ __device__ __forceinline__ PbArrays pb_arrays(unsigned char* sm, int N2) {
     a.tok = (uint32_t*)(sm + 24 * n);
     a.tree = (uint32_t*)sm; a.link = (uint16_t*)sm; a.rank = (uint16_t*)(sm + 8 * n); a.canon = (uint16_t*)(sm + 10 * n);
     a.enode = (uint16_t*)(sm + 12 * n); a.parent = (uint16_t*)(sm + 14 * n); a.first = (uint32_t*)(sm + 16 * n);
-    a.wnode = (uint16_t*)(sm + 20 * n); a.idc = (uint16_t*)(sm + 22 * n); a.deg = (uint32_t*)(sm + 24 * n);
+    a.wnode = (uint16_t*)(sm + 20 * n); a.idc = (uint16_t*)(sm + 22 * n); a.deg = (uint32_t*)(sm + 4 * n); a.llen = (uint16_t*)(sm + 24 * n);
     a.clen = a.rank;
     return a;
 }
@@ -214,26 +217,91 @@ __device__ __forceinline__ uint32_t pb_end(const PbArrays& a, uint32_t hd) { ret
 __device__ __forceinline__ uint32_t pb_id(const PbArrays& a, uint32_t hd) { return hd == PB_ROOT ? 0u : a.idc[hd >> 1] + (hd & 1); }
 __device__ __forceinline__ uint32_t pb_state(const PbArrays& a, uint32_t node) { return node == 0 ? PB_ROOT : a.first[node]; }
 
-// Visit every transition into state u = (p, clone): f(source handle, solid).
+// The states that the transitions into state u = (p, clone) come from, but for the root: a stretch of the suffix links' chain from
+// the prefix before (for a clone, from what that prefix had in common with an earlier one), from the first state shorter than u
+// down to length low (0: the root has one as well).  A link of the chain is two reads that go out together, 40 cycles; reading
+// a state's length from its own arrays made it 130.
+struct PbChain { uint32_t v, lv, low; };
+__device__ __forceinline__ bool pb_more(const PbChain& c) { return c.v != PB_ROOT && c.lv >= c.low; }
+__device__ __forceinline__ void pb_next(const PbArrays& a, PbChain& c) {
+    const uint32_t n = a.link[c.v], l = a.llen[c.v];
+    c.v = l < c.lv ? n : PB_ROOT; c.lv = l;                // (lengths fall along suffix links)
+}
+// Walk a warp's 32 chains: f(v, on, owner, all) by whole warps, v a state of lane `owner`'s chain where `on`; all: the lanes are
+// at the same chain, otherwise each at its own.
+// Most chains have one to three states, and each lane goes along its own.  But a build waits for its longest chain, and where
+// tokens repeat (a run of one token, or of a few in turn) a chain has a state for each repeat, their handles the same distance
+// apart: when few lanes are left, all look at the next 32 states of one chain, as far as that distance holds; where it
+// does not, they take what comes one after the other, 16 states at a time.
+// (Four states of each lane's chain side by side: 4096 prompts of 1024 tokens 10 % slower, the builds being bound by their instructions.)
+constexpr int PB_FEW = 4;                  // lanes left
 template <class F>
-__device__ __forceinline__ void pb_into(const PbArrays& a, uint32_t u, F f) {
-    const uint32_t p = u >> 1;
-    const uint32_t len = pb_len(a, u), low = pb_len(a, a.link[u]);
-    uint32_t v = PB_ROOT, lv = 0;
-    if (len > 1) {
-        if (!(u & 1)) v = (p - 1) << 1;
-        else {                                             // a suffix of what prefix p - 1 had in common with an earlier one
-            v = pb_state(a, a.wnode[p - 1] & 0x7FFFu);
-            while (v != PB_ROOT && pb_len(a, v) >= len) v = a.link[v];
+__device__ __forceinline__ void pb_walk(const PbArrays& a, PbChain& c, int n, int lane, F f) {
+    unsigned rest = __ballot_sync(0xFFFFFFFFu, pb_more(c));
+    for (int turn = 0; rest; turn++) {
+        if (turn >= 4 && __popc(rest) <= PB_FEW) break;
+        const bool on = pb_more(c);
+        const uint32_t v = c.v;
+        if (on) pb_next(a, c);
+        f(v, on, lane, false);
+        rest = __ballot_sync(0xFFFFFFFFu, pb_more(c));
+    }
+    for (; rest; rest &= rest - 1) {
+        const int owner = __ffs(rest) - 1;
+        PbChain x;                                         // the same in all lanes
+        x.v = __shfl_sync(0xFFFFFFFFu, c.v, owner); x.lv = __shfl_sync(0xFFFFFFFFu, c.lv, owner); x.low = __shfl_sync(0xFFFFFFFFu, c.low, owner);
+        while (pb_more(x)) {
+            uint32_t v = x.v + (uint32_t)lane * (a.link[x.v] - x.v);
+            const bool in = v < 2u * (uint32_t)n;
+            const uint32_t nv = in ? a.link[v] : PB_ROOT, nl = in ? a.llen[v] : 0u;
+            uint32_t pv = __shfl_up_sync(0xFFFFFFFFu, nv, 1), pl = __shfl_up_sync(0xFFFFFFFFu, nl, 1);
+            if (lane == 0) { pv = x.v; pl = x.lv; }
+            const unsigned ok = __ballot_sync(0xFFFFFFFFu, in && pv == v && pl >= x.low && nl < pl);
+            const int r = ~ok ? __ffs(~ok) - 1 : 32;
+            if (r >= 4) {
+                f(v, lane < r, owner, true);
+                x.v = __shfl_sync(0xFFFFFFFFu, nv, r - 1); x.lv = __shfl_sync(0xFFFFFFFFu, nl, r - 1);
+                continue;
+            }
+            v = PB_ROOT;
+            for (int i = 0; i < 16 && pb_more(x); i++) {
+                if (lane == i) v = x.v;
+                pb_next(a, x);
+            }
+            f(v, v != PB_ROOT, owner, true);
         }
-        lv = pb_len(a, v);
+        if (lane == owner) c = x;
     }
-    for (uint32_t below = len; lv >= low && lv < below; lv = pb_len(a, v)) {        // (lengths fall along suffix links)
-        below = lv;
-        f(v, lv + 1 == len);
-        if (v == PB_ROOT) break;
-        v = a.link[v];
+}
+// Where the chain of u's transitions begins.  u: live lanes only.  start: kept beside `first` for a second walk.
+__device__ __forceinline__ PbChain pb_chain(const PbArrays& a, bool live, uint32_t u, uint32_t len, int n, int lane) {
+    const uint32_t p = u >> 1;
+    PbChain c;
+    c.v = PB_ROOT; c.lv = 0; c.low = len;
+    if (live && len > 1) {
+        if (!(u & 1)) { c.v = (p - 1) << 1; c.lv = p; }
+        else {
+            const uint32_t x = a.wnode[p - 1] & 0x7FFFu;
+            c.v = x == 0 ? PB_ROOT : reinterpret_cast<const uint16_t*>(a.first)[2 * x];
+            c.lv = a.clen[p - 1];
+        }
     }
+    pb_walk(a, c, n, lane, [](uint32_t, bool, int, bool) {});        // the states that are not shorter
+    if (live) {
+        c.low = a.llen[u];
+        if (u & 1) reinterpret_cast<uint16_t*>(a.first)[2 * p + 1] = (uint16_t)c.v;
+    }
+    return c;
+}
+__device__ __forceinline__ PbChain pb_chain_again(const PbArrays& a, bool live, uint32_t u, uint32_t len) {
+    PbChain c;
+    c.v = PB_ROOT; c.lv = c.low = 0;
+    if (live && len > 1) {
+        if (!(u & 1)) { c.v = ((u >> 1) - 1) << 1; c.lv = u >> 1; }
+        else { c.v = reinterpret_cast<const uint16_t*>(a.first)[2 * (u >> 1) + 1]; c.lv = pb_len(a, c.v); }
+        c.low = a.llen[u];
+    }
+    return c;
 }
 
 // Slabs for a whole prompt, by one warp: all of them or none.  Subtracting and giving back what is too few would do, were it not
@@ -444,7 +512,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         for (int i = tid; i < width; i += nt) a.tree[width + i] = __vminu2(a.tree[2 * (width + i)], a.tree[2 * (width + i) + 1]);
         if (width > 32) pb_sync(nt); else __syncwarp();      // the last levels are warp 0's alone
     }
-    for (int j = tid; j < N2; j += nt) { a.first[j] = 0xFFFFFFFFu; a.deg[j] = 0; }
+    for (int j = tid; j < N2; j += nt) a.first[j] = 0xFFFFFFFFu;
     if (tid == 0) { sh.root_deg = 0; sh.err = 0; }
     if (tid < 16) sh.cls_n[tid] = 0;
     pb_sync(nt);
@@ -529,8 +597,13 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
             // suffix links
             uint32_t x = pb_leaf(a, (uint32_t)p);
             if (x != 0 && pb_h(a, (int)x) == (uint32_t)p + 1u) x = a.parent[x];      // the prefix occurs again: the interval is its own
-            a.link[2 * p] = (uint16_t)pb_state(a, x);
-            if (cl) a.link[2 * p + 1] = (uint16_t)pb_state(a, a.parent[a.wnode[p] & 0x7FFFu]);
+            const uint32_t y = a.wnode[p] & 0x7FFFu, yl = pb_h(a, (int)y);
+            a.link[2 * p] = (uint16_t)pb_state(a, x); a.llen[2 * p] = (uint16_t)pb_h(a, (int)x);    // (h[0] is 0)
+            a.clen[p] = (uint16_t)yl;                      // (only this thread has read the rank that was there)
+            if (cl) {
+                const uint32_t up = a.parent[y];
+                a.link[2 * p + 1] = (uint16_t)pb_state(a, up); a.llen[2 * p + 1] = (uint16_t)pb_h(a, (int)up);
+            }
         }
     }
     // the root's table entries are given out from a bitmap, in place of `canon`, if that is large enough
@@ -538,29 +611,34 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     const bool bitmap = W.root_cap <= 16 * N2;
     pb_sync(nt);
     if (bitmap) for (int j = tid; j < (N2 >> 1); j += nt) taken[j] = 0;
-    for (int p = tid; p < n; p += nt) a.clen[p] = (uint16_t)pb_h(a, a.wnode[p] & 0x7FFF);
+    for (int p = tid; p < n; p += nt) a.deg[p] = 0;
     pb_sync(nt);
 
     // ---- transitions: count them (the root's go to its table at once)
     uint2* root = W.root_tab + (size_t)b * W.root_cap;
     const uint32_t cap_mask = (uint32_t)W.root_cap - 1u, bmask = (uint32_t)(W.root_cap / SAM_ROOT_BUCKET) - 1u;
-    for (int q = tid; q < 2 * n; q += nt) {
+    for (int q = tid; q - lane < 2 * n; q += nt) {         // (whole warps)
         const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1);
-        if ((u & 1) && !pb_clones(a, u >> 1)) continue;
-        pb_into(a, u, [&](uint32_t v, bool solid) {
-            if (v != PB_ROOT) { atomicAdd(&a.deg[v >> 1], (v & 1) ? 0x10000u : 1u); return; }
-            const uint32_t t = (uint32_t)text[pb_end(a, u)];
-            const uint2 val = make_uint2(t, pb_id(a, u) | (solid ? SAM_FLAG : 0u));
-            uint32_t at = (sam_hash1(t) & bmask) * SAM_ROOT_BUCKET;
-            for (uint32_t i = 0; i <= cap_mask; i++, at = (at + 1) & cap_mask) {
-                if (bitmap) {
-                    const uint32_t bit = 1u << (at & 31);
-                    if (!(atomicOr(&taken[at >> 5], bit) & bit)) { root[at] = val; break; }
-                } else if (atomicCAS(reinterpret_cast<unsigned long long*>(root + at), (unsigned long long)SAM_NONE,
-                                     (unsigned long long)val.y << 32 | val.x) == (unsigned long long)SAM_NONE) break;
-            }
-            atomicAdd(&sh.root_deg, 1);
+        const bool live = q < 2 * n && (!(u & 1) || pb_clones(a, u >> 1));
+        const uint32_t len = live ? pb_len(a, u) : 0u;
+        const bool from_root = live && a.llen[u] == 0;
+        uint32_t t = 0;
+        if (from_root) t = (uint32_t)text[pb_end(a, u)];
+        PbChain c = pb_chain(a, live, u, len, n, lane);
+        pb_walk(a, c, n, lane, [&](uint32_t v, bool on, int, bool) {
+            if (on) atomicAdd(&a.deg[v >> 1], (v & 1) ? 0x10000u : 1u);
         });
+        if (!from_root) continue;
+        const uint2 val = make_uint2(t, pb_id(a, u) | (len == 1 ? SAM_FLAG : 0u));
+        uint32_t at = (sam_hash1(t) & bmask) * SAM_ROOT_BUCKET;
+        for (uint32_t i = 0; i <= cap_mask; i++, at = (at + 1) & cap_mask) {
+            if (bitmap) {
+                const uint32_t bit = 1u << (at & 31);
+                if (!(atomicOr(&taken[at >> 5], bit) & bit)) { root[at] = val; break; }
+            } else if (atomicCAS(reinterpret_cast<unsigned long long*>(root + at), (unsigned long long)SAM_NONE,
+                                 (unsigned long long)val.y << 32 | val.x) == (unsigned long long)SAM_NONE) break;
+        }
+        atomicAdd(&sh.root_deg, 1);
     }
     pb_sync(nt);
 
@@ -599,6 +677,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     if (sh.err) { out.err = sh.err; out.s2 = out.l2 = out.e2 = 0; return; }
     const int rps_shift = W.slab_shift - 5;
     const uint32_t* blk_slab = sh.slab + sh.n_rec_slabs;
+    const uint32_t us = W.slab_shift - 7;                  // log2 of the 128-byte units of a slab
     auto record = [&](uint32_t id) {
         return reinterpret_cast<uint4*>(W.pool + ((size_t)sh.slab[id >> rps_shift] << W.slab_shift)) + 2 * (size_t)(id & ((1u << rps_shift) - 1));
     };
@@ -610,8 +689,9 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         uint4 bw = make_uint4(0, 0, 0, 0);
         if (d > 2) {
             const int k = d <= SAM_BLOCK_MIN ? 0 : 28 - __clz(d - 1);
-            const uint32_t at = sh.cls_base[k] + ((uint32_t)(q < n ? a.parent : a.canon)[p] << k);
-            const uint32_t us = W.slab_shift - 7;
+            uint16_t* nth = (q < n ? a.parent : a.canon) + p;
+            const uint32_t at = sh.cls_base[k] + ((uint32_t)*nth << k);
+            *nth = (uint16_t)at;                           // (at most two units for each of 8192 tokens)
             bw = make_uint4((blk_slab[at >> us] << us) + (at & ((1u << us) - 1u)), (uint32_t)SAM_BLOCK_MIN << k, 0, 0);
         }
         uint4* rec = record(pb_id(a, u));
@@ -626,17 +706,22 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     pb_sync(nt);
 
     // ---- transitions: write them
-    for (int q = tid; q < 2 * n; q += nt) {
+    for (int q = tid; q - lane < 2 * n; q += nt) {
         const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1);
-        if ((u & 1) && !pb_clones(a, u >> 1)) continue;
-        const uint32_t t = (uint32_t)text[pb_end(a, u)], idu = pb_id(a, u);
-        pb_into(a, u, [&](uint32_t v, bool solid) {
-            if (v == PB_ROOT) return;
-            const uint32_t was = (v & 1) ? atomicSub(&a.deg[v >> 1], 0x10000u) >> 16 : atomicSub(&a.deg[v >> 1], 1u) & 0xFFFFu;
-            const uint32_t k = (was & 0x7FFFu) - 1u;
-            uint2* rec = reinterpret_cast<uint2*>(record(pb_id(a, v)));
-            uint2* at = (was & 0x8000u) ? reinterpret_cast<uint2*>(W.pool + (size_t)rec[2].x * 128) + k : rec + 2 + k;
-            *at = make_uint2(t, idu | (solid ? SAM_FLAG : 0u));
+        const bool live = q < 2 * n && (!(u & 1) || pb_clones(a, u >> 1));
+        const uint32_t t = live ? (uint32_t)text[pb_end(a, u)] : 0u, idu = live ? pb_id(a, u) : 0u, len = live ? pb_len(a, u) : 0u;
+        PbChain c = pb_chain_again(a, live, u, len);
+        uint32_t to = idu | (c.lv + 1 == len ? SAM_FLAG : 0u);      // (only the first is solid)
+        pb_walk(a, c, n, lane, [&](uint32_t v, bool on, int owner, bool all) {
+            uint2 edge = make_uint2(t, to);
+            if (all) { edge.x = __shfl_sync(0xFFFFFFFFu, t, owner); edge.y = __shfl_sync(0xFFFFFFFFu, to, owner); }
+            to = idu;
+            if (!on) return;
+            const uint32_t h = v >> 1, odd = v & 1, old = atomicSub(&a.deg[h], odd ? 0x10000u : 1u);
+            const uint32_t unit = (odd ? a.canon : a.parent)[h], id = a.idc[h] + odd, was = odd ? old >> 16 : old & 0xFFFFu;
+            uint2* at = (was & 0x8000u) ? reinterpret_cast<uint2*>(W.pool + ((((size_t)blk_slab[unit >> us]) << us) + (unit & ((1u << us) - 1u))) * 128)
+                                        : reinterpret_cast<uint2*>(record(id) + 1);
+            at[(was & 0x7FFFu) - 1u] = edge;
         });
     }
     pb_sync(nt);

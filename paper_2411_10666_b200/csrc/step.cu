@@ -2389,15 +2389,18 @@ int split_kernel_setup(int device) {
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;
 }
-// The build for rows of up to `stride` tokens.  With the static side: two tokens a thread, four where more than two
-// builds share an SM.  Without: four tokens a thread, registers for as many blocks as the shared memory has room for.
+// The build for rows of up to `stride` tokens.  With the static side: a token a thread, as far as threads go, 1024 where a build
+// has the SM to itself (fewer slots than SMs, or rows of which the shared memory holds one), otherwise 512, so that the registers
+// are enough for two.  (With two tokens a thread 1 x 300 took 25.9 us for 21.0 now, 16 x 1000 41 for 37, and of 256 x 1024 only one
+// build fitted an SM: 95 for 78.)  Without: four tokens a thread, registers for as many blocks as the shared memory has room for.
 int launch_prefill(const StepArgs& A, int batch, int device, cudaLaunchConfig_t* cfg) {
     using Kernel = void (*)(const StepArgs);
     const Kernel kernels[4] = {sam_prefill_kernel<true, 1024, 1>, sam_prefill_kernel<false, 256, 5>, sam_prefill_kernel<false, 512, 3>,
                                sam_prefill_kernel<false, 1024, 1>};
     int n2 = 64;
     while (n2 < A.stride && n2 < PB_MAX) n2 <<= 1;
-    int k = 0, threads = 32 + (n2 / 2 < 64 ? 64 : n2 / 2 > 992 ? 992 : n2 / 2), blocks = batch;
+    const int most = batch <= SAM_SMS || n2 > 2048 ? 1024 : 512, rows = A.stride < most ? (A.stride + 31) & ~31 : most;
+    int k = 0, threads = rows + 32 < most ? rows + 32 : most, blocks = batch;
     if (batch > 2 * SAM_SMS) {
         k = n2 <= 1024 ? 1 : n2 <= 2048 ? 2 : 3;
         threads = n2 / 4 < 128 ? 128 : n2 / 4 > 1024 ? 1024 : n2 / 4;

@@ -385,3 +385,19 @@ def test_steps_with_prompts_replayed_from_a_graph(P, B):
             ref = ob.step(t[i], c[i], L, 8)
             for k, v in outs[i].cpu().items():
                 assert np.array_equal(v, getattr(ref, k)), (share, i, k)
+
+
+@pytest.mark.parametrize("B,n", [(148, 991), (149, 480), (149, 481), (149, 1025), (149, 2049)])
+def test_prompts_at_the_edges_of_the_build_blocks(P, B, n):
+    """One and two builds an SM, and rows of as many tokens as the block has threads, one more, and several times as many."""
+    rng = random.Random(B + n)
+    base = [rng.randrange(400) for _ in range(12_000)]
+    corpus = base + base[2000:7000]
+    L = 16
+    rows = np.array([_text(KINDS[i % len(KINDS)], n, rng, corpus) + [rng.randrange(9) for _ in range(8)] for i in range(B)], dtype=np.int32)
+    counts = np.full((1, B), 8, dtype=np.int32)
+    st = P.StaticSam.build(np.array(corpus, dtype=np.int32), VOCAB)
+    ref, ob, _ = oracle_run(np.array(corpus, dtype=np.int32), VOCAB, rows[:, :n], rows[None, :, n:].copy(), counts, L, n + 8, threads=8)
+    got, batch = gpu_run(P, st, VOCAB, rows[:, :n], rows[None, :, n:].copy(), counts, L, n + 8)
+    assert_same(got, ref)
+    assert_dynamic_automata_equal(batch, ob, range(0, B, 7), n + 8)
