@@ -29,7 +29,8 @@ namespace {
 
 constexpr int PB_MAX = 8192;               // longest text: 28 bytes per token of shared memory
 constexpr int PB_BYTES_PER_TOKEN = 28;
-constexpr int PB_LEVELS = 6;               // rank arrays kept for comparing two prefixes
+constexpr int PB_LEVELS = 5;               // rank arrays kept for comparing two prefixes
+constexpr int PB_COUNTED = 128;            // members of a group up to which they are ordered by counting
 constexpr int PB_BLOCK_SLABS = 80;         // slabs the edge blocks of one text can take (at most 64, and a remainder)
 constexpr uint32_t PB_ROOT = 0xFFFFu;      // handle of the root; a state is (p << 1 | clone)
 
@@ -37,11 +38,12 @@ struct PbShared {                          // what the threads of one build exch
     int16_t chunk[PB_MAX / 32];
     uint32_t slab[SAM_MAX_REC_SLABS + PB_BLOCK_SLABS];       // of the records, then of the edge blocks
     uint32_t cls_n[16], cls_base[16];
-    int groups, clones, root_deg, err, n_rec_slabs;
+    int groups[2];                         // counted in rounds in turn: one is cleared while the other is in use
+    int rows, clones, root_deg, err, n_rec_slabs;
 };
 
 struct PbArrays {
-    uint64_t* key; uint16_t* lev; uint16_t* A; uint16_t* B; uint32_t* tok;      // while sorting
+    uint64_t* key; uint16_t* lev; uint16_t* end; uint16_t* A; uint16_t* B; uint32_t* tok;      // while sorting
     uint32_t* tree; uint16_t* rank; uint16_t* canon; uint16_t* enode; uint16_t* parent;
     uint32_t* first; uint16_t* wnode; uint16_t* idc; uint16_t* link; uint16_t* llen; uint32_t* deg; uint16_t* clen;
     int N2;                                // size of the sorted order, a power of two
@@ -54,7 +56,7 @@ __device__ __forceinline__ PbArrays pb_arrays(unsigned char* sm, int N2) {
     PbArrays a;
     const size_t n = (size_t)N2;
     a.N2 = N2;
-    a.key = (uint64_t*)sm; a.lev = (uint16_t*)(sm + 8 * n); a.A = (uint16_t*)(sm + 20 * n); a.B = (uint16_t*)(sm + 22 * n);
+    a.key = (uint64_t*)sm; a.lev = (uint16_t*)(sm + 8 * n); a.end = (uint16_t*)(sm + 18 * n); a.A = (uint16_t*)(sm + 20 * n); a.B = (uint16_t*)(sm + 22 * n);
     a.tok = (uint32_t*)(sm + 24 * n);
     a.tree = (uint32_t*)sm; a.link = (uint16_t*)sm; a.rank = (uint16_t*)(sm + 8 * n); a.canon = (uint16_t*)(sm + 10 * n);
     a.enode = (uint16_t*)(sm + 12 * n); a.parent = (uint16_t*)(sm + 14 * n); a.first = (uint32_t*)(sm + 16 * n);
@@ -69,95 +71,6 @@ __device__ __forceinline__ bool pb_sync_or(int nt, bool x) {
     uint32_t r;
     asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %2, 0; bar.red.or.pred q, 1, %1, p; selp.u32 %0, 1, 0, q; }" : "=r"(r) : "r"(nt), "r"((uint32_t)x) : "memory");
     return r != 0;
-}
-
-__device__ __forceinline__ uint64_t pb_shfl_xor(uint64_t v, int s) {
-    const uint32_t lo = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)v, s), hi = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)(v >> 32), s);
-    return ((uint64_t)hi << 32) | lo;
-}
-__device__ __forceinline__ void pb_step(uint64_t& v, int lane, int stride, bool up) {
-    const uint64_t o = pb_shfl_xor(v, stride);
-    const bool low = (lane & stride) == 0;
-    if ((o < v) == (low == up)) v = o;
-}
-
-// Bitonic sort of key[0, N2).  Strides below 64 stay in the registers of one warp (two keys a lane).
-// (One copy, out of line: with builds in different phases on an SM, fetching instructions is what they wait for most.)
-__device__ __noinline__ void pb_sort(uint64_t* key, int N2, int tid, int nt) {
-    const int lane = tid & 31, w = tid >> 5, nw = nt >> 5;
-    for (int size = 64; size <= N2; size <<= 1) {
-        int stride = size >> 1;
-        for (; stride >= 128; stride >>= 2) {              // two strides a pass
-            const int half = stride >> 1;
-            for (int q = tid; q < (N2 >> 2); q += nt) {
-                const int i = ((q & ~(half - 1)) << 2) | (q & (half - 1));
-                const bool up = (i & size) == 0;
-                uint64_t x0 = key[i], x1 = key[i + half], x2 = key[i + stride], x3 = key[i + stride + half], t;
-                if ((x0 > x2) == up) { t = x0; x0 = x2; x2 = t; }
-                if ((x1 > x3) == up) { t = x1; x1 = x3; x3 = t; }
-                if ((x0 > x1) == up) { t = x0; x0 = x1; x1 = t; }
-                if ((x2 > x3) == up) { t = x2; x2 = x3; x3 = t; }
-                key[i] = x0; key[i + half] = x1; key[i + stride] = x2; key[i + stride + half] = x3;
-            }
-            pb_sync(nt);
-        }
-        for (; stride >= 64; stride >>= 1) {
-            for (int q = tid; q < (N2 >> 1); q += nt) {
-                const int i = ((q & ~(stride - 1)) << 1) | (q & (stride - 1)), k = i + stride;
-                const uint64_t x = key[i], y = key[k];
-                if ((x > y) == ((i & size) == 0)) { key[i] = y; key[k] = x; }
-            }
-            pb_sync(nt);
-        }
-        for (int c = w; c < (N2 >> 6); c += nw) {
-            uint64_t x = key[64 * c + lane], y = key[64 * c + 32 + lane];
-            if (size == 64) {
-#pragma unroll
-                for (int sz = 2; sz <= 32; sz <<= 1)
-#pragma unroll
-                    for (int st = sz >> 1; st; st >>= 1) {
-                        pb_step(x, lane, st, sz == 32 ? true : (lane & sz) == 0);
-                        pb_step(y, lane, st, sz == 32 ? false : (lane & sz) == 0);
-                    }
-            }
-            const bool up = ((64 * c) & size) == 0;
-            if ((x > y) == up) { const uint64_t t = x; x = y; y = t; }
-#pragma unroll
-            for (int st = 16; st; st >>= 1) { pb_step(x, lane, st, up); pb_step(y, lane, st, up); }
-            key[64 * c + lane] = x; key[64 * c + 32 + lane] = y;
-        }
-        pb_sync(nt);
-    }
-}
-
-// rank[p] = first sorted position of p's group of equal keys; returns the number of groups.
-__device__ int pb_rank(const PbArrays& a, PbShared& sh, uint16_t* rank, int n, int ib, int tid, int nt) {
-    const int lane = tid & 31, w = tid >> 5, nw = nt >> 5, chunks = (n + 31) >> 5;
-    if (tid == 0) sh.groups = 0;
-    pb_sync(nt);
-    for (int c = w; c < chunks; c += nw) {
-        const int j = 32 * c + lane;
-        const bool head = j < n && (j == 0 || (a.key[j] >> ib) != (a.key[j - 1] >> ib));
-        const unsigned mask = __ballot_sync(0xFFFFFFFFu, head);
-        if (lane == 0) { sh.chunk[c] = mask ? (int16_t)(32 * c + 31 - __clz(mask)) : (int16_t)-1; atomicAdd(&sh.groups, __popc(mask)); }
-    }
-    pb_sync(nt);
-    const uint32_t im = (1u << ib) - 1u;
-    for (int c = w; c < chunks; c += nw) {
-        const int j = 32 * c + lane;
-        const bool head = j < n && (j == 0 || (a.key[j] >> ib) != (a.key[j - 1] >> ib));
-        const unsigned mask = __ballot_sync(0xFFFFFFFFu, head);
-        int before = 0;                                    // where the group that reaches into this chunk began
-        for (int base = c - 1; base >= 0; base -= 32) {
-            const int v = base - lane >= 0 ? sh.chunk[base - lane] : -1;
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, v >= 0);
-            if (m) { before = __shfl_sync(0xFFFFFFFFu, v, __ffs(m) - 1); break; }
-        }
-        const unsigned mine = mask & (0xFFFFFFFFu >> (31 - lane));
-        if (j < n) rank[(uint32_t)a.key[j] & im] = (uint16_t)(mine ? 32 * c + 31 - __clz(mine) : before);
-    }
-    pb_sync(nt);
-    return sh.groups;
 }
 
 // The tree over the sorted order: leaf j is h[j] << 16 | A[j], an inner node the two minima of its leaves.
@@ -353,7 +266,7 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + 10 * (size_t)N2);             // [size]: positions, then where they begin
     uint16_t* at = reinterpret_cast<uint16_t*>(smem + 18 * (size_t)N2);              // [N2]: a position's table entry
     for (int i = tid; i < size; i += nt) { key[i] = SAM_NONE; cnt[i] = 0; }
-    if (tid == 0) sh.groups = 0;
+    if (tid == 0) sh.groups[0] = sh.groups[1] = sh.rows = 0;
     pb_sync(nt);
     for (int p = tid; p < n; p += nt) {
         const uint32_t t = a.tok[p];
@@ -371,7 +284,7 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
     for (int c = w; c < chunks; c += nw) {
         const uint32_t x = cnt[64 * c + 2 * lane], y = cnt[64 * c + 2 * lane + 1];
         const int sum = __reduce_add_sync(0xFFFFFFFFu, (int)(x + y)), used = __reduce_add_sync(0xFFFFFFFFu, (x != 0) + (y != 0));
-        if (lane == 0) { sh.chunk[c] = (int16_t)sum; if (used) atomicAdd(&sh.groups, used); }
+        if (lane == 0) { sh.chunk[c] = (int16_t)sum; if (used) atomicAdd(&sh.groups[0], used); }
     }
     pb_sync(nt);
     if (w == 0) {
@@ -401,44 +314,153 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
         a.lev[p] = (uint16_t)begin;
     }
     pb_sync(nt);
-    return sh.groups;
+    return sh.groups[0];
 }
 
-// One round of the sort: order the members of each group of equal prefixes (of `span` tokens) by the tokens before those, by
-// counting how many of the group come first.  A -> B, rank -> next; end: room for where each group ends.  Returns the number
-// of groups.
-__device__ int pb_refine(const PbArrays& a, PbShared& sh, const uint16_t* A, uint16_t* B, const uint16_t* rank, uint16_t* next, uint16_t* end,
-                         int span, int n, int tid, int nt) {
-    for (int j = tid; j < n; j += nt) {
-        const int p = A[j], g = rank[p];
+// What is common to the rounds of the sort.  A round orders the members of each group of equal prefixes (of `span` tokens) by the
+// tokens before those: A -> B, rank -> next.  PB_ALONE in A marks the groups of one, which most positions are in after a round or
+// two: they stay where they are.  This is the look at position j: whether it is alone; end: where each group ends.
+constexpr uint32_t PB_ALONE = 0x8000u;
+__device__ __forceinline__ bool pb_alone(uint16_t* A, const uint16_t* rank, uint16_t* end, int j, int n, uint32_t& p, uint32_t& g, bool& ends) {
+    p = A[j];
+    ends = false;
+    if (p & PB_ALONE) { p &= ~PB_ALONE; return true; }
+    g = rank[p];
+    ends = j + 1 == n || rank[A[j + 1] & ~PB_ALONE] != g;
+    if (ends) {
+        end[g] = (uint16_t)(j + 1);
+        if (g == (uint32_t)j) { A[j] = (uint16_t)(p | PB_ALONE); return true; }
+    }
+    return false;
+}
+// The round's end.  Its counter is read after this barrier and cleared in the next round but one's place, after that round's first
+// barrier, when all threads have read it.
+__device__ __forceinline__ int pb_groups(PbShared& sh, int turn, int mine, int tid, int nt) {
+    mine = __reduce_add_sync(0xFFFFFFFFu, mine);
+    if ((tid & 31) == 0) atomicAdd(&sh.groups[turn & 1], mine);
+    pb_sync(nt);
+    return sh.groups[turn & 1];
+}
+
+// A round by counting, for each member, how many of its group come first, by 3 x span tokens.  Returns the number of groups, or 0,
+// with nothing ordered, if there are groups so large that two rounds of pb_double take less: 7 us for 1024 tokens, 35 for
+// 8191, against 2.2 and 9 for counting small groups.  (Counting groups of 870 of 8191 took 50 us, a bitonic sort of all 47;
+// 1000 texts of 1500 tokens, groups of up to 200: 274 us with the sort, 246 with pb_double.)
+__device__ int pb_refine(const PbArrays& a, PbShared& sh, uint16_t* A, uint16_t* B, const uint16_t* rank, uint16_t* next, int span, int turn, int n, int tid, int nt) {
+    uint32_t alone = 0;                                    // of this thread's positions
+    int mine = 0;
+    bool large = false;
+    for (int j = tid, nth = 0; j < n; j += nt, nth++) {
+        uint32_t p, g;
+        bool ends;
+        if (pb_alone(A, rank, a.end, j, n, p, g, ends)) { alone |= 1u << nth; B[j] = (uint16_t)(p | PB_ALONE); next[p] = (uint16_t)j; mine++; continue; }
+        large |= ends && j + 1 - (int)g > PB_COUNTED;
         uint64_t k = 0;
 #pragma unroll
-        for (int q = 1; q < 4; q++) { const int at = p - q * span; k = k << 16 | (at >= 0 ? (uint32_t)rank[at] + 1u : 0u); }
-        a.key[j] = k;
-        if (j + 1 == n || rank[A[j + 1]] != g) end[g] = (uint16_t)(j + 1);
+        for (int q = 1; q < 4; q++) { const int at = (int)p - q * span; k = k << 16 | (at >= 0 ? (uint32_t)rank[at] + 1u : 0u); }
+        a.key[j] = k << 16 | p;
     }
-    if (tid == 0) sh.groups = 0;
-    pb_sync(nt);
-    int mine = 0;
-    for (int j = tid; j < n; j += nt) {
-        const int p = A[j], g = rank[p], e = end[g];
-        int less = 0, same = 0;
-        if (e - g > 1) {
-            const uint64_t k = a.key[j];
+    if (pb_sync_or(nt, large)) return 0;
+    if (tid == 0) sh.groups[~turn & 1] = 0;
+    for (int j = tid, nth = 0; j < n; j += nt, nth++) {
+        if (alone >> nth & 1u) continue;
+        const uint64_t k = a.key[j], same = k & ~0xFFFFull;
+        const uint32_t p = (uint32_t)k & 0xFFFFu, g = rank[p], e = a.end[g];
+        int less = 0, before = 0;                          // the group's that come before this one, and before all equal to it
 #pragma unroll 4
-            for (int i = g; i < e; i++) {
-                const uint64_t x = a.key[i];
-                less += x < k; same += x == k && i < j;
+        for (uint32_t i = g; i < e; i++) {
+            const uint64_t x = a.key[i];
+            less += x < k; before += x < same;
+        }
+        B[g + less] = (uint16_t)p;
+        next[p] = (uint16_t)(g + before);
+        mine += less == before;
+    }
+    return pb_groups(sh, turn, mine, tid, nt);
+}
+
+// A round that looks at `span` tokens more and does not care how large the groups are.  In the order there is, the prefixes that
+// end `span` tokens earlier already lie as the members of each group shall: the i-th of them, q, says where q + span comes in its
+// group, after as many as have come by.  In a group of up to PB_FEW_MEMBERS that is counted; a larger group has a row of bits,
+// one for each i, and a count before each word of them, 32 groups at a time.
+constexpr int PB_FEW_MEMBERS = 64;
+__device__ int pb_double(const PbArrays& a, PbShared& sh, uint16_t* A, uint16_t* B, const uint16_t* rank, uint16_t* next, int span, int turn, int n, int tid, int nt) {
+    const int lane = tid & 31, w = tid >> 5, nw = nt >> 5, W = a.N2 >> 5;
+    uint32_t* key = reinterpret_cast<uint32_t*>(a.key);
+    uint32_t* bits = key + a.N2;                           // [32][W]
+    uint16_t* before = reinterpret_cast<uint16_t*>(a.tok) + a.N2;                    // [32][W]
+    uint16_t* end = a.end;                                 // of a larger group also, one on, its row
+    uint32_t alone = 0;
+    int mine = 0;
+    for (int j = tid, nth = 0; j < n; j += nt, nth++) {
+        uint32_t p, g;
+        bool ends;
+        if (pb_alone(A, rank, end, j, n, p, g, ends)) { alone |= 1u << nth; B[j] = (uint16_t)(p | PB_ALONE); next[p] = (uint16_t)j; mine++; continue; }
+        if (ends && j + 1 - (int)g > PB_FEW_MEMBERS) end[g + 1] = (uint16_t)atomicAdd(&sh.rows, 1);
+        key[j] = ((int)p >= span ? (uint32_t)rank[p - span] + 1u : 0u) << 16 | p;
+    }
+    pb_sync(nt);
+    if (tid == 0) sh.groups[~turn & 1] = 0;
+    for (int j = tid, nth = 0; j < n; j += nt, nth++) {
+        if (alone >> nth & 1u) continue;
+        const uint32_t k = key[j], same = k & ~0xFFFFu, p = k & 0xFFFFu, g = rank[p], e = end[g];
+        if (e - g > PB_FEW_MEMBERS) continue;
+        int less = 0, ahead = 0;
+#pragma unroll 4
+        for (uint32_t i = g; i < e; i++) {
+            const uint32_t x = key[i];
+            less += x < k; ahead += x < same;
+        }
+        B[g + less] = (uint16_t)p;
+        next[p] = (uint16_t)(g + ahead);
+        mine += less == ahead;
+    }
+    const int rows = sh.rows;
+    const uint32_t g0 = rank[span - 1];                    // the group of the one prefix that has `span` tokens: it comes first
+    if (rows > 0 && tid == 0 && end[g0] - (int)g0 > PB_FEW_MEMBERS) { B[g0] = (uint16_t)(span - 1); next[span - 1] = (uint16_t)g0; mine++; }
+    for (int row0 = 0; row0 < rows; row0 += 32) {
+        const int here = min(32, rows - row0);
+        for (int i = tid; i < (here * W + 3) >> 2; i += nt) reinterpret_cast<uint4*>(bits)[i] = make_uint4(0, 0, 0, 0);
+        pb_sync(nt);
+        for (int i = tid; i < n; i += nt) {
+            const int p = (A[i] & ~PB_ALONE) + span;
+            if (p >= n) continue;
+            const uint32_t g = rank[p];
+            if (end[g] - (int)g <= PB_FEW_MEMBERS) continue;
+            const uint32_t row = end[g + 1] - row0;
+            if (row < 32) atomicOr(&bits[row * W + (i >> 5)], 1u << (i & 31));
+        }
+        pb_sync(nt);
+        for (int r = w; r < here; r += nw) {
+            int run = 0;
+            for (int c = 0; c < W; c += 32) {
+                const int v = c + lane < W ? __popc(bits[r * W + c + lane]) : 0;
+                int s = v;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
+                if (c + lane < W) before[r * W + c + lane] = (uint16_t)(run + s - v);
+                run += __shfl_sync(0xFFFFFFFFu, s, 31);
             }
         }
-        B[g + less + same] = (uint16_t)p;
-        next[p] = (uint16_t)(g + less);
-        mine += same == 0;
+        pb_sync(nt);
+        for (int i = tid; i < n; i += nt) {
+            const int q = A[i] & ~PB_ALONE, p = q + span;
+            if (p >= n) continue;
+            const uint32_t g = rank[p];
+            if (end[g] - (int)g <= PB_FEW_MEMBERS) continue;
+            const uint32_t row = end[g + 1] - row0;
+            if (row >= 32) continue;
+            const int word = (int)row * W, h = rank[q], first = g == g0 ? 1 : 0;
+            const int at = first + before[word + (i >> 5)] + __popc(bits[word + (i >> 5)] & ((1u << (i & 31)) - 1u));
+            const int head = first + before[word + (h >> 5)] + __popc(bits[word + (h >> 5)] & ((1u << (h & 31)) - 1u));
+            B[g + at] = (uint16_t)p;
+            next[p] = (uint16_t)(g + head);
+            mine += at == head;
+        }
+        if (row0 + 32 < rows) pb_sync(nt);
     }
-    mine = __reduce_add_sync(0xFFFFFFFFu, mine);
-    if ((tid & 31) == 0) atomicAdd(&sh.groups, mine);
-    pb_sync(nt);
-    return sh.groups;
+    if (rows > 0 && tid == 0) sh.rows = 0;                 // (all threads have passed a barrier since they read it)
+    return pb_groups(sh, turn, mine, tid, nt);
 }
 
 // The automaton of a text of n tokens for the empty slot b: every record, transition and table entry Expand would
@@ -451,8 +473,6 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     const int N2 = pb_size(n);
     const PbArrays a = pb_arrays(smem, N2);
     const int32_t* text = W.text + (size_t)b * W.text_stride;
-    const int ib = 32 - __clz(n - 1), rb = 32 - __clz(n);  // bits of a position, and of a rank plus one
-    const uint32_t im = (1u << ib) - 1u;
 
     // ---- sort
     uint16_t *A = a.A, *B = a.B;
@@ -460,31 +480,22 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     int spans[PB_LEVELS];
 #pragma unroll
     for (int i = 0; i < PB_LEVELS; i++) spans[i] = 1;
-    int groups = pb_group(a, sh, smem, n, tid, nt);
+    int groups = pb_group(a, sh, smem, n, tid, nt), turn = 1;
     while (groups < n && span < n) {                       // (ranks of n tokens are all different)
         const uint16_t* r = a.lev + (size_t)top * N2;
-        bool large = false;                                // groups so large that counting would take longer than sorting all
-        const int most = min(max(64, N2 >> 3), 384);       // (1 x 8191 with groups of 650: 266 us counted, 222 sorted)
-        for (int j = tid; j + most < n; j += nt) large |= r[A[j]] == r[A[j + most]];
         const int to = top < PB_LEVELS - 1 ? top + 1 : top;                          // the last array is used again for longer spans
-        if (pb_sync_or(nt, large) || to == top) {
-            const int parts = min(4, (64 - ib) / rb);
-            for (int j = tid; j < n; j += nt) {
-                uint64_t k = r[j];
-                for (int q = 1; q < parts; q++) { const int at = j - q * span; k = k << rb | (at >= 0 ? (uint32_t)r[at] + 1u : 0u); }
-                a.key[j] = k << ib | (uint32_t)j;
-            }
-            for (int j = n + tid; j < N2; j += nt) a.key[j] = ~0ull;
-            pb_sync(nt);
-            pb_sort(a.key, N2, tid, nt);
-            for (int j = tid; j < n; j += nt) A[j] = (uint16_t)((uint32_t)a.key[j] & im);
-            groups = pb_rank(a, sh, a.lev + (size_t)to * N2, n, ib, tid, nt);
-            span *= parts;
-        } else {
-            groups = pb_refine(a, sh, A, B, r, a.lev + (size_t)to * N2, a.lev + (to == 1 ? 2 * (size_t)N2 : 0), span, n, tid, nt);
+        uint16_t* next = a.lev + (size_t)to * N2;
+        groups = to == top ? 0 : pb_refine(a, sh, A, B, r, next, span, turn, n, tid, nt);
+        if (groups == 0) {
+            uint16_t* between = reinterpret_cast<uint16_t*>(a.tok);
+            groups = pb_double(a, sh, A, B, r, between, span, turn++, n, tid, nt);
             uint16_t* t = A; A = B; B = t;
-            span *= 4;
+            if (groups == n || 2 * span >= n) break;       // (where all ranks differ they say nothing of shared suffixes)
+            groups = pb_double(a, sh, A, B, between, next, 2 * span, turn, n, tid, nt);
         }
+        uint16_t* t = A; A = B; B = t;
+        span *= 4;
+        turn++;
         top = to;
 #pragma unroll
         for (int i = 0; i < PB_LEVELS; i++) if (i == top) spans[i] = span;
@@ -492,22 +503,21 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     // ---- sorted order, shared suffix lengths
     for (int j = tid; j < N2; j += nt) {
         int x = 0, p = 0xFFFF;
-        if (j < n) p = A[j];
+        if (j < n) p = A[j] & ~PB_ALONE;
         if (j > 0 && j < n) {
-            const int q = A[j - 1];
+            const int q = A[j - 1] & ~PB_ALONE;
 #pragma unroll
-            for (int i = PB_LEVELS - 1; i >= 1; i--) {     // (level 0 is not kept: its place is used by later rounds)
+            for (int i = PB_LEVELS - 1; i >= 0; i--) {
                 if (i <= top) {
                     const uint16_t* r = a.lev + (size_t)i * N2;
                     while (p - x >= 0 && q - x >= 0 && r[p - x] == r[q - x]) x += spans[i];
                 }
             }
-            while (p - x >= 0 && q - x >= 0 && a.tok[p - x] == a.tok[q - x]) x++;
         }
         a.tree[N2 + j] = (uint32_t)x << 16 | (uint32_t)p;
     }
     pb_sync(nt);
-    for (int j = tid; j < n; j += nt) a.rank[A[j]] = (uint16_t)j;
+    for (int j = tid; j < n; j += nt) a.rank[A[j] & ~PB_ALONE] = (uint16_t)j;
     for (int width = N2 >> 1; width >= 1; width >>= 1) {
         for (int i = tid; i < width; i += nt) a.tree[width + i] = __vminu2(a.tree[2 * (width + i)], a.tree[2 * (width + i) + 1]);
         if (width > 32) pb_sync(nt); else __syncwarp();      // the last levels are warp 0's alone

@@ -387,7 +387,7 @@ def test_steps_with_prompts_replayed_from_a_graph(P, B):
                 assert np.array_equal(v, getattr(ref, k)), (share, i, k)
 
 
-@pytest.mark.parametrize("B,n", [(148, 991), (149, 480), (149, 481), (149, 1025), (149, 2049)])
+@pytest.mark.parametrize("B,n", [(148, 991), (149, 480), (149, 481), (149, 1025), (149, 2049), (2723, 105)])
 def test_prompts_at_the_edges_of_the_build_blocks(P, B, n):
     """One and two builds an SM, and rows of as many tokens as the block has threads, one more, and several times as many."""
     rng = random.Random(B + n)
