@@ -213,6 +213,21 @@ __device__ __forceinline__ void ensure_rec(Dyn& D, uint32_t s) {
     D.n_rec_slabs = si + 1;
 }
 
+// Make sure of records for n states from s on, fewer than a slab holds; returns how many there are.  Where the pool has no slab left
+// that may be fewer: the tokens before the one that fails are done all the same.
+__device__ __forceinline__ uint32_t ensure_recs(Dyn& D, uint32_t s, uint32_t n) {
+    if ((s + n - 1) >> D.rps_shift < D.n_rec_slabs) return n;
+    for (uint32_t at = s;; at = s + n - 1) {
+        ensure_rec(D, at);
+        if (D.err) {
+            if (at == s) return 0;
+            D.err = 0;
+            return (D.n_rec_slabs << D.rps_shift) - s;
+        }
+        if (at == s + n - 1) return n;
+    }
+}
+
 // edge block of `cap` entries; returns its offset in 128-byte units from the pool base
 __device__ __forceinline__ uint32_t alloc_block(Dyn& D, uint32_t cap) {
     uint32_t need = cap >> 4, slab_units = 1u << (D.slab_shift - 7);
@@ -534,8 +549,9 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
 // do one token each at once.  A token qualifies if its root lookup was settled ahead of time as
 // "absent" and no earlier token of the run shares its home bucket (so slots and tokens differ).
 // Returns r (0 if token j does not qualify).
+template <class F>
 __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt, unsigned bucket_peers,
-                                             uint32_t& last, uint32_t& ntok) {
+                                             uint32_t& last, uint32_t& ntok, F& emit) {
     const unsigned from_j = ~((1u << j) - 1u);
     const unsigned lt = (1u << D.lane) - 1u;
     const bool first_of_bucket = (bucket_peers & from_j & lt) == 0;
@@ -544,9 +560,8 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
     int r = gap ? __ffs(gap) - 1 : 32 - j;
     if (r <= 0) return 0;
     const uint32_t c0 = D.n_states;
-    ensure_rec(D, c0);
-    if (!D.err) ensure_rec(D, c0 + r - 1);
-    if (D.err) return 0;
+    r = (int)ensure_recs(D, c0, (uint32_t)r);
+    if (r == 0) return 0;
     const int idx = D.lane - j;
     const bool mine = idx >= 0 && idx < r;
     const uint32_t c = c0 + (uint32_t)idx;
@@ -566,6 +581,7 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
     if (bucket_peers & run) D.pr_state = 0;                   // those buckets changed
     __syncwarp();
     SAM_COUNT(D.kc.a, 2 * r - (last == 0 ? 1 : 0));            // per token: the previous state's transition (none from the root) and the root's
+    emit(mine, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1);
     D.n_states = c0 + r; D.root_deg += r;
     last = c0 + r - 1; ntok += r;
     return r;
@@ -586,9 +602,10 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
 // is longer, and what a walk reads ahead (its first record) is checked not to be a q_k.
 // On entry (pa, pb) is the record of s2.  Returns the number of tokens taken (0: not such a run; pre
 // then offers the records read on the way to the ordinary Expand of token j).
+template <class F>
 __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cnt, uint32_t& last, uint32_t& ntok,
                                               uint32_t& s2, uint32_t& l2, uint4& pa, uint4& pb, Pre& pre,
-                                              uint32_t (*stage)[12]) {
+                                              uint32_t (*stage)[12], F& emit) {
     pre.valid = false;
     if (pa.w == 0 || pa.w > 2 || cnt - j < 2) return 0;
     const int lane = D.lane;
@@ -673,9 +690,9 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
     *reinterpret_cast<uint4*>(&stage[lane][8]) = make_uint4(tkr, ps, u, 0);
 
     const uint32_t n0 = D.n_states;                            // c_k = n0 + 2k, cl_k = n0 + 2k + 1
-    ensure_rec(D, n0);
-    if (!D.err) ensure_rec(D, n0 + 2 * (uint32_t)r - 1);
-    if (D.err) return 0;
+    pre.valid = false;                                         // (its place has been used again)
+    r = (int)ensure_recs(D, n0, 2 * (uint32_t)r) / 2;
+    if (r < 2) return 0;
 
     // the new states, side by side
     const bool mine = lane < r;
@@ -717,6 +734,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
         SAM_COUNT(D.kc.c, copied);
     }
 
+    emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1);
     const int lr = r - 1;                                      // the last clone is the new match state
     pa = make_uint4(l0 + (uint32_t)r, __shfl_sync(FULL, qa.y, lr), __shfl_sync(FULL, qa.z, lr), __shfl_sync(FULL, qa.w, lr));
     pb = make_uint4(__shfl_sync(FULL, nb.x, lr), __shfl_sync(FULL, nb.y, lr), __shfl_sync(FULL, nb.z, lr), __shfl_sync(FULL, nb.w, lr));
@@ -730,8 +748,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
 // state Transfer (Algorithm 1) reaches.  In and out: the state (s, sf, l) and, where l > 0, its record (ra, rb).
 // early(): called where the match is in the state of a corpus prefix, so that the draft after m tokens can be requested
 // with the first reads; returns true if the match did go on as the corpus does, for all m tokens.
-// LONG: rows of more than 32 tokens are prompts, as a rule; otherwise they are taken token by token.
-template <bool LONG, class F>
+template <class F>
 __device__ __forceinline__ bool static_advance(const SamStaticView& S, int lane, int32_t tok_first, const int32_t* toks, int m,
                                                uint32_t& s, uint32_t& sf, int32_t& l, uint4& ra, uint4& rb, int& err, ChainCounts& kc, F early) {
 #ifdef SAM_COUNTERS
@@ -743,14 +760,8 @@ __device__ __forceinline__ bool static_advance(const SamStaticView& S, int lane,
     }
 #endif
     bool follows = false;
-    if (m > 32) {
-        if (LONG) static_suffix(S, toks, m, lane, s, sf, l, ra, rb, err, kc);
-        else {
-            bool have = s != 0;
-            static_forward(S, toks, 0, m, s, sf, l, ra, rb, have, lane, err, kc);
-            if (l > 0 && !have && !err) static_record(S, s, ra, rb);
-        }
-    } else if (m > 0) {
+    if (m > 32) static_suffix(S, toks, m, lane, s, sf, l, ra, rb, err, kc);
+    else if (m > 0) {
         const uint32_t tk = (uint32_t)tok_first;
         uint32_t re = SAM_NONE;
         if (lane < m) re = __ldg(S.root_row + tk);
@@ -791,7 +802,7 @@ __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane,
     uint32_t s = __shfl_sync(FULL, cw, CB_S1), sf = __shfl_sync(FULL, cw, CB_S1FLAG);
     int32_t l = (int32_t)__shfl_sync(FULL, cw, CB_L1);
     int dl2 = 0;
-    const bool follows = static_advance<true>(A.S, lane, tok_first, toks, m, s, sf, l, ra, rb, err, kc, [&]() {
+    const bool follows = static_advance(A.S, lane, tok_first, toks, m, s, sf, l, ra, rb, err, kc, [&]() {
         if (DRAFT) {
             const int64_t e2 = (int64_t)ra.z + m, room = A.S.n_tokens - e2;
             dl2 = (int)(room < L ? (room < 0 ? 0 : room) : L);
@@ -864,51 +875,68 @@ __device__ __forceinline__ void dyn_open(const SamBatchView& W, int b, int lane,
     if (D.n_states == 0) D.n_states = 1;            // the root exists implicitly (no record is read for it)
 }
 
-// Expand (fused with the dynamic matcher's Transfer) for each of a step's m tokens, then the slot's control words.
-// On return, unless D.err is set, (ra, rb) is the record of s2 if l2 > 0 (also stored in the control block).
+// Expand (fused with the dynamic matcher's Transfer) for each of up to 32 tokens, one in each lane.  emit is called by the whole
+// warp whenever tokens are done, with what holds after them: (whether this lane has one, the lane that held its token, s2, l2,
+// first end position of s2, text length, state of the whole text, number of states); ends: the tokens for which it is wanted.
+struct NoEmit {
+    static constexpr unsigned ends = 0;
+    __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
+};
+template <class F>
+__device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, uint32_t (*sh_run)[12], F& emit) {
+    Dyn& D = X.D;
+    root_precompute(D, tk, D.lane < cnt);           // most walks end in the root table
+    SAM_COUNT(D.kc.rounds, 1);
+    const unsigned bucket_peers = __match_any_sync(FULL, D.pr_bucket);
+    int j = 0;
+    while (j < cnt && !D.err) {
+        if (X.s2 == 0) {
+            const int r = dyn_fresh_run(D, tk, j, cnt, bucket_peers, X.last, X.ntok, emit);
+            if (r > 0) { j += r; X.have = false; continue; }
+            if (D.err) break;
+        }
+        Pre pre;
+        pre.valid = false;
+        if (X.s2 != 0 && X.have) {
+            const int r = dyn_repeat_run(D, tk, j, cnt, X.last, X.ntok, X.s2, X.l2, X.ra, X.rb, pre, sh_run, emit);
+            if (r > 0) { j += r; continue; }
+            if (D.err) break;
+        }
+        D.cur = j;
+        dyn_extend(D, __shfl_sync(FULL, tk, j), X.last, X.ntok, X.s2, X.l2, X.have, X.ra, X.rb, pre);
+        if ((emit.ends >> j & 1u) && !D.err) {
+            if (X.l2 > 0 && !X.have) { const uint4* rs = rec_ptr(D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(D.kc.rounds, 1); }
+            emit(D.lane == j, D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, D.n_states);
+        }
+        j++;
+    }
+}
+// The newest state's record, without a transition yet, and the slot's control words.
+__device__ __forceinline__ void dyn_close(DynChain& X) {
+    uint4* rl = rec_ptr(X.D, X.last);
+    uint32_t* cb = X.D.cb;
+    if (X.D.lane == 0) {
+        rl[0] = make_uint4(X.ntok, X.s2, X.ntok, 0);
+        rl[1] = make_uint4(0, 0, 0, 0);
+        cb[CB_NTOK] = X.ntok; cb[CB_NSTATES] = X.D.n_states; cb[CB_LAST] = X.last;
+        cb[CB_S2] = X.s2; cb[CB_L2] = X.l2; cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end;
+        cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = X.D.root_deg;
+    }
+    __syncwarp();
+}
+// A step's m tokens, then the slot's control words.  On return, unless D.err is set, (ra, rb) is the record of s2 if l2 > 0 (also
+// stored in the control block).
 __device__ __forceinline__ void dyn_feed(DynChain& X, int32_t tok_first, const int32_t* toks, int m, uint32_t (*sh_run)[12]) {
     Dyn& D = X.D;
     const int lane = D.lane;
+    NoEmit none;
     for (int base = 0; base < m && !D.err; base += 32) {
         const int i = base + lane;
         uint32_t tk = 0;
         if (i < m) tk = (uint32_t)(base == 0 ? tok_first : toks[i]);
-        root_precompute(D, tk, i < m);              // most walks end in the root table
-        SAM_COUNT(D.kc.rounds, 1);
-        const unsigned bucket_peers = __match_any_sync(FULL, D.pr_bucket);
-        const int cnt = min(32, m - base);
-        int j = 0;
-        while (j < cnt && !D.err) {
-            if (X.s2 == 0) {
-                const int r = dyn_fresh_run(D, tk, j, cnt, bucket_peers, X.last, X.ntok);
-                if (r > 0) { j += r; X.have = false; continue; }
-                if (D.err) break;
-            }
-            Pre pre;
-            pre.valid = false;
-            if (X.s2 != 0 && X.have) {
-                const int r = dyn_repeat_run(D, tk, j, cnt, X.last, X.ntok, X.s2, X.l2, X.ra, X.rb, pre, sh_run);
-                if (r > 0) { j += r; continue; }
-                if (D.err) break;
-            }
-            D.cur = j;
-            dyn_extend(D, __shfl_sync(FULL, tk, j), X.last, X.ntok, X.s2, X.l2, X.have, X.ra, X.rb, pre);
-            j++;
-        }
+        dyn_tokens(X, tk, min(32, m - base), sh_run, none);
     }
-    if (m > 0 && !D.err) {
-        // the newest state's record, without a transition yet
-        uint4* rl = rec_ptr(D, X.last);
-        uint32_t* cb = D.cb;
-        if (lane == 0) {
-            rl[0] = make_uint4(X.ntok, X.s2, X.ntok, 0);
-            rl[1] = make_uint4(0, 0, 0, 0);
-            cb[CB_NTOK] = X.ntok; cb[CB_NSTATES] = D.n_states; cb[CB_LAST] = X.last;
-            cb[CB_S2] = X.s2; cb[CB_L2] = X.l2; cb[CB_BLK_CUR] = D.blk_cur; cb[CB_BLK_END] = D.blk_end;
-            cb[CB_NRECSLABS] = D.n_rec_slabs; cb[CB_ROOTDEG] = D.root_deg;
-        }
-        __syncwarp();
-    }
+    if (m > 0 && !D.err) dyn_close(X);
     if (X.l2 > 0 && !D.err) SAM_COUNT(D.kc.rounds, 1);   // the draft
     if (X.l2 > 0 && !D.err && m > 0) {                  // the state moved: get its record, keep a copy
         if (!X.have) { const uint4* rs = rec_ptr(D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(D.kc.rounds, 1); }
@@ -956,8 +984,7 @@ __device__ __forceinline__ void write_failed_slot(const StepOut& o, int L, int b
 }
 
 // Choose the source (Section 3.2), read the draft, write the outputs: by a whole warp that has both sides' results
-// (match length, state, first end position; ntok: the text's length).  READ: how the slot's own text is read (gather_draft).
-template <int READ>
+// (match length, state, first end position; ntok: the text's length).  Other blocks of the grid may have written the text.
 __device__ __forceinline__ void write_slot(const StepArgs& A, const StepOut& o, int b, int lane, int l1, int s1, int64_t e1,
                                            int l2, int s2, int64_t e2, int64_t ntok) {
     const int L = A.L;
@@ -970,7 +997,7 @@ __device__ __forceinline__ void write_slot(const StepArgs& A, const StepOut& o, 
     if (src != SAM_SRC_NONE) {
         const int64_t e = use_static ? e1 : e2, room = (use_static ? A.S.n_tokens : ntok) - e;
         dl = (int)(room < L ? (room < 0 ? 0 : room) : L);
-        gather_draft<READ>(use_static ? A.S.corpus : A.W.text + (size_t)b * A.W.text_stride, e, dl, L, lane, d);
+        gather_draft<2>(use_static ? A.S.corpus : A.W.text + (size_t)b * A.W.text_stride, e, dl, L, lane, d);
         dl = cut_at_stop(d, dl, lane, A.W.stop_token);
     }
 #pragma unroll
@@ -1545,7 +1572,7 @@ __device__ __forceinline__ void split_epilogue(const StepArgs& A, int b, int lan
         if (lane == 0) cb[CB_STATUS] = (uint32_t)err_s;
         return;
     }
-    write_slot<2>(A, o, b, lane, (int)__shfl_sync(FULL, cw, CB_L1), (int)__shfl_sync(FULL, cw, CB_S1), (int64_t)__shfl_sync(FULL, cw2, CB_REC1 + 2 - 32),
+    write_slot(A, o, b, lane, (int)__shfl_sync(FULL, cw, CB_L1), (int)__shfl_sync(FULL, cw, CB_S1), (int64_t)__shfl_sync(FULL, cw2, CB_REC1 + 2 - 32),
                   (int)__shfl_sync(FULL, cw, CB_L2), (int)__shfl_sync(FULL, cw, CB_S2), (int64_t)__shfl_sync(FULL, cw2, CB_REC2 + 2 - 32),
                   (int64_t)__shfl_sync(FULL, cw, CB_NTOK));
 }
@@ -1860,51 +1887,26 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
 
 // ------------------------------------------------------------------ many steps in one launch
 // sam_run_steps has every step's tokens at hand and slots never meet, so a slot goes through all its steps without waiting
-// for the slowest slot of each: a launch per step costs that slowest slot (at 4096 slots 29 us a step, of which the
-// average slot needs 5), the launch, and the reads that start a step (control words, first tokens).  Both match
-// states and the automaton's head stay in registers, the next step's tokens are read a step ahead.
+// for the slowest slot of each, its two sides without waiting for each other (a warp each), and both through the tokens of as many
+// steps as fit 32 lanes at a time: what a step costs beside its tokens (the round that looks them all up in the root table, the
+// control words, runs of tokens cut short, the static match's rounds) is then paid once for some nine steps of 3.3 tokens.
+// Both sides leave each step's result in the step's own outputs, and sam_run_finish_kernel, which no chain waits for, chooses the
+// sources and reads the drafts: 32 rows a warp, eight rows' reads under way together.
+// us a step, step after step on each side (static sides on a few lanes, or three warps a slot up to 296 slots) -> so: 200 slots
+// 2.35 -> 1.3, 1000 slots 6.1 -> 2.3, 4096 slots 7.1 -> 3.9, 16384 slots 20.1 -> 12.5.
+// Bound by the dynamic sides' rounds of reads and how many warps fit (16 an SM with 128 registers, nothing spilled; 20 with 96:
+// 4 % slower at 4096 slots).
+// What the two sides leave: match_len, state and status as they will be; the static side's first end position (or minus its
+// error) in draft_len, the dynamic side's in source, the text length in the first word of the draft.
 struct RunArgs {
     StepArgs A;
     int32_t n_steps, keep;       // keep: the outputs have room for every step
-};
-
-// Whether a step's tokens can be fed to a slot: its status if not (the whole step is checked before any state changes).
-__device__ __forceinline__ int check_step(const StepArgs& A, int lane, int32_t tok_first, const int32_t* toks, int m, uint32_t ntok) {
-    if (m < 0 || m > A.stride) return SAM_SEQ_BAD_COUNT;
-    if ((int64_t)ntok + m > A.W.max_seq_len) return SAM_SEQ_CAPACITY;
-    const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
-    bool bad = false;
-    for (int base = 0; base < m; base += 32) {
-        const int i = base + lane;
-        if (i < m) { const int t = base == 0 ? tok_first : toks[i]; bad |= t < 0 || t >= vocab; }
-    }
-    return __any_sync(FULL, bad) ? SAM_SEQ_BAD_TOKEN : 0;
-}
-
-// The rows of slot b, one step after the other, read a step ahead.
-struct RunRows {
-    const int32_t *toks, *counts;
-    int32_t tok, m;
-    __device__ __forceinline__ void start(const StepArgs& A, int b, int lane) {
-        toks = A.new_tokens + (size_t)b * A.stride; counts = A.counts + b;
-        fetch(A, lane);
-    }
-    __device__ __forceinline__ void fetch(const StepArgs& A, int lane) { m = *counts; tok = lane < A.stride ? toks[lane] : 0; }
-    __device__ __forceinline__ void next(const StepArgs& A, int lane, bool more) {
-        toks += (size_t)A.W.batch * A.stride; counts += A.W.batch;
-        if (more) fetch(A, lane);
-    }
 };
 
 struct StaticSide { uint32_t s, sf; int32_t l; uint4 ra, rb; };
 __device__ __forceinline__ void static_open(uint32_t cw, uint32_t cw2, StaticSide& T) {
     T.s = __shfl_sync(FULL, cw, CB_S1); T.sf = __shfl_sync(FULL, cw, CB_S1FLAG); T.l = (int32_t)__shfl_sync(FULL, cw, CB_L1);
     kept_record(cw2, CB_REC1, T.ra, T.rb);
-}
-__device__ __forceinline__ void static_feed(const StepArgs& A, int b, int lane, const RunRows& in, StaticSide& T, int& err) {
-    ChainCounts kc = {1, 0, 0, 0, 0};
-    static_advance<false>(A.S, lane, in.tok, in.toks, in.m, T.s, T.sf, T.l, T.ra, T.rb, err, kc, []() {});
-    flush_counts(b, lane, true, kc, in.m);
 }
 __device__ __forceinline__ void static_close(uint32_t* cb, int lane, uint32_t ntok, const StaticSide& T) {
     if (lane == 0) {
@@ -1913,197 +1915,358 @@ __device__ __forceinline__ void static_close(uint32_t* cb, int lane, uint32_t nt
     }
 }
 
-// Batches of more than two slots per SM: what counts is how much one resident warp carries.
-//   - The static side of a slot needs little help from other lanes (a state is one 32-byte record, a hash bucket eight
-//     16-byte entries), so a few LANES carry it, each group at its own pace (run_static_lanes).
-//   - The dynamic side has a warp per slot, without the static side's registers and waits (sam_run_split_kernel).
-//   - Both leave each step's result in the step's own outputs, and sam_run_finish_kernel, which no chain waits for, chooses the
-//     sources and reads the drafts: 32 rows a warp, eight rows' reads under way together.
-// Per step (a warp for both sides of a slot, before): 1000 slots 18.5 -> 7.3 us, 4096 slots 16.2 -> 7.2, 16384 slots
-// 58 -> 20.3.  Bound by the static chains up to 4096 slots (5 us a step), by the dynamic side's warps beyond.
-// What the two sides leave: match_len, state and status as they will be; the static side's first end position (or minus its
-// error) in draft_len, the dynamic side's in source, the text length in the first word of the draft.
-
-// The static side of 32 / G slots, G lanes each: Transfer (Algorithm 1) for every token of every step.  A pass of the loop
-// is one round of reads: the record of the state, the home bucket of (state, token) if it has hashed transitions, the root-row
-// entry of the token (used when the walk reaches the root in this pass), the token after it and the next step's count.
-// A step's first end position is in the record that the next step's first pass reads, so it is written then.
-// The lanes of a slot hold its state alike; each reads its share of the bucket's entries.
-template <int G>
-__device__ __forceinline__ void run_static_lanes(const RunArgs& R, int w, int lane) {
-    constexpr int E = SAM_HASH_BUCKET / G;
+// A chunk: whole steps (of one with more than 32 tokens a part), planned a chunk ahead so that its tokens are there when it begins.
+struct RunChunk {
+    int32_t tok, step, own;      // this lane's token and the step it belongs to; if it ends the step: that step and those without tokens after it
+    int32_t n_tok, n_steps, lead;         // tokens and steps in it; steps without tokens before the first that has some
+    uint32_t starts;             // where steps begin
+    int32_t refuse;              // why the step behind it is refused (0: it is not, or there is none)
+    int32_t taken;               // tokens of the step behind it that it holds (of a step of more than 32: the first 32)
+};
+__device__ __forceinline__ int32_t run_counts(const RunArgs& R, int b, int lane, int i) {
+    return i + lane < R.n_steps ? R.A.counts[(size_t)(i + lane) * R.A.W.batch + b] : 0;
+}
+// The chunk that begins with step i, of which `taken` tokens are done, whose slot had ntok tokens before it; m: lane k holds the
+// count of step i + k.
+__device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, int i, int taken, uint32_t ntok, int m, int32_t* sh_map) {
     const StepArgs& A = R.A;
-    const SamStaticView& S = A.S;
-    const int sub = lane % G, group = lane - sub, b = (w * 32 + lane) / G;
-    const bool live = b < A.W.batch;
-    uint32_t* cb = A.W.ctrl + (size_t)(live ? b : 0) * SAM_CTRL_WORDS;
-    const int32_t* row = A.new_tokens + (size_t)(live ? b : 0) * A.stride;
-    const int32_t* cnt = A.counts + (live ? b : 0);
-    const size_t row_step = (size_t)A.W.batch * A.stride;
-    uint32_t s = 0, sf = 0, ntok = 0;
-    int32_t l = 0;
-    uint4 a = make_uint4(0, 0, 0, 0), bb = a;
-    bool active = live && R.n_steps > 0;
-    if (live) {
-        s = cb[CB_S1]; l = (int32_t)cb[CB_L1]; sf = cb[CB_S1FLAG]; ntok = cb[CB_NTOK_S];
-        a = *reinterpret_cast<const uint4*>(cb + CB_REC1); bb = *reinterpret_cast<const uint4*>(cb + CB_REC1 + 4);
-        if (cb[CB_STATUS] != 0) active = false;
-    }
-    const bool was = active;
-    bool have = s != 0, need_len = false, begin = true, bad = false;
-    uint32_t s0 = s, sf0 = sf; int32_t l0 = l;             // as the step found it: a refused step changes nothing
-    int i = 0, j = 0, m = 0, due = 0, err = 0, guard = 0;  // due: the first step whose result has not been written
-    int32_t t = 0, tn = row[0], mn = *cnt;
-    [[maybe_unused]] ChainCounts kc = {1, 0, 0, 0, 0};
-    for (;;) {
-        if (active) {
-            // steps begin here: those without tokens pass by, the first with tokens is looked at
-            while (begin && i < R.n_steps) {
-                m = mn; t = tn;
-                if (m < 0 || m > A.stride || (int64_t)ntok + m > A.W.max_seq_len || (m > 0 && (t < 0 || t >= S.vocab))) { bad = true; break; }
-                if (m > 0) { begin = false; j = 0; s0 = s; sf0 = sf; l0 = l; guard = l + 2 * m + 4; break; }
-                i++; row += row_step; cnt += A.W.batch;
-                if (i < R.n_steps) { mn = *cnt; tn = row[0]; }
-            }
-            if (bad || i >= R.n_steps) active = false;
-        }
-        const bool owed = live && was && due < i;          // results that wait for the record of s
-        if (!__any_sync(FULL, active || owed)) break;
-        SAM_COUNT(kc.rounds, active ? 1 : 0);
-        // none of these reads is under a branch: a lane that does not need a line reads one that every such lane shares
-        const bool at_root = s == 0;
-        const bool want_rec = (active || owed) && !at_root && !have;
-        const bool want_bucket = active && !at_root && sf != 0;
-        uint32_t home = want_bucket ? sam_hash2(s, (uint32_t)t) & S.hash_mask : 0u;
-        const uint32_t re = __ldg(S.root_row + (active ? t : 0));
-        const bool last_tok = j + 1 >= m, more = i + 1 < R.n_steps;
-        tn = active ? (last_tok ? (more ? row[row_step] : 0) : row[j + 1]) : 0;
-        mn = active && more ? cnt[A.W.batch] : 0;
-        const size_t ri = want_rec ? (size_t)s : 0;
-        const uint4 ra = __ldg(S.rec + 2 * ri), rb = __ldg(S.rec + 2 * ri + 1);
-        uint4 ent[E];
+    RunChunk C;
+    C.tok = 0;
+    const int left = R.n_steps - i;
+    const bool counted = m >= 0 && m <= A.stride;
+    if (!counted) m = 0;
+    int upto = m;                                          // tokens up to this step's last
 #pragma unroll
-        for (int e = 0; e < E; e++) ent[e] = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + sub * E + e);
-        if (want_rec) { a = ra; bb = rb; have = true; }
-        if (owed) {
-            for (; due < i; due++) {
-                if (sub != 0 || (!R.keep && due + 1 < R.n_steps)) continue;
-                const StepOut o = step_out(A, R.keep ? due : 0);
-                o.match_len[2 * b] = l; o.draft_len[b] = l > 0 ? (int32_t)a.z : 0;
-                if (o.state) o.state[2 * b] = (int32_t)s;
-            }
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, upto, o); if (lane >= o) upto += t; }
+    const bool room = (int64_t)ntok + upto <= A.W.max_seq_len;
+    const unsigned no = ~__ballot_sync(FULL, lane < left && counted && room && upto <= 32);
+    const int n = no ? __ffs(no) - 1 : 32;
+    C.n_steps = n;
+    C.n_tok = n > 0 ? __shfl_sync(FULL, upto, n - 1) : 0;
+    C.refuse = n < 32 ? __shfl_sync(FULL, lane >= left ? 0 : !counted ? SAM_SEQ_BAD_COUNT : !room ? SAM_SEQ_CAPACITY : 0, n & 31) : 0;
+    C.taken = 0;
+    if (n == 0 && left > 0 && C.refuse == 0) {             // a step of more than 32 tokens, checked as a whole
+        const int len = __shfl_sync(FULL, m, 0);
+        const int32_t* row = A.new_tokens + ((size_t)i * A.W.batch + b) * A.stride;
+        C.step = i; C.own = 0; C.lead = 0; C.starts = 1;
+        if (taken == 0) {
+            const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
+            const int32_t t0 = row[lane], t1 = lane + 32 < len ? row[lane + 32] : 0;
+            if (__any_sync(FULL, t0 < 0 || t0 >= vocab || t1 < 0 || t1 >= vocab)) { C.refuse = SAM_SEQ_BAD_TOKEN; return C; }
         }
-        // the transition: from the record, or from the bucket and the buckets after it
-        uint32_t tgt = at_root ? SAM_NONE : inline_target(a, bb, (uint32_t)t);
-        bool search = want_bucket && tgt == SAM_NONE;      // (every reference to a state with hashed transitions carries the flag)
-        for (int probe = 1; __any_sync(FULL, search); probe++) {
-            uint32_t z = SAM_NONE;
-            bool empty = false;
-#pragma unroll
-            for (int e = 0; e < E; e++) {
-                if (ent[e].x == s && ent[e].y == (uint32_t)t) z = ent[e].z;
-                empty |= ent[e].x == SAM_NONE;
-            }
-            const unsigned in_group = (0xFFFFFFFFu >> (32 - G)) << group;
-            const unsigned hit = __ballot_sync(FULL, search && z != SAM_NONE) & in_group, gap = __ballot_sync(FULL, search && empty) & in_group;
-            const uint32_t found = __shfl_sync(FULL, z, hit ? __ffs(hit) - 1 : lane);
-            if (search) {
-                if (hit) tgt = found;
-                if (hit || gap || probe >= S.hash_max_probe) search = false;
-                else {
-                    home = (home + 1) & S.hash_mask;
-#pragma unroll
-                    for (int e = 0; e < E; e++) ent[e] = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + sub * E + e);
-                }
-            }
-        }
-        if (active) {
-            bool advance = false;
-            if (at_root) {                                 // at the root the match length is 0
-                if (re != SAM_NONE) { s = re & SAM_IDMASK; sf = re >> 31; l = 1; have = false; SAM_COUNT(kc.b, 1); } else l = 0;
-                advance = true;
-            } else {
-                if (need_len) { l = (int32_t)a.x; need_len = false; }
-                have = false;
-                if (tgt != SAM_NONE) { s = tgt & SAM_IDMASK; sf = tgt >> 31; l += 1; advance = true; SAM_COUNT(kc.b, 1); }
-                else {                                     // s <- link(s), l <- len(link(s))
-                    SAM_COUNT(kc.a, 1);
-                    s = a.y & SAM_IDMASK; sf = a.y >> 31;
-                    if (s == 0) {                          // the root either has the token or not: known already
-                        if (re != SAM_NONE) { s = re & SAM_IDMASK; sf = re >> 31; l = 1; SAM_COUNT(kc.b, 1); } else l = 0;
-                        advance = true;
-                    } else need_len = true;
-                    if (--guard < 0) { err = SAM_SEQ_WALK_LIMIT; bad = true; }
-                }
-            }
-            if (advance && !bad) {
-                if (++j < m) {
-                    t = tn;
-                    if (t < 0 || t >= S.vocab) bad = true;
-                } else {
-                    ntok += (uint32_t)m;
-                    i++; row += row_step; cnt += A.W.batch;
-                    begin = true;
-                }
-            }
-            if (bad) { active = false; s = s0; sf = sf0; l = l0; have = false; need_len = false; }
-        }
+        C.n_tok = min(32, len - taken);
+        C.tok = lane < C.n_tok ? row[taken + lane] : 0;
+        if (taken + C.n_tok == len) { C.n_steps = 1; C.own = lane == C.n_tok - 1 ? 1 : 0; } else C.taken = C.n_tok;
+        return C;
     }
-    if (!was || sub != 0) return;
-    if (err)
-        for (int k = i; k < R.n_steps; k++) if (R.keep || k + 1 == R.n_steps) step_out(A, R.keep ? k : 0).draft_len[b] = -err;
-    if (l > 0) {
-        if (!have) static_record(S, s, a, bb);
-        *reinterpret_cast<uint4*>(cb + CB_REC1) = a; *reinterpret_cast<uint4*>(cb + CB_REC1 + 4) = bb;
+    const bool some = lane < n && m > 0;
+    const unsigned filled = __ballot_sync(FULL, some);
+    if (some) sh_map[upto - m] = lane;
+    C.starts = __reduce_or_sync(FULL, some ? 1u << (upto - m) : 0u);
+    C.lead = filled ? __ffs(filled) - 1 : n;
+    __syncwarp();
+    const unsigned mine = C.starts & (0xFFFFFFFFu >> (31 - lane));
+    const int begin = mine ? 31 - __clz(mine) : 0, k = mine ? sh_map[begin] : 0;    // this lane's token: its step's first, and the step
+    const int len = __shfl_sync(FULL, m, k);
+    C.step = i + k; C.own = 0; C.tok = 0;
+    if (lane < C.n_tok) {
+        C.tok = A.new_tokens[((size_t)(i + k) * A.W.batch + b) * A.stride + (lane - begin)];
+        const unsigned after = filled & ~((2u << k) - 1u);
+        if (lane - begin == len - 1) C.own = (after ? __ffs(after) - 1 : n) - k;
     }
-    cb[CB_S1] = s; cb[CB_L1] = (uint32_t)l; cb[CB_S1FLAG] = sf; cb[CB_NTOK_S] = ntok;
-#ifdef SAM_COUNTERS
-    if (g_sam_counters && b < g_sam_counter_slots) {
-        unsigned long long* o = g_sam_counters + (size_t)b * SAM_N_COUNTERS;
-        o[SAM_CNT_STATIC_ROUNDS] += kc.rounds; o[SAM_CNT_STATIC_LINK_MOVES] += kc.a; o[SAM_CNT_STATIC_NEXT_MOVES] += kc.b;
-    }
-#endif
+    __syncwarp();
+    return C;
 }
 
-// Blocks [0, n_lane_blocks): the static sides, 32 slots each; the others: the dynamic side of one slot each.
-// G, the lanes of a static side: 1, 2, 4, 8 take 13.4, 8.2, 7.9, 8.4 us a step at 4096 slots (fewer lanes: a pass waits for
-// more lines and holds more registers) and 20.5, 21.4, 22.3, 25.0 at 16384 (more lanes: fewer warps for the dynamic sides).
-// 20 warps an SM: with 96 registers nothing spills (28 or 24 warps, 72 or 80 registers: 9 and 5 % slower).
-constexpr int run_lanes(int batch) { return batch <= 8192 ? 4 : 2; }
-template <int G>
-__global__ void __launch_bounds__(32, 20) sam_run_split_kernel(const __grid_constant__ RunArgs R) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
-    __shared__ __align__(16) uint32_t sh_run[32][12];
+// Its tokens have come: where one is outside the vocabulary the chunk, which begins with step i, ends before that step.
+__device__ __forceinline__ void run_cut(RunChunk& C, int lane, int i, int vocab) {
+    const unsigned wrong = __ballot_sync(FULL, lane < C.n_tok && (C.tok < 0 || C.tok >= vocab));
+    if (!wrong) return;
+    const int t = __ffs(wrong) - 1;
+    C.n_tok = 31 - __clz(C.starts & (0xFFFFFFFFu >> (31 - t)));
+    C.n_steps = __shfl_sync(FULL, C.step, t) - i;
+    C.refuse = SAM_SEQ_BAD_TOKEN;
+    if (lane >= C.n_tok) C.own = 0;
+}
+
+// What a slot's results are written with, and (in shared memory) what holds at the end of the last step that is done.
+struct RunEmit {
+    const RunArgs& R;
+    int b, lane;
+    int32_t step, own;           // of the chunk (this lane's)
+    unsigned ends;
+    uint32_t* done;              // text length, states, state of the whole text, s2, l2; the step after it
+    __device__ __forceinline__ void write(int first, int n, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok) const {
+        const StepArgs& A = R.A;
+        for (int i = first; i < first + n; i++) {
+            if (!R.keep && i + 1 != R.n_steps) continue;
+            const StepOut o = step_out(A, R.keep ? i : 0);
+            o.match_len[2 * b + 1] = (int32_t)l2; o.source[b] = (int32_t)e2; o.status[b] = 0;
+            o.draft[(size_t)b * A.L] = (int32_t)ntok;
+            if (o.state) o.state[2 * b + 1] = (int32_t)s2;
+        }
+    }
+    __device__ __forceinline__ void operator()(bool on, int from, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok, uint32_t last, uint32_t n_states) {
+        const int st = __shfl_sync(FULL, step, from);
+        int n = __shfl_sync(FULL, own, from);
+        if (!on) n = 0;
+        const unsigned ending = __ballot_sync(FULL, n > 0);
+        if (!ending) return;
+        if (n > 0) write(st, n, s2, l2, e2, ntok);
+        if (lane == 31 - __clz(ending)) { done[0] = ntok; done[1] = n_states; done[2] = last; done[3] = s2; done[4] = l2; done[5] = (uint32_t)(st + n); }
+        __syncwarp();
+    }
+};
+
+__device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, uint32_t (*sh_run)[12], int32_t* sh_map) {
     const StepArgs& A = R.A;
-    const int lane = threadIdx.x;
-    if ((int)blockIdx.x < A.n_lane_blocks) { run_static_lanes<G>(R, blockIdx.x, lane); return; }
-    const int b = (int)blockIdx.x - A.n_lane_blocks;
+    __shared__ uint32_t done[6];
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
-    RunRows in;
-    in.start(A, b, lane);
+    int m = run_counts(R, b, lane, 0);
     int status = (int)__shfl_sync(FULL, cw, CB_STATUS);
+    const bool fit = status == 0;
     DynChain X;
     kept_record(cw2, CB_REC2, X.ra, X.rb);
     dyn_open(A.W, b, lane, cb, cw, cw2, X);
-    for (int i = 0; i < R.n_steps; i++) {
-        const RunRows now = in;
-        in.next(A, lane, i + 1 < R.n_steps);
-        if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, X.ntok);
-        if (status == 0) {
-            X.D.kc = ChainCounts{1, 0, 0, 0, 0};
-            dyn_feed(X, now.tok, now.toks, now.m, sh_run);
+    const uint32_t ntok0 = X.ntok;
+    RunEmit emit{R, b, lane, 0, 0, 0u, done};
+    const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
+    if (lane == 0) { done[0] = X.ntok; done[1] = X.D.n_states; done[2] = X.last; done[3] = X.s2; done[4] = X.l2; done[5] = 0; }
+    __syncwarp();
+    int i = 0;
+    RunChunk C;
+    if (fit) { C = run_plan(R, b, lane, 0, 0, X.ntok, m, sh_map); m = run_counts(R, b, lane, C.n_steps); }
+    while (status == 0 && i < R.n_steps) {
+        run_cut(C, lane, i, vocab);
+        const int next = i + C.n_steps;
+        RunChunk N = C;
+        if (C.refuse == 0 && next < R.n_steps) {
+            N = run_plan(R, b, lane, next, C.taken, X.ntok + (uint32_t)(C.n_tok - C.taken), m, sh_map);
+            if (N.n_steps > 0) m = run_counts(R, b, lane, next + N.n_steps);
+        }
+        if (C.lead > 0) {
+            if (lane == 0) { emit.write(i, C.lead, X.s2, X.l2, X.ra.z, X.ntok); done[5] = (uint32_t)(i + C.lead); }
+            __syncwarp();
+        }
+        if (C.n_tok > 0) {
+            emit.step = C.step; emit.own = C.own;
+            emit.ends = __ballot_sync(FULL, C.own > 0);
+            dyn_tokens(X, (uint32_t)C.tok, C.n_tok, sh_run, emit);
             status = X.D.err;
+            if (status != 0) break;
         }
-        if (lane == 0 && (R.keep || i + 1 == R.n_steps)) {
-            const StepOut o = step_out(A, R.keep ? i : 0);
-            o.match_len[2 * b + 1] = (int32_t)X.l2; o.source[b] = (int32_t)X.ra.z; o.status[b] = status;
-            o.draft[(size_t)b * A.L] = (int32_t)X.ntok;
-            if (o.state) o.state[2 * b + 1] = (int32_t)X.s2;
-        }
+        i = next;
+        status = C.refuse;
+        C = N;
     }
-    // (the slot's status is the finish kernel's to write: its static side may begin after this)
+    if (status != 0)
+        for (int k = (int)done[5] + lane; k < R.n_steps; k += 32) if (R.keep || k + 1 == R.n_steps) step_out(A, R.keep ? k : 0).status[b] = status;
+    if (X.D.err) {                                         // the slot is left as the last step that was done left it
+        if (lane == 0) {
+            cb[CB_NTOK] = done[0]; cb[CB_NSTATES] = done[1]; cb[CB_LAST] = done[2]; cb[CB_S2] = done[3]; cb[CB_L2] = done[4];
+            cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end; cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = X.D.root_deg;
+        }
+    } else if (X.ntok != ntok0) {
+        dyn_close(X);
+        if (X.l2 > 0 && lane == 0) { reinterpret_cast<uint4*>(cb + CB_REC2)[0] = X.ra; reinterpret_cast<uint4*>(cb + CB_REC2)[1] = X.rb; }
+    }
+}
+
+// The static side of a slot, a chunk of whole steps at a time: the longest suffix that occurs in the corpus, at the end of each step.
+//   - All suffixes that begin in the chunk are walked side by side from the root, one lane each, a token a round.  Where
+//     the text is new to the corpus they end after two or three tokens, and a chunk of nine steps is done in as many rounds.
+//   - One lane is the chain instead, a match that follows suffix links (Algorithm 1): at first the match so far.  It lives until what
+//     is left of it begins at token `base` or later, where the walks are.
+//   - A match that goes on along a passage of the corpus takes its tokens in one round (static_follow).  A walk that has done
+//     so is the chain from then on, and the walks that began before its end are part of it.
+// What holds at the end of a step is what the earliest suffix that reaches it says: a walk leaves its result when the record that it
+// goes on from is there; walks that began earlier come there later, except that the chain may be ahead: up to `base` and as far as
+// it has come (`sure`) only it has a say.
+struct RunResult { uint32_t s; int32_t l, e1; };
+
+// A run of transitions of a match in state s (record a, b), taken in one round by the whole warp, as static_run takes it; n: tokens
+// that may be taken, lane k's is tkl.  Returns how many were; out (lane k): the result after k + 1 of them.
+__device__ __forceinline__ int static_follow(const SamStaticView& S, uint32_t s, const uint4& a, const uint4& b, int32_t l, uint32_t tkl, int n, int lane,
+                                             uint32_t& ref, RunResult& out) {
+    out.l = l + 1 + lane; out.s = 0; out.e1 = 0; ref = 0;
+    const uint32_t g = inline_target(a, b, __shfl_sync(FULL, tkl, 0));
+    bool ok = false;
+    if (a.x == a.z) {                                      // the state of a corpus prefix: the tokens are the corpus' own, or not
+        const int64_t e = (int64_t)a.z;
+        int32_t cx = -2;
+        if (lane < n && e + lane < S.n_tokens) { cx = __ldg(S.corpus + e + lane); ref = __ldg(S.pstate + e + lane); }
+        ok = lane < n && (uint32_t)cx == tkl;
+        out.s = ref & SAM_IDMASK; out.e1 = (int32_t)a.z + 1 + lane;
+    } else if (g != SAM_NONE) {                            // ids a constant apart are guessed: lane k reads the (k + 1)-th of them
+        const uint32_t d = (g & SAM_IDMASK) - s;
+        if (d != 1 && d != 2) return 0;
+        const uint32_t id = s + d * (uint32_t)(lane + 1);
+        uint4 ka = make_uint4(0, 0, 0, 0), kb = ka;
+        if (lane < n && (int64_t)id < S.n_states) static_record(S, id, ka, kb);
+        const uint32_t nx = inline_target(ka, kb, __shfl_down_sync(FULL, tkl, 1));         // on the next token
+        const uint32_t from = __shfl_up_sync(FULL, nx, 1);
+        ref = lane == 0 ? g : from;                        // the transition that leads to this lane's state
+        ok = lane < n && ref != SAM_NONE && (ref & SAM_IDMASK) == id;
+        out.s = id; out.e1 = (int32_t)ka.z;
+    }
+    const unsigned no = ~__ballot_sync(FULL, ok);
+    return no ? __ffs(no) - 1 : 32;
+}
+
+// One chunk: tk, n: its tokens; ends: the last tokens of its steps; T: the match, moved over the chunk (have: T's record is there; it
+// is on return, if T.l > 0).  res[k]: the result after token k, for the k in ends.
+__device__ __forceinline__ void static_chunk(const SamStaticView& S, uint32_t tk, int n, unsigned ends, int lane, StaticSide& T, RunResult* res, int& err) {
+    uint32_t re = SAM_NONE;
+    if (lane < n) re = __ldg(S.root_row + tk);
+    res[lane] = RunResult{0u, 0, 0};
+    __syncwarp();
+    int base = 0, sure = 0;
+    bool chain = T.s != 0 && lane == 0;
+    bool alive = chain || (lane < n && re != SAM_NONE), have = false, need_len = false;
+    bool came = true;                                      // by a transition, not by a link
+    uint32_t cs = re & SAM_IDMASK, csf = re >> 31;
+    int32_t cl = 1;
+    int pos = lane + 1;                                    // tokens taken
+    uint4 a = T.ra, b = T.rb;
+    if (chain) { cs = T.s; csf = T.sf; cl = T.l; pos = 0; have = true; }
+    int guard = T.l + 2 * n + 4;                           // link moves of the chain
+    for (;;) {
+        const unsigned arrived = __ballot_sync(FULL, alive && pos == n);
+        if (arrived && lane > __ffs(arrived) - 1) alive = false;          // an earlier suffix reaches the end
+        bool go = alive && (pos < n || !have);
+        if (!__any_sync(FULL, go)) break;
+        const uint32_t t = __shfl_sync(FULL, tk, pos & 31);
+        const bool want_bucket = go && pos < n && csf;
+        uint32_t home = 0;
+        uint4 ent[SAM_HASH_BUCKET];
+        if (want_bucket) {
+            home = sam_hash2(cs, t) & S.hash_mask;
+#pragma unroll
+            for (int e = 0; e < SAM_HASH_BUCKET; e++) ent[e] = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + e);
+        }
+        const bool fresh = go && !have;
+        if (fresh) static_record(S, cs, a, b);
+        if (go) {
+            have = true;
+            if (need_len) { cl = (int32_t)a.x; need_len = false; }
+            if (chain && pos - cl >= max(base, 1)) alive = false;        // begins where the walks do
+        }
+        go = go && alive && pos < n;
+        if (fresh && alive && came && pos > 0 && (ends >> (pos - 1) & 1u) && (chain || pos > sure)) res[pos - 1] = RunResult{cs, cl, (int32_t)a.z};
+        uint32_t tgt = SAM_NONE;
+        if (go) tgt = inline_target(a, b, t);
+        // the earliest suffix there is, along the corpus as far as it goes
+        const unsigned live = __ballot_sync(FULL, alive), apart = (tgt & SAM_IDMASK) - cs;
+        const bool may = go && (chain || cl >= 3) && (a.x == a.z ? tgt != SAM_NONE || csf : tgt != SAM_NONE && (apart == 1 || apart == 2));
+        if (live && __shfl_sync(FULL, may, __ffs(live) - 1)) {
+            const int c = __ffs(live) - 1, p0 = __shfl_sync(FULL, pos, c);
+            uint32_t ref;
+            RunResult out;
+            const int r = static_follow(S, __shfl_sync(FULL, cs, c), shfl4(a, c), shfl4(b, c), __shfl_sync(FULL, cl, c),
+                                        __shfl_sync(FULL, tk, (p0 + lane) & 31), n - p0, lane, ref, out);
+            if (r > 0) {
+                if (lane < r && (ends >> (p0 + lane) & 1u)) res[p0 + lane] = out;
+                base = sure = p0 + r;
+                const uint32_t to = __shfl_sync(FULL, ref, r - 1);
+                if (lane == c) { chain = came = true; cs = to & SAM_IDMASK; csf = to >> 31; cl += r; pos = base; have = go = false; }
+                else if (lane < base) alive = go = false;
+            }
+        }
+        if (go) {
+            if (tgt == SAM_NONE && want_bucket) {          // (every reference to a state with hashed transitions carries the flag)
+                for (int probe = 1;; probe++) {
+                    bool empty = false;
+#pragma unroll
+                    for (int e = 0; e < SAM_HASH_BUCKET; e++) {
+                        if (ent[e].x == cs && ent[e].y == t) tgt = ent[e].z;
+                        empty |= ent[e].x == SAM_NONE;
+                    }
+                    if (tgt != SAM_NONE || empty || probe >= S.hash_max_probe) break;
+                    home = (home + 1) & S.hash_mask;
+#pragma unroll
+                    for (int e = 0; e < SAM_HASH_BUCKET; e++) ent[e] = __ldg(S.hash + (size_t)home * SAM_HASH_BUCKET + e);
+                }
+            }
+            have = came = false;
+            if (tgt != SAM_NONE) { cs = tgt & SAM_IDMASK; csf = tgt >> 31; cl++; pos++; came = true; }
+            else if (!chain) alive = false;
+            else {                                         // s <- link(s), l <- len(link(s))
+                cs = a.y & SAM_IDMASK; csf = a.y >> 31;
+                if (cs != 0) need_len = true;
+                else if (pos == 0 && re != SAM_NONE) { cs = re & SAM_IDMASK; csf = re >> 31; cl = 1; pos = 1; came = true; }
+                else alive = false;
+                if (--guard < 0) { err = SAM_SEQ_WALK_LIMIT; alive = false; }
+            }
+        }
+        const unsigned ahead = __ballot_sync(FULL, alive && chain);
+        if (ahead) { const int c = __ffs(ahead) - 1; sure = max(sure, __shfl_sync(FULL, need_len ? 0 : pos, c)); }
+        __syncwarp();
+    }
+    err = (int)__reduce_max_sync(FULL, (uint32_t)err);
+    const unsigned left = __ballot_sync(FULL, alive);
+    if (!left) { T.s = 0; T.sf = 0; T.l = 0; return; }
+    const int first = __ffs(left) - 1;
+    T.s = __shfl_sync(FULL, cs, first); T.sf = __shfl_sync(FULL, csf, first); T.l = __shfl_sync(FULL, cl, first);
+    T.ra = shfl4(a, first); T.rb = shfl4(b, first);
+}
+
+__device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, int32_t* sh_map, RunResult* res) {
+    const StepArgs& A = R.A;
+    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
+    const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
+    int m = run_counts(R, b, lane, 0);
+    if (__shfl_sync(FULL, cw, CB_STATUS) != 0) return;
+    uint32_t ntok = __shfl_sync(FULL, cw, CB_NTOK_S);
+    StaticSide T;
+    static_open(cw, cw2, T);
+    auto write = [&](int first, int n, uint32_t s, int32_t l, int32_t e1) {
+        for (int i = first; i < first + n; i++) {
+            if (!R.keep && i + 1 != R.n_steps) continue;
+            const StepOut o = step_out(A, R.keep ? i : 0);
+            o.match_len[2 * b] = l; o.draft_len[b] = l > 0 ? e1 : 0;
+            if (o.state) o.state[2 * b] = (int32_t)s;
+        }
+    };
+    int i = 0, err = 0;
+    RunChunk C = run_plan(R, b, lane, 0, 0, ntok, m, sh_map);
+    m = run_counts(R, b, lane, C.n_steps);
+    while (i < R.n_steps) {
+        run_cut(C, lane, i, A.S.vocab);
+        const int next = i + C.n_steps;
+        RunChunk N = C;
+        if (C.refuse == 0 && next < R.n_steps) {
+            N = run_plan(R, b, lane, next, C.taken, ntok + (uint32_t)(C.n_tok - C.taken), m, sh_map);
+            if (N.n_steps > 0) m = run_counts(R, b, lane, next + N.n_steps);
+        }
+        if (C.lead > 0 && lane == 0) write(i, C.lead, T.s, T.l, (int32_t)T.ra.z);
+        if (C.n_tok > 0) {
+            static_chunk(A.S, (uint32_t)C.tok, C.n_tok, __ballot_sync(FULL, C.own > 0), lane, T, res, err);
+            if (err) break;
+            __syncwarp();
+            if (C.own > 0) write(C.step, C.own, res[lane].s, res[lane].l, res[lane].e1);
+            __syncwarp();
+        }
+        ntok += (uint32_t)C.n_tok;
+        i = next;
+        if (C.refuse) break;
+        C = N;
+    }
+    if (err)
+        for (int k = i + lane; k < R.n_steps; k += 32) if (R.keep || k + 1 == R.n_steps) step_out(A, R.keep ? k : 0).draft_len[b] = -err;
+    static_close(cb, lane, ntok, T);
+}
+
+// Blocks of one warp: the dynamic side of each slot, then, with a static automaton, the static side of each slot.
+__global__ void __launch_bounds__(32, 16) sam_run_split_kernel(const __grid_constant__ RunArgs R) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    __shared__ __align__(16) uint32_t sh_run[32][12];
+    __shared__ int32_t sh_map[32];
+    const int lane = threadIdx.x, B = R.A.W.batch;
+    if ((int)blockIdx.x < B) run_dynamic(R, (int)blockIdx.x, lane, sh_run, sh_map);
+    else run_static(R, (int)blockIdx.x - B, lane, sh_map, reinterpret_cast<RunResult*>(&sh_run[0][0]));
+    // (the slot's status is the finish kernel's to write: its other side may begin after this)
 }
 
 constexpr int FINISH_ROWS = 8;                             // rows whose reads a warp has under way together
@@ -2175,87 +2338,6 @@ __global__ void __launch_bounds__(128) sam_run_finish_kernel(const __grid_consta
             }
         }
     if (live) A.draft_len[r] = cut;
-}
-
-// Three warps per slot: the static side, the dynamic side, and one that writes the outputs.  For batches that leave
-// the GPU room: each side goes on with its next step at once, at most RUN_RING steps ahead of the outputs.
-constexpr int RUN_RING = 4;
-__device__ __forceinline__ void run_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void run_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-
-__global__ void __launch_bounds__(96, 4) sam_run_block_kernel(const __grid_constant__ RunArgs R) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
-    __shared__ __align__(16) uint32_t sh_run[32][12];
-    __shared__ __align__(16) int4 from_static[RUN_RING], from_dynamic[RUN_RING];   // (l, s, first end position, error or text length)
-    __shared__ int32_t dyn_status[RUN_RING];
-    const StepArgs& A = R.A;
-    const int b = blockIdx.x, lane = threadIdx.x & 31, role = threadIdx.x >> 5;
-    uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
-    const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
-    const int status0 = (int)__shfl_sync(FULL, cw, CB_STATUS);
-    uint32_t ntok = __shfl_sync(FULL, cw, CB_NTOK);
-    __syncthreads();                                     // all three have the slot as it was
-    // barriers: 1 + r, a side's result is in ring entry r (both sides arrive); 5 + r and 9 + r, the entry has been
-    // read and the static or the dynamic side may use it again
-    if (role == 2) {
-        int status = status0;
-        for (int i = 0; i < R.n_steps; i++) {
-            const int r = i % RUN_RING;
-            run_sync(1 + r, 96);
-            const int4 x = from_static[r], y = from_dynamic[r];
-            if (status == 0) status = dyn_status[r] ? dyn_status[r] : x.w;
-            if (i + RUN_RING < R.n_steps) { run_arrive(5 + r, 64); run_arrive(9 + r, 64); }
-            const StepOut o = step_out(A, R.keep ? i : 0);
-            if (status != 0) write_failed_slot(o, A.L, b, lane, status);
-            else write_slot<0>(A, o, b, lane, x.x, x.y, (int64_t)x.z, y.x, y.y, (int64_t)y.z, (int64_t)y.w);
-        }
-        if (lane == 0 && status != status0) cb[CB_STATUS] = (uint32_t)status;
-        return;
-    }
-    RunRows in;
-    in.start(A, b, lane);
-    int status = status0;
-    if (role == 0) {
-        StaticSide T;
-        static_open(cw, cw2, T);
-        for (int i = 0; i < R.n_steps; i++) {
-            const int r = i % RUN_RING;
-            const RunRows now = in;
-            in.next(A, lane, i + 1 < R.n_steps);
-            if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, ntok);
-            int err = 0;
-            if (status == 0) {
-                if (A.has_static) static_feed(A, b, lane, now, T, err);
-                ntok += (uint32_t)now.m;
-                status = err;
-            }
-            if (i >= RUN_RING) run_sync(5 + r, 64);
-            if (lane == 0) from_static[r] = make_int4(T.l, (int)T.s, (int)T.ra.z, err);
-            __syncwarp();
-            run_arrive(1 + r, 96);
-        }
-        if (A.has_static && status0 == 0) static_close(cb, lane, ntok, T);
-    } else {
-        DynChain X;
-        kept_record(cw2, CB_REC2, X.ra, X.rb);
-        dyn_open(A.W, b, lane, cb, cw, cw2, X);
-        for (int i = 0; i < R.n_steps; i++) {
-            const int r = i % RUN_RING;
-            const RunRows now = in;
-            in.next(A, lane, i + 1 < R.n_steps);
-            if (status == 0) status = check_step(A, lane, now.tok, now.toks, now.m, X.ntok);
-            if (status == 0) {
-                X.D.kc = ChainCounts{1, 0, 0, 0, 0};
-                dyn_feed(X, now.tok, now.toks, now.m, sh_run);
-                status = X.D.err;
-            }
-            if (i >= RUN_RING) run_sync(9 + r, 64);
-            if (lane == 0) { from_dynamic[r] = make_int4((int)X.l2, (int)X.s2, (int)X.ra.z, (int)X.ntok); dyn_status[r] = status; }
-            __syncwarp();
-            run_arrive(1 + r, 96);
-        }
-    }
 }
 
 // A batch larger than the GPU holds at once runs in waves, and a step is as long as its last block: a
@@ -2382,8 +2464,7 @@ int split_kernel_setup(int device) {
     cudaError_t e = (cudaError_t)g_split_setup(device, []() -> int {
         cudaError_t e = cudaFuncSetAttribute(sam_step_split_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(order_slots_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel<4>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel<2>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(sam_run_split_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
         return (int)e;
     });
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
@@ -2526,10 +2607,6 @@ int sam_launch_fetch(const sam_batch* b, const int32_t* rows, const int32_t* cou
     return SAM_OK;
 }
 
-// Steps of sam_run_steps in one launch.  Up to two slots per SM three warps a slot are faster (256 slots 2.6 against 3.4 us a
-// step), from there on what the two sides cost in throughput counts (600 slots 4.9 against 4.4, 500 slots of c4's kind 9.7 against 7.2).
-constexpr int SAM_RUN_BLOCK_MAX_BATCH = 296;
-
 int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps, int32_t L, int32_t keep,
                    int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status,
                    cudaStream_t stream) {
@@ -2549,28 +2626,28 @@ int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)b->view.batch); cfg.stream = stream; cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.stream = stream; cfg.attrs = attr; cfg.numAttrs = 1;
     cudaError_t e;
-    if (b->view.batch <= SAM_RUN_BLOCK_MAX_BATCH) {
-        cfg.blockDim = dim3(96);
-        e = cudaLaunchKernelEx(&cfg, sam_run_block_kernel, R);
-    } else {
-        int rc = split_kernel_setup(b->device);
-        if (rc) return rc;
-        const int lanes = run_lanes(b->view.batch);
-        A.n_lane_blocks = A.has_static ? (int)(((int64_t)b->view.batch * lanes + 31) / 32) : 0;
-        cfg.gridDim.x += (unsigned)A.n_lane_blocks; cfg.blockDim = dim3(32);
-        e = lanes == 4 ? cudaLaunchKernelEx(&cfg, sam_run_split_kernel<4>, R) : cudaLaunchKernelEx(&cfg, sam_run_split_kernel<2>, R);
-        const int64_t rows = (int64_t)b->view.batch * (keep ? n_steps : 1);
-        cfg.gridDim = dim3((unsigned)((rows + 127) / 128)); cfg.blockDim = dim3(128);
-        if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, sam_run_finish_kernel, R);
-    }
+    int rc = split_kernel_setup(b->device);
+    if (rc) return rc;
+    cfg.gridDim = dim3((unsigned)b->view.batch * (A.has_static ? 2u : 1u)); cfg.blockDim = dim3(32);
+    e = cudaLaunchKernelEx(&cfg, sam_run_split_kernel, R);
+    const int64_t rows = (int64_t)b->view.batch * (keep ? n_steps : 1);
+    cfg.gridDim = dim3((unsigned)((rows + 127) / 128)); cfg.blockDim = dim3(128);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, sam_run_finish_kernel, R);
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }
     return SAM_OK;
 }
 
-// A launch per step where rows may hold prompts (the whole-text build has a kernel of its own), else one for all.
-bool sam_runs_in_one_launch(int32_t stride, int32_t n_steps) { return n_steps > 1 && stride < SAM_PREFILL_MIN; }
+// A launch per step where rows may hold prompts (the whole-text build has a kernel of its own), else one for all.  (The counters
+// are the step kernels', one step at a time.)
+bool sam_runs_in_one_launch(int32_t stride, int32_t n_steps) {
+#ifdef SAM_COUNTERS
+    return false;
+#else
+    return n_steps > 1 && stride < SAM_PREFILL_MIN;
+#endif
+}
 
 extern "C" int sam_counters_available(void) {
 #ifdef SAM_COUNTERS

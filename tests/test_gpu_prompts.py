@@ -401,3 +401,61 @@ def test_prompts_at_the_edges_of_the_build_blocks(P, B, n):
     got, batch = gpu_run(P, st, VOCAB, rows[:, :n], rows[None, :, n:].copy(), counts, L, n + 8)
     assert_same(got, ref)
     assert_dynamic_automata_equal(batch, ob, range(0, B, 7), n + 8)
+
+
+def _replayed(P, st, B, vocab, msl, toks, counts, L, **more):
+    """The same steps replayed at once and one after the other: (outputs, outputs, batch, batch)."""
+    import torch
+    t, c = torch.from_numpy(toks).cuda(), torch.from_numpy(counts).cuda()
+    once, each = (P.Batch(st, B, msl, max_draft_len=L, vocab=vocab, **more) for _ in range(2))
+    a = once.run_steps(t, c, L, per_step=True).cpu()
+    rows = [each.step(t[i], c[i], L).cpu() for i in range(len(toks))]
+    return a, {k: np.stack([r[k] for r in rows]) for k in KEYS}, once, each
+
+
+@pytest.mark.parametrize("B", [1, 7, 150])
+@pytest.mark.parametrize("K,most", [(1, 1), (3, 3), (16, 16), (33, 33), (47, 47)])
+def test_replayed_chunks_of_steps(P, B, K, most):
+    """Steps of one token to more than a chunk holds, many without tokens, over texts of every kind: what a slot has at the end
+    of each step is the oracle's, wherever chunks, runs and passages of the corpus begin and end."""
+    rng = random.Random(100 * B + K)
+    base = [rng.randrange(400) for _ in range(6000)]
+    corpus = base + base[2000:4000] + base[1000:3000]
+    steps = max(6, 200 // most)
+    texts = np.array([_text(("corpus", "copies", "periodic", "few", "one", "many", "fibonacci")[b % 7], K * steps, rng, corpus) for b in range(B)], dtype=np.int32)
+    r = np.random.default_rng(B + K)
+    counts = np.where(r.random((steps, B)) < 0.25, 0, r.integers(0, most + 1, size=(steps, B))).astype(np.int32)
+    if B > 1:
+        counts[:, 1] = 0; counts[:, 2] = most               # a slot that takes nothing, one whose rows are full
+    toks = np.zeros((steps, B, K), dtype=np.int32)
+    for b in range(B):
+        at = np.concatenate([[0], np.cumsum(counts[:, b])])
+        for i in range(steps):
+            toks[i, b, :counts[i, b]] = texts[b, at[i]:at[i + 1]]
+    L, msl = 6, K * steps
+    st = P.StaticSam.build(np.array(corpus, dtype=np.int32), VOCAB)
+    ob = oracle.Batch(oracle.Sam(np.array(corpus, dtype=np.int32)), np.array(corpus, dtype=np.int32), B, VOCAB, msl)
+    ref = [ob.step(toks[i], counts[i], L, 8) for i in range(steps)]
+    got, each, once, _ = _replayed(P, st, B, VOCAB, msl, toks, counts, L)
+    for k in KEYS:
+        exp = np.stack([getattr(x, k) for x in ref])
+        assert np.array_equal(got[k], exp), (k, np.argwhere(got[k] != exp)[:3])
+        assert np.array_equal(each[k], exp), k
+    assert_dynamic_automata_equal(once, ob, range(0, B, 5), msl)
+
+
+def test_replayed_steps_that_run_out_of_room(P):
+    """A slot the pool has no slab left for fails at the same step, and is left as the step before left it, replayed or not."""
+    rng = random.Random(3)
+    B, K, steps, L, msl = 3, 11, 150, 4, 2000
+    toks = np.zeros((steps, B, K), dtype=np.int32)
+    toks[:, 0] = np.array(_text("copies", K * steps, rng, []), dtype=np.int32).reshape(steps, K)
+    counts = np.zeros((steps, B), dtype=np.int32)
+    counts[:, 0] = [rng.randint(0, K) for _ in range(steps)]
+    for slabs in (2, 3, 6):
+        got, each, once, one = _replayed(P, None, B, VOCAB, msl, toks, counts, L, pool_slabs=slabs, slab_bytes=8192)
+        for k in KEYS:
+            assert np.array_equal(got[k], each[k]), (slabs, k, np.argwhere(got[k] != each[k])[:3])
+        assert (got["status"][-1, 0] == 1) and (got["status"][:, 1:] == 0).all()
+        a, b = (x.dump(0, 4000, 8000) for x in (once, one))
+        assert a["n_tokens"] == b["n_tokens"] and a["n_states"] == b["n_states"]
