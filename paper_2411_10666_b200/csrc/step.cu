@@ -548,22 +548,28 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
 // solid transition, a root transition, the text — and none depends on another, so lanes j..j+r-1
 // do one token each at once.  A token qualifies if its root lookup was settled ahead of time as
 // "absent" and no earlier token of the run shares its home bucket (so slots and tokens differ).
-// Returns r (0 if token j does not qualify).
+// The token that ends the run is in it too if the root has it, by a solid transition: Expand for it is the same without the
+// root transition, and the match goes on from there.  (256 slots fed by verified drafts, a fifth of whose tokens are of this kind:
+// 19.3 -> 18.7 us a step; 300 slots with copied texts 11.9 -> 11.7.  Not in the kernel of 80 registers, where it costs more
+// spilled registers than it gives unless drafts are verified: 1000 slots 18.2 -> 18.5; nor in chunks of replayed steps.)
+// Returns the number of tokens (0: token j does not qualify); s2, l2: the match after them.
 template <class F>
 __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt, unsigned bucket_peers,
-                                             uint32_t& last, uint32_t& ntok, F& emit) {
+                                             uint32_t& last, uint32_t& ntok, uint32_t& s2, uint32_t& l2, F& emit) {
     const unsigned from_j = ~((1u << j) - 1u);
     const unsigned lt = (1u << D.lane) - 1u;
     const bool first_of_bucket = (bucket_peers & from_j & lt) == 0;
     const unsigned elig = __ballot_sync(FULL, D.pr_state == 2 && first_of_bucket && D.lane >= j && D.lane < cnt);
+    const unsigned known = F::seen ? __ballot_sync(FULL, D.pr_state == 1 && (D.pr_tgt & SAM_FLAG) && D.lane < cnt) : 0u;
     const unsigned gap = ~(elig >> j);
-    int r = gap ? __ffs(gap) - 1 : 32 - j;
+    const int fresh = gap ? __ffs(gap) - 1 : 32 - j;          // tokens that are new
+    int r = fresh + (F::seen && j + fresh < 32 ? (int)(known >> (j + fresh) & 1u) : 0);
     if (r <= 0) return 0;
     const uint32_t c0 = D.n_states;
     r = (int)ensure_recs(D, c0, (uint32_t)r);
     if (r == 0) return 0;
     const int idx = D.lane - j;
-    const bool mine = idx >= 0 && idx < r;
+    const bool mine = idx >= 0 && idx < r, is_new = F::seen ? mine && idx < fresh : mine;
     const uint32_t c = c0 + (uint32_t)idx;
     const uint32_t prev = idx == 0 ? last : c - 1;            // the state this token's transition leaves
     const uint32_t plen = ntok + (uint32_t)idx;               // its length = tokens before this one
@@ -573,16 +579,18 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
             rp[0] = make_uint4(plen, 0, plen, 1);             // link is the root: nothing was matched
             rp[1] = make_uint4(tk, c | SAM_FLAG, 0, 0);
         }
-        D.root[D.pr_slot] = make_uint2(tk, c | (plen == 0 ? SAM_FLAG : 0u));
+        if (is_new) D.root[D.pr_slot] = make_uint2(tk, c | (plen == 0 ? SAM_FLAG : 0u));
         D.text[plen] = (int32_t)tk;
         D.pstate[plen] = c;
     }
-    const unsigned run = ((r >= 32 ? 0u : (1u << r)) - 1u) << j;
+    const int n_new = F::seen ? min(r, fresh) : r;
+    const unsigned run = ((n_new >= 32 ? 0u : (1u << n_new)) - 1u) << j;
     if (bucket_peers & run) D.pr_state = 0;                   // those buckets changed
     __syncwarp();
-    SAM_COUNT(D.kc.a, 2 * r - (last == 0 ? 1 : 0));            // per token: the previous state's transition (none from the root) and the root's
-    emit(mine, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1);
-    D.n_states = c0 + r; D.root_deg += r;
+    SAM_COUNT(D.kc.a, r + n_new - (last == 0 ? 1 : 0));        // per token: the previous state's transition (none from the root) and the root's
+    emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1);
+    if (F::seen && r > n_new) { s2 = __shfl_sync(FULL, D.pr_tgt, j + n_new) & SAM_IDMASK; l2 = 1; }
+    D.n_states = c0 + r; D.root_deg += n_new;
     last = c0 + r - 1; ntok += r;
     return r;
 }
@@ -685,6 +693,22 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
         if (r < 2) return 0;
     }
 
+    // Most walks end where they begin: at a state (or the root) whose transition leads elsewhere than to q_k.  Earlier walks do not
+    // change that: they turn transitions from their own q to their own clone.  In long runs (chunks of replayed steps) lanes say so
+    // for all tokens at once where the state's transitions are inline or the root's entry is settled.  (1.5 % there; runs within a
+    // step are too short for it, 1 % the other way.)
+    unsigned walks = FULL;
+    if (F::chunks) {
+        const uint32_t known = __shfl_sync(FULL, D.pr_state, (j + lane) & 31), to = __shfl_sync(FULL, D.pr_tgt, (j + lane) & 31);
+        bool walk = true;
+        if (u == 0) walk = known == 0 || (known == 1 && (to & SAM_IDMASK) == ps);
+        else if (ua.w <= 2) {
+            const uint32_t at = inline_target(ua, ub, tkr);
+            walk = at == SAM_NONE || (at & SAM_IDMASK) == ps;              // (none: the walk reports it)
+        }
+        walks = __ballot_sync(FULL, walk);
+    }
+
     *reinterpret_cast<uint4*>(&stage[lane][0]) = ua;
     *reinterpret_cast<uint4*>(&stage[lane][4]) = ub;
     *reinterpret_cast<uint4*>(&stage[lane][8]) = make_uint4(tkr, ps, u, 0);
@@ -719,6 +743,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
 
     // the redirect walks, one after the other; what each needs was left in shared memory by its lane
     for (int k = 0; k < r && !D.err; k++) {
+        if (F::chunks && !(walks >> k & 1u)) continue;
         D.cur = j + k;
         const uint4 xa = *reinterpret_cast<const uint4*>(&stage[k][0]);
         const uint4 xb = *reinterpret_cast<const uint4*>(&stage[k][4]);
@@ -878,10 +903,18 @@ __device__ __forceinline__ void dyn_open(const SamBatchView& W, int b, int lane,
 // Expand (fused with the dynamic matcher's Transfer) for each of up to 32 tokens, one in each lane.  emit is called by the whole
 // warp whenever tokens are done, with what holds after them: (whether this lane has one, the lane that held its token, s2, l2,
 // first end position of s2, text length, state of the whole text, number of states); ends: the tokens for which it is wanted.
+// seen: runs of new tokens take the known one behind them (dyn_fresh_run).
+template <bool SEEN>
 struct NoEmit {
+    static constexpr bool chunks = false, seen = SEEN;
     static constexpr unsigned ends = 0;
     __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
 };
+template <class F>
+__device__ __forceinline__ void dyn_emit(DynChain& X, int j, F& emit) {    // after token j
+    if (X.l2 > 0 && !X.have) { const uint4* rs = rec_ptr(X.D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(X.D.kc.rounds, 1); }
+    emit(X.D.lane == j, X.D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, X.D.n_states);
+}
 template <class F>
 __device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, uint32_t (*sh_run)[12], F& emit) {
     Dyn& D = X.D;
@@ -891,8 +924,12 @@ __device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, ui
     int j = 0;
     while (j < cnt && !D.err) {
         if (X.s2 == 0) {
-            const int r = dyn_fresh_run(D, tk, j, cnt, bucket_peers, X.last, X.ntok, emit);
-            if (r > 0) { j += r; X.have = false; continue; }
+            const int r = dyn_fresh_run(D, tk, j, cnt, bucket_peers, X.last, X.ntok, X.s2, X.l2, emit);
+            if (r > 0) {
+                j += r;
+                X.have = false;
+                continue;
+            }
             if (D.err) break;
         }
         Pre pre;
@@ -904,10 +941,7 @@ __device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, ui
         }
         D.cur = j;
         dyn_extend(D, __shfl_sync(FULL, tk, j), X.last, X.ntok, X.s2, X.l2, X.have, X.ra, X.rb, pre);
-        if ((emit.ends >> j & 1u) && !D.err) {
-            if (X.l2 > 0 && !X.have) { const uint4* rs = rec_ptr(D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(D.kc.rounds, 1); }
-            emit(D.lane == j, D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, D.n_states);
-        }
+        if ((emit.ends >> j & 1u) && !D.err) dyn_emit(X, j, emit);
         j++;
     }
 }
@@ -926,10 +960,11 @@ __device__ __forceinline__ void dyn_close(DynChain& X) {
 }
 // A step's m tokens, then the slot's control words.  On return, unless D.err is set, (ra, rb) is the record of s2 if l2 > 0 (also
 // stored in the control block).
+template <bool SEEN>
 __device__ __forceinline__ void dyn_feed(DynChain& X, int32_t tok_first, const int32_t* toks, int m, uint32_t (*sh_run)[12]) {
     Dyn& D = X.D;
     const int lane = D.lane;
-    NoEmit none;
+    NoEmit<SEEN> none;
     for (int base = 0; base < m && !D.err; base += 32) {
         const int i = base + lane;
         uint32_t tk = 0;
@@ -1183,7 +1218,8 @@ __device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 64;" :::
 // VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
 // AHEAD: a third warp reads ahead of the dynamic side (read_ahead).
 // INLINE: the rows and counts came with the launch (sam_step_host).
-template <bool VERIFY, bool AHEAD, bool INLINE>
+// SEEN: dyn_feed's.
+template <bool VERIFY, bool AHEAD, bool INLINE, bool SEEN>
 __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_tokens, const int32_t* counts) {
     // Programmatic dependent launch: this grid may be scheduled while the previous kernel of the stream
     // is still finishing.  Nothing is read before that kernel has completed and flushed; the kernel
@@ -1310,7 +1346,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
         DynChain X;
         X.ra = ra; X.rb = rb;
         dyn_open(A.W, b, lane, cb, cw, cw2, X);
-        dyn_feed(X, tok_first, toks, built ? 0 : m, sh_run);
+        dyn_feed<SEEN>(X, tok_first, toks, built ? 0 : m, sh_run);
         err = X.D.err; my_l = (int32_t)X.l2; my_s = (int32_t)X.s2;
         if (X.l2 > 0 && !err) {
             const int64_t e = (int64_t)X.ra.z;                  // min_endpos
@@ -1337,7 +1373,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
 // waves: 20.5 / 18.5) 17.0, 1180 slots with two warps a slot 19.2, with three 17.4.
 template <bool VERIFY, int AHEAD>
 __global__ void __launch_bounds__(AHEAD ? 96 : 64, AHEAD ? AHEAD : 10) sam_step_kernel(const __grid_constant__ StepArgs A) {
-    step_body<VERIFY, AHEAD != 0, false>(A, A.new_tokens, A.counts);
+    step_body<VERIFY, AHEAD != 0, false, VERIFY || AHEAD != 8>(A, A.new_tokens, A.counts);
 }
 
 // A host-array step whose rows and counts fit the launch's arguments: reading them from host memory, in the kernel's first
@@ -1346,7 +1382,7 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64, AHEAD ? AHEAD : 10) sam_step_
 constexpr int SAM_INLINE_WORDS = 896;                    // within 4 KB of arguments
 struct StepArgsInline { StepArgs A; int32_t in[SAM_INLINE_WORDS]; };                // rows, then counts
 __global__ void __launch_bounds__(96, 5) sam_step_inline_kernel(const __grid_constant__ StepArgsInline I) {
-    step_body<false, true, true>(I.A, I.in, I.in + (size_t)I.A.W.batch * I.A.stride);
+    step_body<false, true, true, true>(I.A, I.in, I.in + (size_t)I.A.W.batch * I.A.stride);
 }
 
 // Larger ones: the rows and counts are brought over in whole lines by this kernel, launched ahead of the step's.
@@ -1806,7 +1842,7 @@ __device__ __forceinline__ bool dynamic_slot(const StepArgs& A, int b, int lane,
         DynChain X;
         kept_record(cw2, CB_REC2, X.ra, X.rb);
         dyn_open(A.W, b, lane, cb, cw, cw2, X);
-        dyn_feed(X, tok_first, toks, m, sh_run);
+        dyn_feed<true>(X, tok_first, toks, m, sh_run);
         err = X.D.err;
         if (err) { status = err; fresh_fail = true; }
     }
@@ -1991,6 +2027,7 @@ __device__ __forceinline__ void run_cut(RunChunk& C, int lane, int i, int vocab)
 
 // What a slot's results are written with, and (in shared memory) what holds at the end of the last step that is done.
 struct RunEmit {
+    static constexpr bool chunks = true, seen = false;
     const RunArgs& R;
     int b, lane;
     int32_t step, own;           // of the chunk (this lane's)

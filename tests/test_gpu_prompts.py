@@ -459,3 +459,36 @@ def test_replayed_steps_that_run_out_of_room(P):
         assert (got["status"][-1, 0] == 1) and (got["status"][:, 1:] == 0).all()
         a, b = (x.dump(0, 4000, 8000) for x in (once, one))
         assert a["n_tokens"] == b["n_tokens"] and a["n_states"] == b["n_states"]
+
+
+@pytest.mark.parametrize("B", [64, 700, 1100, 1300])
+def test_runs_of_new_tokens_with_a_known_one_behind(P, B):
+    """Steps of r new tokens, a known one and what may follow it, for every r up to more than a warp holds: known by a solid
+    transition of the root or not (a clone), the first token of the text, a token of the step itself."""
+    import torch
+    rng = random.Random(B)
+    K, steps = 47, 4
+    toks, counts = np.zeros((steps, B, K), dtype=np.int32), np.zeros((steps, B), dtype=np.int32)
+    for b in range(B):
+        fresh = iter(rng.sample(range(1000, VOCAB), 300))
+        past = []
+        for i in range(steps):
+            row = [next(fresh) for _ in range(b % 42)]
+            if past:
+                row.append(past[0] if rng.random() < 0.2 else rng.choice(past))
+            elif row:
+                row.append(row[rng.randrange(len(row))])
+            row += [rng.choice(past + row + [3, 4]) for _ in range(rng.randint(0, 3))]
+            row = row[:K]
+            past += row
+            counts[i, b] = len(row)
+            toks[i, b, :len(row)] = row
+    L, msl = 5, K * steps
+    ob = oracle.Batch(None, None, B, VOCAB, msl)
+    batch = P.Batch(None, B, msl, max_draft_len=L, vocab=VOCAB)
+    for i in range(steps):
+        ref = ob.step(toks[i], counts[i], L, 8)
+        got = batch.step(torch.from_numpy(toks[i]).cuda(), torch.from_numpy(counts[i]).cuda(), L).cpu()
+        for k in KEYS:
+            assert np.array_equal(got[k], getattr(ref, k)), (i, k)
+    assert_dynamic_automata_equal(batch, ob, range(0, B, 13), msl)
