@@ -74,6 +74,14 @@ __device__ __forceinline__ bool pb_sync_or(int nt, bool x) {
 }
 
 // The tree over the sorted order: leaf j is h[j] << 16 | A[j], an inner node the two minima of its leaves.
+// The levels above 32 nodes of a level of `width` (a power of two), by a warp whose lane k has node at + k in v.
+__device__ __forceinline__ void pb_grow(const PbArrays& a, uint32_t v, int width, int at, int lane) {
+#pragma unroll
+    for (int l = 1; l <= 5; l++) {
+        v = __vminu2(v, __shfl_xor_sync(0xFFFFFFFFu, v, 1 << (l - 1)));
+        if ((lane & ((1 << l) - 1)) == 0 && lane < width && (width >> l) > 0) a.tree[(width >> l) + ((at + lane) >> l)] = v;
+    }
+}
 // First boundary to the left of sorted position j (inclusive) with h < l; acc: smallest A met, that position's included.
 __device__ __forceinline__ int pb_left(const PbArrays& a, int j, uint32_t l, uint32_t& acc) {
     int i = a.N2 + j;
@@ -265,7 +273,10 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
     uint32_t* key = reinterpret_cast<uint32_t*>(a.key);                              // [size]: tokens
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + 10 * (size_t)N2);             // [size]: positions, then where they begin
     uint16_t* at = reinterpret_cast<uint16_t*>(smem + 18 * (size_t)N2);              // [N2]: a position's table entry
-    for (int i = tid; i < size; i += nt) { key[i] = SAM_NONE; cnt[i] = 0; }
+    for (int i = tid; i < size >> 2; i += nt) {
+        reinterpret_cast<uint4*>(key)[i] = make_uint4(SAM_NONE, SAM_NONE, SAM_NONE, SAM_NONE);
+        reinterpret_cast<uint4*>(cnt)[i] = make_uint4(0, 0, 0, 0);
+    }
     if (tid == 0) sh.groups[0] = sh.groups[1] = sh.rows = 0;
     pb_sync(nt);
     for (int p = tid; p < n; p += nt) {
@@ -514,14 +525,17 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
                 }
             }
         }
-        a.tree[N2 + j] = (uint32_t)x << 16 | (uint32_t)p;
+        const uint32_t leaf = (uint32_t)x << 16 | (uint32_t)p;
+        a.tree[N2 + j] = leaf;
+        pb_grow(a, leaf, N2, j - lane, lane);                // (N2 and nt are whole warps)
     }
     pb_sync(nt);
     for (int j = tid; j < n; j += nt) a.rank[A[j] & ~PB_ALONE] = (uint16_t)j;
-    for (int width = N2 >> 1; width >= 1; width >>= 1) {
-        for (int i = tid; i < width; i += nt) a.tree[width + i] = __vminu2(a.tree[2 * (width + i)], a.tree[2 * (width + i) + 1]);
-        if (width > 32) pb_sync(nt); else __syncwarp();      // the last levels are warp 0's alone
-    }
+    if (w == 0)                                              // the other levels, of at most 256 nodes
+        for (int width = N2 >> 5; width > 1; width >>= 5) {
+            for (int at = 0; at < width; at += 32) pb_grow(a, a.tree[width + at + (lane & (width - 1))], width, at, lane);
+            __syncwarp();
+        }
     for (int j = tid; j < N2; j += nt) a.first[j] = 0xFFFFFFFFu;
     if (tid == 0) { sh.root_deg = 0; sh.err = 0; }
     if (tid < 16) sh.cls_n[tid] = 0;
@@ -547,12 +561,15 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         }
         a.canon[j] = (uint16_t)c;
     }
+    pb_sync(nt);
     for (bool moved = true; moved;) {                      // each boundary to the first of its interval, jumping over jumps
-        pb_sync(nt);
         bool m = false;
         for (int j = tid; j < n; j += nt) {
-            const uint32_t c = a.canon[j], d = a.canon[c];
-            if (c != d) { a.canon[j] = (uint16_t)d; m = true; }
+            const uint32_t was = a.canon[j];
+            uint32_t c = was, d = a.canon[c];
+            for (int k = 0; k < 3 && c != d; k++) { c = d; d = a.canon[c]; }
+            if (c != was) a.canon[j] = (uint16_t)c;
+            m |= c != d;
         }
         moved = pb_sync_or(nt, m);
     }
@@ -621,16 +638,22 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     const bool bitmap = W.root_cap <= 16 * N2;
     pb_sync(nt);
     if (bitmap) for (int j = tid; j < (N2 >> 1); j += nt) taken[j] = 0;
-    for (int p = tid; p < n; p += nt) a.deg[p] = 0;
+    uint16_t* clone = a.parent;                            // the positions that clone, one after the other: all states are n + n_clones
+    for (int p = tid; p < n; p += nt) {
+        a.deg[p] = 0;
+        if (pb_clones(a, (uint32_t)p)) clone[a.idc[p] - p - 1] = (uint16_t)p;
+    }
     pb_sync(nt);
+    const int states = n + sh.clones;
+    auto state = [&](int q) { return q < n ? 2u * (uint32_t)q : 2u * clone[q - n] + 1u; };
+    auto block_of = [&](uint32_t u) { return (u & 1) ? a.canon + (u >> 1) : reinterpret_cast<uint16_t*>(a.first) + (u & ~1u); };
 
     // ---- transitions: count them (the root's go to its table at once)
     uint2* root = W.root_tab + (size_t)b * W.root_cap;
     const uint32_t cap_mask = (uint32_t)W.root_cap - 1u, bmask = (uint32_t)(W.root_cap / SAM_ROOT_BUCKET) - 1u;
-    for (int q = tid; q - lane < 2 * n; q += nt) {         // (whole warps)
-        const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1);
-        const bool live = q < 2 * n && (!(u & 1) || pb_clones(a, u >> 1));
-        const uint32_t len = live ? pb_len(a, u) : 0u;
+    for (int q = tid; q - lane < states; q += nt) {        // (whole warps)
+        const bool live = q < states;
+        const uint32_t u = live ? state(q) : 0u, len = live ? pb_len(a, u) : 0u;
         const bool from_root = live && a.llen[u] == 0;
         uint32_t t = 0;
         if (from_root) t = (uint32_t)text[pb_end(a, u)];
@@ -655,11 +678,12 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
     // ---- room: records, and edge blocks by size, largest first, so that none crosses a slab
     unsigned long long pool = 0;                           // (read here, where nobody waits for it)
     if (tid == 0) pool = *reinterpret_cast<const volatile unsigned long long*>(W.pool_hdr);
-    for (int q = tid; q < 2 * n; q += nt) {
-        const uint32_t p = (uint32_t)(q < n ? q : q - n), d = q < n ? a.deg[p] & 0xFFFFu : a.deg[p] >> 16;
+    for (int q = tid; q < states; q += nt) {
+        const uint32_t u = state(q), d = a.deg[u >> 1] >> ((u & 1) * 16) & 0xFFFFu;
         if (d > 2) {
             const int k = d <= SAM_BLOCK_MIN ? 0 : 28 - __clz(d - 1);                // 16 << k entries
-            (q < n ? a.parent : a.canon)[p] = (uint16_t)atomicAdd(&sh.cls_n[k], 1u); // its number among those of its size
+            *block_of(u) = (uint16_t)atomicAdd(&sh.cls_n[k], 1u);                    // its number among those of its size
+            atomicOr(&a.deg[u >> 1], (u & 1) ? 0x80000000u : 0x8000u);               // from here on: it has an edge block
         }
     }
     pb_sync(nt);
@@ -692,14 +716,12 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         return reinterpret_cast<uint4*>(W.pool + ((size_t)sh.slab[id >> rps_shift] << W.slab_shift)) + 2 * (size_t)(id & ((1u << rps_shift) - 1));
     };
     // ---- records
-    for (int q = tid; q < 2 * n; q += nt) {
-        const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1), p = u >> 1;
-        if ((u & 1) && !pb_clones(a, p)) continue;
-        const uint32_t d = (u & 1) ? a.deg[p] >> 16 : a.deg[p] & 0xFFFFu;
+    for (int q = tid; q < states; q += nt) {
+        const uint32_t u = state(q), d = a.deg[u >> 1] >> ((u & 1) * 16) & 0x7FFFu;
         uint4 bw = make_uint4(0, 0, 0, 0);
         if (d > 2) {
             const int k = d <= SAM_BLOCK_MIN ? 0 : 28 - __clz(d - 1);
-            uint16_t* nth = (q < n ? a.parent : a.canon) + p;
+            uint16_t* nth = block_of(u);
             const uint32_t at = sh.cls_base[k] + ((uint32_t)*nth << k);
             *nth = (uint16_t)at;                           // (at most two units for each of 8192 tokens)
             bw = make_uint4((blk_slab[at >> us] << us) + (at & ((1u << us) - 1u)), (uint32_t)SAM_BLOCK_MIN << k, 0, 0);
@@ -709,16 +731,11 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         rec[1] = bw;
     }
     pb_sync(nt);
-    for (int p = tid; p < n; p += nt) {                    // bit 15 of a count: the state has an edge block
-        const uint32_t v = a.deg[p];
-        a.deg[p] = v | ((v & 0xFFFFu) > 2 ? 0x8000u : 0u) | ((v >> 16) > 2 ? 0x80000000u : 0u);
-    }
-    pb_sync(nt);
 
     // ---- transitions: write them
-    for (int q = tid; q - lane < 2 * n; q += nt) {
-        const uint32_t u = (uint32_t)(q < n ? 2 * q : 2 * (q - n) + 1);
-        const bool live = q < 2 * n && (!(u & 1) || pb_clones(a, u >> 1));
+    for (int q = tid; q - lane < states; q += nt) {
+        const bool live = q < states;
+        const uint32_t u = live ? state(q) : 0u;
         const uint32_t t = live ? (uint32_t)text[pb_end(a, u)] : 0u, idu = live ? pb_id(a, u) : 0u, len = live ? pb_len(a, u) : 0u;
         PbChain c = pb_chain_again(a, live, u, len);
         uint32_t to = idu | (c.lv + 1 == len ? SAM_FLAG : 0u);      // (only the first is solid)
@@ -728,7 +745,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
             to = idu;
             if (!on) return;
             const uint32_t h = v >> 1, odd = v & 1, old = atomicSub(&a.deg[h], odd ? 0x10000u : 1u);
-            const uint32_t unit = (odd ? a.canon : a.parent)[h], id = a.idc[h] + odd, was = odd ? old >> 16 : old & 0xFFFFu;
+            const uint32_t unit = *block_of(v), id = a.idc[h] + odd, was = odd ? old >> 16 : old & 0xFFFFu;
             uint2* at = (was & 0x8000u) ? reinterpret_cast<uint2*>(W.pool + ((((size_t)blk_slab[unit >> us]) << us) + (unit & ((1u << us) - 1u))) * 128)
                                         : reinterpret_cast<uint2*>(record(id) + 1);
             at[(was & 0x7FFFu) - 1u] = edge;
