@@ -39,7 +39,7 @@ struct PbShared {                          // what the threads of one build exch
     uint32_t slab[SAM_MAX_REC_SLABS + PB_BLOCK_SLABS];       // of the records, then of the edge blocks
     uint32_t cls_n[16], cls_base[16];
     int groups[2];                         // counted in rounds in turn: one is cleared while the other is in use
-    int rows, clones, root_deg, err, n_rec_slabs;
+    int rows, placed, clones, root_deg, err, n_rec_slabs;
 };
 
 struct PbArrays {
@@ -265,11 +265,12 @@ __device__ __forceinline__ uint32_t pb_take_slabs(const SamBatchView& W, unsigne
 
 struct PbResult { int32_t s2, l2, e2; int err; };          // e2: first end position of the match state
 
-// The first round: positions grouped by their token, the groups in the order of a hash table (any order of the tokens will do).
+// The first round: positions grouped by their token, the groups in any order of the tokens (the order in which warps ask for room).
 // A: the positions, group after group; rank 0 of `lev`: where a position's group begins.  Returns the number of groups.
-// (Counting in a table costs 3 us for 1024 tokens; sorting keys of three tokens cost 10.)
+// (Counting in a table costs 2 us for 1024 tokens, with a scan of the table for the groups' places 3; sorting keys of three
+// tokens cost 10.)
 __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, int n, int tid, int nt) {
-    const int lane = tid & 31, w = tid >> 5, nw = nt >> 5, N2 = a.N2, size = 2 * N2;
+    const int lane = tid & 31, N2 = a.N2, size = 2 * N2;
     uint32_t* key = reinterpret_cast<uint32_t*>(a.key);                              // [size]: tokens
     uint32_t* cnt = reinterpret_cast<uint32_t*>(smem + 10 * (size_t)N2);             // [size]: positions, then where they begin
     uint16_t* at = reinterpret_cast<uint16_t*>(smem + 18 * (size_t)N2);              // [N2]: a position's table entry
@@ -277,13 +278,14 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
         reinterpret_cast<uint4*>(key)[i] = make_uint4(SAM_NONE, SAM_NONE, SAM_NONE, SAM_NONE);
         reinterpret_cast<uint4*>(cnt)[i] = make_uint4(0, 0, 0, 0);
     }
-    if (tid == 0) sh.groups[0] = sh.groups[1] = sh.rows = 0;
+    if (tid == 0) sh.groups[0] = sh.groups[1] = sh.rows = sh.placed = 0;
     pb_sync(nt);
     for (int p = tid; p < n; p += nt) {
         const uint32_t t = a.tok[p];
         uint32_t h = sam_hash1(t) & (size - 1);
         for (int probe = 0; probe < size; probe++) {       // (at most half full)
-            const uint32_t old = atomicCAS(&key[h], SAM_NONE, t);
+            uint32_t old = key[h];
+            if (old == SAM_NONE) old = atomicCAS(&key[h], SAM_NONE, t);
             if (old == SAM_NONE || old == t) break;
             h = (h + 1) & (size - 1);
         }
@@ -291,32 +293,17 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
         a.B[p] = (uint16_t)atomicAdd(&cnt[h], 1u);
     }
     pb_sync(nt);
-    const int chunks = size >> 6;                          // of 64 entries, two a lane
-    for (int c = w; c < chunks; c += nw) {
-        const uint32_t x = cnt[64 * c + 2 * lane], y = cnt[64 * c + 2 * lane + 1];
-        const int sum = __reduce_add_sync(0xFFFFFFFFu, (int)(x + y)), used = __reduce_add_sync(0xFFFFFFFFu, (x != 0) + (y != 0));
-        if (lane == 0) { sh.chunk[c] = (int16_t)sum; if (used) atomicAdd(&sh.groups[0], used); }
-    }
-    pb_sync(nt);
-    if (w == 0) {
-        int run = 0;
-        for (int base = 0; base < chunks; base += 32) {
-            const int v = base + lane < chunks ? sh.chunk[base + lane] : 0;
-            int s = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
-            if (base + lane < chunks) sh.chunk[base + lane] = (int16_t)(run + s - v);
-            run += __shfl_sync(0xFFFFFFFFu, s, 31);
-        }
-    }
-    pb_sync(nt);
-    for (int c = w; c < chunks; c += nw) {
-        const int x = (int)cnt[64 * c + 2 * lane], y = (int)cnt[64 * c + 2 * lane + 1];
-        int s = x + y;
+    for (int p = tid; p - lane < n; p += nt) {             // (whole warps) the first position of each group sees to its place
+        const bool first = p < n && a.B[p] == 0;
+        const int c = first ? (int)cnt[at[p]] : 0;
+        int s = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
-        const int begin = sh.chunk[c] + s - x - y;
-        cnt[64 * c + 2 * lane] = (uint32_t)begin; cnt[64 * c + 2 * lane + 1] = (uint32_t)(begin + x);
+        const unsigned firsts = __ballot_sync(0xFFFFFFFFu, first);
+        int base = 0;
+        if (lane == 31 && firsts) { base = atomicAdd(&sh.placed, s); atomicAdd(&sh.groups[0], __popc(firsts)); }
+        base = __shfl_sync(0xFFFFFFFFu, base, 31);
+        if (first) cnt[at[p]] = (uint32_t)(base + s - c);
     }
     pb_sync(nt);
     for (int p = tid; p < n; p += nt) {
@@ -517,9 +504,12 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         if (j < n) p = A[j] & ~PB_ALONE;
         if (j > 0 && j < n) {
             const int q = A[j - 1] & ~PB_ALONE;
+            int equal = -1;                                // the last level whose ranks are equal: most neighbours differ at the first
+#pragma unroll
+            for (int i = 0; i < PB_LEVELS; i++) if (equal == i - 1 && i <= top && a.lev[(size_t)i * N2 + p] == a.lev[(size_t)i * N2 + q]) equal = i;
 #pragma unroll
             for (int i = PB_LEVELS - 1; i >= 0; i--) {
-                if (i <= top) {
+                if (i <= equal) {
                     const uint16_t* r = a.lev + (size_t)i * N2;
                     while (p - x >= 0 && q - x >= 0 && r[p - x] == r[q - x]) x += spans[i];
                 }
@@ -613,6 +603,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         }
     pb_sync(nt);
     uint32_t* pstate = W.pstate + (size_t)b * W.text_stride;
+    if (32 * tid < n) asm volatile("prefetch.global.L1 [%0];" ::"l"(text + 32 * tid));       // for the transitions' tokens
     for (int c = w; c < chunks; c += nw) {
         const int p = 32 * c + lane;
         const bool cl = p < n && pb_clones(a, (uint32_t)p);
