@@ -18,10 +18,10 @@
 //     along the suffix links of w without that token, down to length k.
 // Nothing here depends on a guess: each of these statements is the definition of the automaton of the text.
 //
-// What bounds it: for short texts the chain of some 50 barriers, for long ones one SM's shared memory (everything but the
-// outputs stays there, 28 bytes per token), and a step waits for its slowest build.  Walking the suffix links' chains with one
-// read a link, and the longest of them by whole warps (pb_walk), took the slowest of 64 x 1024 tokens from 70 us to 47, of
-// 256 x 1024 from 110 to 53.
+// What bounds it: for short texts the chain of some 40 barriers (1 x 300 tokens 17 us), for long ones one SM's issue slots (8191 tokens:
+// 64 % of them, 3900 instructions of a warp for 32 tokens, a third of the time in the sort; everything but the outputs stays
+// in shared memory, 28 bytes per token), for many the same (4096 x 1024 tokens: 9.5 tokens a ns), and a step waits for its slowest
+// build: 64 x 1024 tokens 34 to 51 us by text, mean 25.
 #pragma once
 #include "common.h"
 

@@ -1414,7 +1414,7 @@ __global__ void __launch_bounds__(128) fetch_inputs_kernel(const int32_t* rows, 
 //   five to an SM instead of three (4096 prompts of 1024 tokens).  There are as many blocks as are resident at once, and they share
 //   out the slots with prompts: those that order_slots_kernel has listed, or, in batches that are not ordered, what they find in the counts.
 //   (A block per slot costs an ordinary step of 1000 slots with rows of 8192 tokens 3 us.)
-// From how many tokens (SAM_PREFILL_MIN): the build takes 14 us for its shortest texts, one Expand after the other 0.3 to 0.5
+// From how many tokens (SAM_PREFILL_MIN): a step with one such prompt takes 18 us, reset included, one Expand after the other 0.3 to 0.5
 // us a token.
 __device__ __forceinline__ bool is_prompt(const StepArgs& A, int m) {
     return m >= SAM_PREFILL_MIN && m <= A.stride && m <= PB_MAX && m <= A.W.max_seq_len;
@@ -1929,7 +1929,7 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
 // Both sides leave each step's result in the step's own outputs, and sam_run_finish_kernel, which no chain waits for, chooses the
 // sources and reads the drafts: 32 rows a warp, eight rows' reads under way together.
 // us a step, step after step on each side (static sides on a few lanes, or three warps a slot up to 296 slots) -> so: 200 slots
-// 2.35 -> 1.3, 1000 slots 6.1 -> 2.3, 4096 slots 7.1 -> 3.9, 16384 slots 20.1 -> 12.5.
+// 2.35 -> 1.3, 1000 slots 6.1 -> 2.2, 4096 slots 7.1 -> 3.6, 16384 slots 20.1 -> 11.8.
 // Bound by the dynamic sides' rounds of reads and how many warps fit (16 an SM with 128 registers, nothing spilled; 20 with 96:
 // 4 % slower at 4096 slots).
 // What the two sides leave: match_len, state and status as they will be; the static side's first end position (or minus its
