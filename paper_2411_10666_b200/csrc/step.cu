@@ -588,7 +588,7 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
     if (bucket_peers & run) D.pr_state = 0;                   // those buckets changed
     __syncwarp();
     SAM_COUNT(D.kc.a, r + n_new - (last == 0 ? 1 : 0));        // per token: the previous state's transition (none from the root) and the root's
-    emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1);
+    emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1, D.root_deg + (uint32_t)idx + 1);
     if (F::seen && r > n_new) { s2 = __shfl_sync(FULL, D.pr_tgt, j + n_new) & SAM_IDMASK; l2 = 1; }
     D.n_states = c0 + r; D.root_deg += n_new;
     last = c0 + r - 1; ntok += r;
@@ -759,7 +759,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
         SAM_COUNT(D.kc.c, copied);
     }
 
-    emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1);
+    emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1, D.root_deg);
     const int lr = r - 1;                                      // the last clone is the new match state
     pa = make_uint4(l0 + (uint32_t)r, __shfl_sync(FULL, qa.y, lr), __shfl_sync(FULL, qa.z, lr), __shfl_sync(FULL, qa.w, lr));
     pb = make_uint4(__shfl_sync(FULL, nb.x, lr), __shfl_sync(FULL, nb.y, lr), __shfl_sync(FULL, nb.z, lr), __shfl_sync(FULL, nb.w, lr));
@@ -902,18 +902,19 @@ __device__ __forceinline__ void dyn_open(const SamBatchView& W, int b, int lane,
 
 // Expand (fused with the dynamic matcher's Transfer) for each of up to 32 tokens, one in each lane.  emit is called by the whole
 // warp whenever tokens are done, with what holds after them: (whether this lane has one, the lane that held its token, s2, l2,
-// first end position of s2, text length, state of the whole text, number of states); ends: the tokens for which it is wanted.
+// first end position of s2, text length, state of the whole text, number of states, transitions of the root); ends: the tokens for
+// which it is wanted.
 // seen: runs of new tokens take the known one behind them (dyn_fresh_run).
 template <bool SEEN>
 struct NoEmit {
     static constexpr bool chunks = false, seen = SEEN;
     static constexpr unsigned ends = 0;
-    __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
+    __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
 };
 template <class F>
 __device__ __forceinline__ void dyn_emit(DynChain& X, int j, F& emit) {    // after token j
     if (X.l2 > 0 && !X.have) { const uint4* rs = rec_ptr(X.D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(X.D.kc.rounds, 1); }
-    emit(X.D.lane == j, X.D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, X.D.n_states);
+    emit(X.D.lane == j, X.D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, X.D.n_states, X.D.root_deg);
 }
 template <class F>
 __device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, uint32_t (*sh_run)[12], F& emit) {
@@ -2032,7 +2033,7 @@ struct RunEmit {
     int b, lane;
     int32_t step, own;           // of the chunk (this lane's)
     unsigned ends;
-    uint32_t* done;              // text length, states, state of the whole text, s2, l2; the step after it
+    uint32_t* done;              // text length, states, state of the whole text, s2, l2; the step after it; the root's transitions
     __device__ __forceinline__ void write(int first, int n, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok) const {
         const StepArgs& A = R.A;
         for (int i = first; i < first + n; i++) {
@@ -2043,21 +2044,23 @@ struct RunEmit {
             if (o.state) o.state[2 * b + 1] = (int32_t)s2;
         }
     }
-    __device__ __forceinline__ void operator()(bool on, int from, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok, uint32_t last, uint32_t n_states) {
+    __device__ __forceinline__ void operator()(bool on, int from, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok, uint32_t last, uint32_t n_states, uint32_t root_deg) {
         const int st = __shfl_sync(FULL, step, from);
         int n = __shfl_sync(FULL, own, from);
         if (!on) n = 0;
         const unsigned ending = __ballot_sync(FULL, n > 0);
         if (!ending) return;
         if (n > 0) write(st, n, s2, l2, e2, ntok);
-        if (lane == 31 - __clz(ending)) { done[0] = ntok; done[1] = n_states; done[2] = last; done[3] = s2; done[4] = l2; done[5] = (uint32_t)(st + n); }
+        if (lane == 31 - __clz(ending)) {
+            done[0] = ntok; done[1] = n_states; done[2] = last; done[3] = s2; done[4] = l2; done[5] = (uint32_t)(st + n); done[6] = root_deg;
+        }
         __syncwarp();
     }
 };
 
 __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, uint32_t (*sh_run)[12], int32_t* sh_map) {
     const StepArgs& A = R.A;
-    __shared__ uint32_t done[6];
+    __shared__ uint32_t done[7];
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
     int m = run_counts(R, b, lane, 0);
@@ -2069,7 +2072,7 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
     const uint32_t ntok0 = X.ntok;
     RunEmit emit{R, b, lane, 0, 0, 0u, done};
     const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
-    if (lane == 0) { done[0] = X.ntok; done[1] = X.D.n_states; done[2] = X.last; done[3] = X.s2; done[4] = X.l2; done[5] = 0; }
+    if (lane == 0) { done[0] = X.ntok; done[1] = X.D.n_states; done[2] = X.last; done[3] = X.s2; done[4] = X.l2; done[5] = 0; done[6] = X.D.root_deg; }
     __syncwarp();
     int i = 0;
     RunChunk C;
@@ -2099,10 +2102,17 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
     }
     if (status != 0)
         for (int k = (int)done[5] + lane; k < R.n_steps; k += 32) if (R.keep || k + 1 == R.n_steps) step_out(A, R.keep ? k : 0).status[b] = status;
-    if (X.D.err) {                                         // the slot is left as the last step that was done left it
+    if (X.D.err) {
+        // The slot is left as the last step that was done left it, but for what the tokens after it have made.  The first of them
+        // completes the newest state's record; where the pool had no state for it, that is done here, without a transition.
+        const uint32_t newest = done[2];
+        uint4* rl = rec_ptr(X.D, newest);
+        const uint4* rs = rec_ptr(X.D, done[3]);
         if (lane == 0) {
-            cb[CB_NTOK] = done[0]; cb[CB_NSTATES] = done[1]; cb[CB_LAST] = done[2]; cb[CB_S2] = done[3]; cb[CB_L2] = done[4];
-            cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end; cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = X.D.root_deg;
+            if (newest != 0 && X.D.n_states == done[1]) { rl[0] = make_uint4(done[0], done[3], done[0], 0); rl[1] = make_uint4(0, 0, 0, 0); }
+            if (done[4] > 0) { reinterpret_cast<uint4*>(cb + CB_REC2)[0] = rs[0]; reinterpret_cast<uint4*>(cb + CB_REC2)[1] = rs[1]; }
+            cb[CB_NTOK] = done[0]; cb[CB_NSTATES] = done[1]; cb[CB_LAST] = newest; cb[CB_S2] = done[3]; cb[CB_L2] = done[4];
+            cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end; cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = done[6];
         }
     } else if (X.ntok != ntok0) {
         dyn_close(X);

@@ -444,6 +444,14 @@ def test_replayed_chunks_of_steps(P, B, K, most):
     assert_dynamic_automata_equal(once, ob, range(0, B, 5), msl)
 
 
+DUMP = ("n_tokens", "n_states", "n_edges", "length", "link", "min_endpos", "deg")
+
+
+def _dump(batch, slot):
+    d = batch.dump(slot, 4000, 8000)
+    return {k: d[k].tolist() if hasattr(d[k], "tolist") else d[k] for k in DUMP}, sorted(zip(*(d["edge_" + k].tolist() for k in ("src", "tok", "tgt"))))
+
+
 def test_replayed_steps_that_run_out_of_room(P):
     """A slot the pool has no slab left for fails at the same step, and is left as the step before left it, replayed or not."""
     rng = random.Random(3)
@@ -459,6 +467,49 @@ def test_replayed_steps_that_run_out_of_room(P):
         assert (got["status"][-1, 0] == 1) and (got["status"][:, 1:] == 0).all()
         a, b = (x.dump(0, 4000, 8000) for x in (once, one))
         assert a["n_tokens"] == b["n_tokens"] and a["n_states"] == b["n_states"]
+        assert _dump(once, 0) == _dump(one, 0)
+
+
+@pytest.mark.parametrize("static", [False, True])
+@pytest.mark.parametrize("kind,m,parts", [("distinct", 5, 1), ("distinct", 5, 2), ("distinct", 7, 1), ("distinct", 43, 1), ("one", 3, 1),
+                                          ("fibonacci", 1, 1), ("copies", 1, 1), ("copies", 6, 2), ("corpus", 4, 1)])
+def test_the_newest_state_of_a_replay_that_ran_out_of_room(P, kind, m, parts, static):
+    """The pool ends exactly at a step's end (255 states: 51 steps of 5 new tokens, each token a state; the last also as the first
+    step of a second launch) or inside a step: every record of the slot, the newest state's too, is that of the slot stepped one
+    call at a time, and the steps before are the oracle's.  The pool holds garbage to begin with."""
+    import torch
+    rng = random.Random(m)
+    L, msl, slabs, slab = 4, 1000, 2, 4096
+    steps = 2 * 255 // m
+    corpus = np.array([rng.randrange(400) for _ in range(3000)], dtype=np.int32)
+    st = P.StaticSam.build(corpus, VOCAB) if static else None
+    text = np.array(_text(kind, steps * m, rng, corpus.tolist()), dtype=np.int32)
+    toks, counts = text.reshape(steps, 1, m), np.full((steps, 1), m, dtype=np.int32)
+    t, c = torch.from_numpy(toks).cuda(), torch.from_numpy(counts).cuda()
+    once, one = (P.Batch(st, 1, msl, max_draft_len=L, vocab=VOCAB, pool_slabs=slabs, slab_bytes=slab) for _ in range(2))
+    for b in (once, one):
+        b.workspace[-slabs * slab:] = 0xEE
+    rows = [one.step(t[i], c[i], L).cpu() for i in range(steps)]
+    each = {k: np.stack([r[k] for r in rows]) for k in KEYS}
+    ok = int((each["status"][:, 0] == 0).sum())
+    assert 0 < ok < steps and (each["status"][ok:] == 1).all()
+    cuts = [0, ok, steps] if parts == 2 else [0, steps]
+    outs = [once.run_steps(t[a:b].contiguous(), c[a:b].contiguous(), L, per_step=True).cpu() for a, b in zip(cuts, cuts[1:])]
+    got = {k: np.concatenate([o[k] for o in outs]) for k in KEYS}
+    ob = oracle.Batch(oracle.Sam(corpus) if static else None, corpus if static else None, 1, VOCAB, msl)
+    for i in range(ok):
+        ref = ob.step(toks[i], counts[i], L)
+        for k in KEYS:
+            assert np.array_equal(got[k][i], getattr(ref, k)) and np.array_equal(each[k][i], getattr(ref, k)), (i, k)
+    for k in KEYS:
+        assert np.array_equal(got[k][ok:], each[k][ok:]), k
+    a, b = _dump(once, 0), _dump(one, 0)
+    assert a == b
+    assert a[0]["n_tokens"] == ok * m and ok * m in a[0]["length"]
+    # exactly at a step's end: nothing of the next step has been made, so all of it is the oracle's
+    if kind == "distinct" and m == 5:
+        assert a[0]["n_states"] == 256
+        assert_dynamic_automata_equal(once, ob, [0], msl)
 
 
 @pytest.mark.parametrize("B", [64, 700, 1100, 1300])
