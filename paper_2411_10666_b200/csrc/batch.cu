@@ -138,52 +138,53 @@ cudaError_t launch_after(K kernel, int blocks, int threads, cudaStream_t s, Args
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// one warp copies a slot's automaton into flat arrays
+// one warp copies a slot's automaton into flat arrays; of records and edge blocks it reads what lies in the pool, whatever they say
 __global__ void dump_kernel(SamBatchView W, int32_t slot, int32_t* hdr, int32_t* length, int32_t* link,
                             int32_t* min_endpos, int32_t* deg, int32_t max_states,
                             int32_t* e_src, int32_t* e_tok, int32_t* e_tgt, int32_t max_edges) {
     const int lane = threadIdx.x;
     const uint32_t* cb = W.ctrl + (size_t)slot * SAM_CTRL_WORDS;
-    const uint32_t n_states = cb[CB_NSTATES] ? cb[CB_NSTATES] : 1;
     const int rps_shift = W.slab_shift - 5;
-    int n_edges = 0;
+    const size_t slab_bytes = (size_t)1 << W.slab_shift, pool_bytes = (size_t)W.pool_slabs << W.slab_shift;
+    const uint32_t most = (uint32_t)SAM_MAX_REC_SLABS << rps_shift;       // (a slab is at most 2^30 bytes)
+    const uint32_t n_states = cb[CB_NSTATES] == 0 ? 1 : cb[CB_NSTATES] < most ? cb[CB_NSTATES] : most;
+    int64_t n_edges = 0;
+    auto put = [&](int64_t k, uint32_t from, uint32_t tok, uint32_t to) {
+        if (k < max_edges) { e_src[k] = (int32_t)from; e_tok[k] = (int32_t)tok; e_tgt[k] = (int32_t)(to & SAM_IDMASK); }
+    };
     // root: state 0
     if (lane == 0 && max_states > 0) { length[0] = 0; link[0] = -1; min_endpos[0] = 0; deg[0] = (int32_t)cb[CB_ROOTDEG]; }
     const uint2* root = W.root_tab + (size_t)slot * W.root_cap;
     for (int base = 0; base < W.root_cap; base += 32) {
         uint2 e = root[base + lane];
         unsigned has = __ballot_sync(0xFFFFFFFFu, e.x != SAM_NONE);
-        if (e.x != SAM_NONE) {
-            int k = n_edges + __popc(has & ((1u << lane) - 1));
-            if (k < max_edges) { e_src[k] = 0; e_tok[k] = (int32_t)e.x; e_tgt[k] = (int32_t)(e.y & SAM_IDMASK); }
-        }
+        if (e.x != SAM_NONE) put(n_edges + __popc(has & ((1u << lane) - 1)), 0, e.x, e.y);
         n_edges += __popc(has);
     }
     for (uint32_t s = 1; s < n_states; s++) {
-        uint32_t slab = cb[CB_SLABTAB + (s >> rps_shift)];
-        const uint4* rp = reinterpret_cast<const uint4*>(W.pool + ((size_t)slab << W.slab_shift) +
-                                                         ((size_t)(s & ((1u << rps_shift) - 1)) << 5));
-        const uint4 a = rp[0], b = rp[1];
+        const uint32_t slab = cb[CB_SLABTAB + (s >> rps_shift)];
+        uint4 a = make_uint4(0, 0, 0, 0), b = a;
+        if (slab < (uint32_t)W.pool_slabs) {
+            const uint4* rp = reinterpret_cast<const uint4*>(W.pool + ((size_t)slab << W.slab_shift) +
+                                                             ((size_t)(s & ((1u << rps_shift) - 1)) << 5));
+            a = rp[0]; b = rp[1];
+        }
         if (lane == 0 && s < (uint32_t)max_states) {
             length[s] = (int32_t)a.x; link[s] = (int32_t)a.y; min_endpos[s] = (int32_t)a.z; deg[s] = (int32_t)a.w;
         }
         if (a.w <= 2) {
-            if (lane == 0) {
-                if (a.w >= 1 && n_edges < max_edges) { e_src[n_edges] = (int32_t)s; e_tok[n_edges] = (int32_t)b.x; e_tgt[n_edges] = (int32_t)(b.y & SAM_IDMASK); }
-                if (a.w == 2 && n_edges + 1 < max_edges) { e_src[n_edges + 1] = (int32_t)s; e_tok[n_edges + 1] = (int32_t)b.z; e_tgt[n_edges + 1] = (int32_t)(b.w & SAM_IDMASK); }
-            }
-            n_edges += (int)a.w;
+            if (lane == 0 && a.w >= 1) put(n_edges, s, b.x, b.y);
+            if (lane == 0 && a.w == 2) put(n_edges + 1, s, b.z, b.w);
+            n_edges += a.w;
         } else {
-            const uint2* blk = reinterpret_cast<const uint2*>(W.pool + (size_t)b.x * 128);
-            for (uint32_t i = lane; i < a.w; i += 32) {
-                uint2 e = blk[i];
-                int k = n_edges + (int)i;
-                if (k < max_edges) { e_src[k] = (int32_t)s; e_tok[k] = (int32_t)e.x; e_tgt[k] = (int32_t)(e.y & SAM_IDMASK); }
-            }
-            n_edges += (int)a.w;
+            const size_t at = (size_t)b.x * 128, bytes = (size_t)a.w * 8;
+            if (bytes > slab_bytes || at + bytes > pool_bytes) continue;             // no edge block
+            const uint2* blk = reinterpret_cast<const uint2*>(W.pool + at);
+            for (uint32_t i = lane; i < a.w; i += 32) { const uint2 e = blk[i]; put(n_edges + i, s, e.x, e.y); }
+            n_edges += a.w;
         }
     }
-    if (lane == 0) { hdr[0] = (int32_t)cb[CB_NTOK]; hdr[1] = (int32_t)n_states; hdr[2] = n_edges; }
+    if (lane == 0) { hdr[0] = (int32_t)cb[CB_NTOK]; hdr[1] = (int32_t)n_states; hdr[2] = (int32_t)(n_edges < INT32_MAX ? n_edges : INT32_MAX); }
 }
 
 }  // namespace

@@ -512,6 +512,30 @@ def test_the_newest_state_of_a_replay_that_ran_out_of_room(P, kind, m, parts, st
         assert_dynamic_automata_equal(once, ob, [0], msl)
 
 
+@pytest.mark.parametrize("record,slab", [((5, 1, 5, 1000, 0x7FFFFFFF, 16, 0, 0), None), ((5, 1, 5, 0xFFFFFFF0, 0, 16, 0, 0), None),
+                                         ((5, 1, 5, 200, 95, 16, 0, 0), None), (None, 0x7FFFFFFF)])
+def test_dumps_read_inside_the_pool(P, record, slab):
+    """A record that names an edge block outside the pool (or one that is none) has no edges in a dump, a state slab outside it
+    holds no states; the other states' are as they were."""
+    import torch
+    batch = P.Batch(None, 2, 100, max_draft_len=4, vocab=VOCAB, slab_bytes=4096, pool_slabs=3)
+    toks = torch.tensor([[1, 2, 3, 4, 1, 2, 9, 9, 1, 5]] * 2, dtype=torch.int32, device="cuda")
+    batch.step(toks, torch.tensor([10, 0], dtype=torch.int32, device="cuda"), 4)
+    before = batch.dump(0, 100, 100)
+    words = batch.workspace.view(torch.int32)
+    pool = words[-3 * 1024:]
+    state = 4
+    at = int(words[64 + 16]) * 1024 + state * 8             # the slot's first slab, behind the pool's header and 16 control words
+    assert pool[at].item() == before["length"][state] == 4
+    if slab is None:
+        pool[at:at + 8] = torch.tensor(np.array(record, dtype=np.uint32).view(np.int32), device="cuda")
+    else:
+        words[64 + 16] = slab
+    after = batch.dump(0, 100, 100)
+    edges = [[e for e in zip(*(d["edge_" + k].tolist() for k in ("src", "tok", "tgt"))) if e[0] == 0 or (slab is None and e[0] != state)] for d in (before, after)]
+    assert after["n_states"] == before["n_states"] and after["n_edges"] == len(edges[1]) and edges[0] == edges[1]
+
+
 @pytest.mark.parametrize("B", [64, 700, 1100, 1300])
 def test_runs_of_new_tokens_with_a_known_one_behind(P, B):
     """Steps of r new tokens, a known one and what may follow it, for every r up to more than a warp holds: known by a solid
