@@ -2213,6 +2213,7 @@ __device__ __forceinline__ void static_chunk(const SamStaticView& S, uint32_t tk
             const int r = static_follow(S, __shfl_sync(FULL, cs, c), shfl4(a, c), shfl4(b, c), __shfl_sync(FULL, cl, c),
                                         __shfl_sync(FULL, tk, (p0 + lane) & 31), n - p0, lane, ref, out);
             if (r > 0) {
+                __syncwarp();                              // (walks that are ahead may just have left theirs where this one's count)
                 if (lane < r && (ends >> (p0 + lane) & 1u)) res[p0 + lane] = out;
                 base = sure = p0 + r;
                 const uint32_t to = __shfl_sync(FULL, ref, r - 1);
