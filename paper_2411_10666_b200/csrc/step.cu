@@ -2162,8 +2162,9 @@ __device__ __forceinline__ int static_follow(const SamStaticView& S, uint32_t s,
 }
 
 // One chunk: tk, n: its tokens; ends: the last tokens of its steps; T: the match, moved over the chunk (have: T's record is there; it
-// is on return, if T.l > 0).  res[k]: the result after token k, for the k in ends.
-__device__ __forceinline__ void static_chunk(const SamStaticView& S, uint32_t tk, int n, unsigned ends, int lane, StaticSide& T, RunResult* res, int& err) {
+// is on return, if T.l > 0).  res[k]: the result after token k, for the k in ends.  Returns for how many tokens the results hold: all n,
+// or, with err, as many as the match had taken when its links went on for too long.
+__device__ __forceinline__ int static_chunk(const SamStaticView& S, uint32_t tk, int n, unsigned ends, int lane, StaticSide& T, RunResult* res, int& err) {
     uint32_t re = SAM_NONE;
     if (lane < n) re = __ldg(S.root_row + tk);
     res[lane] = RunResult{0u, 0, 0};
@@ -2251,12 +2252,14 @@ __device__ __forceinline__ void static_chunk(const SamStaticView& S, uint32_t tk
         if (ahead) { const int c = __ffs(ahead) - 1; sure = max(sure, __shfl_sync(FULL, need_len ? 0 : pos, c)); }
         __syncwarp();
     }
-    err = (int)__reduce_max_sync(FULL, (uint32_t)err);
+    const unsigned failed = __ballot_sync(FULL, err != 0);
+    if (failed) { err = SAM_SEQ_WALK_LIMIT; n = __shfl_sync(FULL, pos, __ffs(failed) - 1); }
     const unsigned left = __ballot_sync(FULL, alive);
-    if (!left) { T.s = 0; T.sf = 0; T.l = 0; return; }
+    if (!left) { T.s = 0; T.sf = 0; T.l = 0; return n; }
     const int first = __ffs(left) - 1;
     T.s = __shfl_sync(FULL, cs, first); T.sf = __shfl_sync(FULL, csf, first); T.l = __shfl_sync(FULL, cl, first);
     T.ra = shfl4(a, first); T.rb = shfl4(b, first);
+    return n;
 }
 
 __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, int32_t* sh_map, RunResult* res) {
@@ -2289,11 +2292,12 @@ __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, in
         }
         if (C.lead > 0 && lane == 0) write(i, C.lead, T.s, T.l, (int32_t)T.ra.z);
         if (C.n_tok > 0) {
-            static_chunk(A.S, (uint32_t)C.tok, C.n_tok, __ballot_sync(FULL, C.own > 0), lane, T, res, err);
-            if (err) break;
+            const int held = static_chunk(A.S, (uint32_t)C.tok, C.n_tok, __ballot_sync(FULL, C.own > 0), lane, T, res, err);
             __syncwarp();
-            if (C.own > 0) write(C.step, C.own, res[lane].s, res[lane].l, res[lane].e1);
+            const bool mine = C.own > 0 && lane < held;
+            if (mine) write(C.step, C.own, res[lane].s, res[lane].l, res[lane].e1);
             __syncwarp();
+            if (err) { i = max(i + C.lead, (int)__reduce_max_sync(FULL, mine ? (uint32_t)(C.step + C.own) : 0u)); break; }     // the step that fails
         }
         ntok += (uint32_t)C.n_tok;
         i = next;

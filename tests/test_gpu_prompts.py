@@ -512,6 +512,32 @@ def test_the_newest_state_of_a_replay_that_ran_out_of_room(P, kind, m, parts, st
         assert_dynamic_automata_equal(once, ob, [0], msl)
 
 
+def test_steps_before_the_one_whose_links_go_on_for_too_long(P, tmp_path):
+    """In an automaton with a state whose suffix link leads to itself the walk's limit ends the step that meets it; the steps before
+    it, in the same chunk of a replay too, are reported as they are one call at a time."""
+    import torch
+    path = str(tmp_path / "linked_to_itself.sam")
+    st = P.StaticSam.build(np.array([1, 2, 3, 4, 5, 6, 7, 8, 9, 50, 5, 6, 7, 60], dtype=np.int32), 1000)
+    st.save(path)
+    words = np.fromfile(path, dtype=np.uint64)
+    recs = words[16:16 + 4 * st.info.n_states].view(np.uint32).reshape(-1, 8)     # {len, link, first end position, ...} behind the header
+    bad = int(np.flatnonzero((recs[:, 0] == 7) & (recs[:, 2] == 7))[0])           # the prefix of seven tokens
+    recs[bad, 1] = bad
+    total = 0xCBF29CE484222325
+    for w in words[16:].tolist():
+        total = (total ^ w) * 0x100000001B3 & 0xFFFFFFFFFFFFFFFF
+    words[15] = total
+    words.tofile(path)
+    rows = [[1, 2], [3, 4, 5], [], [6, 7], [999], [1]]
+    toks, counts = np.zeros((6, 1, 3), dtype=np.int32), np.array([[len(r)] for r in rows], dtype=np.int32)
+    for i, r in enumerate(rows):
+        toks[i, 0, :len(r)] = r
+    got, each, _, _ = _replayed(P, P.StaticSam.load(path), 1, 1000, 64, toks, counts, 4)
+    assert each["status"][:, 0].tolist() == [0, 0, 0, 0, 2, 2] and each["match_len"][3, 0, 0] == 7
+    for k in KEYS:
+        assert np.array_equal(got[k], each[k]), k
+
+
 @pytest.mark.parametrize("record,slab", [((5, 1, 5, 1000, 0x7FFFFFFF, 16, 0, 0), None), ((5, 1, 5, 0xFFFFFFF0, 0, 16, 0, 0), None),
                                          ((5, 1, 5, 200, 95, 16, 0, 0), None), (None, 0x7FFFFFFF)])
 def test_dumps_read_inside_the_pool(P, record, slab):

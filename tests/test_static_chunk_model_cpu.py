@@ -212,3 +212,23 @@ def test_results_do_not_depend_on_the_order_of_stores(seed):
 
 def test_a_walk_ahead_and_the_run_that_overtakes_it_need_the_barrier():
     assert any(wrong(s, False) for s in range(400))
+
+
+def test_what_holds_when_the_links_go_on_for_too_long():
+    """A state whose link leads to itself: the results of the tokens before the one that it fails at hold."""
+    seen = 0
+    for seed in range(600):
+        rng = random.Random(seed)
+        corpus, text = texts(rng)
+        C = Corpus(corpus)
+        exp, match = longest(C, text), (0, 0)
+        bad = rng.choice([s for s in range(1, len(C.len)) if C.len[s] > 2])
+        C.link[bad] = bad
+        for at, toks, ends in chunks_of(text, rng):
+            match, res, held, failed = chunk(C, toks, ends, match, rng)
+            for k in ends:
+                assert k >= held or res[k] == exp[at + k], (seed, at, k)
+            if failed:
+                seen += held > min(ends)
+                break
+    assert seen > 20
