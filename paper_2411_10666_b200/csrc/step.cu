@@ -212,20 +212,55 @@ __device__ __forceinline__ void ensure_rec(Dyn& D, uint32_t s) {
     if (D.lane == 0) D.cb[CB_SLABTAB + si] = (uint32_t)slab;
     D.n_rec_slabs = si + 1;
 }
+// State slabs of a slot that has n_rec_slabs of them, up to number `upto` or as many as there are: {this lane's slab, how many now}.
+__device__ __noinline__ uint2 take_rec_slabs(int32_t* pool_hdr, int32_t* free_stack, int32_t* slab_owner, int seq, uint32_t* cb,
+                                             uint32_t upto, uint32_t n_rec_slabs, uint32_t tab) {
+    for (; n_rec_slabs <= upto && n_rec_slabs < SAM_MAX_REC_SLABS; n_rec_slabs++) {
+        const int slab = take_slab(pool_hdr, free_stack, slab_owner, seq);
+        if (slab < 0) break;
+        if ((threadIdx.x & 31) == n_rec_slabs) tab = (uint32_t)slab;
+        if ((threadIdx.x & 31) == 0) cb[CB_SLABTAB + n_rec_slabs] = (uint32_t)slab;
+    }
+    return make_uint2(tab, n_rec_slabs);
+}
 
 // Make sure of records for n states from s on, fewer than a slab holds; returns how many there are.  Where the pool has no slab left
 // that may be fewer: the tokens before the one that fails are done all the same.
+// How that rare case is written matters, since it stands in four places of the chain that a step waits for (us a step):
+//   - F::call, a call: the single steps' kernels.  With a loop in each place they spilled on every token's way (sam_step_kernel<false, 0>
+//     56/92 bytes stored/loaded, 8/40 now; the split kernel 62/100, 6/8 now): 2000 slots 15.1, now 14.8; 8191 slots 40.0, 39.3;
+//     12000 slots 48.1, 47.6; 1000 slots 12.9, 12.6;
+//   - in place, all tokens of a run or none: the verified steps' kernel of 80 registers, 1000 slots 18.4 (a call: 19.0);
+//   - F::chunks, in place and as many tokens as there are: replays, whose kernels spill nothing (a call: 1 to 2 % slower).
+template <class F>
 __device__ __forceinline__ uint32_t ensure_recs(Dyn& D, uint32_t s, uint32_t n) {
-    if ((s + n - 1) >> D.rps_shift < D.n_rec_slabs) return n;
-    for (uint32_t at = s;; at = s + n - 1) {
-        ensure_rec(D, at);
-        if (D.err) {
-            if (at == s) return 0;
-            D.err = 0;
-            return (D.n_rec_slabs << D.rps_shift) - s;
-        }
-        if (at == s + n - 1) return n;
+    const uint32_t upto = (s + n - 1) >> D.rps_shift;
+    if (upto < D.n_rec_slabs) return n;
+    if (F::call) {
+        const uint2 r = take_rec_slabs(D.pool_hdr, D.free_stack, D.slab_owner, D.seq, D.cb, upto, D.n_rec_slabs, D.tab);
+        D.tab = r.x; D.n_rec_slabs = r.y;
+    } else {
+        ensure_rec(D, s);
+        if (!D.err) ensure_rec(D, s + n - 1);
+        D.err = 0;
     }
+    const uint32_t there = D.n_rec_slabs << D.rps_shift;
+    if (there <= s) { D.err = SAM_SEQ_CAPACITY; return 0; }
+    return min(n, there - s);
+}
+template <class F>
+__device__ __forceinline__ void ensure_next(Dyn& D, uint32_t s) {        // of one state
+    if (F::call) ensure_recs<F>(D, s, 1);
+    else ensure_rec(D, s);
+}
+// of a run of r tokens that make `per` states each; returns how many tokens there are records for (all or none in a kernel that neither
+// calls nor has steps to end inside the run)
+template <class F>
+__device__ __forceinline__ int ensure_run(Dyn& D, uint32_t s, int r, int per) {
+    if (F::call || F::chunks) return (int)ensure_recs<F>(D, s, (uint32_t)(per * r)) / per;
+    ensure_rec(D, s);
+    if (!D.err) ensure_rec(D, s + (uint32_t)(per * r) - 1);
+    return D.err ? 0 : r;
 }
 
 // edge block of `cap` entries; returns its offset in 128-byte units from the pool base
@@ -423,6 +458,7 @@ __device__ __forceinline__ void redirect_walk(Dyn& D, uint32_t pp, uint32_t t, u
 // last: state of the whole text; ntok: text length; (s2, l2): match state = link[last], its length.
 // On entry, if have_rec, (pa, pb) is the record of s2 as it stands; on exit have_rec says whether
 // (pa, pb) is the record of the new s2 (known without a read when s2 is a fresh clone).
+template <class F>
 __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, uint32_t& ntok,
                                            uint32_t& s2, uint32_t& l2, bool& have_rec, uint4& pa, uint4& pb,
                                            const Pre& pre) {
@@ -430,7 +466,7 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
     have_rec = false;
     const uint32_t k = ntok + 1;                       // max_length after this token
     const uint32_t c = D.n_states;
-    ensure_rec(D, c);
+    ensure_next<F>(D, c);
     if (D.err) return;
     D.n_states = c + 1;
 
@@ -485,7 +521,7 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
         } else {
             // clone q as cl with len[p] + 1
             const uint32_t cl = D.n_states;
-            ensure_rec(D, cl);
+            ensure_next<F>(D, cl);
             if (D.err) return;
             D.n_states = cl + 1;
             uint4* rq = rec_ptr(D, q);
@@ -550,8 +586,9 @@ __device__ __forceinline__ void dyn_extend(Dyn& D, uint32_t t, uint32_t& last, u
 // "absent" and no earlier token of the run shares its home bucket (so slots and tokens differ).
 // The token that ends the run is in it too if the root has it, by a solid transition: Expand for it is the same without the
 // root transition, and the match goes on from there.  (256 slots fed by verified drafts, a fifth of whose tokens are of this kind:
-// 19.3 -> 18.7 us a step; 300 slots with copied texts 11.9 -> 11.7.  Not in the kernel of 80 registers, where it costs more
-// spilled registers than it gives unless drafts are verified: 1000 slots 18.2 -> 18.5; nor in chunks of replayed steps.)
+// 19.3 -> 18.7 us a step; 300 slots with copied texts 11.9 -> 11.7.  Up to 888 slots, in the kernels of three warps a slot with 96
+// registers and more: beyond, where throughput counts, it gives nothing or takes, us a step with / without it: 2000 slots 14.7 / 14.7,
+// 4096 28.8 / 28.6, 8192 41.5 / 41.2, 12000 59.1 / 58.7, verified 1000 18.3 / 18.4, 1400 21.0 / 21.0.  Nor in chunks of replayed steps.)
 // Returns the number of tokens (0: token j does not qualify); s2, l2: the match after them.
 template <class F>
 __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt, unsigned bucket_peers,
@@ -566,7 +603,7 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
     int r = fresh + (F::seen && j + fresh < 32 ? (int)(known >> (j + fresh) & 1u) : 0);
     if (r <= 0) return 0;
     const uint32_t c0 = D.n_states;
-    r = (int)ensure_recs(D, c0, (uint32_t)r);
+    r = ensure_run<F>(D, c0, r, 1);
     if (r == 0) return 0;
     const int idx = D.lane - j;
     const bool mine = idx >= 0 && idx < r, is_new = F::seen ? mine && idx < fresh : mine;
@@ -715,7 +752,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
 
     const uint32_t n0 = D.n_states;                            // c_k = n0 + 2k, cl_k = n0 + 2k + 1
     pre.valid = false;                                         // (its place has been used again)
-    r = (int)ensure_recs(D, n0, 2 * (uint32_t)r) / 2;
+    r = ensure_run<F>(D, n0, r, 2);
     if (r < 2) return 0;
 
     // the new states, side by side
@@ -904,10 +941,10 @@ __device__ __forceinline__ void dyn_open(const SamBatchView& W, int b, int lane,
 // warp whenever tokens are done, with what holds after them: (whether this lane has one, the lane that held its token, s2, l2,
 // first end position of s2, text length, state of the whole text, number of states, transitions of the root); ends: the tokens for
 // which it is wanted.
-// seen: runs of new tokens take the known one behind them (dyn_fresh_run).
-template <bool SEEN>
+// seen: runs of new tokens take the known one behind them (dyn_fresh_run).  call, chunks: ensure_recs.
+template <bool SEEN, bool CALL>
 struct NoEmit {
-    static constexpr bool chunks = false, seen = SEEN;
+    static constexpr bool chunks = false, seen = SEEN, call = CALL;
     static constexpr unsigned ends = 0;
     __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
 };
@@ -941,7 +978,7 @@ __device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, ui
             if (D.err) break;
         }
         D.cur = j;
-        dyn_extend(D, __shfl_sync(FULL, tk, j), X.last, X.ntok, X.s2, X.l2, X.have, X.ra, X.rb, pre);
+        dyn_extend<F>(D, __shfl_sync(FULL, tk, j), X.last, X.ntok, X.s2, X.l2, X.have, X.ra, X.rb, pre);
         if ((emit.ends >> j & 1u) && !D.err) dyn_emit(X, j, emit);
         j++;
     }
@@ -961,11 +998,11 @@ __device__ __forceinline__ void dyn_close(DynChain& X) {
 }
 // A step's m tokens, then the slot's control words.  On return, unless D.err is set, (ra, rb) is the record of s2 if l2 > 0 (also
 // stored in the control block).
-template <bool SEEN>
+template <bool SEEN, bool CALL>
 __device__ __forceinline__ void dyn_feed(DynChain& X, int32_t tok_first, const int32_t* toks, int m, uint32_t (*sh_run)[12]) {
     Dyn& D = X.D;
     const int lane = D.lane;
-    NoEmit<SEEN> none;
+    NoEmit<SEEN, CALL> none;
     for (int base = 0; base < m && !D.err; base += 32) {
         const int i = base + lane;
         uint32_t tk = 0;
@@ -1219,8 +1256,8 @@ __device__ __forceinline__ void step_sync() { asm volatile("bar.sync 1, 64;" :::
 // VERIFY: the accepted tokens are derived from the previous draft and the target's tokens (sam_step_verified).
 // AHEAD: a third warp reads ahead of the dynamic side (read_ahead).
 // INLINE: the rows and counts came with the launch (sam_step_host).
-// SEEN: dyn_feed's.
-template <bool VERIFY, bool AHEAD, bool INLINE, bool SEEN>
+// SEEN, CALL: dyn_feed's.
+template <bool VERIFY, bool AHEAD, bool INLINE, bool SEEN, bool CALL>
 __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_tokens, const int32_t* counts) {
     // Programmatic dependent launch: this grid may be scheduled while the previous kernel of the stream
     // is still finishing.  Nothing is read before that kernel has completed and flushed; the kernel
@@ -1347,7 +1384,7 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
         DynChain X;
         X.ra = ra; X.rb = rb;
         dyn_open(A.W, b, lane, cb, cw, cw2, X);
-        dyn_feed<SEEN>(X, tok_first, toks, built ? 0 : m, sh_run);
+        dyn_feed<SEEN, CALL>(X, tok_first, toks, built ? 0 : m, sh_run);
         err = X.D.err; my_l = (int32_t)X.l2; my_s = (int32_t)X.s2;
         if (X.l2 > 0 && !err) {
             const int64_t e = (int64_t)X.ra.z;                  // min_endpos
@@ -1369,12 +1406,12 @@ __device__ __forceinline__ void step_body(const StepArgs& A, const int32_t* new_
 }
 
 // AHEAD: blocks of three warps an SM has to hold, 0 for blocks of two.  Registers come in quarters of an SM: 5 blocks (740
-// slots) have 120 a thread and spill nothing, 6 (888) have 96, 8 (1184) have 80 and spill 188 bytes.  Prompt-copying
+// slots) have 120 a thread and spill nothing, 6 (888) have 96, 8 (1184) have 80 and spill 192 bytes.  Prompt-copying
 // slots, us a step with 5 / 6 / 8 blocks: 740 slots 14.6 / 15.0 / -, 880 slots - / 15.5 / 16.4, 1000 slots (in two
 // waves: 20.5 / 18.5) 17.0, 1180 slots with two warps a slot 19.2, with three 17.4.
 template <bool VERIFY, int AHEAD>
 __global__ void __launch_bounds__(AHEAD ? 96 : 64, AHEAD ? AHEAD : 10) sam_step_kernel(const __grid_constant__ StepArgs A) {
-    step_body<VERIFY, AHEAD != 0, false, VERIFY || AHEAD != 8>(A, A.new_tokens, A.counts);
+    step_body<VERIFY, AHEAD != 0, false, AHEAD == 5 || AHEAD == 6, !(VERIFY && AHEAD == 8)>(A, A.new_tokens, A.counts);
 }
 
 // A host-array step whose rows and counts fit the launch's arguments: reading them from host memory, in the kernel's first
@@ -1383,7 +1420,7 @@ __global__ void __launch_bounds__(AHEAD ? 96 : 64, AHEAD ? AHEAD : 10) sam_step_
 constexpr int SAM_INLINE_WORDS = 896;                    // within 4 KB of arguments
 struct StepArgsInline { StepArgs A; int32_t in[SAM_INLINE_WORDS]; };                // rows, then counts
 __global__ void __launch_bounds__(96, 5) sam_step_inline_kernel(const __grid_constant__ StepArgsInline I) {
-    step_body<false, true, true, true>(I.A, I.in, I.in + (size_t)I.A.W.batch * I.A.stride);
+    step_body<false, true, true, true, true>(I.A, I.in, I.in + (size_t)I.A.W.batch * I.A.stride);
 }
 
 // Larger ones: the rows and counts are brought over in whole lines by this kernel, launched ahead of the step's.
@@ -1843,7 +1880,7 @@ __device__ __forceinline__ bool dynamic_slot(const StepArgs& A, int b, int lane,
         DynChain X;
         kept_record(cw2, CB_REC2, X.ra, X.rb);
         dyn_open(A.W, b, lane, cb, cw, cw2, X);
-        dyn_feed<true>(X, tok_first, toks, m, sh_run);
+        dyn_feed<false, true>(X, tok_first, toks, m, sh_run);
         err = X.D.err;
         if (err) { status = err; fresh_fail = true; }
     }
@@ -2028,7 +2065,7 @@ __device__ __forceinline__ void run_cut(RunChunk& C, int lane, int i, int vocab)
 
 // What a slot's results are written with, and (in shared memory) what holds at the end of the last step that is done.
 struct RunEmit {
-    static constexpr bool chunks = true, seen = false;
+    static constexpr bool chunks = true, seen = false, call = false;
     const RunArgs& R;
     int b, lane;
     int32_t step, own;           // of the chunk (this lane's)
