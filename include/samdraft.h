@@ -198,8 +198,8 @@ int sam_step(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t stride,
  * between: new_tokens_dev [n_steps, B, stride], counts_dev [n_steps, B].  If out_per_step is
  * non-zero every output array has a leading n_steps dimension and keeps each step's results,
  * otherwise the arrays are those of sam_step and hold the last step's.  A slot's steps follow one another,
- * different slots are not kept in step: short rows (stride below 48) take one launch for all n_steps (two for
- * large batches), rows that may hold prompts the launches of sam_step for each step. */
+ * different slots are not kept in step: short rows (stride below 48) take two launches for all n_steps (one for
+ * few steps of up to 296 slots), a single step and rows that may hold prompts those of sam_step for each step. */
 int sam_run_steps(sam_batch_t* b, const int32_t* new_tokens_dev, int32_t stride,
                   const int32_t* counts_dev, int32_t n_steps, int32_t L, int32_t out_per_step,
                   int32_t* draft_tokens_dev, int32_t* draft_len_dev, int32_t* match_len_dev,

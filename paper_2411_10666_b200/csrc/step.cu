@@ -25,7 +25,7 @@
 //     map, or ids two apart), read in one round trip and checked (dyn_repeat_run);
 //   - the static match is not advanced token by token: all suffixes of the row are walked side by side, and a
 //     match that goes on as the corpus does is taken in one round (static_match.cuh);
-//   - steps whose tokens are all at hand (sam_run_steps) run in one launch, no slot waiting for another;
+//   - steps whose tokens are all at hand (sam_run_steps) run in one launch or two, no slot waiting for another;
 //   - a prompt that fills an empty slot is not extended token by token either: its automaton is built at once by all
 //     threads of a block (prefill_build.cuh, sam_prefill_kernel);
 //   - when the batch is larger than the GPU holds at once, the slots with the most tokens are started
@@ -625,7 +625,7 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
     if (bucket_peers & run) D.pr_state = 0;                   // those buckets changed
     __syncwarp();
     SAM_COUNT(D.kc.a, r + n_new - (last == 0 ? 1 : 0));        // per token: the previous state's transition (none from the root) and the root's
-    emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1, D.root_deg + (uint32_t)idx + 1);
+    if (emit.ends >> j & (FULL >> (32 - r))) emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1, D.root_deg + (uint32_t)idx + 1);
     if (F::seen && r > n_new) { s2 = __shfl_sync(FULL, D.pr_tgt, j + n_new) & SAM_IDMASK; l2 = 1; }
     D.n_states = c0 + r; D.root_deg += n_new;
     last = c0 + r - 1; ntok += r;
@@ -796,7 +796,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
         SAM_COUNT(D.kc.c, copied);
     }
 
-    emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1, D.root_deg);
+    if (emit.ends >> j & (FULL >> (32 - r))) emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1, D.root_deg);
     const int lr = r - 1;                                      // the last clone is the new match state
     pa = make_uint4(l0 + (uint32_t)r, __shfl_sync(FULL, qa.y, lr), __shfl_sync(FULL, qa.z, lr), __shfl_sync(FULL, qa.w, lr));
     pb = make_uint4(__shfl_sync(FULL, nb.x, lr), __shfl_sync(FULL, nb.y, lr), __shfl_sync(FULL, nb.z, lr), __shfl_sync(FULL, nb.w, lr));
@@ -1975,6 +1975,7 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
 struct RunArgs {
     StepArgs A;
     int32_t n_steps, keep;       // keep: the outputs have room for every step
+    int32_t finish;              // sam_run_block_kernel finishes the rows
 };
 
 struct StaticSide { uint32_t s, sf; int32_t l; uint4 ra, rb; };
@@ -1996,6 +1997,7 @@ struct RunChunk {
     uint32_t starts;             // where steps begin
     int32_t refuse;              // why the step behind it is refused (0: it is not, or there is none)
     int32_t taken;               // tokens of the step behind it that it holds (of a step of more than 32: the first 32)
+    int32_t tail;                // a token of that step behind those
 };
 __device__ __forceinline__ int32_t run_counts(const RunArgs& R, int b, int lane, int i) {
     return i + lane < R.n_steps ? R.A.counts[(size_t)(i + lane) * R.A.W.batch + b] : 0;
@@ -2005,10 +2007,16 @@ __device__ __forceinline__ int32_t run_counts(const RunArgs& R, int b, int lane,
 __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, int i, int taken, uint32_t ntok, int m, int32_t* sh_map) {
     const StepArgs& A = R.A;
     RunChunk C;
-    C.tok = 0;
+    C.tok = C.tail = C.taken = C.refuse = 0;
     const int left = R.n_steps - i;
     const bool counted = m >= 0 && m <= A.stride;
     if (!counted) m = 0;
+    const int m0 = __shfl_sync(FULL, m, 0), m1 = __shfl_sync(FULL, m, 1);
+    if (m0 >= 1 && m0 <= 32 && m0 + m1 > 32 && (int64_t)ntok + m0 <= A.W.max_seq_len) {          // a wide step, alone
+        C.n_steps = 1; C.n_tok = m0; C.step = i; C.own = lane == m0 - 1 ? 1 : 0; C.lead = 0; C.starts = 1;
+        if (lane < m0) C.tok = A.new_tokens[((size_t)i * A.W.batch + b) * A.stride + lane];
+        return C;
+    }
     int upto = m;                                          // tokens up to this step's last
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, upto, o); if (lane >= o) upto += t; }
@@ -2018,19 +2026,13 @@ __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, 
     C.n_steps = n;
     C.n_tok = n > 0 ? __shfl_sync(FULL, upto, n - 1) : 0;
     C.refuse = n < 32 ? __shfl_sync(FULL, lane >= left ? 0 : !counted ? SAM_SEQ_BAD_COUNT : !room ? SAM_SEQ_CAPACITY : 0, n & 31) : 0;
-    C.taken = 0;
-    if (n == 0 && left > 0 && C.refuse == 0) {             // a step of more than 32 tokens, checked as a whole
-        const int len = __shfl_sync(FULL, m, 0);
+    if (n == 0 && left > 0 && C.refuse == 0) {             // a step of more than 32 tokens, checked as a whole when it begins
         const int32_t* row = A.new_tokens + ((size_t)i * A.W.batch + b) * A.stride;
         C.step = i; C.own = 0; C.lead = 0; C.starts = 1;
-        if (taken == 0) {
-            const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
-            const int32_t t0 = row[lane], t1 = lane + 32 < len ? row[lane + 32] : 0;
-            if (__any_sync(FULL, t0 < 0 || t0 >= vocab || t1 < 0 || t1 >= vocab)) { C.refuse = SAM_SEQ_BAD_TOKEN; return C; }
-        }
-        C.n_tok = min(32, len - taken);
-        C.tok = lane < C.n_tok ? row[taken + lane] : 0;
-        if (taken + C.n_tok == len) { C.n_steps = 1; C.own = lane == C.n_tok - 1 ? 1 : 0; } else C.taken = C.n_tok;
+        C.n_tok = min(32, m0 - taken);
+        if (lane < C.n_tok) C.tok = row[taken + lane];
+        if (taken + C.n_tok == m0) { C.n_steps = 1; C.own = lane == C.n_tok - 1 ? 1 : 0; }
+        else { C.taken = C.n_tok; if (lane + 32 < m0) C.tail = row[lane + 32]; }
         return C;
     }
     const bool some = lane < n && m > 0;
@@ -2054,8 +2056,9 @@ __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, 
 
 // Its tokens have come: where one is outside the vocabulary the chunk, which begins with step i, ends before that step.
 __device__ __forceinline__ void run_cut(RunChunk& C, int lane, int i, int vocab) {
-    const unsigned wrong = __ballot_sync(FULL, lane < C.n_tok && (C.tok < 0 || C.tok >= vocab));
+    const unsigned wrong = __ballot_sync(FULL, (lane < C.n_tok && (C.tok < 0 || C.tok >= vocab)) || C.tail < 0 || C.tail >= vocab);
     if (!wrong) return;
+    C.taken = 0;
     const int t = __ffs(wrong) - 1;
     C.n_tok = 31 - __clz(C.starts & (0xFFFFFFFFu >> (31 - t)));
     C.n_steps = __shfl_sync(FULL, C.step, t) - i;
@@ -2359,19 +2362,16 @@ __global__ void __launch_bounds__(32, 16) sam_run_split_kernel(const __grid_cons
 }
 
 constexpr int FINISH_ROWS = 8;                             // rows whose reads a warp has under way together
-__global__ void __launch_bounds__(128) sam_run_finish_kernel(const __grid_constant__ RunArgs R) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+// n <= 32 rows of the outputs from r0 on, `apart` from one another, by a warp.
+__device__ __forceinline__ void run_finish(const RunArgs& R, int64_t r0, int64_t apart, int n, int lane) {
     const StepArgs& A = R.A;
-    const int lane = threadIdx.x & 31, L = A.L;
+    const int L = A.L;
     const int64_t rows = (int64_t)A.W.batch * (R.keep ? R.n_steps : 1);
-    const int64_t r0 = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * 32;
-    if (r0 >= rows) return;
-    const int64_t r = r0 + lane;
-    const bool live = r < rows;
+    const int64_t r = r0 + lane * apart;
+    const bool live = lane < n;
     int src = SAM_SRC_NONE, dl = 0;
     const int32_t* from = A.S.corpus;
-    if (live) {                                            // lane k: row r0 + k
+    if (live) {                                            // this lane's row
         const int b = (int)(r % A.W.batch);
         int status = A.status[r], l1 = 0, s1 = 0, e1 = 0;
         int l2 = A.match_len[2 * r + 1];
@@ -2404,7 +2404,6 @@ __global__ void __launch_bounds__(128) sam_run_finish_kernel(const __grid_consta
     __syncwarp();                                          // (every lane has read its row's first word)
     const int32_t stop = A.W.stop_token;
     int cut = dl;
-    const int n = (int)(rows - r0 < 32 ? rows - r0 : 32);
     for (int base = 0; base < L; base += 32)
         for (int k0 = 0; k0 < n; k0 += FINISH_ROWS) {
             int32_t v[FINISH_ROWS];
@@ -2423,10 +2422,37 @@ __global__ void __launch_bounds__(128) sam_run_finish_kernel(const __grid_consta
                     if (hit) c = base + __ffs(hit) - 1;
                     if (lane == k0 + k) cut = c;
                 }
-                if (k0 + k < n && base + lane < L) A.draft_tokens[(r0 + k0 + k) * L + base + lane] = base + lane < c ? v[k] : -1;
+                if (k0 + k < n && base + lane < L) A.draft_tokens[(r0 + (k0 + k) * apart) * L + base + lane] = base + lane < c ? v[k] : -1;
             }
         }
     if (live) A.draft_len[r] = cut;
+}
+__global__ void __launch_bounds__(128) sam_run_finish_kernel(const __grid_constant__ RunArgs R) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int64_t rows = (int64_t)R.A.W.batch * (R.keep ? R.n_steps : 1);
+    const int64_t r0 = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * 32;
+    if (r0 < rows) run_finish(R, r0, 1, (int)(rows - r0 < 32 ? rows - r0 : 32), threadIdx.x & 31);
+}
+
+// Up to two slots an SM: the two sides of a slot are the warps of a block, which have the SM's L1 to themselves (the other kernel asks
+// for half of it as shared memory; 1 to 296 slots with 24 tokens a step 5 to 10 % faster), and few rows are finished by the block
+// itself: calls of two steps 2.4 (one slot) to 4.4 us (200 slots) shorter, of four 1.0 to 4.7.
+__global__ void __launch_bounds__(64, 8) sam_run_block_kernel(const __grid_constant__ RunArgs R) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    __shared__ __align__(16) uint32_t sh_run[32][12];
+    __shared__ RunResult res[32];
+    __shared__ int32_t sh_map[2][32];
+    const int lane = threadIdx.x & 31, side = threadIdx.x >> 5, b = blockIdx.x, B = R.A.W.batch;
+    if (lane < R.n_steps)                                  // (which tokens are read first depends on the counts)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(R.A.new_tokens + ((size_t)lane * B + b) * R.A.stride));
+    if (side == 0) run_dynamic(R, b, lane, sh_run, sh_map[0]);
+    else if (R.A.has_static) run_static(R, b, lane, sh_map[1], res);
+    if (!R.finish) return;
+    __syncthreads();
+    const int n = R.keep ? R.n_steps : 1;
+    for (int i = 32 * side; i < n; i += 64) run_finish(R, (int64_t)i * B + b, B, min(32, n - i), lane);
 }
 
 // A batch larger than the GPU holds at once runs in waves, and a step is as long as its last block: a
@@ -2696,6 +2722,9 @@ int sam_launch_fetch(const sam_batch* b, const int32_t* rows, const int32_t* cou
     return SAM_OK;
 }
 
+// Up to SAM_RUN_FINISH_MAX times 32 draft tokens of a slot are read by its own block: 64 rows of 16 tokens as fast as by a launch of their
+// own (1, 64, 296 slots: 75 / 74, 242 / 245, 171 / 171 us a call with its prompts), 192 rows 160 / 153, 192 of 128 tokens 185 / 148.
+constexpr int SAM_RUN_BLOCK_MAX_BATCH = 2 * SAM_SMS, SAM_RUN_FINISH_MAX = 64;
 int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride, const int32_t* counts, int32_t n_steps, int32_t L, int32_t keep,
                    int32_t* draft_tokens, int32_t* draft_len, int32_t* match_len, int32_t* source, int32_t* state, int32_t* status,
                    cudaStream_t stream) {
@@ -2719,9 +2748,16 @@ int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride
     cudaError_t e;
     int rc = split_kernel_setup(b->device);
     if (rc) return rc;
-    cfg.gridDim = dim3((unsigned)b->view.batch * (A.has_static ? 2u : 1u)); cfg.blockDim = dim3(32);
-    e = cudaLaunchKernelEx(&cfg, sam_run_split_kernel, R);
     const int64_t rows = (int64_t)b->view.batch * (keep ? n_steps : 1);
+    if (b->view.batch <= SAM_RUN_BLOCK_MAX_BATCH) {
+        R.finish = (keep ? n_steps : 1) * ((L + 31) / 32) <= SAM_RUN_FINISH_MAX;
+        cfg.gridDim = dim3((unsigned)b->view.batch); cfg.blockDim = dim3(64);
+        e = cudaLaunchKernelEx(&cfg, sam_run_block_kernel, R);
+    } else {
+        cfg.gridDim = dim3((unsigned)b->view.batch * (A.has_static ? 2u : 1u)); cfg.blockDim = dim3(32);
+        e = cudaLaunchKernelEx(&cfg, sam_run_split_kernel, R);
+    }
+    if (R.finish && e == cudaSuccess) return SAM_OK;
     cfg.gridDim = dim3((unsigned)((rows + 127) / 128)); cfg.blockDim = dim3(128);
     if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, sam_run_finish_kernel, R);
     if (e != cudaSuccess) { sam_set_cuda_error(e); return SAM_ERR_CUDA; }

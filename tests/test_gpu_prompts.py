@@ -120,7 +120,7 @@ def test_many_prompts_at_once(P, n):
 
 @pytest.mark.parametrize("B,per_step", [(1, True), (296, True), (297, True), (297, False), (8193, True)])
 def test_steps_in_one_launch(P, B, per_step):
-    """sam_run_steps over each kernel's range: ragged counts, steps without tokens, slots that are refused on the way,
+    """sam_run_steps up to and beyond 296 slots, where its kernels change: ragged counts, steps without tokens, slots that are refused on the way,
     rows of up to 47 tokens, with and without room for every step's outputs, with and without a static automaton."""
     import torch
     rng = np.random.default_rng(B)
@@ -442,6 +442,43 @@ def test_replayed_chunks_of_steps(P, B, K, most):
         assert np.array_equal(got[k], exp), (k, np.argwhere(got[k] != exp)[:3])
         assert np.array_equal(each[k], exp), k
     assert_dynamic_automata_equal(once, ob, range(0, B, 5), msl)
+
+
+@pytest.mark.parametrize("B", [1, 296, 297])
+@pytest.mark.parametrize("steps,L", [(2, 128), (16, 128), (17, 128), (32, 33), (33, 33), (64, 32), (65, 32), (64, 1)])
+def test_replays_of_few_steps_and_of_wide_ones(P, B, steps, L):
+    """Up to 296 slots the rows are finished by the slot's own block as long as there are few, else by a launch of their own, as for
+    more slots.  Steps of 16 and 17, 31 to 33 and 47 tokens side by side, where a chunk holds one step, two or a part, and slots
+    refused at one of them: a token outside the vocabulary among the first 32 or behind them, a count, the capacity."""
+    import torch
+    K, vocab = 47, 300
+    rng = np.random.default_rng(steps * 1000 + L + B)
+    corpus = rng.integers(0, vocab, size=4000, dtype=np.int32)
+    corpus[2000:3000] = corpus[:1000]
+    counts = rng.choice([0, 1, 16, 17, 31, 32, 33, 47], size=(steps, B)).astype(np.int32)
+    toks = rng.integers(0, vocab, size=(steps, B, K), dtype=np.int32)
+    for i in range(steps):                                  # every second step goes on along the corpus
+        if i % 2:
+            at = rng.integers(0, 3900, size=B)
+            toks[i] = corpus[at[:, None] + np.arange(K)]
+    msl = max(int(counts.sum()), 1) if B == 1 else K * steps - 1
+    if B > 10:
+        mid = steps // 2
+        counts[mid, :6] = (40, 40, 20, 33, K + 1, -1)
+        toks[mid, 0, 39] = vocab; toks[mid, 1, 31] = -3; toks[mid, 2, 19] = vocab; toks[mid, 3, 32] = -1
+        toks[:, 6] = 5; counts[:, 6] = 47                   # ... and slot 6 runs over the longest text there is
+    st = P.StaticSam.build(corpus, vocab)
+    ob = oracle.Batch(oracle.Sam(corpus), corpus, B, vocab, msl, 1, 2, 5)
+    ref = [ob.step(toks[i], counts[i], L, 8) for i in range(steps)]
+    assert B == 1 or ((ref[-1].status[:7] != 0).all() and (ref[-1].status[7:] == 0).any())
+    t, c = torch.from_numpy(toks).cuda(), torch.from_numpy(counts).cuda()
+    for per_step in (True, False):
+        batch = P.Batch(st, B, msl, max_draft_len=L, l_bias=1, min_match=2, vocab=vocab, stop_token=5)
+        got = batch.run_steps(t, c, L, per_step=per_step).cpu()
+        for k in KEYS:
+            exp = np.stack([getattr(r, k) for r in ref]) if per_step else getattr(ref[-1], k)
+            assert np.array_equal(got[k], exp), (per_step, k, np.argwhere(got[k] != exp)[:3])
+        assert_dynamic_automata_equal(batch, ob, [b for b in (0, 7, 100) if b < B and ref[-1].status[b] == 0], msl)
 
 
 DUMP = ("n_tokens", "n_states", "n_edges", "length", "link", "min_endpos", "deg")
