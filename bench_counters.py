@@ -1,10 +1,10 @@
 #!/usr/bin/env python
 """Operation counts of the step kernels on a workload, from the library built with -DSAM_COUNTERS.
 
-    python bench_counters.py --workload c5 [--warmup 8 --steps 512] [--batch N] [--corpus-tokens N] [--from-reset]
+    python bench_counters.py --workload c5 [--warmup 8 --steps 512] [--batch N] [--corpus-tokens N] [--from-reset] [--replay]
 
-Runs the workload's prompt prefill and decoding steps through `sam_step` with the counters attached and
-prints one JSON line: per counter the sum over all slots for the decoding steps [warmup, warmup + steps)
+Runs the workload's prompt prefill and decoding steps through `sam_step` (with --replay: the decoding steps through one
+`sam_run_steps`) with the counters attached and prints one JSON line: per counter the sum over all slots for the decoding steps [warmup, warmup + steps)
 (or, with --from-reset, for everything since the empty batch: prefill and all steps), and the means per
 sequence-step that `bench.py` turns into the dependent-access bound.  The counters build is a second
 compilation of the same sources; this script re-runs itself with SAMDRAFT_VARIANT=counters so that the
@@ -33,6 +33,7 @@ def parse_args(argv=None):
     ap.add_argument("--prompt-len", type=int, default=0)
     ap.add_argument("--gen-len", type=int, default=0)
     ap.add_argument("--from-reset", action="store_true", help="count the prefill and every decoding step")
+    ap.add_argument("--replay", action="store_true", help="the decoding steps in one sam_run_steps call")
     return ap.parse_args(argv)
 
 
@@ -64,18 +65,22 @@ def main():
     cnt = torch.zeros((B, sd.N_COUNTERS), dtype=torch.int64, device=dev)
     nt = torch.from_numpy(new_tokens[:hi]).to(dev)
     ct = torch.from_numpy(counts[:hi]).to(dev)
+    def run(a, b):
+        if args.replay and b > a:
+            batch.run_steps(nt[a:b], ct[a:b], L, per_step=False, out=out)
+        for i in range(a, a if args.replay else b):
+            batch.step(nt[i], ct[i], L, out)
+
     torch.cuda.synchronize()
     if args.from_reset:
         sd.sam_counters_attach(cnt, B)
     batch.step(torch.from_numpy(np.ascontiguousarray(seqs[:, :spec.prompt_len])).to(dev),
                torch.full((B,), spec.prompt_len, dtype=torch.int32, device=dev), L, out)
-    if lo > 0:
-        batch.run_steps(nt[:lo], ct[:lo], L, per_step=False, out=out)
+    run(0, lo)
     torch.cuda.synchronize()
     if not args.from_reset:
         sd.sam_counters_attach(cnt, B)
-    if hi > lo:
-        batch.run_steps(nt[lo:hi], ct[lo:hi], L, per_step=False, out=out)
+    run(lo, hi)
     torch.cuda.synchronize()
     sd.sam_counters_attach(None)
     ok = bool((out.status == 0).all().item())

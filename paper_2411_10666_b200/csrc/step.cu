@@ -54,10 +54,10 @@ namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-// counts of one chain of one slot in one step (registers; dropped by the compiler in the regular build)
+// counts of one chain of one slot in one step, or in all of a replay (registers; dropped by the compiler in the regular build)
 struct ChainCounts { uint32_t rounds, a, b, c, d; };
 
-__device__ __forceinline__ void flush_counts(int slot, int lane, bool is_static, const ChainCounts& k, int m) {
+__device__ __forceinline__ void flush_counts(int slot, int lane, bool is_static, const ChainCounts& k, int m, int steps) {
 #ifdef SAM_COUNTERS
     if (g_sam_counters && lane == 0 && slot < g_sam_counter_slots) {
         unsigned long long* o = g_sam_counters + (size_t)slot * SAM_N_COUNTERS;
@@ -66,7 +66,7 @@ __device__ __forceinline__ void flush_counts(int slot, int lane, bool is_static,
         } else {
             o[SAM_CNT_DYNAMIC_ROUNDS] += k.rounds; o[SAM_CNT_WALK_INSERTS] += k.a; o[SAM_CNT_CLONES] += k.b;
             o[SAM_CNT_COPIED_EDGES] += k.c; o[SAM_CNT_REDIRECTS] += k.d;
-            o[SAM_CNT_TOKENS] += (unsigned)m; o[SAM_CNT_SEQ_STEPS] += m > 0 ? 1u : 0u;
+            o[SAM_CNT_TOKENS] += (unsigned)m; o[SAM_CNT_SEQ_STEPS] += (unsigned)steps;
         }
     }
 #endif
@@ -873,7 +873,7 @@ __device__ __forceinline__ void static_chain(const StepArgs& A, int b, int lane,
     });
     l_out = l; s_out = s; sf_out = sf;
     if (l > 0 && !err) SAM_COUNT(kc.rounds, DRAFT && !follows ? 1 : 0);
-    flush_counts(b, lane, true, kc, m);
+    flush_counts(b, lane, true, kc, m, m > 0);
     if (DRAFT && l > 0 && !err) {
         if (follows) my_dl = dl2;
         else {
@@ -1015,7 +1015,7 @@ __device__ __forceinline__ void dyn_feed(DynChain& X, int32_t tok_first, const i
         if (!X.have) { const uint4* rs = rec_ptr(D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(D.kc.rounds, 1); }
         if (lane == 0) { reinterpret_cast<uint4*>(D.cb + CB_REC2)[0] = X.ra; reinterpret_cast<uint4*>(D.cb + CB_REC2)[1] = X.rb; }
     }
-    if (!D.err) flush_counts(D.seq, lane, false, D.kc, m);
+    if (!D.err) flush_counts(D.seq, lane, false, D.kc, m, m > 0);
 }
 
 // Called by one thread of a block after the block's outputs are written (and made known to that
@@ -2115,6 +2115,7 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
     if (lane == 0) { done[0] = X.ntok; done[1] = X.D.n_states; done[2] = X.last; done[3] = X.s2; done[4] = X.l2; done[5] = 0; done[6] = X.D.root_deg; }
     __syncwarp();
     int i = 0;
+    [[maybe_unused]] int n_fed = 0;                        // steps with tokens
     RunChunk C;
     if (fit) { C = run_plan(R, b, lane, 0, 0, X.ntok, m, sh_map); m = run_counts(R, b, lane, C.n_steps); }
     while (status == 0 && i < R.n_steps) {
@@ -2133,6 +2134,7 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
             emit.step = C.step; emit.own = C.own;
             emit.ends = __ballot_sync(FULL, C.own > 0);
             dyn_tokens(X, (uint32_t)C.tok, C.n_tok, sh_run, emit);
+            SAM_COUNT(n_fed, __popc(emit.ends));
             status = X.D.err;
             if (status != 0) break;
         }
@@ -2155,6 +2157,8 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
             cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end; cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = done[6];
         }
     } else if (X.ntok != ntok0) {
+        SAM_COUNT(X.D.kc.rounds, 1);                       // (the first tokens)
+        flush_counts(b, lane, false, X.D.kc, (int)(X.ntok - ntok0), n_fed);
         dyn_close(X);
         if (X.l2 > 0 && lane == 0) { reinterpret_cast<uint4*>(cb + CB_REC2)[0] = X.ra; reinterpret_cast<uint4*>(cb + CB_REC2)[1] = X.rb; }
     }
@@ -2204,7 +2208,7 @@ __device__ __forceinline__ int static_follow(const SamStaticView& S, uint32_t s,
 // One chunk: tk, n: its tokens; ends: the last tokens of its steps; T: the match, moved over the chunk (have: T's record is there; it
 // is on return, if T.l > 0).  res[k]: the result after token k, for the k in ends.  Returns for how many tokens the results hold: all n,
 // or, with err, as many as the match had taken when its links went on for too long.
-__device__ __forceinline__ int static_chunk(const SamStaticView& S, uint32_t tk, int n, unsigned ends, int lane, StaticSide& T, RunResult* res, int& err) {
+__device__ __forceinline__ int static_chunk(const SamStaticView& S, uint32_t tk, int n, unsigned ends, int lane, StaticSide& T, RunResult* res, int& err, ChainCounts& kc) {
     uint32_t re = SAM_NONE;
     if (lane < n) re = __ldg(S.root_row + tk);
     res[lane] = RunResult{0u, 0, 0};
@@ -2219,11 +2223,13 @@ __device__ __forceinline__ int static_chunk(const SamStaticView& S, uint32_t tk,
     uint4 a = T.ra, b = T.rb;
     if (chain) { cs = T.s; csf = T.sf; cl = T.l; pos = 0; have = true; }
     int guard = T.l + 2 * n + 4;                           // link moves of the chain
+    SAM_COUNT(kc.rounds, 1);
     for (;;) {
         const unsigned arrived = __ballot_sync(FULL, alive && pos == n);
         if (arrived && lane > __ffs(arrived) - 1) alive = false;          // an earlier suffix reaches the end
         bool go = alive && (pos < n || !have);
         if (!__any_sync(FULL, go)) break;
+        SAM_COUNT(kc.rounds, 1);
         const uint32_t t = __shfl_sync(FULL, tk, pos & 31);
         const bool want_bucket = go && pos < n && csf;
         uint32_t home = 0;
@@ -2249,6 +2255,7 @@ __device__ __forceinline__ int static_chunk(const SamStaticView& S, uint32_t tk,
         const bool may = go && (chain || cl >= 3) && (a.x == a.z ? tgt != SAM_NONE || csf : tgt != SAM_NONE && (apart == 1 || apart == 2));
         if (live && __shfl_sync(FULL, may, __ffs(live) - 1)) {
             const int c = __ffs(live) - 1, p0 = __shfl_sync(FULL, pos, c);
+            SAM_COUNT(kc.rounds, 1);
             uint32_t ref;
             RunResult out;
             const int r = static_follow(S, __shfl_sync(FULL, cs, c), shfl4(a, c), shfl4(b, c), __shfl_sync(FULL, cl, c),
@@ -2320,6 +2327,7 @@ __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, in
         }
     };
     int i = 0, err = 0;
+    [[maybe_unused]] ChainCounts kc = {2, 0, 0, 0, 0};       // two rounds already: the control words and counts, the first tokens
     RunChunk C = run_plan(R, b, lane, 0, 0, ntok, m, sh_map);
     m = run_counts(R, b, lane, C.n_steps);
     while (i < R.n_steps) {
@@ -2332,7 +2340,18 @@ __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, in
         }
         if (C.lead > 0 && lane == 0) write(i, C.lead, T.s, T.l, (int32_t)T.ra.z);
         if (C.n_tok > 0) {
-            const int held = static_chunk(A.S, (uint32_t)C.tok, C.n_tok, __ballot_sync(FULL, C.own > 0), lane, T, res, err);
+#ifdef SAM_COUNTERS
+            {                                              // the moves Algorithm 1 itself makes over these tokens
+                uint32_t ts = T.s, tsf = T.sf; int32_t tl = T.l;
+                const uint32_t rounds = kc.rounds;
+                for (int j = 0; j < C.n_tok && !err; j++) {
+                    const uint32_t t = (uint32_t)__shfl_sync(FULL, C.tok, j);
+                    static_transfer(A.S, ts, tsf, tl, t, __ldg(A.S.root_row + t), lane, err, false, T.ra, T.rb, kc);
+                }
+                kc.rounds = rounds; err = 0;
+            }
+#endif
+            const int held = static_chunk(A.S, (uint32_t)C.tok, C.n_tok, __ballot_sync(FULL, C.own > 0), lane, T, res, err, kc);
             __syncwarp();
             const bool mine = C.own > 0 && lane < held;
             if (mine) write(C.step, C.own, res[lane].s, res[lane].l, res[lane].e1);
@@ -2347,6 +2366,7 @@ __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, in
     if (err)
         for (int k = i + lane; k < R.n_steps; k += 32) if (R.keep || k + 1 == R.n_steps) step_out(A, R.keep ? k : 0).draft_len[b] = -err;
     static_close(cb, lane, ntok, T);
+    flush_counts(b, lane, true, kc, 0, 0);
 }
 
 // Blocks of one warp: the dynamic side of each slot, then, with a static automaton, the static side of each slot.
@@ -2764,15 +2784,9 @@ int sam_launch_run(const sam_batch* b, const int32_t* new_tokens, int32_t stride
     return SAM_OK;
 }
 
-// A launch per step where rows may hold prompts (the whole-text build has a kernel of its own), else one for all.  (The counters
-// are the step kernels', one step at a time.)
-bool sam_runs_in_one_launch(int32_t stride, int32_t n_steps) {
-#ifdef SAM_COUNTERS
-    return false;
-#else
-    return n_steps > 1 && stride < SAM_PREFILL_MIN;
-#endif
-}
+// The launches of sam_step for each step where rows may hold prompts (the whole-text build has a kernel of its own), else one or two
+// for all.
+bool sam_runs_in_one_launch(int32_t stride, int32_t n_steps) { return n_steps > 1 && stride < SAM_PREFILL_MIN; }
 
 extern "C" int sam_counters_available(void) {
 #ifdef SAM_COUNTERS

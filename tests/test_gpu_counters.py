@@ -46,3 +46,15 @@ def test_counts_equal_the_oracles(name, corpus, batch, pl, gl):
     # the rounds of dependent reads are the kernels' own figure: at least the control words and the draft
     c = got["counters"]
     assert c["static_rounds"] >= c["seq_steps"] and c["dynamic_rounds"] >= 2 * c["seq_steps"]
+
+
+@pytest.mark.parametrize("name,corpus,batch,pl,gl", [("c2", 300_000, 24, 300, 500), ("c5", 200_000, 1700, 60, 90)])
+def test_replays_count_the_same_operations(name, corpus, batch, pl, gl):
+    """The replays' kernels, both of them: the algorithms' operations are the single steps', in fewer rounds."""
+    args = ["--workload", name, "--corpus-tokens", str(corpus), "--batch", str(batch), "--prompt-len", str(pl), "--gen-len", str(gl)]
+    steps, replay = _device_counts(args), _device_counts(args + ["--replay"])
+    assert replay["status_all_ok"]
+    for k in SAME:
+        assert replay["counters"][k] == steps["counters"][k], k
+    for k in ("static_rounds", "dynamic_rounds"):
+        assert 0 < replay["counters"][k] < steps["counters"][k], k
