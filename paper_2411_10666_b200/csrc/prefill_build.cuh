@@ -295,10 +295,7 @@ __device__ int pb_group(const PbArrays& a, PbShared& sh, unsigned char* smem, in
     pb_sync(nt);
     for (int p = tid; p - lane < n; p += nt) {             // (whole warps) the first position of each group sees to its place
         const bool first = p < n && a.B[p] == 0;
-        const int c = first ? (int)cnt[at[p]] : 0;
-        int s = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
+        const int c = first ? (int)cnt[at[p]] : 0, s = sum_upto(c, lane);
         const unsigned firsts = __ballot_sync(0xFFFFFFFFu, first);
         int base = 0;
         if (lane == 31 && firsts) { base = atomicAdd(&sh.placed, s); atomicAdd(&sh.groups[0], __popc(firsts)); }
@@ -433,9 +430,7 @@ __device__ int pb_double(const PbArrays& a, PbShared& sh, uint16_t* A, uint16_t*
             int run = 0;
             for (int c = 0; c < W; c += 32) {
                 const int v = c + lane < W ? __popc(bits[r * W + c + lane]) : 0;
-                int s = v;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
+                const int s = sum_upto(v, lane);
                 if (c + lane < W) before[r * W + c + lane] = (uint16_t)(run + s - v);
                 run += __shfl_sync(0xFFFFFFFFu, s, 31);
             }
@@ -588,9 +583,7 @@ __device__ void pb_build(const SamBatchView& W, int b, uint32_t* cb, int n, unsi
         int run = 0;
         for (int base = 0; base < chunks; base += 32) {
             const int v = base + lane < chunks ? sh.chunk[base + lane] : 0;
-            int s = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xFFFFFFFFu, s, o); if (lane >= o) s += t; }
+            const int s = sum_upto(v, lane);
             if (base + lane < chunks) sh.chunk[base + lane] = (int16_t)(run + s - v);
             run += __shfl_sync(0xFFFFFFFFu, s, 31);
         }

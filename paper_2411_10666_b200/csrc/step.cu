@@ -54,6 +54,13 @@ namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
+// The sum of v over a warp's lanes up to this one.
+__device__ __forceinline__ int sum_upto(int v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, v, o); if (lane >= o) v += t; }
+    return v;
+}
+
 // counts of one chain of one slot in one step, or in all of a replay (registers; dropped by the compiler in the regular build)
 struct ChainCounts { uint32_t rounds, a, b, c, d; };
 
@@ -2017,9 +2024,7 @@ __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, 
         if (lane < m0) C.tok = A.new_tokens[((size_t)i * A.W.batch + b) * A.stride + lane];
         return C;
     }
-    int upto = m;                                          // tokens up to this step's last
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(FULL, upto, o); if (lane >= o) upto += t; }
+    const int upto = sum_upto(m, lane);                    // tokens up to this step's last
     const bool room = (int64_t)ntok + upto <= A.W.max_seq_len;
     const unsigned no = ~__ballot_sync(FULL, lane < left && counted && room && upto <= 32);
     const int n = no ? __ffs(no) - 1 : 32;
