@@ -632,7 +632,7 @@ __device__ __forceinline__ int dyn_fresh_run(Dyn& D, uint32_t tk, int j, int cnt
     if (bucket_peers & run) D.pr_state = 0;                   // those buckets changed
     __syncwarp();
     SAM_COUNT(D.kc.a, r + n_new - (last == 0 ? 1 : 0));        // per token: the previous state's transition (none from the root) and the root's
-    if (emit.ends >> j & (FULL >> (32 - r))) emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1, D.root_deg + (uint32_t)idx + 1);
+    emit(is_new, D.lane, 0u, 0u, 0u, plen + 1, c, c + 1);
     if (F::seen && r > n_new) { s2 = __shfl_sync(FULL, D.pr_tgt, j + n_new) & SAM_IDMASK; l2 = 1; }
     D.n_states = c0 + r; D.root_deg += n_new;
     last = c0 + r - 1; ntok += r;
@@ -803,7 +803,7 @@ __device__ __forceinline__ int dyn_repeat_run(Dyn& D, uint32_t tk, int j, int cn
         SAM_COUNT(D.kc.c, copied);
     }
 
-    if (emit.ends >> j & (FULL >> (32 - r))) emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1, D.root_deg);
+    emit(mine, (j + lane) & 31, clk, l0 + 1 + (uint32_t)lane, qa.z, ntok + (uint32_t)lane + 1, ck, clk + 1);
     const int lr = r - 1;                                      // the last clone is the new match state
     pa = make_uint4(l0 + (uint32_t)r, __shfl_sync(FULL, qa.y, lr), __shfl_sync(FULL, qa.z, lr), __shfl_sync(FULL, qa.w, lr));
     pb = make_uint4(__shfl_sync(FULL, nb.x, lr), __shfl_sync(FULL, nb.y, lr), __shfl_sync(FULL, nb.z, lr), __shfl_sync(FULL, nb.w, lr));
@@ -946,19 +946,18 @@ __device__ __forceinline__ void dyn_open(const SamBatchView& W, int b, int lane,
 
 // Expand (fused with the dynamic matcher's Transfer) for each of up to 32 tokens, one in each lane.  emit is called by the whole
 // warp whenever tokens are done, with what holds after them: (whether this lane has one, the lane that held its token, s2, l2,
-// first end position of s2, text length, state of the whole text, number of states, transitions of the root); ends: the tokens for
-// which it is wanted.
+// first end position of s2, text length, state of the whole text, number of states); ends: the tokens for which it is wanted.
 // seen: runs of new tokens take the known one behind them (dyn_fresh_run).  call, chunks: ensure_recs.
 template <bool SEEN, bool CALL>
 struct NoEmit {
     static constexpr bool chunks = false, seen = SEEN, call = CALL;
     static constexpr unsigned ends = 0;
-    __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
+    __device__ __forceinline__ void operator()(bool, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t) const {}
 };
 template <class F>
 __device__ __forceinline__ void dyn_emit(DynChain& X, int j, F& emit) {    // after token j
     if (X.l2 > 0 && !X.have) { const uint4* rs = rec_ptr(X.D, X.s2); X.ra = rs[0]; X.rb = rs[1]; X.have = true; SAM_COUNT(X.D.kc.rounds, 1); }
-    emit(X.D.lane == j, X.D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, X.D.n_states, X.D.root_deg);
+    emit(X.D.lane == j, X.D.lane, X.s2, X.l2, X.ra.z, X.ntok, X.last, X.D.n_states);
 }
 template <class F>
 __device__ __forceinline__ void dyn_tokens(DynChain& X, uint32_t tk, int cnt, uint32_t (*sh_run)[12], F& emit) {
@@ -2009,8 +2008,12 @@ struct RunChunk {
 __device__ __forceinline__ int32_t run_counts(const RunArgs& R, int b, int lane, int i) {
     return i + lane < R.n_steps ? R.A.counts[(size_t)(i + lane) * R.A.W.batch + b] : 0;
 }
+// WIDE: sam_run_block_kernel's, for few slots, whose steps may be wide: a step that fills a chunk by itself is planned without the scan, and
+// one of more than 32 tokens is checked when it begins instead of here, where that waits for the tokens (64 slots, up to 47 tokens a
+// step, 5 to 10 % faster).  For many slots it costs registers and gives nothing (4096 slots x 192 steps 1180 -> 1200 us).
 // The chunk that begins with step i, of which `taken` tokens are done, whose slot had ntok tokens before it; m: lane k holds the
 // count of step i + k.
+template <bool WIDE>
 __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, int i, int taken, uint32_t ntok, int m, int32_t* sh_map) {
     const StepArgs& A = R.A;
     RunChunk C;
@@ -2018,8 +2021,8 @@ __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, 
     const int left = R.n_steps - i;
     const bool counted = m >= 0 && m <= A.stride;
     if (!counted) m = 0;
-    const int m0 = __shfl_sync(FULL, m, 0), m1 = __shfl_sync(FULL, m, 1);
-    if (m0 >= 1 && m0 <= 32 && m0 + m1 > 32 && (int64_t)ntok + m0 <= A.W.max_seq_len) {          // a wide step, alone
+    const int m0 = __shfl_sync(FULL, m, 0), m1 = WIDE ? __shfl_sync(FULL, m, 1) : 0;
+    if (WIDE && m0 >= 1 && m0 <= 32 && m0 + m1 > 32 && (int64_t)ntok + m0 <= A.W.max_seq_len) {          // a wide step, alone
         C.n_steps = 1; C.n_tok = m0; C.step = i; C.own = lane == m0 - 1 ? 1 : 0; C.lead = 0; C.starts = 1;
         if (lane < m0) C.tok = A.new_tokens[((size_t)i * A.W.batch + b) * A.stride + lane];
         return C;
@@ -2031,13 +2034,18 @@ __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, 
     C.n_steps = n;
     C.n_tok = n > 0 ? __shfl_sync(FULL, upto, n - 1) : 0;
     C.refuse = n < 32 ? __shfl_sync(FULL, lane >= left ? 0 : !counted ? SAM_SEQ_BAD_COUNT : !room ? SAM_SEQ_CAPACITY : 0, n & 31) : 0;
-    if (n == 0 && left > 0 && C.refuse == 0) {             // a step of more than 32 tokens, checked as a whole when it begins
+    if (n == 0 && left > 0 && C.refuse == 0) {             // a step of more than 32 tokens, checked as a whole
         const int32_t* row = A.new_tokens + ((size_t)i * A.W.batch + b) * A.stride;
         C.step = i; C.own = 0; C.lead = 0; C.starts = 1;
+        if (!WIDE && taken == 0) {
+            const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
+            const int32_t t0 = row[lane], t1 = lane + 32 < m0 ? row[lane + 32] : 0;
+            if (__any_sync(FULL, t0 < 0 || t0 >= vocab || t1 < 0 || t1 >= vocab)) { C.refuse = SAM_SEQ_BAD_TOKEN; C.n_tok = 0; return C; }
+        }
         C.n_tok = min(32, m0 - taken);
         if (lane < C.n_tok) C.tok = row[taken + lane];
         if (taken + C.n_tok == m0) { C.n_steps = 1; C.own = lane == C.n_tok - 1 ? 1 : 0; }
-        else { C.taken = C.n_tok; if (lane + 32 < m0) C.tail = row[lane + 32]; }
+        else { C.taken = C.n_tok; if (WIDE && lane + 32 < m0) C.tail = row[lane + 32]; }
         return C;
     }
     const bool some = lane < n && m > 0;
@@ -2060,8 +2068,9 @@ __device__ __forceinline__ RunChunk run_plan(const RunArgs& R, int b, int lane, 
 }
 
 // Its tokens have come: where one is outside the vocabulary the chunk, which begins with step i, ends before that step.
+template <bool WIDE>
 __device__ __forceinline__ void run_cut(RunChunk& C, int lane, int i, int vocab) {
-    const unsigned wrong = __ballot_sync(FULL, (lane < C.n_tok && (C.tok < 0 || C.tok >= vocab)) || C.tail < 0 || C.tail >= vocab);
+    const unsigned wrong = __ballot_sync(FULL, (lane < C.n_tok && (C.tok < 0 || C.tok >= vocab)) || (WIDE && (C.tail < 0 || C.tail >= vocab)));
     if (!wrong) return;
     C.taken = 0;
     const int t = __ffs(wrong) - 1;
@@ -2078,7 +2087,7 @@ struct RunEmit {
     int b, lane;
     int32_t step, own;           // of the chunk (this lane's)
     unsigned ends;
-    uint32_t* done;              // text length, states, state of the whole text, s2, l2; the step after it; the root's transitions
+    uint32_t* done;              // text length, states, state of the whole text, s2, l2; the step after it
     __device__ __forceinline__ void write(int first, int n, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok) const {
         const StepArgs& A = R.A;
         for (int i = first; i < first + n; i++) {
@@ -2089,23 +2098,22 @@ struct RunEmit {
             if (o.state) o.state[2 * b + 1] = (int32_t)s2;
         }
     }
-    __device__ __forceinline__ void operator()(bool on, int from, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok, uint32_t last, uint32_t n_states, uint32_t root_deg) {
+    __device__ __forceinline__ void operator()(bool on, int from, uint32_t s2, uint32_t l2, uint32_t e2, uint32_t ntok, uint32_t last, uint32_t n_states) {
         const int st = __shfl_sync(FULL, step, from);
         int n = __shfl_sync(FULL, own, from);
         if (!on) n = 0;
         const unsigned ending = __ballot_sync(FULL, n > 0);
         if (!ending) return;
         if (n > 0) write(st, n, s2, l2, e2, ntok);
-        if (lane == 31 - __clz(ending)) {
-            done[0] = ntok; done[1] = n_states; done[2] = last; done[3] = s2; done[4] = l2; done[5] = (uint32_t)(st + n); done[6] = root_deg;
-        }
+        if (lane == 31 - __clz(ending)) { done[0] = ntok; done[1] = n_states; done[2] = last; done[3] = s2; done[4] = l2; done[5] = (uint32_t)(st + n); }
         __syncwarp();
     }
 };
 
+template <bool WIDE>
 __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, uint32_t (*sh_run)[12], int32_t* sh_map) {
     const StepArgs& A = R.A;
-    __shared__ uint32_t done[7];
+    __shared__ uint32_t done[6];
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
     const uint32_t cw = cb[lane], cw2 = cb[32 + lane];
     int m = run_counts(R, b, lane, 0);
@@ -2117,18 +2125,18 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
     const uint32_t ntok0 = X.ntok;
     RunEmit emit{R, b, lane, 0, 0, 0u, done};
     const int vocab = A.has_static ? A.S.vocab : A.W.vocab;
-    if (lane == 0) { done[0] = X.ntok; done[1] = X.D.n_states; done[2] = X.last; done[3] = X.s2; done[4] = X.l2; done[5] = 0; done[6] = X.D.root_deg; }
+    if (lane == 0) { done[0] = X.ntok; done[1] = X.D.n_states; done[2] = X.last; done[3] = X.s2; done[4] = X.l2; done[5] = 0; }
     __syncwarp();
     int i = 0;
     [[maybe_unused]] int n_fed = 0;                        // steps with tokens
     RunChunk C;
-    if (fit) { C = run_plan(R, b, lane, 0, 0, X.ntok, m, sh_map); m = run_counts(R, b, lane, C.n_steps); }
+    if (fit) { C = run_plan<WIDE>(R, b, lane, 0, 0, X.ntok, m, sh_map); m = run_counts(R, b, lane, C.n_steps); }
     while (status == 0 && i < R.n_steps) {
-        run_cut(C, lane, i, vocab);
+        run_cut<WIDE>(C, lane, i, vocab);
         const int next = i + C.n_steps;
         RunChunk N = C;
         if (C.refuse == 0 && next < R.n_steps) {
-            N = run_plan(R, b, lane, next, C.taken, X.ntok + (uint32_t)(C.n_tok - C.taken), m, sh_map);
+            N = run_plan<WIDE>(R, b, lane, next, C.taken, X.ntok + (uint32_t)(C.n_tok - C.taken), m, sh_map);
             if (N.n_steps > 0) m = run_counts(R, b, lane, next + N.n_steps);
         }
         if (C.lead > 0) {
@@ -2153,13 +2161,20 @@ __device__ __forceinline__ void run_dynamic(const RunArgs& R, int b, int lane, u
         // The slot is left as the last step that was done left it, but for what the tokens after it have made.  The first of them
         // completes the newest state's record; where the pool had no state for it, that is done here, without a transition.
         const uint32_t newest = done[2];
+        __syncwarp();
+        uint32_t root_deg = X.D.root_deg;                  // without the transitions that tokens after that step have given it
+        for (uint32_t at = done[0]; at < X.ntok; at++) {
+            bool seen = false;
+            for (uint32_t k = lane; k < at; k += 32) seen |= X.D.text[k] == X.D.text[at];
+            if (!__any_sync(FULL, seen)) root_deg--;
+        }
         uint4* rl = rec_ptr(X.D, newest);
         const uint4* rs = rec_ptr(X.D, done[3]);
         if (lane == 0) {
             if (newest != 0 && X.D.n_states == done[1]) { rl[0] = make_uint4(done[0], done[3], done[0], 0); rl[1] = make_uint4(0, 0, 0, 0); }
             if (done[4] > 0) { reinterpret_cast<uint4*>(cb + CB_REC2)[0] = rs[0]; reinterpret_cast<uint4*>(cb + CB_REC2)[1] = rs[1]; }
             cb[CB_NTOK] = done[0]; cb[CB_NSTATES] = done[1]; cb[CB_LAST] = newest; cb[CB_S2] = done[3]; cb[CB_L2] = done[4];
-            cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end; cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = done[6];
+            cb[CB_BLK_CUR] = X.D.blk_cur; cb[CB_BLK_END] = X.D.blk_end; cb[CB_NRECSLABS] = X.D.n_rec_slabs; cb[CB_ROOTDEG] = root_deg;
         }
     } else if (X.ntok != ntok0) {
         SAM_COUNT(X.D.kc.rounds, 1);                       // (the first tokens)
@@ -2314,6 +2329,7 @@ __device__ __forceinline__ int static_chunk(const SamStaticView& S, uint32_t tk,
     return n;
 }
 
+template <bool WIDE>
 __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, int32_t* sh_map, RunResult* res) {
     const StepArgs& A = R.A;
     uint32_t* cb = A.W.ctrl + (size_t)b * SAM_CTRL_WORDS;
@@ -2333,14 +2349,14 @@ __device__ __forceinline__ void run_static(const RunArgs& R, int b, int lane, in
     };
     int i = 0, err = 0;
     [[maybe_unused]] ChainCounts kc = {2, 0, 0, 0, 0};       // two rounds already: the control words and counts, the first tokens
-    RunChunk C = run_plan(R, b, lane, 0, 0, ntok, m, sh_map);
+    RunChunk C = run_plan<WIDE>(R, b, lane, 0, 0, ntok, m, sh_map);
     m = run_counts(R, b, lane, C.n_steps);
     while (i < R.n_steps) {
-        run_cut(C, lane, i, A.S.vocab);
+        run_cut<WIDE>(C, lane, i, A.S.vocab);
         const int next = i + C.n_steps;
         RunChunk N = C;
         if (C.refuse == 0 && next < R.n_steps) {
-            N = run_plan(R, b, lane, next, C.taken, ntok + (uint32_t)(C.n_tok - C.taken), m, sh_map);
+            N = run_plan<WIDE>(R, b, lane, next, C.taken, ntok + (uint32_t)(C.n_tok - C.taken), m, sh_map);
             if (N.n_steps > 0) m = run_counts(R, b, lane, next + N.n_steps);
         }
         if (C.lead > 0 && lane == 0) write(i, C.lead, T.s, T.l, (int32_t)T.ra.z);
@@ -2381,8 +2397,8 @@ __global__ void __launch_bounds__(32, 16) sam_run_split_kernel(const __grid_cons
     __shared__ __align__(16) uint32_t sh_run[32][12];
     __shared__ int32_t sh_map[32];
     const int lane = threadIdx.x, B = R.A.W.batch;
-    if ((int)blockIdx.x < B) run_dynamic(R, (int)blockIdx.x, lane, sh_run, sh_map);
-    else run_static(R, (int)blockIdx.x - B, lane, sh_map, reinterpret_cast<RunResult*>(&sh_run[0][0]));
+    if ((int)blockIdx.x < B) run_dynamic<false>(R, (int)blockIdx.x, lane, sh_run, sh_map);
+    else run_static<false>(R, (int)blockIdx.x - B, lane, sh_map, reinterpret_cast<RunResult*>(&sh_run[0][0]));
     // (the slot's status is the finish kernel's to write: its other side may begin after this)
 }
 
@@ -2472,8 +2488,8 @@ __global__ void __launch_bounds__(64, 8) sam_run_block_kernel(const __grid_const
     const int lane = threadIdx.x & 31, side = threadIdx.x >> 5, b = blockIdx.x, B = R.A.W.batch;
     if (lane < R.n_steps)                                  // (which tokens are read first depends on the counts)
         asm volatile("prefetch.global.L1 [%0];" ::"l"(R.A.new_tokens + ((size_t)lane * B + b) * R.A.stride));
-    if (side == 0) run_dynamic(R, b, lane, sh_run, sh_map[0]);
-    else if (R.A.has_static) run_static(R, b, lane, sh_map[1], res);
+    if (side == 0) run_dynamic<true>(R, b, lane, sh_run, sh_map[0]);
+    else if (R.A.has_static) run_static<true>(R, b, lane, sh_map[1], res);
     if (!R.finish) return;
     __syncthreads();
     const int n = R.keep ? R.n_steps : 1;
