@@ -120,7 +120,7 @@ def test_many_prompts_at_once(P, n):
 
 @pytest.mark.parametrize("B,per_step", [(1, True), (296, True), (297, True), (297, False), (8193, True)])
 def test_steps_in_one_launch(P, B, per_step):
-    """sam_run_steps up to and beyond 296 slots, where its kernels change: ragged counts, steps without tokens, slots that are refused on the way,
+    """sam_run_steps over each kernel's range: ragged counts, steps without tokens, slots that are refused on the way,
     rows of up to 47 tokens, with and without room for every step's outputs, with and without a static automaton."""
     import torch
     rng = np.random.default_rng(B)
