@@ -18,8 +18,9 @@
 //     along the suffix links of w without that token, down to length k.
 // Nothing here depends on a guess: each of these statements is the definition of the automaton of the text.
 //
-// What bounds it: for short texts the chain of some 40 barriers (1 x 300 tokens 17 us), for long ones one SM's issue slots (8191 tokens:
-// 64 % of them, 3900 instructions of a warp for 32 tokens, a third of the time in the sort; everything but the outputs stays
+// What bounds it: for short texts the chain of some 40 barriers (1 x 300 tokens 17 us), for long ones one SM's issue slots (8191 tokens, 206 us
+// under ncu in the version that was captured, 173 us now: 64 % of them, 3900 instructions of a warp for 32 tokens, a third of the time in
+// the sort; everything but the outputs stays
 // in shared memory, 28 bytes per token), for many the same (4096 x 1024 tokens: 9.5 tokens a ns), and a step waits for its slowest
 // build: 64 x 1024 tokens 34 to 51 us by text, mean 25.
 #pragma once

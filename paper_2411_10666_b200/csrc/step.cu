@@ -1973,7 +1973,7 @@ __global__ void __launch_bounds__(32) sam_step_split_kernel(const __grid_constan
 // Both sides leave each step's result in the step's own outputs, and sam_run_finish_kernel, which no chain waits for, chooses the
 // sources and reads the drafts: 32 rows a warp, eight rows' reads under way together.
 // us a step, step after step on each side (static sides on a few lanes, or three warps a slot up to 296 slots) -> so: 200 slots
-// 2.35 -> 1.3, 1000 slots 6.1 -> 2.2, 4096 slots 7.1 -> 3.6, 16384 slots 20.1 -> 11.8.
+// 2.35 -> 1.3, 1000 slots 6.1 -> 2.2, 4096 slots 7.1 -> 4.0, 16384 slots 20.1 -> 11.8.
 // Bound by the dynamic sides' rounds of reads and how many warps fit (16 an SM with 128 registers, nothing spilled; 20 with 96:
 // 4 % slower at 4096 slots).
 // What the two sides leave: match_len, state and status as they will be; the static side's first end position (or minus its
